@@ -24,9 +24,9 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
                           cudaStream_t stream, std::string& err);
 
 int piko_backward_launch(int W, int H, int mode, int unclamped, int T, int V, const int* tris, const int4* vtx,
-                         const float* color, const float* normal, const float* light, const float* invw,
-                         const float* pos, const float* mvp, const unsigned long long* key,
-                         const float* dl_drgba, float* dcolor, float* dnormal, float* dlight, int num_sms,
+                         const float* vdot, const float* color, const float* normal, const float* light,
+                         const float* invw, const float* pos, const float* mvp, const unsigned long long* key,
+                         const float* dl_drgba, float4* acc, float* dcolor, float* dnormal, float* dlight, int num_sms,
                          cudaStream_t s);
 
 struct piko_raster {
@@ -55,6 +55,9 @@ struct piko_raster {
   long long dcap = 0;
   float* invw = nullptr;  // 1 / clip w per vertex, with perspective-correct attributes
   long long icap = 0;
+  float4* gacc = nullptr;  // gradient sums per vertex, zero between calls
+  long long gcap = 0;
+  bool gacc_dirty = false;  // a failed backward launch may have left sums behind
   BinRect* rect = nullptr;
   long long tcap = 0;
   unsigned* bin_count = nullptr;  // 2 * nbins, zero between frames
@@ -137,6 +140,18 @@ int grow(piko_raster* h, T** ptr, long long* cap, long long need, const char* wh
   return PIKO_OK;
 }
 
+// The gradient accumulators, zero between calls.  Grown with the vertex
+// buffer (forward and reserve too), so that a backward call recorded into a
+// graph after a forward of the same scene allocates nothing.
+int grow_gacc(piko_raster* h, long long need) {
+  if (need <= h->gcap) return PIKO_OK;
+  const int r = grow(h, &h->gacc, &h->gcap, need, "gradient sums");
+  if (r != PIKO_OK) return r;
+  cudaError_t e = cudaMemset(h->gacc, 0, (size_t)h->gcap * sizeof(float4));
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  return e == cudaSuccess ? PIKO_OK : cuda_fail(h, e, "gradient sums");
+}
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace
@@ -190,6 +205,7 @@ void piko_raster_destroy(piko_raster* h) {
   cudaFree(h->vtx);
   cudaFree(h->vdot);
   cudaFree(h->invw);
+  cudaFree(h->gacc);
   cudaFree(h->rect);
   cudaFree(h->bin_count);
   cudaFree(h->bin_off);
@@ -295,6 +311,7 @@ int piko_raster_reserve(piko_raster* h, int64_t max_vertices, int64_t max_triang
   int r;
   if ((r = grow(h, &h->vtx, &h->vcap, max_vertices, "vertex buffer")) != PIKO_OK) return r;
   if ((r = grow(h, &h->vdot, &h->dcap, max_vertices, "vertex light terms")) != PIKO_OK) return r;
+  if ((r = grow_gacc(h, max_vertices)) != PIKO_OK) return r;
   // 1/w too, so that turning perspective-correct attributes on later needs no allocation
   if ((r = grow(h, &h->invw, &h->icap, max_vertices, "vertex 1/w")) != PIKO_OK) return r;
   if ((r = grow(h, &h->rect, &h->tcap, max_triangles, "bin rectangles")) != PIKO_OK) return r;
@@ -466,7 +483,7 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   h->last_stream = st;
   const int V = s->num_vertices, T = s->num_triangles;
-  if ((r = grow(h, &h->vtx, &h->vcap, V, "vertex buffer")) != PIKO_OK) return r;
+  if ((r = grow(h, &h->vtx, &h->vcap, V, "vertex buffer")) != PIKO_OK || (r = grow_gacc(h, V)) != PIKO_OK) return r;
   const bool lambert = s->shade_mode == PIKO_SHADE_LAMBERT;
   if (lambert && (r = grow(h, &h->vdot, &h->dcap, V, "vertex light terms")) != PIKO_OK) return r;
   if (h->perspective && (r = grow(h, &h->invw, &h->icap, V, "vertex 1/w")) != PIKO_OK) return r;
@@ -719,17 +736,27 @@ int piko_raster_backward(piko_raster* h, const piko_scene* s, const piko_framebu
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   h->last_stream = st;
   if ((r = grow(h, &h->vtx, &h->vcap, s->num_vertices, "vertex buffer")) != PIKO_OK) return r;
+  if ((r = grow_gacc(h, s->num_vertices)) != PIKO_OK) return r;
+  const bool lambert = s->shade_mode == PIKO_SHADE_LAMBERT;
+  if (lambert && (r = grow(h, &h->vdot, &h->dcap, s->num_vertices, "vertex light terms")) != PIKO_OK) return r;
   if (h->perspective && (r = grow(h, &h->invw, &h->icap, s->num_vertices, "vertex 1/w")) != PIKO_OK) return r;
   float* invw = h->perspective ? h->invw : nullptr;
+  if (h->gacc_dirty) {
+    const cudaError_t e = cudaMemsetAsync(h->gacc, 0, (size_t)h->gcap * sizeof(float4), st);
+    if (e != cudaSuccess) return cuda_fail(h, e, "gradient sums");
+    h->gacc_dirty = false;
+  }
   // the vertex stage runs again so that backward does not depend on which
   // scene the handle rasterized last
-  launch_vertex(h->W, h->H, s->num_vertices, s->pos, s->mvp, h->vtx, nullptr, nullptr, nullptr, invw, h->num_sms,
-                st);
+  launch_vertex(h->W, h->H, s->num_vertices, s->pos, s->mvp, h->vtx, lambert ? s->normal : nullptr, s->light_dir,
+                lambert ? h->vdot : nullptr, invw, h->num_sms, st);
   if (piko_backward_launch(h->W, h->H, s->shade_mode, h->unclamped, s->num_triangles, s->num_vertices, s->tris,
-                           h->vtx, s->color, s->normal, s->light_dir, invw, h->clip ? s->pos : nullptr, s->mvp,
-                           reinterpret_cast<const unsigned long long*>(fwd->key), dl_drgba, dl_dcolor,
-                           dl_dnormal, dl_dlight, h->num_sms, st) != 0)
+                           h->vtx, h->vdot, s->color, s->normal, s->light_dir, invw, h->clip ? s->pos : nullptr,
+                           s->mvp, reinterpret_cast<const unsigned long long*>(fwd->key), dl_drgba, h->gacc, dl_dcolor,
+                           dl_dnormal, dl_dlight, h->num_sms, st) != 0) {
+    h->gacc_dirty = true;
     return cuda_fail(h, cudaGetLastError(), "backward launch");
+  }
   return PIKO_OK;
 }
 

@@ -40,9 +40,7 @@ struct BatchScene {
   uint2* galb_out;
   // backward
   const float4* dl;
-  float* dcolor;
-  float* dnormal;
-  float* dlight;
+  float4* acc;  // the gradient sums of the scene's vertices (NULL: no gradients wanted)
 };
 
 struct BatchSync {
@@ -468,6 +466,10 @@ struct BatchBwdParams {
   int total_btiles;
   const int4* vtx;
   const float* invw;  // as in BatchParams
+  // accumulators (GradAcc) of the finishing pass and the prefix of their chunks
+  int ngroups, total_chunks;
+  const GradAcc* groups;
+  const int* chunk_prefix;
 };
 
 // Warp form: each warp takes whole tiles (grid-stride over the batch's
@@ -492,7 +494,7 @@ __global__ void __launch_bounds__(BWD_THREADS, PIKO_BWD_MINB) k_batch_backward(B
   for (int i = blockIdx.x * BATCH_BWD_WARPS + warp; i < b.total_btiles; i += nwarps) {
     const int s = find_scene(b.btile_prefix, b.n, i);
     const BatchScene& d = b.sc[s];
-    if (d.dl == nullptr || d.mode == PIKO_SHADE_GBUFFER) continue;  // the same for the whole warp
+    if (d.acc == nullptr) continue;  // the same for the whole warp
     __syncwarp();  // the previous tile's reads of c are done
     if (lane == 0) {
       c.W = d.g.W; c.H = d.g.H; c.mode = d.mode; c.unclamped = d.unclamped; c.T = d.T; c.V = d.V;
@@ -500,7 +502,7 @@ __global__ void __launch_bounds__(BWD_THREADS, PIKO_BWD_MINB) k_batch_backward(B
       c.invw = b.invw ? b.invw + d.vtx_base : nullptr;
       c.pos = nullptr;  // batches do not clip
       c.mvp = nullptr;
-      c.key = d.key_out; c.dl = d.dl; c.dcolor = d.dcolor; c.dnormal = d.dnormal; c.dlight = d.dlight;
+      c.key = d.key_out; c.dl = d.dl; c.acc = d.acc;
     }
     __syncwarp();
     float L0 = 0.f, L1 = 0.f, L2 = 0.f;
@@ -515,6 +517,16 @@ __global__ void __launch_bounds__(BWD_THREADS, PIKO_BWD_MINB) k_batch_backward(B
   }
 }
 constexpr size_t BATCH_BWD_SMEM = sizeof(BatchBwdSmem);
+
+// Sums of all vertices into the gradient arrays, a chunk of one group per CTA step.
+__global__ void __launch_bounds__(GRAD_CHUNK) k_batch_finish(BatchBwdParams b) {
+  __shared__ GradFinishSmem sm;
+  pdl_wait();  // the accumulators
+  for (int i = blockIdx.x; i < b.total_chunks; i += gridDim.x) {
+    const int g = find_scene(b.chunk_prefix, b.ngroups, i);
+    grad_finish_chunk(b.groups[g], i - __ldg(b.chunk_prefix + g), sm);
+  }
+}
 
 }  // namespace piko
 
@@ -554,11 +566,16 @@ struct BatchState {
   long long bcap = 0;  // bins
   unsigned* bin_tris = nullptr;
   long long ecap = 0;
+  float4* gacc = nullptr;  // gradient sums, zero between calls
+  long long gcap = 0;
+  bool gacc_dirty = false;  // a failed backward launch may have left sums behind
   BatchSync* sync = nullptr;
   unsigned epoch = 0;
   // host staging (pinned) and the last layout
   void* staging = nullptr;
   size_t staging_cap = 0;
+  size_t desc_bytes = 0;   // of the last layout: scenes, 6 prefix arrays, gradient groups and their prefix
+  size_t group_off = 0;    // where the gradient groups start
   cudaEvent_t uploaded = nullptr;
   BatchParams params;
   std::vector<BatchScene> host_desc;  // the uploaded descriptors
@@ -587,7 +604,7 @@ int grow_dev(T** p, long long* cap, long long need, bool zero, std::string& err)
     err = "cudaMalloc of batch scratch failed";
     return PIKO_ERR_OOM;
   }
-  if (zero && cudaMemset(*p, 0, (size_t)n * sizeof(T)) != cudaSuccess) {
+  if (zero && (cudaMemset(*p, 0, (size_t)n * sizeof(T)) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)) {
     err = "cudaMemset of batch scratch failed";
     return PIKO_ERR_CUDA;
   }
@@ -612,6 +629,7 @@ void batch_state_free(BatchState* bs) {
   cudaFree(bs->cursor);
   cudaFree(bs->chunk_state);
   cudaFree(bs->bin_tris);
+  cudaFree(bs->gacc);
   cudaFree(bs->sync);
   if (bs->staging) cudaFreeHost(bs->staging);
   if (bs->uploaded) cudaEventDestroy(bs->uploaded);
@@ -686,6 +704,8 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   if ((r = grow_dev(&bs->vdot, &bs->dcap, tv, false, err)) != PIKO_OK) return r;
   if (persp && (r = grow_dev(&bs->invw, &bs->icap, tv, false, err)) != PIKO_OK) return r;
   if ((r = grow_dev(&bs->rect, &bs->tcap, tt, false, err)) != PIKO_OK) return r;
+  // here and not in the backward call, which may be recorded into a graph
+  if ((r = grow_dev(&bs->gacc, &bs->gcap, tv, true, err)) != PIKO_OK) return r;
   if (tb > bs->bcap) {
     // counts must start at zero; offsets/cursors/chunk states are rewritten
     cudaFree(bs->cnt); cudaFree(bs->bin_off); cudaFree(bs->cursor); cudaFree(bs->chunk_state);
@@ -711,10 +731,12 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
       return PIKO_ERR_OOM;
     }
   }
-  // descriptors + 6 prefix arrays, uploaded from pinned memory
+  // descriptors + 6 prefix arrays, uploaded from pinned memory; room after
+  // them for the backward's gradient groups and their prefix
   const size_t dbytes = sizeof(BatchScene) * n;
   const size_t pbytes = sizeof(int) * (n + 1);
-  const size_t total = dbytes + 6 * pbytes;
+  const size_t group_off = (dbytes + 6 * pbytes + 15) / 16 * 16;
+  const size_t total = group_off + sizeof(GradAcc) * n + pbytes;
   if (!bs->uploaded && cudaEventCreateWithFlags(&bs->uploaded, cudaEventDisableTiming) != cudaSuccess) {
     err = "cudaEventCreate failed";
     return PIKO_ERR_CUDA;
@@ -742,7 +764,7 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   std::memcpy(h, d.data(), dbytes);
   const std::vector<int>* arrays[6] = {&pv, &pt, &pb, &ps, &pd, &pp};
   for (int a = 0; a < 6; ++a) std::memcpy(h + dbytes + a * pbytes, arrays[a]->data(), pbytes);
-  if (cudaMemcpyAsync(bs->desc, bs->staging, total, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
+  if (cudaMemcpyAsync(bs->desc, bs->staging, group_off, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
       cudaEventRecord(bs->uploaded, stream) != cudaSuccess) {
     err = "upload of batch descriptors failed";
     return PIKO_ERR_CUDA;
@@ -779,6 +801,8 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
     return PIKO_ERR_CUDA;
   }
   bs->grid = per_sm * num_sms;
+  bs->desc_bytes = total;
+  bs->group_off = group_off;
   bs->n = n;
   bs->persp = persp ? 1 : 0;
   bs->host_desc = d;
@@ -855,8 +879,13 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
     err = "backward_batch needs a forward_batch of the same scenes first";
     return PIKO_ERR_INVALID_ARG;
   }
-  // per-scene gradient pointers go into the descriptors (same layout)
+  // per-scene accumulators go into the descriptors (same layout); scenes in a
+  // row with the same attributes and gradient arrays (views of one mesh) share
+  // one group of accumulators, which is finished once
   std::vector<BatchScene> d = bs->host_desc;
+  std::vector<GradAcc> groups;
+  std::vector<int> chunk_prefix(1, 0);
+  long long acc_used = 0;
   for (int i = 0; i < n; ++i) {
     if (scenes[i].num_triangles != d[i].T || scenes[i].num_vertices != d[i].V ||
         reinterpret_cast<unsigned long long*>(fbs[i].key) != d[i].key_out) {
@@ -868,18 +897,50 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
       return PIKO_ERR_INVALID_ARG;
     }
     d[i].dl = dl ? reinterpret_cast<const float4*>(dl[i]) : nullptr;
-    d[i].dcolor = dc ? dc[i] : nullptr;
-    d[i].dnormal = dn ? dn[i] : nullptr;
-    d[i].dlight = dlt ? dlt[i] : nullptr;
     d[i].color = scenes[i].color;
     d[i].normal = scenes[i].normal;
     d[i].light = scenes[i].light_dir;
+    const bool lambert = d[i].mode == PIKO_SHADE_LAMBERT;
+    GradAcc g;
+    g.V = d[i].V;
+    g.normal = lambert ? d[i].normal : nullptr;
+    g.light = lambert ? d[i].light : nullptr;
+    g.dcolor = dc && (!lambert || d[i].color) ? dc[i] : nullptr;
+    g.dnormal = dn && lambert ? dn[i] : nullptr;
+    g.dlight = dlt && lambert ? dlt[i] : nullptr;
+    d[i].acc = nullptr;
+    if (!d[i].dl || d[i].mode == PIKO_SHADE_GBUFFER || g.V == 0 || (!g.dcolor && !g.dnormal && !g.dlight)) continue;
+    if (!groups.empty()) {
+      const GradAcc& q = groups.back();
+      if (q.V == g.V && q.normal == g.normal && q.light == g.light && q.dcolor == g.dcolor &&
+          q.dnormal == g.dnormal && q.dlight == g.dlight) {
+        d[i].acc = q.acc;
+        continue;
+      }
+    }
+    g.acc = d[i].acc = bs->gacc + acc_used;
+    acc_used += g.V;  // at most the batch's vertices
+    groups.push_back(g);
+    chunk_prefix.push_back(chunk_prefix.back() + (g.V + GRAD_CHUNK - 1) / GRAD_CHUNK);
+  }
+  if (groups.empty()) return PIKO_OK;  // nothing to add
+  if (bs->gacc_dirty) {
+    if (cudaMemsetAsync(bs->gacc, 0, (size_t)bs->gcap * sizeof(float4), stream) != cudaSuccess) {
+      err = "gradient sums reset failed";
+      return PIKO_ERR_CUDA;
+    }
+    bs->gacc_dirty = false;
   }
   cudaStreamCaptureStatus cap_status = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(stream, &cap_status);
   if (cap_status == cudaStreamCaptureStatusNone) cudaEventSynchronize(bs->uploaded);
-  std::memcpy(bs->staging, d.data(), sizeof(BatchScene) * n);
-  if (cudaMemcpyAsync(bs->desc, bs->staging, sizeof(BatchScene) * n, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
+  char* h = static_cast<char*>(bs->staging);
+  const size_t prefix_off = bs->group_off + sizeof(GradAcc) * n;
+  std::memcpy(h, d.data(), sizeof(BatchScene) * n);
+  std::memcpy(h + bs->group_off, groups.data(), sizeof(GradAcc) * groups.size());
+  std::memcpy(h + prefix_off, chunk_prefix.data(), sizeof(int) * chunk_prefix.size());
+  // the prefix arrays of the layout are still in the staging block
+  if (cudaMemcpyAsync(bs->desc, bs->staging, bs->desc_bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
       cudaEventRecord(bs->uploaded, stream) != cudaSuccess) {
     err = "upload of backward descriptors failed";
     return PIKO_ERR_CUDA;
@@ -891,6 +952,10 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
   p.total_btiles = bs->params.total_btiles;
   p.vtx = bs->vtx;
   p.invw = bs->params.invw;  // the interpolation of the last forward_batch
+  p.ngroups = (int)groups.size();
+  p.total_chunks = chunk_prefix.back();
+  p.groups = reinterpret_cast<const GradAcc*>(static_cast<const char*>(bs->desc) + bs->group_off);
+  p.chunk_prefix = reinterpret_cast<const int*>(static_cast<const char*>(bs->desc) + prefix_off);
   static int per_sm_of[64] = {0};  // the shared-memory opt-in is per device
   int dev = 0;
   cudaGetDevice(&dev);
@@ -916,8 +981,11 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
     k_batch_backward<true><<<(int)blocks, BWD_THREADS, BATCH_BWD_SMEM, stream>>>(p);
   else
     k_batch_backward<false><<<(int)blocks, BWD_THREADS, BATCH_BWD_SMEM, stream>>>(p);
-  const cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = launch_pdl(k_batch_finish, p.total_chunks < 8 * num_sms ? p.total_chunks : 8 * num_sms, GRAD_CHUNK, 0, stream, p);
   if (e != cudaSuccess) {
+    bs->gacc_dirty = true;
     err = std::string("batch backward launch: ") + cudaGetErrorString(e);
     return PIKO_ERR_CUDA;
   }

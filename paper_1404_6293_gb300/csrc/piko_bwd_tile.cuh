@@ -10,15 +10,21 @@
 //   dL/dn_i += (g . albedo) b_i L   when s > 0 (or unclamped)
 //   dL/dL   += (g . albedo) n
 //
+// The normal and light gradients are linear in the sums of G b_i, G = g .
+// albedo, so a vertex needs four sums only: three of the colour and one of G.
+// They live in an accumulator of one float4 per vertex (GradAcc below), which
+// a pass over the vertices (grad_finish_chunk) turns into the three gradient
+// arrays and leaves zero for the next call.
+//
 // A warp takes a 16 x 16 or 16 x 32 tile (backward_warp_tile, below) with no
 // CTA barrier: the warps of a CTA work on separate tiles.  Each lane walks a
 // column of the tile and keeps, for as long as its pixels keep the same
 // winning triangle (a run), that triangle's setup (vertex indices, snapped
 // positions, 2 x area) and the sums of its 12 per-pixel terms (below) in
 // registers; a run that ends is summed with the other lanes' runs of the same
-// triangle and added to the gradient arrays with one set of atomics.  A
-// triangle is set up once per run rather than per pixel, and a triangle that
-// covers a column of the tile is flushed once for it.
+// triangle and added to the accumulators of its three vertices.  A triangle
+// is set up once per run rather than per pixel, and a triangle that covers a
+// column of the tile is flushed once for it.
 #pragma once
 
 #include "piko_internal.cuh"
@@ -44,7 +50,7 @@ constexpr int BWD_THREADS = 256;             // CTA size of the backward kernels
 // vertex j (g_c b_j for Gouraud); q = 9 + j is G b_j with G = g . albedo
 // (0 where the clamp is inactive).  The normal and light gradients are
 // linear in the G b_j sums: dL/dn_j = L sum(G b_j) and dL/dL = sum_j n_j
-// sum(G b_j), so they are formed once per slot from the sums.
+// sum(G b_j), so they are formed once per vertex from the sums.
 constexpr int BWD_VALS = 12;
 constexpr unsigned BWD_NONE = 0xFFFFFFFFu;
 
@@ -60,10 +66,78 @@ struct BwdScene {
   const float* mvp;
   const unsigned long long* key;
   const float4* dl;
-  float* dcolor;
+  float4* acc;  // per vertex: sums of g s b (colour) and of G b (zero between calls)
+};
+
+// ------------------------------------------------------------ accumulators
+// One 16-byte vector reduction per vertex and flushed run.  The L2 takes a
+// reduction per sector and instruction, whatever its width: adding the 18
+// scalars of a run (9 colour, 9 normal) one by one kept it at its limit, and
+// three vector reductions carry the same sums.
+__device__ __forceinline__ void grad_add(float4* acc, float c0, float c1, float c2, float G) {
+  if (c0 != 0.f || c1 != 0.f || c2 != 0.f || G != 0.f)
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(acc), "f"(c0), "f"(c1), "f"(c2), "f"(G)
+                 : "memory");
+}
+
+// A group of vertices with one accumulator: the vertices of a scene, or of
+// several scenes of a batch that share their attributes and gradient arrays.
+struct GradAcc {
+  int V;
+  float4* acc;
+  const float* normal;  // Lambert (NULL for Gouraud: no normal or light gradients)
+  const float* light;
+  float* dcolor;   // NULL: not wanted
   float* dnormal;
   float* dlight;
 };
+
+constexpr int GRAD_CHUNK = 256;  // vertices per CTA step of the finishing pass, one per thread
+
+struct GradFinishSmem {
+  float4 a[GRAD_CHUNK];
+  float light[GRAD_CHUNK / 32][3];
+};
+
+// Vertices [GRAD_CHUNK chunk, + GRAD_CHUNK) of a group; called by a CTA of
+// GRAD_CHUNK threads.  The sums go through shared memory so that the
+// gradient arrays (three floats a vertex) are added to in whole sectors.
+// Atomic, as several calls on different streams may share the arrays.
+__device__ __forceinline__ void grad_finish_chunk(const GradAcc& f, int chunk, GradFinishSmem& sm) {
+  const int tid = threadIdx.x, lane = tid & 31, base = chunk * GRAD_CHUNK, v = base + tid;
+  float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (v < f.V) a = __ldcg(f.acc + v);
+  const bool hit = a.x != 0.f || a.y != 0.f || a.z != 0.f || a.w != 0.f;
+  if (hit) f.acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (!__syncthreads_or(hit)) return;  // (the barrier also ends the last chunk's reads of sm)
+  sm.a[tid] = a;
+  if (f.normal && f.dlight) {
+    float g[3] = {0.f, 0.f, 0.f};
+    if (a.w != 0.f) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) g[k] = a.w * __ldg(f.normal + 3 * (size_t)v + k);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      for (int o = 16; o > 0; o >>= 1) g[k] += __shfl_xor_sync(FULL_MASK, g[k], o);
+      if (lane == 0) sm.light[tid >> 5][k] = g[k];
+    }
+  }
+  __syncthreads();
+  if (f.normal && f.dlight && tid < 3) {
+    float s = 0.f;
+    for (int w = 0; w < GRAD_CHUNK / 32; ++w) s += sm.light[w][tid];
+    if (s != 0.f) atomicAdd(f.dlight + tid, s);
+  }
+  const float* s = reinterpret_cast<const float*>(sm.a);
+  const int n = 3 * min(GRAD_CHUNK, f.V - base);
+  for (int i = tid; i < n; i += GRAD_CHUNK) {
+    const int q = i / 3, c = i - 3 * q;
+    if (f.dcolor && s[4 * q + c] != 0.f) atomicAdd(f.dcolor + 3 * (size_t)base + i, s[4 * q + c]);
+    if (f.normal && f.dnormal && s[4 * q + 3] != 0.f)
+      atomicAdd(f.dnormal + 3 * (size_t)base + i, s[4 * q + 3] * __ldg(f.light + c));
+  }
+}
 
 // ---------------------------------------------------------------- warp form
 // One warp takes a BWD_TILE_W x TILE_H tile in passes of 16 x 2 pixels:
@@ -183,51 +257,24 @@ __device__ __forceinline__ void bwd_run_terms(const BwdScene& sc, const BwdRun& 
   }
 }
 
-// Adds term q (see BWD_VALS) with value val of a triangle whose vertex j (the
-// vertex of term q) is vj to the scene's gradients: a colour term goes to
-// dL/dc of the vertex; a G b_j sum goes to dL/dn_j (times L) and, when
-// `light` is set, to this thread's share of dL/dL (times n_j).
-__device__ __forceinline__ void bwd_add_term_v(const BwdScene& sc, int vj, int q, float val, bool has_c, bool has_n,
-                                               bool light, float L0, float L1, float L2, float& gl0, float& gl1,
-                                               float& gl2) {
-  if (q < 9) {
-    if (has_c) atomicAdd(sc.dcolor + 3 * (size_t)vj + (q % 3), val);
-    return;
-  }
-  const size_t vb = 3 * (size_t)vj;
-  if (has_n) {
-    atomicAdd(sc.dnormal + vb, val * L0);
-    atomicAdd(sc.dnormal + vb + 1, val * L1);
-    atomicAdd(sc.dnormal + vb + 2, val * L2);
-  }
-  if (light) {
-    gl0 += val * __ldg(sc.normal + vb);
-    gl1 += val * __ldg(sc.normal + vb + 1);
-    gl2 += val * __ldg(sc.normal + vb + 2);
-  }
-}
-
 // Flushes the runs of the lanes with fl set (t: their triangle, r: its
 // setup, acc: their sums, cleared here).  Warp-collective.
 __device__ __forceinline__ void bwd_run_flush(const BwdScene& sc, bool fl, unsigned t, const BwdRun& r,
-                                              float (&acc)[BWD_VALS], float (*stage)[33], bool has_c, bool has_n,
-                                              bool has_l, float L0, float L1, float L2, float& gl0, float& gl1,
-                                              float& gl2) {
+                                              float (&acc)[BWD_VALS], float (*stage)[33]) {
   const int lane = threadIdx.x & 31;
   const unsigned grp = __match_any_sync(FULL_MASK, fl ? t : BWD_NONE);
   const bool own = fl && __popc(grp) <= 2;
   if (own) {
-    const int vid[3] = {r.v0, r.v1, r.v2};
-#pragma unroll
-    for (int q = 0; q < BWD_VALS; ++q)
-      if (acc[q] != 0.f)
-        bwd_add_term_v(sc, vid[q < 9 ? q / 3 : q - 9], q, acc[q], has_c, has_n, has_l, L0, L1, L2, gl0, gl1, gl2);
+    grad_add(sc.acc + r.v0, acc[0], acc[1], acc[2], acc[9]);
+    grad_add(sc.acc + r.v1, acc[3], acc[4], acc[5], acc[10]);
+    grad_add(sc.acc + r.v2, acc[6], acc[7], acc[8], acc[11]);
   }
   unsigned big = __ballot_sync(FULL_MASK, fl && !own);
   if (big != 0u) {
 #pragma unroll
     for (int q = 0; q < BWD_VALS; ++q) stage[q][lane] = acc[q];
     __syncwarp();
+    const int j = lane < 3 ? lane : 0;  // the vertex a lane adds to
     // every round removes at least the round's leader lane
     for (int round = 0; big != 0u && round < 32; ++round) {
       const int ld = __ffs(big) - 1;
@@ -235,14 +282,12 @@ __device__ __forceinline__ void bwd_run_flush(const BwdScene& sc, bool fl, unsig
       const int u0 = __shfl_sync(FULL_MASK, r.v0, ld), u1 = __shfl_sync(FULL_MASK, r.v1, ld),
                 u2 = __shfl_sync(FULL_MASK, r.v2, ld);
       big &= ~gm;
-      if (lane < BWD_VALS) {
-        float sum = 0.f;
+      float sum = 0.f;
+      if (lane < BWD_VALS)
         for (unsigned m = gm; m; m &= m - 1) sum += stage[lane][__ffs(m) - 1];
-        const int j = lane < 9 ? lane / 3 : lane - 9;
-        if (sum != 0.f)
-          bwd_add_term_v(sc, j == 0 ? u0 : (j == 1 ? u1 : u2), lane, sum, has_c, has_n, has_l, L0, L1, L2, gl0, gl1,
-                         gl2);
-      }
+      const float c0 = __shfl_sync(FULL_MASK, sum, 3 * j), c1 = __shfl_sync(FULL_MASK, sum, 3 * j + 1),
+                  c2 = __shfl_sync(FULL_MASK, sum, 3 * j + 2), G = __shfl_sync(FULL_MASK, sum, 9 + j);
+      if (lane < 3) grad_add(sc.acc + (j == 0 ? u0 : (j == 1 ? u1 : u2)), c0, c1, c2, G);
     }
     __syncwarp();  // the staging area is rewritten by the next flush
   }
@@ -254,18 +299,13 @@ __device__ __forceinline__ void bwd_run_flush(const BwdScene& sc, bool fl, unsig
 
 // One tile with its top-left pixel (x0, y0), taken by one warp (all 32 lanes
 // call it with the same arguments); stage is the warp's own staging area.
-// The tile's share of dL/dL is added at its end.  A triangle that starts a
-// run is set up by the lowest lane of the warp that holds it and broadcast to
+// A triangle that starts a run is set up by the lowest lane of the warp that holds it and broadcast to
 // the lanes that need it; a lane whose run goes on keeps its setup.
 // CLIP: near/far clipping may be on (sc.pos set).
 template <bool PERSP = false, bool CLIP = false, int TILE_H = BWD_TILE_H>
 __device__ __forceinline__ void backward_warp_tile(const BwdScene& sc, int x0, int y0, float (*stage)[33], float L0,
                                                    float L1, float L2) {
   const int lane = threadIdx.x & 31;
-  const bool has_c = sc.dcolor != nullptr && (sc.mode == PIKO_SHADE_GOURAUD || sc.color != nullptr);
-  const bool has_n = sc.dnormal != nullptr && sc.mode == PIKO_SHADE_LAMBERT;
-  const bool has_l = sc.dlight != nullptr && sc.mode == PIKO_SHADE_LAMBERT;
-  float gl0 = 0.f, gl1 = 0.f, gl2 = 0.f;
   float acc[BWD_VALS];
 #pragma unroll
   for (int q = 0; q < BWD_VALS; ++q) acc[q] = 0.f;
@@ -290,7 +330,7 @@ __device__ __forceinline__ void backward_warp_tile(const BwdScene& sc, int x0, i
     const bool change = t != cur;
     const bool ends = change && r.kind != 0;
     if (__any_sync(FULL_MASK, ends))
-      bwd_run_flush(sc, ends, cur, r, acc, stage, has_c, has_n, has_l, L0, L1, L2, gl0, gl1, gl2);
+      bwd_run_flush(sc, ends, cur, r, acc, stage);
     const bool need = change && t != BWD_NONE;
     if (__any_sync(FULL_MASK, need)) {
       const int leader = __ffs(__match_any_sync(FULL_MASK, t)) - 1;
@@ -304,20 +344,7 @@ __device__ __forceinline__ void backward_warp_tile(const BwdScene& sc, int x0, i
     if (r.kind != 0) bwd_run_terms<PERSP, CLIP>(sc, r, x, y, g, acc);
   }
   const bool ends = r.kind != 0;
-  if (__any_sync(FULL_MASK, ends))
-    bwd_run_flush(sc, ends, cur, r, acc, stage, has_c, has_n, has_l, L0, L1, L2, gl0, gl1, gl2);
-  if (has_l) {
-    for (int o = 16; o > 0; o >>= 1) {
-      gl0 += __shfl_xor_sync(FULL_MASK, gl0, o);
-      gl1 += __shfl_xor_sync(FULL_MASK, gl1, o);
-      gl2 += __shfl_xor_sync(FULL_MASK, gl2, o);
-    }
-    if (lane == 0) {
-      if (gl0 != 0.f) atomicAdd(sc.dlight, gl0);
-      if (gl1 != 0.f) atomicAdd(sc.dlight + 1, gl1);
-      if (gl2 != 0.f) atomicAdd(sc.dlight + 2, gl2);
-    }
-  }
+  if (__any_sync(FULL_MASK, ends)) bwd_run_flush(sc, ends, cur, r, acc, stage);
 }
 
 }  // namespace piko
