@@ -4,6 +4,7 @@
 
 #include <string>
 
+#include "piko_direct.cuh"
 #include "piko_internal.cuh"
 #include "piko_scan.cuh"
 
@@ -24,7 +25,8 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
                           cudaStream_t stream, std::string& err);
 
 int piko_backward_launch(int W, int H, int mode, int unclamped, int T, int V, const int* tris, const int4* vtx,
-                         const float* vdot, const float* color, const float* normal, const float* light,
+                         const float* vdot, const float4* vattr, const float* color, const float* normal,
+                         const float* light,
                          const float* invw, const float* pos, const float* mvp, const unsigned long long* key,
                          const float* dl_drgba, float4* acc, float* dcolor, float* dnormal, float* dlight, int num_sms,
                          cudaStream_t s);
@@ -49,15 +51,15 @@ struct piko_raster {
   bool use_stage_ev = false;
   int device = 0, num_sms = 0;
   // scratch (device)
-  int4* vtx = nullptr;
+  // per vertex, carved from one allocation (vertex_block) of vcap vertices
+  void* vertex_block = nullptr;
   long long vcap = 0;
-  float* vdot = nullptr;  // n . L per vertex for Lambert
-  long long dcap = 0;
-  float* invw = nullptr;  // 1 / clip w per vertex, with perspective-correct attributes
-  long long icap = 0;
-  float4* gacc = nullptr;  // gradient sums per vertex, zero between calls
-  long long gcap = 0;
-  bool gacc_dirty = false;  // a failed backward launch may have left sums behind
+  int4* vtx = nullptr;      // snapped position
+  float4* vattr = nullptr;  // colour and n . L, for Lambert with colours
+  float4* gacc = nullptr;   // gradient sums, zero between calls
+  float* vdot = nullptr;    // n . L, for Lambert without colours
+  float* invw = nullptr;    // 1 / clip w, with perspective-correct attributes
+  bool gacc_dirty = false;  // gacc is not zero: new, or a backward launch failed
   BinRect* rect = nullptr;
   long long tcap = 0;
   unsigned* bin_count = nullptr;  // 2 * nbins, zero between frames
@@ -71,6 +73,8 @@ struct piko_raster {
   // spread over whole CTAs), and the count pass's parity
   uint2* heavy = nullptr;
   unsigned heavy_epoch = 0;
+  unsigned long long* dkeys = nullptr;  // a key per pixel of directly rasterized triangles (piko_direct.cuh)
+  long long dkcap = 0;
   // fragment buffers of the unfused pipeline (PIKO_SCHED_UNFUSED)
   unsigned* frag_pix = nullptr;
   unsigned long long* frag_key = nullptr;
@@ -95,8 +99,11 @@ struct piko_raster {
   long long hcap_pos = 0, hcap_tris = 0, hcap_color = 0, hcap_normal = 0, hcap_small = 0, hcap_key = 0,
             hcap_rgba = 0, hcap_gn = 0, hcap_ga = 0;
   DevStatus* status = nullptr;
-  unsigned long long* h_needed = nullptr;  // pinned
+  unsigned long long* h_needed = nullptr;  // pinned, written by the scan (ScanReport): bin entries needed, those of
+                                           // them in the lists, clipped sub-triangles, the report's tag
+  unsigned long long report_tag = 0;
   long long last_entries = 0;              // bin entries of the last frame read back (0: none yet)
+  int last_tris = -1;                      // triangles of that frame
   cudaStream_t last_stream = nullptr;
   std::string err;
 };
@@ -140,16 +147,32 @@ int grow(piko_raster* h, T** ptr, long long* cap, long long need, const char* wh
   return PIKO_OK;
 }
 
-// The gradient accumulators, zero between calls.  Grown with the vertex
-// buffer (forward and reserve too), so that a backward call recorded into a
-// graph after a forward of the same scene allocates nothing.
-int grow_gacc(piko_raster* h, long long need) {
-  if (need <= h->gcap) return PIKO_OK;
-  const int r = grow(h, &h->gacc, &h->gcap, need, "gradient sums");
-  if (r != PIKO_OK) return r;
-  cudaError_t e = cudaMemset(h->gacc, 0, (size_t)h->gcap * sizeof(float4));
-  if (e == cudaSuccess) e = cudaDeviceSynchronize();
-  return e == cudaSuccess ? PIKO_OK : cuda_fail(h, e, "gradient sums");
+// The per-vertex arrays, in one allocation: allocating costs a first frame
+// more than its kernels, and a later call with other options (perspective,
+// gradients) on the same scene, possibly being captured, allocates nothing.
+int grow_vertices(piko_raster* h, long long need) {
+  if (need <= h->vcap) return PIKO_OK;
+  char* block = static_cast<char*>(h->vertex_block);
+  long long cap = 0;
+  h->vcap = 0;
+  const long long per_vertex = sizeof(int4) + 2 * sizeof(float4) + 2 * sizeof(float);
+  long long bytes = 0;
+  h->vertex_block = nullptr;
+  const int r = grow(h, &block, &bytes, need * per_vertex, "vertex buffer");
+  if (r != PIKO_OK) {
+    h->vertex_block = block;
+    return r;
+  }
+  cap = bytes / per_vertex / 4 * 4;
+  h->vertex_block = block;
+  h->vtx = reinterpret_cast<int4*>(block);
+  h->vattr = reinterpret_cast<float4*>(h->vtx + cap);
+  h->gacc = h->vattr + cap;
+  h->vdot = reinterpret_cast<float*>(h->gacc + cap);
+  h->invw = h->vdot + cap;
+  h->gacc_dirty = true;
+  h->vcap = cap;
+  return PIKO_OK;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -185,7 +208,7 @@ piko_raster* piko_raster_create(int width, int height, int bin_w, int bin_h, int
             cudaMemset(h->chunk_state, 0, sizeof(unsigned long long) * scan_chunks(h->nbins)) == cudaSuccess &&
             cudaMalloc(&h->status, sizeof(DevStatus)) == cudaSuccess &&
             cudaMalloc(&h->heavy, sizeof(uint2) * HEAVY_LIST_CAP) == cudaSuccess &&
-            cudaMallocHost(&h->h_needed, sizeof(unsigned long long)) == cudaSuccess &&
+            cudaMallocHost(&h->h_needed, 4 * sizeof(unsigned long long)) == cudaSuccess &&
             cudaMallocHost(&h->h_frags, sizeof(unsigned)) == cudaSuccess &&
             cudaMallocHost(&h->h_clips, sizeof(unsigned)) == cudaSuccess &&
             cudaMemset(h->bin_count, 0, sizeof(unsigned) * 2 * h->nbins) == cudaSuccess &&
@@ -196,16 +219,14 @@ piko_raster* piko_raster_create(int width, int height, int bin_w, int bin_h, int
     piko_raster_destroy(h);
     return nullptr;
   }
+  memset(h->h_needed, 0, 4 * sizeof(unsigned long long));
   return h;
 }
 
 void piko_raster_destroy(piko_raster* h) {
   if (!h) return;
   cudaDeviceSynchronize();
-  cudaFree(h->vtx);
-  cudaFree(h->vdot);
-  cudaFree(h->invw);
-  cudaFree(h->gacc);
+  cudaFree(h->vertex_block);
   cudaFree(h->rect);
   cudaFree(h->bin_count);
   cudaFree(h->bin_off);
@@ -213,6 +234,7 @@ void piko_raster_destroy(piko_raster* h) {
   cudaFree(h->chunk_state);
   cudaFree(h->bin_tris);
   cudaFree(h->heavy);
+  cudaFree(h->dkeys);
   cudaFree(h->frag_pix);
   cudaFree(h->frag_key);
   cudaFree(h->frag_rgba);
@@ -239,6 +261,31 @@ void piko_raster_destroy(piko_raster* h) {
 const char* piko_raster_last_error(const piko_raster* h) {
   if (!h) return "null handle";
   return h->err.c_str();
+}
+
+// Colour and n . L packed per vertex for a Lambert scene with colours.
+static float4* packed_attributes(piko_raster* h, const piko_scene* s) {
+  return s->shade_mode == PIKO_SHADE_LAMBERT && s->color ? h->vattr : nullptr;
+}
+
+// The keys of direct rasterization for a frame of T triangles, or NULL when
+// every triangle is binned: a frame of larger triangles, one whose work is
+// counted or binned exactly, or no memory for the keys (nothing is allocated
+// while the stream is being captured).
+static unsigned long long* direct_keys(piko_raster* h, int T, int V, cudaStream_t st) {
+  if (h->stats || h->exact_bins || h->small_px < 1 || h->schedule > PIKO_SCHED_HARDWARE ||
+      !direct_scene(T, V, h->W, h->H))
+    return nullptr;
+  const long long need = (long long)h->W * h->H;
+  if (need > h->dkcap) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
+        grow(h, &h->dkeys, &h->dkcap, need, "direct keys") != PIKO_OK) {
+      cudaGetLastError();
+      return nullptr;
+    }
+  }
+  return h->dkeys;
 }
 
 // Chunks the heavy-triangle list may hold: none under test hook bit 2, so
@@ -309,13 +356,14 @@ int piko_raster_reserve(piko_raster* h, int64_t max_vertices, int64_t max_triang
       max_triangles > INT32_MAX || max_bin_entries > 0xFFFFFFF0LL)
     return fail(h, PIKO_ERR_INVALID_ARG, "reserve sizes out of range");
   int r;
-  if ((r = grow(h, &h->vtx, &h->vcap, max_vertices, "vertex buffer")) != PIKO_OK) return r;
-  if ((r = grow(h, &h->vdot, &h->dcap, max_vertices, "vertex light terms")) != PIKO_OK) return r;
-  if ((r = grow_gacc(h, max_vertices)) != PIKO_OK) return r;
-  // 1/w too, so that turning perspective-correct attributes on later needs no allocation
-  if ((r = grow(h, &h->invw, &h->icap, max_vertices, "vertex 1/w")) != PIKO_OK) return r;
+  if ((r = grow_vertices(h, max_vertices)) != PIKO_OK) return r;
   if ((r = grow(h, &h->rect, &h->tcap, max_triangles, "bin rectangles")) != PIKO_OK) return r;
   if ((r = grow(h, &h->bin_tris, &h->ecap, max_bin_entries, "bin lists")) != PIKO_OK) return r;
+  // keys of direct rasterization, if such scenes can take it (else, or without
+  // the memory, every triangle is binned)
+  if (direct_scene(max_triangles, max_vertices, h->W, h->H) &&
+      grow(h, &h->dkeys, &h->dkcap, (long long)h->W * h->H, "direct keys") != PIKO_OK)
+    cudaGetLastError();
   cudaError_t e = cudaDeviceSynchronize();
   return e == cudaSuccess ? PIKO_OK : cuda_fail(h, e, "reserve");
 }
@@ -360,11 +408,28 @@ static int check_scene(piko_raster* h, const piko_scene* s) {
   return PIKO_OK;
 }
 
-// Near/far clipping: the sub-triangle list for this frame.  With the
-// capacity check the count is read back (one host sync) and the list grown
-// and refilled once if it overflowed; without it an overflow is reported as
-// PIKO_ERR_OVERFLOW and the frame writes nothing.
-static int clip_pass(piko_raster* h, const piko_scene* s, cudaStream_t st) {
+// Waits until the scan's report of this frame (tag h->report_tag) is in
+// h_needed.  The scan writes it to host memory itself, so the kernels launched
+// behind the scan keep running meanwhile.  Ends with the stream at the latest.
+static int wait_report(piko_raster* h, cudaStream_t st) {
+  const auto arrived = [&] { return __atomic_load_n(h->h_needed + 3, __ATOMIC_ACQUIRE) == h->report_tag; };
+  for (unsigned spin = 1; !arrived(); ++spin) {
+    if (spin & 2047u) continue;
+    const cudaError_t e = cudaStreamQuery(st);
+    if (e == cudaErrorNotReady) continue;
+    if (e != cudaSuccess) return cuda_fail(h, e, "bin-list size read-back");
+    if (arrived()) break;
+    return fail(h, PIKO_ERR_CUDA, "the scan reported nothing");
+  }
+  return PIKO_OK;
+}
+
+// Near/far clipping: the sub-triangle list for this frame.  With wait, the
+// capacity check's, the count is read back (one host sync) and the list grown
+// and refilled once if it overflowed; without it an overflow is recorded as
+// PIKO_ERR_OVERFLOW, the later stages write nothing, and the caller looks at
+// the count in the scan's report (zeroed: the vertex stage cleared the count).
+static int clip_pass(piko_raster* h, const piko_scene* s, cudaStream_t st, bool wait, bool zeroed) {
   const int T = s->num_triangles;
   long long want = T / 8 + 1024;
   int r;
@@ -375,11 +440,12 @@ static int clip_pass(piko_raster* h, const piko_scene* s, cudaStream_t st) {
         return r;
     }
     const long long cap = h->ccap_tris / 3 < h->ccap_orig ? h->ccap_tris / 3 : h->ccap_orig;
-    cudaError_t e = cudaMemsetAsync(&h->status->clip_count, 0, sizeof(unsigned), st);
+    cudaError_t e = cudaSuccess;
+    if (!zeroed || attempt > 0) e = cudaMemsetAsync(&h->status->clip_count, 0, sizeof(unsigned), st);
     if (e != cudaSuccess) return cuda_fail(h, e, "clip count clear");
     launch_clip(h->W, h->H, T, s->tris, s->num_vertices, s->pos, s->mvp, h->vtx, h->clip_tris, h->clip_orig,
                 (unsigned)cap, h->status, h->num_sms, st);
-    if (!h->check_capacity) return PIKO_OK;
+    if (!wait) return PIKO_OK;
     e = cudaMemcpyAsync(h->h_clips, &h->status->clip_count, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(h, e, "clip count read-back");
@@ -413,7 +479,7 @@ static int forward_other_mapping(piko_raster* h, const piko_scene* s, piko_frame
   in.pos = s->pos; in.mvp = s->mvp;
   in.clip_tris = h->clip ? h->clip_tris : nullptr;
   in.clip_orig = h->clip ? h->clip_orig : nullptr;
-  in.clip_cap = h->clip ? (unsigned)(h->ccap_tris < h->ccap_orig ? h->ccap_tris : h->ccap_orig) : 0u;
+  in.clip_cap = h->clip ? (unsigned)(h->ccap_tris / 3 < h->ccap_orig ? h->ccap_tris / 3 : h->ccap_orig) : 0u;
   const bool persp = h->perspective != 0;
   const size_t key_bytes = sizeof(unsigned long long) * (size_t)h->W * h->H;
   int r;
@@ -473,79 +539,15 @@ static int forward_other_mapping(piko_raster* h, const piko_scene* s, piko_frame
   return PIKO_OK;
 }
 
-int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* fb, void* cuda_stream) {
-  if (!h) return PIKO_ERR_INVALID_ARG;
-  int r = check_scene(h, s);
-  if (r != PIKO_OK) return r;
-  if (!fb || !fb->key) return fail(h, PIKO_ERR_INVALID_ARG, "framebuffer key is required");
-  if (s->shade_mode == PIKO_SHADE_GBUFFER && (!fb->gbuf_normal || !fb->gbuf_albedo))
-    return fail(h, PIKO_ERR_INVALID_ARG, "G-buffer mode needs gbuf_normal and gbuf_albedo");
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
-  h->last_stream = st;
+// The scatter pass and the Process stage of a frame whose scan is launched.
+static int scatter_and_process(piko_raster* h, const piko_scene* s, piko_framebuffer* fb, cudaStream_t st, bool ev,
+                               const DirectRaster& direct, const float4* vattr, const int4* clip_tris,
+                               unsigned clip_cap) {
   const int V = s->num_vertices, T = s->num_triangles;
-  if ((r = grow(h, &h->vtx, &h->vcap, V, "vertex buffer")) != PIKO_OK || (r = grow_gacc(h, V)) != PIKO_OK) return r;
-  const bool lambert = s->shade_mode == PIKO_SHADE_LAMBERT;
-  if (lambert && (r = grow(h, &h->vdot, &h->dcap, V, "vertex light terms")) != PIKO_OK) return r;
-  if (h->perspective && (r = grow(h, &h->invw, &h->icap, V, "vertex 1/w")) != PIKO_OK) return r;
-  if ((r = grow(h, &h->rect, &h->tcap, T, "bin rectangles")) != PIKO_OK) return r;
-  if (h->ecap == 0 && (r = grow(h, &h->bin_tris, &h->ecap, (long long)T * 2 + 4096, "bin lists")) != PIKO_OK)
-    return r;
-
-  const bool ev = h->use_stage_ev;
-  h->use_stage_ev = false;
-  if (ev) cudaEventRecord(h->stage_ev[0], st);
-  if (h->stats) cudaMemsetAsync(&h->status->tests, 0, 4 * sizeof(unsigned long long), st);
-  launch_vertex(h->W, h->H, V, s->pos, s->mvp, h->vtx, lambert ? s->normal : nullptr, s->light_dir,
-                lambert ? h->vdot : nullptr, h->perspective ? h->invw : nullptr, h->num_sms, st);
-  if (h->clip && (r = clip_pass(h, s, st)) != PIKO_OK) return r;
-  const int4* clip_tris = h->clip ? h->clip_tris : nullptr;
-  const unsigned clip_cap = h->clip ? (unsigned)(h->ccap_tris < h->ccap_orig ? h->ccap_tris : h->ccap_orig) : 0u;
-  if (clip_cap && (r = grow(h, &h->rect, &h->tcap, (long long)T + clip_cap, "bin rectangles")) != PIKO_OK) return r;
-  if (ev) cudaEventRecord(h->stage_ev[1], st);
-  if (h->schedule == PIKO_SCHED_FUSED || h->schedule == PIKO_SCHED_UNFUSED)
-    return forward_other_mapping(h, s, fb, st, ev);
-  for (int attempt = 0;; ++attempt) {
-    if (h->stats && attempt > 0) cudaMemsetAsync(&h->status->binned, 0, sizeof(unsigned long long), st);
-    // a frame of one scan chunk of bins is scanned by the count pass's last
-    // CTA (one launch fewer on the chain); larger frames take the scan kernel
-    // (with stage events on, the count and scan launches stay apart)
-    const unsigned heavy_epoch = ++h->heavy_epoch, scan_epoch = ++h->scan_epoch;
-    const bool fused = !ev && launch_count_and_scan(h->g, T, s->tris, V, h->vtx, h->rect, h->bin_count, h->status,
-                                                    h->stats, h->num_sms, st, clip_tris, clip_cap, h->exact_bins,
-                                                    h->heavy, heavy_cap(h), heavy_epoch, h->bin_off, h->cursor,
-                                                    (unsigned long long)h->ecap, h->chunk_state, scan_epoch);
-    if (!fused) {
-      launch_setup_count(h->g, T, s->tris, V, h->vtx, h->rect, h->bin_count, h->status, h->stats, h->num_sms, st,
-                         clip_tris, clip_cap, h->exact_bins, h->heavy, heavy_cap(h), heavy_epoch);
-      if (ev) cudaEventRecord(h->stage_ev[2], st);
-      launch_scan(h->nbins, h->bin_count, h->bin_off, h->cursor, (unsigned long long)h->ecap, h->status,
-                  h->chunk_state, scan_epoch, st, h->wait_budget, h->withhold);
-      if (ev) cudaEventRecord(h->stage_ev[3], st);
-    }
-    if (!h->check_capacity) break;
-    cudaError_t e = cudaMemcpyAsync(h->h_needed, &h->status->needed, sizeof(unsigned long long),
-                                    cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(h, e, "bin-list size read-back");
-    const long long need = (long long)*h->h_needed;
-    if (need <= h->ecap) break;
-    if (attempt > 0 || need > 0xFFFFFFF0LL) return fail(h, PIKO_ERR_OVERFLOW, "bin lists too large");
-    if ((r = grow(h, &h->bin_tris, &h->ecap, need, "bin lists")) != PIKO_OK) return r;
-    // the failed scan recorded an overflow and zeroed the counts: clear and count again
-    e = cudaMemsetAsync(h->status, 0, sizeof(unsigned) * 2, st);
-    if (e != cudaSuccess) return cuda_fail(h, e, "status clear");
-  }
-  launch_scatter(h->g, T, h->rect, h->bin_off, h->cursor, h->bin_tris, (unsigned long long)h->ecap, h->status,
-                 h->num_sms, st, clip_tris, clip_cap, h->exact_bins ? s->tris : nullptr, V, h->vtx, h->heavy,
-                 heavy_cap(h), h->heavy_epoch);
-  if (ev) cudaEventRecord(h->stage_ev[4], st);
-
   ProcessParams p;
   p.g = h->g;
   p.ntiles = h->nbins;
-  // records sized from this frame's bin-list total when it was read back,
-  // else from the last one read back
-  if (h->check_capacity) h->last_entries = (long long)*h->h_needed;
+  // records sized from the last bin-list total read back
   p.slots_hint = slots_for_entries(h->last_entries, h->nbins);
   p.schedule = h->schedule;
   p.small_px = h->small_px;
@@ -559,6 +561,7 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
   p.normal = s->normal;
   p.light = s->light_dir;
   p.vdot = h->vdot;
+  p.vattr = vattr;
   p.invw = h->perspective ? h->invw : nullptr;
   p.clip_tris = clip_tris;
   p.clip_orig = h->clip ? h->clip_orig : nullptr;
@@ -566,11 +569,22 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
   p.mvp = s->mvp;
   p.bin_off = h->bin_off;
   p.bin_tris = h->bin_tris;
+  p.dkeys = direct.keys;
   p.key_out = reinterpret_cast<unsigned long long*>(fb->key);
   p.rgba_out = reinterpret_cast<float4*>(fb->rgba);
   p.gnorm_out = reinterpret_cast<uint2*>(fb->gbuf_normal);
   p.galb_out = reinterpret_cast<uint2*>(fb->gbuf_albedo);
   p.st = h->status;
+  if (direct.keys) {
+    const cudaError_t e = launch_scatter_shade(p, h->rect, h->cursor, h->bin_tris, (unsigned long long)h->ecap,
+                                               h->num_sms, st, clip_cap, h->heavy, heavy_cap(h), h->heavy_epoch);
+    if (e != cudaSuccess) return cuda_fail(h, e, "scatter launch");
+  } else {
+    launch_scatter(h->g, T, h->rect, h->bin_off, h->cursor, h->bin_tris, (unsigned long long)h->ecap, h->status,
+                   h->num_sms, st, clip_tris, clip_cap, h->exact_bins ? s->tris : nullptr, V, h->vtx, h->heavy,
+                   heavy_cap(h), h->heavy_epoch);
+  }
+  if (ev) cudaEventRecord(h->stage_ev[4], st);
   int grid = h->nbins;
   if (h->schedule != PIKO_SCHED_HARDWARE) {
     int per_sm = 0;
@@ -583,6 +597,113 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
   if (e != cudaSuccess) return cuda_fail(h, e, "process launch");
   if (ev) cudaEventRecord(h->stage_ev[5], st);
   return PIKO_OK;
+}
+
+int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* fb, void* cuda_stream) {
+  if (!h) return PIKO_ERR_INVALID_ARG;
+  int r = check_scene(h, s);
+  if (r != PIKO_OK) return r;
+  if (!fb || !fb->key) return fail(h, PIKO_ERR_INVALID_ARG, "framebuffer key is required");
+  if (s->shade_mode == PIKO_SHADE_GBUFFER && (!fb->gbuf_normal || !fb->gbuf_albedo))
+    return fail(h, PIKO_ERR_INVALID_ARG, "G-buffer mode needs gbuf_normal and gbuf_albedo");
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
+  h->last_stream = st;
+  const int V = s->num_vertices, T = s->num_triangles;
+  if ((r = grow_vertices(h, V)) != PIKO_OK) return r;
+  const bool lambert = s->shade_mode == PIKO_SHADE_LAMBERT;
+  if ((r = grow(h, &h->rect, &h->tcap, T, "bin rectangles")) != PIKO_OK) return r;
+  if (h->ecap == 0 && (r = grow(h, &h->bin_tris, &h->ecap, (long long)T * 2 + 4096, "bin lists")) != PIKO_OK)
+    return r;
+
+  const bool ev = h->use_stage_ev;
+  h->use_stage_ev = false;
+  if (ev) cudaEventRecord(h->stage_ev[0], st);
+  if (h->stats) cudaMemsetAsync(&h->status->tests, 0, 4 * sizeof(unsigned long long), st);
+  float4* vattr = packed_attributes(h, s);
+  DirectRaster direct;
+  direct.keys = direct_keys(h, T, V, st);
+  direct.max_px = h->small_px < DIRECT_MAX_PX ? h->small_px : DIRECT_MAX_PX;
+  launch_vertex(h->W, h->H, V, s->pos, s->mvp, h->vtx, lambert ? s->normal : nullptr, s->light_dir,
+                lambert ? h->vdot : nullptr, h->perspective ? h->invw : nullptr, h->num_sms, st, direct.keys,
+                h->clip ? h->status : nullptr, s->color, vattr);
+  const bool other = h->schedule == PIKO_SCHED_FUSED || h->schedule == PIKO_SCHED_UNFUSED;
+  // With the capacity check the host has to see the bin-list size.  On a
+  // handle's first frame, or one of another triangle count, it waits for it
+  // before scattering, as the lists' size also sizes the Process stage's
+  // records; from then on the scatter and Process kernels are launched behind
+  // the scan, with the last size (they skip a frame whose lists overflowed),
+  // and the host reads the scan's report while they run.
+  const bool check = h->check_capacity != 0;
+  const bool ahead = check && !other && h->last_entries > 0 && h->last_tris == T;
+  if (h->clip && (r = clip_pass(h, s, st, check && !ahead, V > 0)) != PIKO_OK) return r;
+  if (ev) cudaEventRecord(h->stage_ev[1], st);
+  if (other) return forward_other_mapping(h, s, fb, st, ev);
+  bool clip_grown = false, bins_grown = false;
+  for (bool again = false;; again = true) {
+    if (h->stats && again) cudaMemsetAsync(&h->status->binned, 0, sizeof(unsigned long long), st);
+    const int4* clip_tris = h->clip ? h->clip_tris : nullptr;
+    const long long ccap = h->ccap_tris / 3 < h->ccap_orig ? h->ccap_tris / 3 : h->ccap_orig;
+    const unsigned clip_cap = h->clip ? (unsigned)ccap : 0u;
+    if (clip_cap && (r = grow(h, &h->rect, &h->tcap, (long long)T + clip_cap, "bin rectangles")) != PIKO_OK) return r;
+    direct.clip_orig = h->clip ? h->clip_orig : nullptr;
+    // a frame of one scan chunk of bins is scanned by the count pass's last
+    // CTA (one launch fewer on the chain); larger frames take the scan kernel
+    // (with stage events on, the count and scan launches stay apart)
+    const unsigned heavy_epoch = ++h->heavy_epoch, scan_epoch = ++h->scan_epoch;
+    ScanReport report;
+    if (check) {
+      report.host = h->h_needed;
+      report.tag = ++h->report_tag;
+    }
+    const bool fused = !ev && launch_count_and_scan(h->g, T, s->tris, V, h->vtx, h->rect, h->bin_count, h->status,
+                                                    h->stats, h->num_sms, st, clip_tris, clip_cap, h->exact_bins,
+                                                    h->heavy, heavy_cap(h), heavy_epoch, h->bin_off, h->cursor,
+                                                    (unsigned long long)h->ecap, h->chunk_state, scan_epoch, direct,
+                                                    report);
+    if (!fused) {
+      launch_setup_count(h->g, T, s->tris, V, h->vtx, h->rect, h->bin_count, h->status, h->stats, h->num_sms, st,
+                         clip_tris, clip_cap, h->exact_bins, h->heavy, heavy_cap(h), heavy_epoch, direct);
+      if (ev) cudaEventRecord(h->stage_ev[2], st);
+      launch_scan(h->nbins, h->bin_count, h->bin_off, h->cursor, (unsigned long long)h->ecap, h->status,
+                  h->chunk_state, scan_epoch, st, h->wait_budget, h->withhold, &report);
+      if (ev) cudaEventRecord(h->stage_ev[3], st);
+    }
+    bool fits = true;
+    for (int step = 0; step < 2; ++step) {
+      // ahead: launch, then look at the report; else the other way round
+      if ((step == 0) == ahead || !check) {
+        if ((r = scatter_and_process(h, s, fb, st, ev, direct, vattr, clip_tris, clip_cap)) != PIKO_OK) return r;
+        if (!check) return PIKO_OK;
+        continue;
+      }
+      if ((r = wait_report(h, st)) != PIKO_OK) return r;
+      const long long need = (long long)h->h_needed[0], clips = (long long)h->h_needed[2];
+      if (h->clip && clips > ccap) {
+        if (clip_grown) return fail(h, PIKO_ERR_OVERFLOW, "clipped triangle list too large");
+        clip_grown = true;
+        const long long want = clips + clips / 8 + 1024;
+        if ((r = grow(h, &h->clip_tris, &h->ccap_tris, 3 * want, "clipped triangles")) != PIKO_OK ||
+            (r = grow(h, &h->clip_orig, &h->ccap_orig, want, "clipped triangle indices")) != PIKO_OK)
+          return r;
+        fits = false;
+      } else if (need > h->ecap) {
+        if (bins_grown || need > 0xFFFFFFF0LL) return fail(h, PIKO_ERR_OVERFLOW, "bin lists too large");
+        bins_grown = true;
+        if ((r = grow(h, &h->bin_tris, &h->ecap, need, "bin lists")) != PIKO_OK) return r;
+        fits = false;
+      }
+      if (!fits) {
+        // the failed pass recorded an overflow and zeroed the counts: clear and count again
+        const cudaError_t e = cudaMemsetAsync(h->status, 0, sizeof(unsigned) * 2, st);
+        if (e != cudaSuccess) return cuda_fail(h, e, "status clear");
+        if (h->clip && clips > ccap && (r = clip_pass(h, s, st, false, false)) != PIKO_OK) return r;
+        break;
+      }
+      h->last_entries = h->h_needed[1] > 0 ? (long long)h->h_needed[1] : 1;
+      h->last_tris = T;
+    }
+    if (fits) return PIKO_OK;
+  }
 }
 
 int piko_raster_forward_host(piko_raster* h, const piko_scene* s, piko_framebuffer* fb, void* cuda_stream) {
@@ -670,12 +791,12 @@ int piko_raster_forward_batch(piko_raster* h, const piko_scene* scenes, int n, p
                                   h->withhold)) != PIKO_OK)
       return r;
     if (!h->check_capacity) return PIKO_OK;
-    cudaError_t e = cudaMemcpyAsync(h->h_needed, &h->status->needed, sizeof(unsigned long long),
+    cudaError_t e = cudaMemcpyAsync(h->h_needed, &h->status->needed, 2 * sizeof(unsigned long long),
                                     cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(h, e, "batch bin-list size read-back");
     const long long need = (long long)*h->h_needed;
-    batch_note_entries(h->batch, need);
+    batch_note_entries(h->batch, h->h_needed[1] > 0 ? (long long)h->h_needed[1] : 1);
     if (need <= batch_capacity(h->batch)) return PIKO_OK;
     if (attempt > 0 || need > 0xFFFFFFF0LL) return fail(h, PIKO_ERR_OVERFLOW, "batch bin lists too large");
     if ((r = batch_grow_entries(h->batch, need, h->err)) != PIKO_OK) return r;
@@ -735,23 +856,23 @@ int piko_raster_backward(piko_raster* h, const piko_scene* s, const piko_framebu
   if (!aligned16(dl_drgba)) return fail(h, PIKO_ERR_INVALID_ARG, "dl_drgba must be 16-byte aligned");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   h->last_stream = st;
-  if ((r = grow(h, &h->vtx, &h->vcap, s->num_vertices, "vertex buffer")) != PIKO_OK) return r;
-  if ((r = grow_gacc(h, s->num_vertices)) != PIKO_OK) return r;
+  if ((r = grow_vertices(h, s->num_vertices)) != PIKO_OK) return r;
   const bool lambert = s->shade_mode == PIKO_SHADE_LAMBERT;
-  if (lambert && (r = grow(h, &h->vdot, &h->dcap, s->num_vertices, "vertex light terms")) != PIKO_OK) return r;
-  if (h->perspective && (r = grow(h, &h->invw, &h->icap, s->num_vertices, "vertex 1/w")) != PIKO_OK) return r;
   float* invw = h->perspective ? h->invw : nullptr;
   if (h->gacc_dirty) {
-    const cudaError_t e = cudaMemsetAsync(h->gacc, 0, (size_t)h->gcap * sizeof(float4), st);
+    const cudaError_t e = cudaMemsetAsync(h->gacc, 0, (size_t)h->vcap * sizeof(float4), st);
     if (e != cudaSuccess) return cuda_fail(h, e, "gradient sums");
-    h->gacc_dirty = false;
+    // a captured clear has not run
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    h->gacc_dirty = cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
   }
   // the vertex stage runs again so that backward does not depend on which
   // scene the handle rasterized last
+  float4* vattr = packed_attributes(h, s);
   launch_vertex(h->W, h->H, s->num_vertices, s->pos, s->mvp, h->vtx, lambert ? s->normal : nullptr, s->light_dir,
-                lambert ? h->vdot : nullptr, invw, h->num_sms, st);
+                lambert ? h->vdot : nullptr, invw, h->num_sms, st, nullptr, nullptr, s->color, vattr);
   if (piko_backward_launch(h->W, h->H, s->shade_mode, h->unclamped, s->num_triangles, s->num_vertices, s->tris,
-                           h->vtx, h->vdot, s->color, s->normal, s->light_dir, invw, h->clip ? s->pos : nullptr,
+                           h->vtx, h->vdot, vattr, s->color, s->normal, s->light_dir, invw, h->clip ? s->pos : nullptr,
                            s->mvp, reinterpret_cast<const unsigned long long*>(fwd->key), dl_drgba, h->gacc, dl_dcolor,
                            dl_dnormal, dl_dlight, h->num_sms, st) != 0) {
     h->gacc_dirty = true;

@@ -16,8 +16,8 @@
 #include <string>
 #include <vector>
 
+#include "piko_direct.cuh"
 #include "piko_scan.cuh"
-#include "piko_tile.cuh"
 #include "piko_bwd_tile.cuh"
 
 namespace piko {
@@ -25,7 +25,9 @@ namespace piko {
 struct BatchScene {
   RasterGeom g;
   int V, T, mode, schedule;
-  int vtx_base, tri_base, bin_base, pix_base;
+  int vtx_base, tri_base, bin_base;
+  int direct;         // small triangles are rasterized by the count pass (piko_direct.cuh)
+  unsigned key_base;  // into the direct keys
   int slot_bits, nslots, rec_stride;
   int unclamped;  // Lambert without the clamp (the handle's option)
   const float4* pos;
@@ -60,12 +62,16 @@ struct BatchParams {
   const int* bin_prefix;
   const int* stat_prefix;  // tiles of static scenes
   const int* dyn_prefix;   // tiles of dynamic scenes
-  const int* btile_prefix;  // backward tiles (BWD_TILE_W x BATCH_BWD_TILE_H)
+  const int* btile_prefix;  // backward tiles (BWD_TILE_W x BATCH_BWD_TILE_H) of the tile form's scenes
+  const int* pblock_prefix;  // 8 x 4 pixel blocks of the pixel form's scenes
+  int total_pblocks;
   int total_v, total_t, total_bins, total_static, total_dyn, total_btiles;
   int4* vtx;
-  float* vdot;
+  float4* vattr;  // colour and n . L per vertex (Lambert; the colour only where the scene has one)
   float* invw;  // 1 / clip w per vertex (perspective-correct attributes), else NULL
   BinRect* rect;
+  unsigned long long* dkeys;  // a key per pixel of the scenes with direct rasterization
+  unsigned total_dkeys;
   unsigned* cnt;  // 2 * total_bins, zero between frames
   unsigned* bin_off;
   unsigned* cursor;
@@ -91,6 +97,15 @@ __device__ __forceinline__ int find_scene(const int* __restrict__ prefix, int n,
     else hi = mid;
   }
   return lo;
+}
+
+// find_scene for the item base + lane of a warp: one search, of the warp's
+// first item with every lane reading the same words, and a step per scene
+// boundary inside the warp (base is below the batch's total)
+__device__ __forceinline__ int find_scene_lane(const int* __restrict__ prefix, int n, int base, int i) {
+  int s = find_scene(prefix, n, base);
+  while (s + 1 < n && __ldg(prefix + s + 1) <= i) ++s;
+  return s;
 }
 
 __device__ __forceinline__ bool skip_flags(const DevStatus* st) {
@@ -150,8 +165,9 @@ __device__ bool cta_should_stop(const DevStatus* st) {
 // ------------------------------------------------------------------ phases
 template <bool PERSP>
 __device__ void phase_vertex(const BatchParams& b) {
+  if (b.total_dkeys) clear_keys(b.dkeys, b.total_dkeys);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < b.total_v; i += gridDim.x * blockDim.x) {
-    const int s = find_scene(b.vtx_prefix, b.n, i);
+    const int s = find_scene_lane(b.vtx_prefix, b.n, i & ~31, i);
     const BatchScene& d = b.sc[s];
     const int v = i - d.vtx_base;
     if (PERSP) {
@@ -163,7 +179,11 @@ __device__ void phase_vertex(const BatchParams& b) {
     }
     if (d.mode == PIKO_SHADE_LAMBERT) {
       const float* n = d.normal + 3 * (size_t)v;
-      b.vdot[i] = __ldg(n) * __ldg(d.light) + __ldg(n + 1) * __ldg(d.light + 1) + __ldg(n + 2) * __ldg(d.light + 2);
+      const float* c = d.color + 3 * (size_t)v;
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (d.color) a = make_float4(__ldg(c), __ldg(c + 1), __ldg(c + 2), 0.f);
+      a.w = __ldg(n) * __ldg(d.light) + __ldg(n + 1) * __ldg(d.light + 1) + __ldg(n + 2) * __ldg(d.light + 2);
+      b.vattr[i] = a;
     }
   }
 }
@@ -172,14 +192,21 @@ struct LaneBins {
   bool valid, single;
   int bx0, by0, bx1, by1;
   int nbx, bin_base;
+  unsigned dentries;  // bin entries a directly rasterized triangle would have had
 };
 
-__device__ __forceinline__ LaneBins lane_setup(const BatchParams& b, int t) {
+__device__ __forceinline__ LaneBins no_bins() {
   LaneBins r;
   r.valid = false; r.single = false;
   r.bx0 = 0; r.by0 = 0; r.bx1 = -1; r.by1 = -1; r.nbx = 1; r.bin_base = 0;
+  r.dentries = 0u;
+  return r;
+}
+
+__device__ __forceinline__ LaneBins lane_setup(const BatchParams& b, int t, int lane) {
+  LaneBins r = no_bins();
   if (t >= b.total_t) return r;
-  const int s = find_scene(b.tri_prefix, b.n, t);
+  const int s = find_scene_lane(b.tri_prefix, b.n, t - lane, t);
   const BatchScene& d = b.sc[s];
   r.nbx = d.g.nbx;
   r.bin_base = d.bin_base;
@@ -193,15 +220,21 @@ __device__ __forceinline__ LaneBins lane_setup(const BatchParams& b, int t) {
   const int4* vtx = b.vtx + d.vtx_base;
   const int4 p0 = __ldg(vtx + ia), p1 = __ldg(vtx + ib), p2 = __ldg(vtx + ic);
   if (!(p0.w & p1.w & p2.w)) return r;
-  const long long A = (long long)(p1.x - p0.x) * (p2.y - p0.y) - (long long)(p2.x - p0.x) * (p1.y - p0.y);
-  if (A == 0) return r;
+  const int minx = min(p0.x, min(p1.x, p2.x)), maxx = max(p0.x, max(p1.x, p2.x));
+  const int miny = min(p0.y, min(p1.y, p2.y)), maxy = max(p0.y, max(p1.y, p2.y));
   int px0, px1, py0, py1;
-  centre_range(min(p0.x, min(p1.x, p2.x)), max(p0.x, max(p1.x, p2.x)), 0, d.g.W - 1, px0, px1);
-  centre_range(min(p0.y, min(p1.y, p2.y)), max(p0.y, max(p1.y, p2.y)), 0, d.g.H - 1, py0, py1);
+  centre_range(minx, maxx, 0, d.g.W - 1, px0, px1);
+  centre_range(miny, maxy, 0, d.g.H - 1, py0, py1);
   if (px0 > px1 || py0 > py1) return r;
-  r.valid = true;
   r.bx0 = px0 >> d.g.bshift_x; r.bx1 = px1 >> d.g.bshift_x;
   r.by0 = py0 >> d.g.bshift_y; r.by1 = py1 >> d.g.bshift_y;
+  if (d.direct && direct_small(maxx - minx, maxy - miny, px0, px1, py0, py1, DIRECT_MAX_PX)) {
+    if (direct_triangle(p0, p1, p2, (unsigned)tl, px0, px1, py0, py1, d.g.W, b.dkeys + d.key_base))
+      r.dentries = (unsigned)((r.bx1 - r.bx0 + 1) * (r.by1 - r.by0 + 1));
+    return r;  // no bin entries
+  }
+  r.valid = (long long)(p1.x - p0.x) * (p2.y - p0.y) - (long long)(p2.x - p0.x) * (p1.y - p0.y) != 0;
+  if (!r.valid) return r;
   r.single = r.bx0 == r.bx1 && r.by0 == r.by1;
   return r;
 }
@@ -241,12 +274,18 @@ __device__ __forceinline__ void for_multi_pairs(const LaneBins& r, int lane, F&&
 
 __device__ void phase_count(const BatchParams& b) {
   const int lane = threadIdx.x & 31;
+  unsigned dentries = 0u;
   const unsigned lt_mask = (1u << lane) - 1u;
   const int warps_total = gridDim.x * (blockDim.x >> 5);
   for (int base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; base < b.total_t;
        base += warps_total * 32) {
     const int t = base + lane;
-    const LaneBins r = lane_setup(b, t);
+    const LaneBins r = lane_setup(b, t, lane);
+    dentries += r.dentries;
+    if (!__any_sync(FULL_MASK, r.valid)) {  // nothing to bin
+      if (t < b.total_t) b.rect[t] = BinRect{0xFFFFFFFFu, 0u};
+      continue;
+    }
     const unsigned bin = r.single ? (unsigned)(r.bin_base + r.by0 * r.nbx + r.bx0) : 0xFFFFFFFFu;
     const unsigned grp = __match_any_sync(FULL_MASK, bin);
     const int leader = __ffs(grp) - 1;
@@ -266,6 +305,8 @@ __device__ void phase_count(const BatchParams& b) {
     }
     for_multi_pairs(r, lane, [&](int, int gbin) { atomicAdd(b.cnt + b.total_bins + gbin, 1u); });
   }
+  const unsigned long long sum = __reduce_add_sync(FULL_MASK, dentries);
+  if (lane == 0 && sum) atomicAdd(&b.st->direct_entries, sum);
 }
 
 __device__ void phase_scan(const BatchParams& b, ScanSmem& sm) {
@@ -296,13 +337,11 @@ __device__ void phase_scatter(const BatchParams& b) {
   for (int base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; base < b.total_t;
        base += warps_total * 32) {
     const int t = base + lane;
-    LaneBins r;
-    r.valid = false; r.single = false;
-    r.bx0 = 0; r.by0 = 0; r.bx1 = -1; r.by1 = -1; r.nbx = 1; r.bin_base = 0;
+    LaneBins r = no_bins();
     if (t < b.total_t) {
       const BinRect q = b.rect[t];
       if (q.lo != 0xFFFFFFFFu) {
-        const BatchScene& d = b.sc[find_scene(b.tri_prefix, b.n, t)];
+        const BatchScene& d = b.sc[find_scene_lane(b.tri_prefix, b.n, base, t)];
         r.valid = true;
         r.nbx = d.g.nbx;
         r.bin_base = d.bin_base;
@@ -344,13 +383,15 @@ __device__ void load_tile_scene(const BatchParams& b, int s, TileScene& t) {
   t.color = d.color;
   t.normal = d.normal;
   t.light = d.light;
-  t.vdot = b.vdot + d.vtx_base;
+  t.vdot = nullptr;
+  t.vattr = b.vattr + d.vtx_base;
   t.invw = b.invw ? b.invw + d.vtx_base : nullptr;
   t.T = d.T;
   t.clip_tris = nullptr;  // batches do not clip
   t.clip_orig = nullptr;
   t.pos = nullptr;
   t.mvp = nullptr;
+  t.dkeys = d.direct ? b.dkeys + d.key_base : nullptr;
   t.key_out = d.key_out;
   t.rgba_out = d.rgba_out;
   t.gnorm_out = d.gnorm_out;
@@ -378,6 +419,7 @@ __device__ void process_one(const BatchParams& b, const int* prefix, int i, Proc
     __syncthreads();
     return;
   }
+  if (sc.dkeys && beg == end) shade_direct_tile<PERSP, false>(sc, ps.tile);
   process_tile<false, PERSP>(sc, ps.tile, beg, end, b.bin_tris, sm, big_base, st);
 }
 
@@ -462,8 +504,9 @@ __global__ void __maxnreg__(PIKO_BATCH_MAXNREG) k_batch_forward(BatchParams b) {
 struct BatchBwdParams {
   int n;
   const BatchScene* sc;
-  const int* btile_prefix;  // [n+1] backward tiles per scene
-  int total_btiles;
+  const int* btile_prefix;  // [n+1] backward tiles per scene (tile form; 0 for a scene of the pixel form)
+  const int* pblock_prefix;  // [n+1] 8 x 4 pixel blocks per scene (pixel form; else 0)
+  int total_btiles, total_pblocks;
   const int4* vtx;
   const float* invw;  // as in BatchParams
   // accumulators (GradAcc) of the finishing pass and the prefix of their chunks
@@ -471,6 +514,15 @@ struct BatchBwdParams {
   const GradAcc* groups;
   const int* chunk_prefix;
 };
+
+__device__ __forceinline__ void fill_bwd_scene(const BatchBwdParams& b, const BatchScene& d, BwdScene& c) {
+  c.W = d.g.W; c.H = d.g.H; c.mode = d.mode; c.unclamped = d.unclamped; c.T = d.T; c.V = d.V;
+  c.tris = d.tris; c.vtx = b.vtx + d.vtx_base; c.color = d.color; c.normal = d.normal; c.light = d.light;
+  c.invw = b.invw ? b.invw + d.vtx_base : nullptr;
+  c.pos = nullptr;  // batches do not clip
+  c.mvp = nullptr;
+  c.key = d.key_out; c.dl = d.dl; c.acc = d.acc;
+}
 
 // Warp form: each warp takes whole tiles (grid-stride over the batch's
 // tiles), with no CTA barrier; the scene of a tile is found by every lane
@@ -496,14 +548,7 @@ __global__ void __launch_bounds__(BWD_THREADS, PIKO_BWD_MINB) k_batch_backward(B
     const BatchScene& d = b.sc[s];
     if (d.acc == nullptr) continue;  // the same for the whole warp
     __syncwarp();  // the previous tile's reads of c are done
-    if (lane == 0) {
-      c.W = d.g.W; c.H = d.g.H; c.mode = d.mode; c.unclamped = d.unclamped; c.T = d.T; c.V = d.V;
-      c.tris = d.tris; c.vtx = b.vtx + d.vtx_base; c.color = d.color; c.normal = d.normal; c.light = d.light;
-      c.invw = b.invw ? b.invw + d.vtx_base : nullptr;
-      c.pos = nullptr;  // batches do not clip
-      c.mvp = nullptr;
-      c.key = d.key_out; c.dl = d.dl; c.acc = d.acc;
-    }
+    if (lane == 0) fill_bwd_scene(b, d, c);
     __syncwarp();
     float L0 = 0.f, L1 = 0.f, L2 = 0.f;
     if (c.mode == PIKO_SHADE_LAMBERT) {
@@ -517,6 +562,41 @@ __global__ void __launch_bounds__(BWD_THREADS, PIKO_BWD_MINB) k_batch_backward(B
   }
 }
 constexpr size_t BATCH_BWD_SMEM = sizeof(BatchBwdSmem);
+
+// Pixel form: a warp takes BATCH_PIX_RUN blocks of 8 x 4 pixels in a row, so
+// that it looks its scene up once for most of them.
+constexpr int BATCH_PIX_RUN = 4;
+template <bool PERSP>
+__global__ void __launch_bounds__(PIX_THREADS, 4) k_batch_backward_pixel(BatchBwdParams b) {
+  __shared__ float sval[PIX_THREADS / 32][BWD_VALS][32];
+  __shared__ BwdScene ssc[PIX_THREADS / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int first = (blockIdx.x * (PIX_THREADS / 32) + warp) * BATCH_PIX_RUN;
+  if (first >= b.total_pblocks) return;  // the same for the whole warp
+  BwdScene& c = ssc[warp];
+  int s = find_scene(b.pblock_prefix, b.n, first), held = -1;
+  float L0 = 0.f, L1 = 0.f, L2 = 0.f;
+  for (int i = first; i < min(first + BATCH_PIX_RUN, b.total_pblocks); ++i) {
+    while (s + 1 < b.n && __ldg(b.pblock_prefix + s + 1) <= i) ++s;
+    const BatchScene& d = b.sc[s];
+    if (d.acc == nullptr) continue;
+    if (s != held) {
+      __syncwarp();  // the previous scene's reads of c are done
+      if (lane == 0) fill_bwd_scene(b, d, c);
+      __syncwarp();
+      held = s;
+      if (c.mode == PIKO_SHADE_LAMBERT) {
+        L0 = __ldg(c.light); L1 = __ldg(c.light + 1); L2 = __ldg(c.light + 2);
+      }
+    }
+    const int lt = i - __ldg(b.pblock_prefix + s);
+    const int ntx = (c.W + PIX_W - 1) / PIX_W;
+    const int ty = lt / ntx, tx = lt - ty * ntx;
+    backward_warp_pixels<PERSP>(c, nullptr, nullptr, tx * PIX_W + (lane & (PIX_W - 1)), ty * PIX_H + lane / PIX_W, sval[warp], L0,
+                                L1, L2);
+    __syncwarp();  // sval is rewritten by the next block
+  }
+}
 
 // Sums of all vertices into the gradient arrays, a chunk of one group per CTA step.
 __global__ void __launch_bounds__(GRAD_CHUNK) k_batch_finish(BatchBwdParams b) {
@@ -553,7 +633,7 @@ struct BatchState {
   size_t desc_cap = 0;
   int4* vtx = nullptr;
   long long vcap = 0;
-  float* vdot = nullptr;
+  float4* vattr = nullptr;
   long long dcap = 0;
   float* invw = nullptr;
   long long icap = 0;
@@ -566,15 +646,17 @@ struct BatchState {
   long long bcap = 0;  // bins
   unsigned* bin_tris = nullptr;
   long long ecap = 0;
+  unsigned long long* dkeys = nullptr;  // keys of direct rasterization
+  long long dkcap = 0;
   float4* gacc = nullptr;  // gradient sums, zero between calls
   long long gcap = 0;
-  bool gacc_dirty = false;  // a failed backward launch may have left sums behind
+  bool gacc_dirty = false;  // gacc is not zero: new, or a backward launch failed
   BatchSync* sync = nullptr;
   unsigned epoch = 0;
   // host staging (pinned) and the last layout
   void* staging = nullptr;
   size_t staging_cap = 0;
-  size_t desc_bytes = 0;   // of the last layout: scenes, 6 prefix arrays, gradient groups and their prefix
+  size_t desc_bytes = 0;   // of the last layout: scenes, 7 prefix arrays, gradient groups and their prefix
   size_t group_off = 0;    // where the gradient groups start
   cudaEvent_t uploaded = nullptr;
   BatchParams params;
@@ -621,7 +703,7 @@ void batch_state_free(BatchState* bs) {
   if (!bs) return;
   cudaFree(bs->desc);
   cudaFree(bs->vtx);
-  cudaFree(bs->vdot);
+  cudaFree(bs->vattr);
   cudaFree(bs->invw);
   cudaFree(bs->rect);
   cudaFree(bs->cnt);
@@ -630,6 +712,7 @@ void batch_state_free(BatchState* bs) {
   cudaFree(bs->chunk_state);
   cudaFree(bs->bin_tris);
   cudaFree(bs->gacc);
+  cudaFree(bs->dkeys);
   cudaFree(bs->sync);
   if (bs->staging) cudaFreeHost(bs->staging);
   if (bs->uploaded) cudaEventDestroy(bs->uploaded);
@@ -645,8 +728,8 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   if (!bs) bs = new BatchState();
   if (n < 1 || !scenes || !fbs) { err = "batch needs n >= 1 scenes and framebuffers"; return PIKO_ERR_INVALID_ARG; }
   std::vector<BatchScene> d(n);
-  std::vector<int> pv(n + 1), pt(n + 1), pb(n + 1), ps(n + 1), pd(n + 1), pp(n + 1);
-  long long tv = 0, tt = 0, tb = 0, tsd = 0, tdy = 0, tp = 0;
+  std::vector<int> pv(n + 1), pt(n + 1), pb(n + 1), ps(n + 1), pd(n + 1), pp(n + 1), pq(n + 1);
+  long long tv = 0, tt = 0, tb = 0, tsd = 0, tdy = 0, tp = 0, tq = 0, tk = 0;
   int max_bin_px = 64, max_rec = 0;
   // shading records per tile from the last frame's mean entries per bin
   const int slots_hint = bs ? slots_for_entries(bs->last_entries, (int)(bs->last_bins > 0 ? bs->last_bins : 1)) : 0;
@@ -673,7 +756,14 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
     x.g.bshift_x = ilog2i(bw); x.g.bshift_y = ilog2i(bh);
     x.g.nbx = (s.width + bw - 1) / bw; x.g.nby = (s.height + bh - 1) / bh;
     x.V = s.num_vertices; x.T = s.num_triangles; x.mode = s.shade_mode; x.schedule = sched;
-    x.vtx_base = (int)tv; x.tri_base = (int)tt; x.bin_base = (int)tb; x.pix_base = 0;
+    x.vtx_base = (int)tv; x.tri_base = (int)tt; x.bin_base = (int)tb;
+    // key indices are 32-bit; scenes past that, or without the memory below, bin every triangle
+    const long long px = (long long)s.width * s.height;
+    if (direct_scene(x.T, x.V, s.width, s.height) && tk + px < (1LL << 32)) {
+      x.direct = 1;
+      x.key_base = (unsigned)tk;
+      tk += px;
+    }
     tile_layout(s.num_triangles, bw * bh, s.shade_mode, s.color != nullptr, persp != 0, 255, x.slot_bits, x.nslots,
                 x.rec_stride, slots_hint);
     x.unclamped = unclamped;
@@ -684,28 +774,32 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
     x.gnorm_out = reinterpret_cast<uint2*>(f.gbuf_normal);
     x.galb_out = reinterpret_cast<uint2*>(f.gbuf_albedo);
     const int ntiles = x.g.nbx * x.g.nby;
-    pv[i] = (int)tv; pt[i] = (int)tt; pb[i] = (int)tb; ps[i] = (int)tsd; pd[i] = (int)tdy; pp[i] = (int)tp;
+    pv[i] = (int)tv; pt[i] = (int)tt; pb[i] = (int)tb; ps[i] = (int)tsd; pd[i] = (int)tdy; pp[i] = (int)tp; pq[i] = (int)tq;
     tv += x.V; tt += x.T; tb += ntiles;
-    tp += (long long)((s.width + BWD_TILE_W - 1) / BWD_TILE_W) *
-          ((s.height + BATCH_BWD_TILE_H - 1) / BATCH_BWD_TILE_H);
+    if (bwd_pixel_form(x.T, s.width, s.height))
+      tq += (long long)((s.width + PIX_W - 1) / PIX_W) * ((s.height + PIX_H - 1) / PIX_H);
+    else
+      tp += (long long)((s.width + BWD_TILE_W - 1) / BWD_TILE_W) *
+            ((s.height + BATCH_BWD_TILE_H - 1) / BATCH_BWD_TILE_H);
     if (sched == PIKO_SCHED_STATIC) tsd += ntiles;
     else tdy += ntiles;
     if (bw * bh > max_bin_px) max_bin_px = bw * bh;
     if (x.nslots * x.rec_stride > max_rec) max_rec = x.nslots * x.rec_stride;
   }
-  pv[n] = (int)tv; pt[n] = (int)tt; pb[n] = (int)tb; ps[n] = (int)tsd; pd[n] = (int)tdy; pp[n] = (int)tp;
-  if (tv >= (1LL << 31) || tt >= (1LL << 31) || tb >= (1LL << 31) || tp >= (1LL << 31)) {
+  pv[n] = (int)tv; pt[n] = (int)tt; pb[n] = (int)tb; ps[n] = (int)tsd; pd[n] = (int)tdy; pp[n] = (int)tp; pq[n] = (int)tq;
+  if (tv >= (1LL << 31) || tt >= (1LL << 31) || tb >= (1LL << 31) || tp + tq >= (1LL << 31)) {
     err = "batch too large (a total reaches 2^31)";
     return PIKO_ERR_INVALID_ARG;
   }
   // device scratch
   int r;
   if ((r = grow_dev(&bs->vtx, &bs->vcap, tv, false, err)) != PIKO_OK) return r;
-  if ((r = grow_dev(&bs->vdot, &bs->dcap, tv, false, err)) != PIKO_OK) return r;
+  if ((r = grow_dev(&bs->vattr, &bs->dcap, tv, false, err)) != PIKO_OK) return r;
   if (persp && (r = grow_dev(&bs->invw, &bs->icap, tv, false, err)) != PIKO_OK) return r;
   if ((r = grow_dev(&bs->rect, &bs->tcap, tt, false, err)) != PIKO_OK) return r;
   // here and not in the backward call, which may be recorded into a graph
-  if ((r = grow_dev(&bs->gacc, &bs->gcap, tv, true, err)) != PIKO_OK) return r;
+  if (tv > bs->gcap) bs->gacc_dirty = true;
+  if ((r = grow_dev(&bs->gacc, &bs->gcap, tv, false, err)) != PIKO_OK) return r;
   if (tb > bs->bcap) {
     // counts must start at zero; offsets/cursors/chunk states are rewritten
     cudaFree(bs->cnt); cudaFree(bs->bin_off); cudaFree(bs->cursor); cudaFree(bs->chunk_state);
@@ -724,6 +818,14 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
     }
     bs->bcap = cap;
   }
+  cudaStreamCaptureStatus cap_status = cudaStreamCaptureStatusNone;
+  cudaStreamIsCapturing(stream, &cap_status);
+  if (tk > bs->dkcap && (cap_status != cudaStreamCaptureStatusNone ||
+                         grow_dev(&bs->dkeys, &bs->dkcap, tk, false, err) != PIKO_OK)) {
+    err.clear();
+    tk = 0;
+    for (BatchScene& x : d) x.direct = 0;
+  }
   if (bs->ecap == 0 && (r = grow_dev(&bs->bin_tris, &bs->ecap, 2 * tt + 4096, false, err)) != PIKO_OK) return r;
   if (!bs->sync) {
     if (cudaMalloc(&bs->sync, sizeof(BatchSync)) != cudaSuccess || cudaMemset(bs->sync, 0, sizeof(BatchSync)) != cudaSuccess) {
@@ -731,18 +833,16 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
       return PIKO_ERR_OOM;
     }
   }
-  // descriptors + 6 prefix arrays, uploaded from pinned memory; room after
+  // descriptors + 7 prefix arrays, uploaded from pinned memory; room after
   // them for the backward's gradient groups and their prefix
   const size_t dbytes = sizeof(BatchScene) * n;
   const size_t pbytes = sizeof(int) * (n + 1);
-  const size_t group_off = (dbytes + 6 * pbytes + 15) / 16 * 16;
+  const size_t group_off = (dbytes + 7 * pbytes + 15) / 16 * 16;
   const size_t total = group_off + sizeof(GradAcc) * n + pbytes;
   if (!bs->uploaded && cudaEventCreateWithFlags(&bs->uploaded, cudaEventDisableTiming) != cudaSuccess) {
     err = "cudaEventCreate failed";
     return PIKO_ERR_CUDA;
   }
-  cudaStreamCaptureStatus cap_status = cudaStreamCaptureStatusNone;
-  cudaStreamIsCapturing(stream, &cap_status);
   if (cap_status == cudaStreamCaptureStatusNone && bs->staging) cudaEventSynchronize(bs->uploaded);
   if (total > bs->staging_cap) {
     if (cap_status != cudaStreamCaptureStatusNone) {
@@ -762,8 +862,8 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   }
   char* h = static_cast<char*>(bs->staging);
   std::memcpy(h, d.data(), dbytes);
-  const std::vector<int>* arrays[6] = {&pv, &pt, &pb, &ps, &pd, &pp};
-  for (int a = 0; a < 6; ++a) std::memcpy(h + dbytes + a * pbytes, arrays[a]->data(), pbytes);
+  const std::vector<int>* arrays[7] = {&pv, &pt, &pb, &ps, &pd, &pp, &pq};
+  for (int a = 0; a < 7; ++a) std::memcpy(h + dbytes + a * pbytes, arrays[a]->data(), pbytes);
   if (cudaMemcpyAsync(bs->desc, bs->staging, group_off, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
       cudaEventRecord(bs->uploaded, stream) != cudaSuccess) {
     err = "upload of batch descriptors failed";
@@ -780,9 +880,12 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   b.stat_prefix = reinterpret_cast<const int*>(dd + dbytes + 3 * pbytes);
   b.dyn_prefix = reinterpret_cast<const int*>(dd + dbytes + 4 * pbytes);
   b.btile_prefix = reinterpret_cast<const int*>(dd + dbytes + 5 * pbytes);
+  b.pblock_prefix = reinterpret_cast<const int*>(dd + dbytes + 6 * pbytes);
+  b.total_pblocks = (int)tq;
   b.total_v = (int)tv; b.total_t = (int)tt; b.total_bins = (int)tb; b.total_static = (int)tsd;
   b.total_dyn = (int)tdy; b.total_btiles = (int)tp;
-  b.vtx = bs->vtx; b.vdot = bs->vdot; b.invw = persp ? bs->invw : nullptr; b.rect = bs->rect; b.cnt = bs->cnt; b.bin_off = bs->bin_off;
+  b.vtx = bs->vtx; b.vattr = bs->vattr; b.invw = persp ? bs->invw : nullptr; b.rect = bs->rect; b.cnt = bs->cnt; b.bin_off = bs->bin_off;
+  b.dkeys = bs->dkeys; b.total_dkeys = (unsigned)tk;
   b.cursor = bs->cursor; b.chunk_state = bs->chunk_state; b.bin_tris = bs->bin_tris;
   b.capacity = (unsigned long long)bs->ecap; b.sync = bs->sync;
   b.max_bin_px = max_bin_px;
@@ -929,7 +1032,9 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
       err = "gradient sums reset failed";
       return PIKO_ERR_CUDA;
     }
-    bs->gacc_dirty = false;
+    // a captured clear has not run
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    bs->gacc_dirty = cudaStreamIsCapturing(stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
   }
   cudaStreamCaptureStatus cap_status = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(stream, &cap_status);
@@ -950,6 +1055,8 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
   p.sc = bs->params.sc;
   p.btile_prefix = bs->params.btile_prefix;
   p.total_btiles = bs->params.total_btiles;
+  p.pblock_prefix = bs->params.pblock_prefix;
+  p.total_pblocks = bs->params.total_pblocks;
   p.vtx = bs->vtx;
   p.invw = bs->params.invw;  // the interpolation of the last forward_batch
   p.ngroups = (int)groups.size();
@@ -976,11 +1083,20 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
   long long blocks = (long long)per_sm * num_sms;
   const long long need = (p.total_btiles + BATCH_BWD_WARPS - 1) / BATCH_BWD_WARPS;  // a tile per warp
   if (blocks > need) blocks = need;
-  if (blocks < 1) blocks = 1;
-  if (bs->persp)
-    k_batch_backward<true><<<(int)blocks, BWD_THREADS, BATCH_BWD_SMEM, stream>>>(p);
-  else
-    k_batch_backward<false><<<(int)blocks, BWD_THREADS, BATCH_BWD_SMEM, stream>>>(p);
+  if (p.total_btiles > 0) {
+    if (bs->persp)
+      k_batch_backward<true><<<(int)blocks, BWD_THREADS, BATCH_BWD_SMEM, stream>>>(p);
+    else
+      k_batch_backward<false><<<(int)blocks, BWD_THREADS, BATCH_BWD_SMEM, stream>>>(p);
+  }
+  if (p.total_pblocks > 0) {
+    const int per_cta = PIX_THREADS / 32 * BATCH_PIX_RUN;
+    const int pblocks = (p.total_pblocks + per_cta - 1) / per_cta;
+    if (bs->persp)
+      k_batch_backward_pixel<true><<<pblocks, PIX_THREADS, 0, stream>>>(p);
+    else
+      k_batch_backward_pixel<false><<<pblocks, PIX_THREADS, 0, stream>>>(p);
+  }
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)
     e = launch_pdl(k_batch_finish, p.total_chunks < 8 * num_sms ? p.total_chunks : 8 * num_sms, GRAD_CHUNK, 0, stream, p);

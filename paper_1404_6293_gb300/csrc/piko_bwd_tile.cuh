@@ -347,4 +347,141 @@ __device__ __forceinline__ void backward_warp_tile(const BwdScene& sc, int x0, i
   if (__any_sync(FULL_MASK, ends)) bwd_run_flush(sc, ends, cur, r, acc, stage);
 }
 
+// ---------------------------------------------------------------- pixel form
+// For scenes of tiny triangles (a tile would hold nearly as many triangles as
+// pixels, so the tile form's runs are a pixel or two long): a warp takes an
+// 8 x 4 block of pixels, which shares more winners than a row of 32; lanes
+// whose pixels share a winning triangle are summed in shared memory and one
+// lane adds the sums to the three vertices' accumulators.  Bound by the latency
+// of its gathers (key, indices, vertices) and by the L2's reductions, so every
+// block is its own warp and CTAs are many.
+constexpr int PIX_THREADS = 256;
+constexpr int PIX_W = 8, PIX_H = 4;  // pixels of a warp
+
+// Scenes with a triangle for every 16 pixels or fewer take the pixel form (in
+// a batch of 64 uneven scenes the line at 4 pixels took 895 us, at 16 815 us).
+__host__ __device__ inline bool bwd_pixel_form(int T, int W, int H) { return 16LL * T > (long long)W * H; }
+
+// Pixel (x, y) of each lane; sval is the warp's own staging area.  vattr:
+// colour and n . L per vertex; without it vdot: n . L; without both it is
+// formed from the normals and the light (L0, L1, L2).
+template <bool PERSP>
+__device__ __forceinline__ void backward_warp_pixels(const BwdScene& sc, const float* __restrict__ vdot,
+                                                     const float4* __restrict__ vattr, int x, int y, float (*sval)[32], float L0, float L1, float L2) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt_mask = (1u << lane) - 1u;
+  // the key and dL/drgba do not come from the vertex stage before this kernel
+  const size_t o = (size_t)y * sc.W + x;
+  unsigned t = BWD_NONE;
+  float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (x < sc.W && y < sc.H) {
+    t = __ldg(reinterpret_cast<const unsigned*>(sc.key) + 2 * o);  // the key's triangle word
+    g = __ldg(sc.dl + o);
+  }
+  // a key naming a triangle outside this scene, or one the vertex stage
+  // culls, contributes nothing (it cannot come from this scene's forward)
+  bool hit = t < (unsigned)sc.T;
+  int ia = 0, ib = 0, ic = 0;
+  if (hit) {
+    ia = __ldg(sc.tris + 3 * (size_t)t); ib = __ldg(sc.tris + 3 * (size_t)t + 1); ic = __ldg(sc.tris + 3 * (size_t)t + 2);
+  }
+  pdl_wait();  // snapped vertices and light terms
+  pdl_launch_dependents();
+  TriSetup s;
+  s.v0 = s.v1 = s.v2 = 0;
+  bool clipped = false;
+  if (hit) {
+    const bool in_range = ia >= 0 && ia < sc.V && ib >= 0 && ib < sc.V && ic >= 0 && ic < sc.V;
+    hit = in_range && setup_triangle(ia, ib, ic, sc.vtx, s);
+    if (!hit && in_range && sc.pos) {  // a winner the vertex stage rejected was clipped
+      clipped = hit = true;
+      s.v0 = ia; s.v1 = ib; s.v2 = ic;
+    }
+  }
+  if (!hit) t = BWD_NONE;
+  float v[BWD_VALS];
+#pragma unroll
+  for (int q = 0; q < BWD_VALS; ++q) v[q] = 0.f;
+  if (hit) {
+    const int vid[3] = {s.v0, s.v1, s.v2};
+    float b[3];
+    if (clipped) {
+      clip_ray_weights(sc.pos, sc.mvp, sc.W, sc.H, vid, x, y, b[0], b[1], b[2]);
+    } else {
+      const float fA = f32_from_i64(s.A);
+      if (s.A < (1LL << 31)) {  // the covered pixel's edge functions lie in [0, A]: exact in 32 bits
+        const int Px = 256 * x + 128, Py = 256 * y + 128;
+        const int w1 = edge_fn_wrap32(s.X2, s.Y2, s.X0, s.Y0, Px, Py), w2 = edge_fn_wrap32(s.X0, s.Y0, s.X1, s.Y1, Px, Py);
+        b[0] = __fdiv_rn((float)((int)s.A - w1 - w2), fA);
+        b[1] = __fdiv_rn((float)w1, fA);
+        b[2] = __fdiv_rn((float)w2, fA);
+      } else {
+        const long long Px = 256LL * x + 128, Py = 256LL * y + 128;
+        const long long w1 = (long long)(s.X0 - s.X2) * (Py - s.Y2) - (long long)(s.Y0 - s.Y2) * (Px - s.X2);
+        const long long w2 = (long long)(s.X1 - s.X0) * (Py - s.Y0) - (long long)(s.Y1 - s.Y0) * (Px - s.X0);
+        b[0] = __fdiv_rn(f32_from_i64(s.A - w1 - w2), fA);
+        b[1] = __fdiv_rn(f32_from_i64(w1), fA);
+        b[2] = __fdiv_rn(f32_from_i64(w2), fA);
+      }
+      if (PERSP)
+        perspective_bary(b[0], b[1], b[2], __ldg(sc.invw + vid[0]), __ldg(sc.invw + vid[1]), __ldg(sc.invw + vid[2]));
+    }
+    if (sc.mode == PIKO_SHADE_GOURAUD) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        v[3 * j] = g.x * b[j]; v[3 * j + 1] = g.y * b[j]; v[3 * j + 2] = g.z * b[j];
+      }
+    } else {
+      float a0 = 0.80f, a1 = 0.75f, a2 = 0.65f;  // material of Listing 1 without colours
+      float d = 0.f;                             // n . L = sum_j b_j (n_j . L), by linearity
+      if (sc.color) a0 = a1 = a2 = 0.f;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        if (vattr) {
+          const float4 q = __ldg(vattr + vid[j]);
+          a0 += b[j] * q.x; a1 += b[j] * q.y; a2 += b[j] * q.z;
+          d += b[j] * q.w;
+          continue;
+        }
+        if (sc.color) {
+          const float* c = sc.color + 3 * (size_t)vid[j];
+          a0 += b[j] * __ldg(c); a1 += b[j] * __ldg(c + 1); a2 += b[j] * __ldg(c + 2);
+        }
+        const float* nj = sc.normal + 3 * (size_t)vid[j];
+        d += b[j] * (vdot ? __ldg(vdot + vid[j]) : __ldg(nj) * L0 + __ldg(nj + 1) * L1 + __ldg(nj + 2) * L2);
+      }
+      const bool active = sc.unclamped || d > 0.f;
+      const float sh = sc.unclamped ? d : fmaxf(d, 0.f);
+      const float G = active ? (g.x * a0 + g.y * a1 + g.z * a2) : 0.f;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        if (sc.color) {
+          v[3 * j] = g.x * sh * b[j]; v[3 * j + 1] = g.y * sh * b[j]; v[3 * j + 2] = g.z * sh * b[j];
+        }
+        v[9 + j] = G * b[j];
+      }
+    }
+  }
+  // group lanes by winning triangle; the lowest lane of each group sums
+  // the group's contributions and adds them to the vertices
+  const unsigned grp = __match_any_sync(FULL_MASK, t);
+  const bool leader = hit && (grp & lt_mask) == 0u;
+  const bool alone = __popc(grp) == 1;
+  if (!alone) {
+#pragma unroll
+    for (int q = 0; q < BWD_VALS; ++q) sval[q][lane] = v[q];
+  }
+  __syncwarp();
+  if (leader) {
+    for (unsigned rest = grp & ~(1u << lane); rest; rest &= rest - 1) {
+      const int src = __ffs(rest) - 1;
+#pragma unroll
+      for (int q = 0; q < BWD_VALS; ++q) v[q] += sval[q][src];
+    }
+    grad_add(sc.acc + s.v0, v[0], v[1], v[2], v[9]);
+    grad_add(sc.acc + s.v1, v[3], v[4], v[5], v[10]);
+    grad_add(sc.acc + s.v2, v[6], v[7], v[8], v[11]);
+  }
+}
+
 }  // namespace piko

@@ -9,6 +9,7 @@
 //   k_scatter      triangle indices into the bin lists
 // The per-tile Process stage is in piko_process.cu.
 
+#include "piko_direct.cuh"
 #include "piko_scan.cuh"
 
 namespace piko {
@@ -20,7 +21,9 @@ template <bool INVW>
 __global__ void __launch_bounds__(256) k_vertex(int W, int H, int V, const float4* __restrict__ pos,
                                                 const float* __restrict__ mvp, int4* __restrict__ vtx,
                                                 const float* __restrict__ normal, const float* __restrict__ light,
-                                                float* __restrict__ vdot, float* __restrict__ invw) {
+                                                float* __restrict__ vdot, float* __restrict__ invw,
+                                                unsigned long long* __restrict__ dkeys, DevStatus* clip_st,
+                                                const float* __restrict__ color, float4* __restrict__ vattr) {
   pdl_launch_dependents();  // the count pass may be scheduled; it waits for this grid before reading
   __shared__ float m[16];
   const bool has_m = mvp != nullptr;
@@ -28,14 +31,22 @@ __global__ void __launch_bounds__(256) k_vertex(int W, int H, int V, const float
     if (threadIdx.x < 16) m[threadIdx.x] = mvp[threadIdx.x];
     __syncthreads();
   }
+  if (dkeys) clear_keys(dkeys, (size_t)W * H);
+  if (clip_st && blockIdx.x == 0 && threadIdx.x == 0) clip_st->clip_count = 0u;
   const float fW = (float)W, fH = (float)H;
   float L0 = 0.f, L1 = 0.f, L2 = 0.f;
   if (vdot) {
     L0 = __ldg(light); L1 = __ldg(light + 1); L2 = __ldg(light + 2);
   }
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < V; i += gridDim.x * blockDim.x) {
-    if (vdot) vdot[i] = __ldg(normal + 3 * (size_t)i) * L0 + __ldg(normal + 3 * (size_t)i + 1) * L1 +
-                        __ldg(normal + 3 * (size_t)i + 2) * L2;
+    if (vdot) {
+      const size_t j = 3 * (size_t)i;
+      const float d = __ldg(normal + j) * L0 + __ldg(normal + j + 1) * L1 + __ldg(normal + j + 2) * L2;
+      if (vattr)
+        vattr[i] = make_float4(__ldg(color + j), __ldg(color + j + 1), __ldg(color + j + 2), d);
+      else
+        vdot[i] = d;
+    }
     // one 16-byte load per vertex, coalesced across the warp
     if (INVW) {
       float w;
@@ -50,17 +61,19 @@ __global__ void __launch_bounds__(256) k_vertex(int W, int H, int V, const float
 }
 
 void launch_vertex(int W, int H, int V, const float* pos, const float* mvp, int4* vtx, const float* normal,
-                   const float* light, float* vdot, float* invw, int num_sms, cudaStream_t s) {
+                   const float* light, float* vdot, float* invw, int num_sms, cudaStream_t s,
+                   unsigned long long* dkeys, DevStatus* clip_st, const float* color, float4* vattr) {
   if (V <= 0) return;
-  // one vertex per thread: every load is in flight at once
-  (void)num_sms;
-  const int blocks = (V + 255) / 256;
+  // one vertex per thread: every load is in flight at once; at least a wave
+  // of CTAs when there are keys to clear
+  int blocks = (V + 255) / 256;
+  if (dkeys && blocks < 8 * num_sms) blocks = 8 * num_sms;
   if (invw)
     k_vertex<true><<<blocks, 256, 0, s>>>(W, H, V, reinterpret_cast<const float4*>(pos), mvp, vtx, normal, light, vdot,
-                                          invw);
+                                          invw, dkeys, clip_st, color, vattr);
   else
     k_vertex<false><<<blocks, 256, 0, s>>>(W, H, V, reinterpret_cast<const float4*>(pos), mvp, vtx, normal, light,
-                                           vdot, nullptr);
+                                           vdot, nullptr, dkeys, clip_st, color, vattr);
 }
 
 // ======================================================================
@@ -333,7 +346,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan(int nbins, unsigned* __re
                                                        unsigned* __restrict__ bin_off, unsigned* __restrict__ cursor,
                                                        unsigned long long capacity, DevStatus* st,
                                                        unsigned long long* __restrict__ chunk_state, unsigned epoch,
-                                                       long long wait_budget, int withhold) {
+                                                       long long wait_budget, int withhold, ScanReport report) {
   __shared__ ScanSmem sm;
   pdl_wait();  // counts and the ticket reset of the count pass
   pdl_launch_dependents();
@@ -343,7 +356,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan(int nbins, unsigned* __re
   const int nchunks = (nbins + SCAN_CHUNK - 1) / SCAN_CHUNK;
   if (chunk >= nchunks) return;  // only with a corrupted ticket; the count pass resets it every frame
   scan_chunk(chunk, nchunks, nbins, cnt, bin_off, cursor, capacity, st, chunk_state, epoch, sm, &st->queue_head,
-             wait_budget, withhold);
+             wait_budget, withhold, report);
   // one CTA per chunk: every ticket was taken before the last chunk's
   // look-back ended, so the last chunk may reset the ticket
   if (chunk == nchunks - 1 && threadIdx.x == 0) st->scan_ticket = 0u;
@@ -375,34 +388,57 @@ __device__ __forceinline__ TriVerts gather_verts(int3 idx, int V, const int4* __
   return v;
 }
 
+// The vertices of frame triangle t (of T input triangles, idx its indices,
+// and clipped sub-triangles up to TT), or in_range false.
+__device__ __forceinline__ TriVerts fetch_tri(int T, int TT, int t, int3 idx, int V, const int4* __restrict__ vtx,
+                                              const int4* __restrict__ clip_tris) {
+  TriVerts v = gather_verts(idx, V, vtx, t < T);
+  if (t >= T && t < TT) {  // a clipped sub-triangle: its snapped points
+    const int4* c = clip_tris + 3 * (size_t)(t - T);
+    v.p0 = c[0]; v.p1 = c[1]; v.p2 = c[2];
+    v.in_range = true;
+  }
+  return v;
+}
+
 // Count-pass work for one batch of 32 triangles (one per lane).  EXACT:
-// multi-bin pairs pass the exact overlap test first.
-template <bool EXACT>
-__device__ __forceinline__ void count_batch(const RasterGeom& g, int T, int t, int3 idx, const TriVerts& v,
+// multi-bin pairs pass the exact overlap test first.  DIRECT: triangles of a
+// few pixels are rasterized here into the direct keys (piko_direct.cuh) and
+// get no bin entries; *dentries counts those they would have had.
+template <bool EXACT, bool DIRECT>
+__device__ __forceinline__ void count_batch(const RasterGeom& g, int T, int t, const TriVerts& v,
                                             BinRect* __restrict__ rect, unsigned* __restrict__ cnt, int nbins,
                                             DevStatus* st, int stats, int lane, unsigned lt_mask,
-                                            uint2* __restrict__ heavy, unsigned heavy_cap, unsigned* heavy_n) {
+                                            uint2* __restrict__ heavy, unsigned heavy_cap, unsigned* heavy_n,
+                                            const DirectRaster& direct, unsigned key_tri, unsigned* dentries) {
   bool valid = false;
+
   int bx0 = 0, by0 = 0, bx1 = -1, by1 = -1;
   if (t < T) {
     if (!v.in_range) {
       record_error(st, PIKO_ERR_BAD_INDEX);
     } else if (v.p0.w & v.p1.w & v.p2.w) {
-      const long long A = (long long)(v.p1.x - v.p0.x) * (v.p2.y - v.p0.y) -
-                          (long long)(v.p2.x - v.p0.x) * (v.p1.y - v.p0.y);
-      if (A != 0) {
-        int px0, px1, py0, py1;
-        centre_range(min(v.p0.x, min(v.p1.x, v.p2.x)), max(v.p0.x, max(v.p1.x, v.p2.x)), 0, g.W - 1, px0, px1);
-        centre_range(min(v.p0.y, min(v.p1.y, v.p2.y)), max(v.p0.y, max(v.p1.y, v.p2.y)), 0, g.H - 1, py0, py1);
-        if (px0 <= px1 && py0 <= py1) {  // some pixel centre inside the bounding box
-          valid = true;
-          bx0 = px0 >> g.bshift_x; bx1 = px1 >> g.bshift_x;
-          by0 = py0 >> g.bshift_y; by1 = py1 >> g.bshift_y;
+      const int minx = min(v.p0.x, min(v.p1.x, v.p2.x)), maxx = max(v.p0.x, max(v.p1.x, v.p2.x));
+      const int miny = min(v.p0.y, min(v.p1.y, v.p2.y)), maxy = max(v.p0.y, max(v.p1.y, v.p2.y));
+      int px0, px1, py0, py1;
+      centre_range(minx, maxx, 0, g.W - 1, px0, px1);
+      centre_range(miny, maxy, 0, g.H - 1, py0, py1);
+      if (px0 <= px1 && py0 <= py1) {  // some pixel centre inside the bounding box
+        bx0 = px0 >> g.bshift_x; bx1 = px1 >> g.bshift_x;
+        by0 = py0 >> g.bshift_y; by1 = py1 >> g.bshift_y;
+        if (DIRECT && direct_small(maxx - minx, maxy - miny, px0, px1, py0, py1, direct.max_px)) {
+          if (direct_triangle(v.p0, v.p1, v.p2, key_tri, px0, px1, py0, py1, g.W, direct.keys))
+            *dentries += (unsigned)((bx1 - bx0 + 1) * (by1 - by0 + 1));
+        } else {
+          valid = (long long)(v.p1.x - v.p0.x) * (v.p2.y - v.p0.y) - (long long)(v.p2.x - v.p0.x) * (v.p1.y - v.p0.y) != 0;
         }
       }
     }
   }
-  (void)idx;
+  if (DIRECT && !__any_sync(FULL_MASK, valid)) {  // nothing to bin
+    if (t < T) rect[t] = BinRect{RECT_CULLED, 0u};
+    return;
+  }
   if (stats) {
     const unsigned nv = __popc(__ballot_sync(FULL_MASK, valid));
     if (lane == 0 && nv) atomicAdd(&st->binned, (unsigned long long)nv);
@@ -484,17 +520,20 @@ struct FusedScan {
   unsigned long long capacity;
   unsigned long long* chunk_state;
   unsigned epoch;
+  ScanReport report;
 };
 
 // eight CTAs of 256 threads per SM (32 registers) for the default binning,
 // four (64 registers) with the exact overlap test
-template <bool EXACT, bool SCAN = false>
-__global__ void __launch_bounds__(256, EXACT ? 4 : 8) k_setup_count(RasterGeom g, int T, const int* __restrict__ tris, int V,
+template <bool EXACT, bool SCAN = false, bool DIRECT = false>
+__global__ void __launch_bounds__(256, EXACT || DIRECT ? 4 : 8) k_setup_count(RasterGeom g, int T, const int* __restrict__ tris, int V,
                                                      const int4* __restrict__ vtx, BinRect* __restrict__ rect,
                                                      unsigned* __restrict__ cnt, int nbins, DevStatus* st,
                                                      int stats, const int4* __restrict__ clip_tris,
                                                      unsigned clip_cap, uint2* __restrict__ heavy,
-                                                     unsigned heavy_cap, unsigned heavy_epoch, FusedScan fs) {
+                                                     unsigned heavy_cap, unsigned heavy_epoch, FusedScan fs,
+                                                     DirectRaster direct) {
+  unsigned dentries = 0u;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   // the vertex stage does not touch the status word, and everything before
   // it has completed (it is launched without the early-start attribute)
@@ -513,16 +552,44 @@ __global__ void __launch_bounds__(256, EXACT ? 4 : 8) k_setup_count(RasterGeom g
   // batches in flight per warp needed 48 registers, five CTAs, and ran 2%
   // slower end to end)
   const int TT = frame_triangles(T, clip_tris, clip_cap, st);
-  for (int base = (blockIdx.x * (blockDim.x >> 5) + wib) * 32; base < TT; base += step) {
-    const int t = base + lane;
-    const int3 ia = load_tri(tris, T, t);
-    TriVerts va = gather_verts(ia, V, vtx, t < T);
-    if (t >= T && t < TT) {  // a clipped sub-triangle: its snapped points
-      const int4* c = clip_tris + 3 * (size_t)(t - T);
-      va.p0 = c[0]; va.p1 = c[1]; va.p2 = c[2];
-      va.in_range = true;
+  if (!DIRECT) {
+    for (int base = (blockIdx.x * (blockDim.x >> 5) + wib) * 32; base < TT; base += step) {
+      const int t = base + lane;
+      const TriVerts va = fetch_tri(T, TT, t, load_tri(tris, T, t), V, vtx, clip_tris);
+      count_batch<EXACT, false>(g, TT, t, va, rect, cnt, nbins, st, stats, lane, lt_mask, heavy, heavy_cap, heavy_n,
+                                direct, (unsigned)t, &dentries);
     }
-    count_batch<EXACT>(g, TT, t, ia, va, rect, cnt, nbins, st, stats, lane, lt_mask, heavy, heavy_cap, heavy_n);
+  } else {
+    // rasterizing holds 64 registers a thread, half the warps: the next
+    // batch's vertices and the indices of the one after are loaded before a
+    // batch is rasterized
+    auto after = [&](int b) { return b < TT - step ? b + step : TT; };  // this warp's next batch, or the end
+    int base = (blockIdx.x * (blockDim.x >> 5) + wib) * 32;
+    if (base > TT) base = TT;
+    int next = after(base);
+    TriVerts va = fetch_tri(T, TT, base + lane, load_tri(tris, T, base + lane), V, vtx, clip_tris);
+    int3 idx = load_tri(tris, T, next + lane);
+    while (base < TT) {
+      const int t = base + lane;
+      const TriVerts vn = fetch_tri(T, TT, next + lane, idx, V, vtx, clip_tris);
+      base = next;
+      next = after(next);
+      idx = load_tri(tris, T, next + lane);
+      // a clipped sub-triangle's keys carry its triangle
+      const unsigned key_tri = t >= T && t < TT ? direct.clip_orig[t - T] : (unsigned)t;
+      count_batch<EXACT, true>(g, TT, t, va, rect, cnt, nbins, st, stats, lane, lt_mask, heavy, heavy_cap, heavy_n,
+                               direct, key_tri, &dentries);
+      va = vn;
+    }
+  }
+  if (DIRECT) {
+    __shared__ unsigned s_dentries;
+    if (threadIdx.x == 0) s_dentries = 0u;
+    __syncthreads();
+    dentries = __reduce_add_sync(FULL_MASK, dentries);
+    if (lane == 0 && dentries) atomicAdd(&s_dentries, dentries);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_dentries) atomicAdd(&st->direct_entries, (unsigned long long)s_dentries);
   }
   if (SCAN) {
     __shared__ ScanSmem scan_sm;
@@ -535,7 +602,7 @@ __global__ void __launch_bounds__(256, EXACT ? 4 : 8) k_setup_count(RasterGeom g
       __threadfence();
       if (threadIdx.x == 0) st->count_done = 0u;  // for the next frame
       scan_chunk(0, 1, nbins, cnt, fs.bin_off, fs.cursor, fs.capacity, st, fs.chunk_state, fs.epoch, scan_sm,
-                 &st->queue_head);
+                 &st->queue_head, WAIT_BUDGET_CYCLES, 0, fs.report);
     }
   }
 }
@@ -554,27 +621,34 @@ static int resident_per_sm(K kernel, int threads) {
 void launch_setup_count(const RasterGeom& g, int T, const int* tris, int V, const int4* vtx, BinRect* rect,
                         unsigned* bin_count, DevStatus* st, int stats, int num_sms, cudaStream_t s,
                         const int4* clip_tris, unsigned clip_cap, int exact, uint2* heavy, unsigned heavy_cap,
-                        unsigned heavy_epoch) {
-  static const int per_sm = resident_per_sm(k_setup_count<false>, 256);
+                        unsigned heavy_epoch, DirectRaster direct) {
+  static const int per_sm_of[2] = {resident_per_sm(k_setup_count<false>, 256),
+                                   resident_per_sm(k_setup_count<false, false, true>, 256)};
+  const int per_sm = per_sm_of[direct.keys != nullptr];
+  const auto kernel = exact ? k_setup_count<true> : (direct.keys ? k_setup_count<false, false, true> : k_setup_count<false>);
   const long long TT = (long long)T + (clip_tris ? clip_cap : 0u);
   int warps = (int)((TT + 31) / 32);
   int blocks = (warps + 7) / 8;
   blocks = blocks < num_sms * per_sm ? blocks : num_sms * per_sm;
   if (blocks < 1) blocks = 1;  // with no triangles the kernel still resets the scan ticket
-  launch_pdl(exact ? k_setup_count<true> : k_setup_count<false>, blocks, 256, 0, s, g, T, tris, V, vtx, rect,
-             bin_count, g.nbx * g.nby, st, stats, clip_tris, clip_cap, heavy_cap ? heavy : nullptr, heavy_cap,
-             heavy_epoch, FusedScan{});
+  launch_pdl(kernel, blocks, 256, 0, s, g, T, tris, V, vtx, rect, bin_count, g.nbx * g.nby, st, stats, clip_tris,
+             clip_cap, heavy_cap ? heavy : nullptr, heavy_cap, heavy_epoch, FusedScan{}, direct);
 }
 
 bool launch_count_and_scan(const RasterGeom& g, int T, const int* tris, int V, const int4* vtx, BinRect* rect,
                            unsigned* bin_count, DevStatus* st, int stats, int num_sms, cudaStream_t s,
                            const int4* clip_tris, unsigned clip_cap, int exact, uint2* heavy, unsigned heavy_cap,
                            unsigned heavy_epoch, unsigned* bin_off, unsigned* cursor, unsigned long long capacity,
-                           unsigned long long* chunk_state, unsigned scan_epoch) {
+                           unsigned long long* chunk_state, unsigned scan_epoch, DirectRaster direct,
+                           const ScanReport& report) {
   const int nbins = g.nbx * g.nby;
   // one chunk of the count pass's 256 threads x SCAN_PER bins
   if (nbins > 256 * SCAN_PER) return false;
-  static const int per_sm = resident_per_sm(k_setup_count<false, true>, 256);
+  static const int per_sm_of[2] = {resident_per_sm(k_setup_count<false, true>, 256),
+                                   resident_per_sm(k_setup_count<false, true, true>, 256)};
+  const int per_sm = per_sm_of[direct.keys != nullptr];
+  const auto kernel =
+      exact ? k_setup_count<true, true> : (direct.keys ? k_setup_count<false, true, true> : k_setup_count<false, true>);
   const long long TT = (long long)T + (clip_tris ? clip_cap : 0u);
   int warps = (int)((TT + 31) / 32);
   int blocks = (warps + 7) / 8;
@@ -586,17 +660,17 @@ bool launch_count_and_scan(const RasterGeom& g, int T, const int* tris, int V, c
   fs.capacity = capacity;
   fs.chunk_state = chunk_state;
   fs.epoch = scan_epoch;
-  launch_pdl(exact ? k_setup_count<true, true> : k_setup_count<false, true>, blocks, 256, 0, s, g, T, tris, V, vtx,
-             rect, bin_count, nbins, st, stats, clip_tris, clip_cap, heavy_cap ? heavy : nullptr, heavy_cap,
-             heavy_epoch, fs);
+  fs.report = report;
+  launch_pdl(kernel, blocks, 256, 0, s, g, T, tris, V, vtx, rect, bin_count, nbins, st, stats, clip_tris, clip_cap,
+             heavy_cap ? heavy : nullptr, heavy_cap, heavy_epoch, fs, direct);
   return true;
 }
 
 void launch_scan(int nbins, unsigned* bin_count, unsigned* bin_off, unsigned* cursor, unsigned long long capacity,
                  DevStatus* st, unsigned long long* chunk_state, unsigned epoch, cudaStream_t s, long long wait_budget,
-                 int withhold) {
+                 int withhold, const ScanReport* report) {
   launch_pdl(k_scan, scan_chunks(nbins), SCAN_THREADS, 0, s, nbins, bin_count, bin_off, cursor, capacity, st,
-             chunk_state, epoch, wait_budget, withhold);
+             chunk_state, epoch, wait_budget, withhold, report ? *report : ScanReport());
 }
 
 // ======================================================================
@@ -668,30 +742,25 @@ __device__ __forceinline__ unsigned single_pos(const RasterGeom& g, BinRect r, c
   return __ldg(bin_off + bin) + r.hi;
 }
 
-// eight CTAs of 256 threads per SM (32 registers); the exact test's
-// instance keeps its vertices in registers (four CTAs)
+// The pass of CTA `block` of nblocks.
 template <bool EXACT>
-__global__ void __launch_bounds__(256, EXACT ? 4 : 8) k_scatter(RasterGeom g, int T, const BinRect* __restrict__ rect,
-                                                 const unsigned* __restrict__ bin_off,
-                                                 unsigned* __restrict__ cursor, unsigned* __restrict__ bin_tris,
-                                                 unsigned long long capacity, const DevStatus* st,
-                                                 const int4* __restrict__ clip_tris, unsigned clip_cap,
-                                                 const int* __restrict__ tris, int V, const int4* __restrict__ vtx,
-                                                 const uint2* __restrict__ heavy, unsigned heavy_cap,
-                                                 unsigned heavy_epoch) {
-  pdl_wait();  // offsets, cursors and the status of the scan
-  pdl_launch_dependents();
-  if (st->flags & STATUS_SKIP_MASK) return;
+__device__ __forceinline__ void scatter_cta(const RasterGeom& g, int T, const BinRect* __restrict__ rect,
+                                            const unsigned* __restrict__ bin_off, unsigned* __restrict__ cursor,
+                                            unsigned* __restrict__ bin_tris, unsigned long long capacity,
+                                            const DevStatus* st, const int4* __restrict__ clip_tris, unsigned clip_cap,
+                                            const int* __restrict__ tris, int V, const int4* __restrict__ vtx,
+                                            const uint2* __restrict__ heavy, unsigned heavy_cap, unsigned heavy_epoch,
+                                            int block, int nblocks) {
   const int T_in = T;
   T = frame_triangles(T, clip_tris, clip_cap, st);
   // the heavy list's length is loaded now and used after the per-warp work
   const unsigned nheavy = heavy ? heavy_count(st, heavy_epoch, heavy_cap) : 0u;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int step = gridDim.x * (blockDim.x >> 5) * 32;
+  const int step = nblocks * (blockDim.x >> 5) * 32;
   BinRect none;
   none.lo = RECT_CULLED; none.hi = 0u;
   // two batches per iteration, loads first
-  for (int base = (blockIdx.x * (blockDim.x >> 5) + wib) * 32; base < T; base += 2 * step) {
+  for (int base = (block * (blockDim.x >> 5) + wib) * 32; base < T; base += 2 * step) {
     const int baseB = base + step;
     const bool hasB = baseB < T;
     const BinRect ra = base + lane < T ? rect[base + lane] : none;
@@ -706,7 +775,7 @@ __global__ void __launch_bounds__(256, EXACT ? 4 : 8) k_scatter(RasterGeom g, in
     if (hasB) scatter_batch<EXACT>(g, baseB, rb, pb, cursor, bin_tris, capacity, lane, ob);
   }
   // the heavy list's chunks, one per CTA step, a pair per thread
-  for (unsigned e = blockIdx.x; e < nheavy; e += gridDim.x) {
+  for (unsigned e = block; e < nheavy; e += nblocks) {
     const uint2 h = heavy[e];
     if (h.x == HEAVY_NONE || threadIdx.x >= HEAVY_CHUNK) continue;
     const int k = (int)h.y * HEAVY_CHUNK + (int)threadIdx.x;
@@ -724,6 +793,95 @@ __global__ void __launch_bounds__(256, EXACT ? 4 : 8) k_scatter(RasterGeom g, in
   }
 }
 
+// eight CTAs of 256 threads per SM (32 registers); the exact test's
+// instance keeps its vertices in registers (four CTAs)
+template <bool EXACT>
+__global__ void __launch_bounds__(256, EXACT ? 4 : 8) k_scatter(RasterGeom g, int T, const BinRect* __restrict__ rect,
+                                                 const unsigned* __restrict__ bin_off,
+                                                 unsigned* __restrict__ cursor, unsigned* __restrict__ bin_tris,
+                                                 unsigned long long capacity, const DevStatus* st,
+                                                 const int4* __restrict__ clip_tris, unsigned clip_cap,
+                                                 const int* __restrict__ tris, int V, const int4* __restrict__ vtx,
+                                                 const uint2* __restrict__ heavy, unsigned heavy_cap,
+                                                 unsigned heavy_epoch) {
+  pdl_wait();  // offsets, cursors and the status of the scan
+  pdl_launch_dependents();
+  if (st->flags & STATUS_SKIP_MASK) return;
+  scatter_cta<EXACT>(g, T, rect, bin_off, cursor, bin_tris, capacity, st, clip_tris, clip_cap, tris, V, vtx, heavy,
+                     heavy_cap, heavy_epoch, blockIdx.x, gridDim.x);
+}
+
+// A frame with direct keys: the first scatter_blocks CTAs scatter, the others
+// shade the tiles without bin entries, 8 x 4 pixels per warp and step.  Shading
+// is bound by the latency of a chain of dependent gathers (bin offsets and key,
+// indices, vertices and attributes), so a warp loads the keys of the block
+// after next and the indices of the next before it shades a block.
+struct ScatterShade {
+  TileScene sc;
+  const BinRect* rect;
+  const unsigned* bin_off;
+  unsigned* cursor;
+  unsigned* bin_tris;
+  unsigned long long capacity;
+  const DevStatus* st;
+  unsigned clip_cap;
+  const uint2* heavy;
+  unsigned heavy_cap, heavy_epoch;
+  int scatter_blocks;
+};
+template <bool PERSP, bool CLIP>
+__global__ void __launch_bounds__(256, CLIP ? 4 : 5) k_scatter_shade(const __grid_constant__ ScatterShade a) {
+  pdl_wait();  // offsets, cursors and the status of the scan; the direct keys
+  pdl_launch_dependents();
+  if (a.st->flags & STATUS_SKIP_MASK) return;
+  const TileScene& sc = a.sc;
+  const RasterGeom& g = sc.g;
+  if ((int)blockIdx.x < a.scatter_blocks) {
+    scatter_cta<false>(g, sc.T, a.rect, a.bin_off, a.cursor, a.bin_tris, a.capacity, a.st, sc.clip_tris, a.clip_cap,
+                       nullptr, 0, nullptr, a.heavy, a.heavy_cap, a.heavy_epoch, blockIdx.x, a.scatter_blocks);
+    return;
+  }
+  const int lane = threadIdx.x & 31;
+  const int per_row = (g.W + SHADE_W - 1) / SHADE_W, blocks = per_row * ((g.H + SHADE_H - 1) / SHADE_H);
+  const int step = ((int)gridDim.x - a.scatter_blocks) * 8;
+  // a lane's pixel of block b (past the framebuffer: nothing), and its key,
+  // EMPTY where the block is the Process stage's (mine false).  Bins are at
+  // least 8 x 8 pixels, so a block lies in one.
+  struct Block {
+    int x, y;
+    unsigned long long k;
+    bool mine;
+  };
+  auto load = [&](int b) {
+    Block r;
+    r.mine = false;
+    r.k = KEY_EMPTY;
+    r.x = r.y = 0;
+    if (b < blocks) {
+      const int by = b / per_row, x0 = (b - by * per_row) * SHADE_W, y0 = by * SHADE_H;
+      const int bin = (y0 >> g.bshift_y) * g.nbx + (x0 >> g.bshift_x);
+      r.x = x0 + (lane & (SHADE_W - 1));
+      r.y = y0 + lane / SHADE_W;
+      r.k = direct_key(sc, r.x, r.y);
+      r.mine = __ldg(a.bin_off + bin) == __ldg(a.bin_off + bin + 1);
+    }
+    return r;
+  };
+  int b = ((int)blockIdx.x - a.scatter_blocks) * 8 + (int)(threadIdx.x >> 5);
+  Block cur = load(b), next = load(b < blocks - step ? b + step : blocks);
+  int3 id = make_int3(0, 0, 0), idn = id;
+  if (cur.k != KEY_EMPTY) id = tri_indices(sc.tris, (unsigned)cur.k);
+  while (b < blocks) {
+    if (next.k != KEY_EMPTY) idn = tri_indices(sc.tris, (unsigned)next.k);
+    b = b < blocks - step ? b + step : blocks;
+    const Block after = load(b < blocks - step ? b + step : blocks);
+    if (cur.mine) shade_direct_block<PERSP, CLIP>(sc, cur.k, id, cur.x, cur.y);
+    cur = next;
+    next = after;
+    id = idn;
+  }
+}
+
 void launch_scatter(const RasterGeom& g, int T, const BinRect* rect, const unsigned* bin_off, unsigned* cursor,
                     unsigned* bin_tris, unsigned long long capacity, DevStatus* st, int num_sms, cudaStream_t s,
                     const int4* clip_tris, unsigned clip_cap, const int* tris, int V, const int4* vtx,
@@ -736,6 +894,29 @@ void launch_scatter(const RasterGeom& g, int T, const BinRect* rect, const unsig
   blocks = blocks < num_sms * per_sm ? blocks : num_sms * per_sm;
   launch_pdl(tris ? k_scatter<true> : k_scatter<false>, blocks, 256, 0, s, g, T, rect, bin_off, cursor, bin_tris,
              capacity, st, clip_tris, clip_cap, tris, V, vtx, heavy_cap ? heavy : nullptr, heavy_cap, heavy_epoch);
+}
+
+cudaError_t launch_scatter_shade(const ProcessParams& p, const BinRect* rect, unsigned* cursor, unsigned* bin_tris,
+                                 unsigned long long capacity, int num_sms, cudaStream_t s, unsigned clip_cap,
+                                 const uint2* heavy, unsigned heavy_cap, unsigned heavy_epoch) {
+  const long long TT = (long long)p.num_triangles + (p.clip_tris ? clip_cap : 0u);
+  const long long need = ((TT + 31) / 32 + 7) / 8;
+  ScatterShade a;
+  a.sc = scene_of(p);
+  a.rect = rect; a.bin_off = p.bin_off; a.cursor = cursor; a.bin_tris = bin_tris; a.capacity = capacity; a.st = p.st;
+  a.clip_cap = clip_cap;
+  a.heavy = heavy_cap ? heavy : nullptr; a.heavy_cap = heavy_cap; a.heavy_epoch = heavy_epoch;
+  a.scatter_blocks = (int)(need < 6LL * num_sms ? need : 6LL * num_sms);
+  const long long warps = (long long)((p.g.W + SHADE_W - 1) / SHADE_W) * ((p.g.H + SHADE_H - 1) / SHADE_H);
+  const bool clip = p.clip_tris != nullptr;
+  const auto kernel = p.invw ? (clip ? k_scatter_shade<true, true> : k_scatter_shade<true, false>)
+                             : (clip ? k_scatter_shade<false, true> : k_scatter_shade<false, false>);
+  // one wave of CTAs shades
+  static const int per_sm_of[4] = {
+      resident_per_sm(k_scatter_shade<false, false>, 256), resident_per_sm(k_scatter_shade<false, true>, 256),
+      resident_per_sm(k_scatter_shade<true, false>, 256), resident_per_sm(k_scatter_shade<true, true>, 256)};
+  const long long wave = (long long)per_sm_of[(p.invw ? 2 : 0) + (clip ? 1 : 0)] * num_sms, all = (warps + 7) / 8;
+  return launch_pdl(kernel, a.scatter_blocks + (int)(all < wave ? all : wave), 256, 0, s, a);
 }
 
 }  // namespace piko

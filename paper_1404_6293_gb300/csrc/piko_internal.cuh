@@ -49,6 +49,7 @@ struct DevStatus {
   unsigned int flags;           // bit c set when PIKO_ERR c was recorded
   unsigned int first_code;      // first PIKO_ERR_* recorded (0 = none)
   unsigned long long needed;    // bin entries the last scan required
+  unsigned long long listed;    // those of them in the lists (the rest: direct_entries; read back together with needed)
   unsigned int queue_head;      // tile counter of the dynamic schedule
   unsigned int scan_ticket;     // next chunk number of the scan (reset by its last chunk)
   unsigned int frag_count;      // fragments emitted by the unfused pipeline's rasterizer
@@ -59,6 +60,7 @@ struct DevStatus {
   unsigned long long binned;    // triangles that reached at least one bin
   unsigned int heavy_n[2];      // chunks in the heavy-triangle list of AssignBin, by count-pass parity
   unsigned int count_done;      // count-pass CTAs finished (its last CTA scans small frames; then 0 again)
+  unsigned long long direct_entries;  // bin entries of the triangles the count pass rasterized itself (0 after the scan)
 };
 
 // Screen and bin geometry of one framebuffer.
@@ -352,6 +354,7 @@ struct ProcessParams {
   const float* normal;
   const float* light;
   const float* vdot;  // n_v . L per vertex (Lambert)
+  const float4* vattr;  // colour and n_v . L per vertex (Lambert with colours; NULL: color and vdot)
   const float* invw;  // 1 / clip w per vertex: perspective-correct attributes (NULL: screen-space)
   const int4* clip_tris;   // near/far clipping: sub-triangles (NULL: off)
   const unsigned* clip_orig;
@@ -359,6 +362,7 @@ struct ProcessParams {
   const float* mvp;
   const unsigned* bin_off;
   const unsigned* bin_tris;
+  const unsigned long long* dkeys;  // keys of the count pass's direct rasterization (NULL: none)
   unsigned long long* key_out;
   float4* rgba_out;
   uint2* gnorm_out;  // binary16 x4
@@ -366,11 +370,25 @@ struct ProcessParams {
   DevStatus* st;
 };
 
+struct ScanReport;  // piko_scan.cuh
+
+// Small triangles rasterized by the count pass itself (piko_direct.cuh).
+struct DirectRaster {
+  unsigned long long* keys = nullptr;  // W * H keys, KEY_EMPTY before the pass (NULL: every triangle is binned)
+  int max_px = 0;                      // largest box taken, in pixels
+  const unsigned* clip_orig = nullptr; // triangle of each clipped sub-triangle
+};
+
 // Vertex stage.  If vdot is not NULL it also stores n_v . L per vertex (the
 // Lambert term is linear in the interpolated normal, so per-vertex dots
 // interpolate to the same value).
+// dkeys (optional): W * H keys of the count pass's direct rasterization, set
+// to KEY_EMPTY here; clip_st (optional): its clip_count is set to 0; vattr
+// (optional, with vdot): takes each vertex's colour and n . L in vdot's place.
 void launch_vertex(int W, int H, int V, const float* pos, const float* mvp, int4* vtx, const float* normal,
-                   const float* light, float* vdot, float* invw, int num_sms, cudaStream_t s);
+                   const float* light, float* vdot, float* invw, int num_sms, cudaStream_t s,
+                   unsigned long long* dkeys = nullptr, DevStatus* clip_st = nullptr, const float* color = nullptr,
+                   float4* vattr = nullptr);
 // Count pass and scan (two launches): bin_count holds 2 * nbins counters
 // (single-bin and multi-bin entries), zero between frames; the scan turns
 // them into CSR offsets and scatter cursors (capacity: entries the bin lists
@@ -390,7 +408,8 @@ constexpr unsigned HEAVY_LIST_CAP = 16384;
 void launch_setup_count(const RasterGeom& g, int T, const int* tris, int V, const int4* vtx,
                         BinRect* rect, unsigned* bin_count, DevStatus* st, int stats, int num_sms, cudaStream_t s,
                         const int4* clip_tris = nullptr, unsigned clip_cap = 0, int exact = 0,
-                        uint2* heavy = nullptr, unsigned heavy_cap = 0, unsigned heavy_epoch = 0);
+                        uint2* heavy = nullptr, unsigned heavy_cap = 0, unsigned heavy_epoch = 0,
+                        DirectRaster direct = DirectRaster());
 // Count pass and scan in one launch for a frame of at most one scan chunk of
 // bins (scan_chunks(nbins) == 1): the count pass's last CTA scans.  Returns
 // false (nothing launched) for larger frames, which take launch_setup_count
@@ -399,7 +418,8 @@ bool launch_count_and_scan(const RasterGeom& g, int T, const int* tris, int V, c
                            unsigned* bin_count, DevStatus* st, int stats, int num_sms, cudaStream_t s,
                            const int4* clip_tris, unsigned clip_cap, int exact, uint2* heavy, unsigned heavy_cap,
                            unsigned heavy_epoch, unsigned* bin_off, unsigned* cursor, unsigned long long capacity,
-                           unsigned long long* chunk_state, unsigned scan_epoch);
+                           unsigned long long* chunk_state, unsigned scan_epoch, DirectRaster direct,
+                           const ScanReport& report);
 // Near/far clipping of the triangles with a rejected vertex: sub-triangles
 // (3 snapped points each) and their triangle's index appended at
 // st->clip_count (PIKO_ERR_OVERFLOW past cap).
@@ -411,7 +431,7 @@ void launch_clip(int W, int H, int T, const int* tris, int V, const float* pos, 
 // test hook bits (piko_scan.cuh).
 void launch_scan(int nbins, unsigned* bin_count, unsigned* bin_off, unsigned* cursor, unsigned long long capacity,
                  DevStatus* st, unsigned long long* chunk_state, unsigned epoch, cudaStream_t s,
-                 long long wait_budget = 40000000, int withhold = 0);
+                 long long wait_budget = 40000000, int withhold = 0, const ScanReport* report = nullptr);
 int scan_chunks(int nbins);
 void launch_scatter(const RasterGeom& g, int T, const BinRect* rect, const unsigned* bin_off, unsigned* cursor,
                     unsigned* bin_tris, unsigned long long capacity, DevStatus* st, int num_sms, cudaStream_t s,
@@ -419,6 +439,11 @@ void launch_scatter(const RasterGeom& g, int T, const BinRect* rect, const unsig
                     const int4* vtx = nullptr, const uint2* heavy = nullptr, unsigned heavy_cap = 0,
                     unsigned heavy_epoch = 0);
 cudaError_t launch_process(const ProcessParams& p, int threads, int grid, cudaStream_t s);
+// launch_scatter of a frame with direct keys (default binning), and the
+// shading of the tiles without bin entries, in one launch.
+cudaError_t launch_scatter_shade(const ProcessParams& p, const BinRect* rect, unsigned* cursor, unsigned* bin_tris,
+                                 unsigned long long capacity, int num_sms, cudaStream_t s, unsigned clip_cap,
+                                 const uint2* heavy, unsigned heavy_cap, unsigned heavy_epoch);
 cudaError_t process_occupancy(const ProcessParams& p, int threads, int* blocks_per_sm);
 
 // Boxes (pixels of a triangle's bounding box inside a tile) up to this size

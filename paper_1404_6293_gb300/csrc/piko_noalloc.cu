@@ -224,6 +224,7 @@ extern "C" int piko_raster_forward_noalloc(const piko_scene* s, piko_framebuffer
   p.normal = s->normal;
   p.light = s->light_dir;
   p.vdot = vdot;
+  p.vattr = nullptr;
   p.invw = nullptr;  // screen-space attributes only
   p.clip_tris = nullptr;  // no clipping: out-of-range vertices cull their triangles
   p.clip_orig = nullptr;
@@ -231,6 +232,7 @@ extern "C" int piko_raster_forward_noalloc(const piko_scene* s, piko_framebuffer
   p.mvp = s->mvp;
   p.bin_off = bin_off;
   p.bin_tris = bin_tris;
+  p.dkeys = nullptr;  // every triangle is binned: the array has no room for a key per pixel
   p.key_out = reinterpret_cast<unsigned long long*>(fb->key);
   p.rgba_out = reinterpret_cast<float4*>(fb->rgba);
   p.gnorm_out = reinterpret_cast<uint2*>(fb->gbuf_normal);

@@ -62,6 +62,13 @@ __device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned l
   asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// What the host reads of a scan without waiting for the stream: pinned words
+// written by the scan itself (needed, listed, clipped sub-triangles, then tag).
+struct ScanReport {
+  unsigned long long* host = nullptr;  // 4 words (NULL: no report)
+  unsigned long long tag = 0;          // differs between consecutive reports of a handle
+};
+
 // Scans chunk `chunk` of nchunks (all threads of the CTA call it; it
 // contains barriers).  The last chunk writes the total, checks the capacity
 // and resets *queue_to_reset (the Process stage's tile queue).
@@ -70,7 +77,7 @@ __device__ __forceinline__ void scan_chunk(int chunk, int nchunks, int nbins, un
                                            unsigned long long capacity, DevStatus* st,
                                            unsigned long long* __restrict__ chunk_state, unsigned epoch, ScanSmem& sm,
                                            unsigned* queue_to_reset, long long wait_budget = WAIT_BUDGET_CYCLES,
-                                           int withhold = 0) {
+                                           int withhold = 0, ScanReport report = ScanReport()) {
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
   const unsigned long long tag = (unsigned long long)(epoch & 0xFFFFu) << 46;
   unsigned* __restrict__ multi = cnt + nbins;
@@ -156,12 +163,25 @@ __device__ __forceinline__ void scan_chunk(int chunk, int nchunks, int nbins, un
       }
   }
   if (chunk == nchunks - 1 && tid == 0) {
-    const unsigned long long total = sm.excl + agg;
+    // entries of directly rasterized triangles count toward the bin lists'
+    // size (what is needed and what overflows does not depend on the route)
+    const unsigned long long listed = sm.excl + agg;
+    const unsigned long long total = listed + *reinterpret_cast<volatile unsigned long long*>(&st->direct_entries);
+    st->direct_entries = 0ull;
     const bool ok = total <= capacity;
-    if (ok) bin_off[nbins] = (unsigned)total;
+    if (ok) bin_off[nbins] = (unsigned)listed;
     st->needed = total;
+    st->listed = listed;
     *queue_to_reset = 0u;
     if (!ok) record_error(st, PIKO_ERR_OVERFLOW);
+    if (report.host) {
+      volatile unsigned long long* r = report.host;
+      r[0] = total;
+      r[1] = listed;
+      r[2] = *reinterpret_cast<volatile unsigned*>(&st->clip_count);
+      __threadfence_system();
+      r[3] = report.tag;
+    }
   }
 }
 

@@ -12,8 +12,9 @@
 //     and the vertex attributes) in a shared-memory record.  A small box
 //     inside the tile is walked by the thread for coverage only, and the
 //     warp then shares out the covered samples of all its small boxes for
-//     their depths (fragment_pass); larger boxes go to a queue that whole
-//     warps rasterize 32 pixels at a time with a coverage ballot;
+//     their depths (fragment_pass); larger boxes of triangles up to 128
+//     pixels a side are shared out by rows and samples (medium_pass); larger
+//     triangles go to a queue that whole warps rasterize one at a time;
 //  2. every covered sample does a 64-bit atomic minimum on the tile's key,
 //     key = depth << 40 | triangle << slot_bits | record slot: ordered by
 //     (depth, triangle) exactly like depth << 32 | triangle, since a
@@ -41,6 +42,7 @@ struct TileScene {
   const float* normal;
   const float* light;
   const float* vdot;
+  const float4* vattr;  // Lambert: colour (if there is one) and n . L per vertex (NULL: from color and vdot)
   const float* invw;  // 1 / clip w per vertex, or NULL for screen-space attributes
   // near/far clipping: triangles T.. of the frame are clipped sub-triangles
   // (3 snapped points each in clip_tris, their triangle in clip_orig); pos
@@ -51,11 +53,14 @@ struct TileScene {
   const unsigned* clip_orig;
   const float4* pos;
   const float* mvp;
+  const unsigned long long* dkeys;  // keys of directly rasterized triangles (NULL: none), one per pixel
   unsigned long long* key_out;
   float4* rgba_out;
   uint2* gnorm_out;
   uint2* galb_out;
 };
+
+TileScene scene_of(const ProcessParams& p);  // piko_process.cu
 
 // Per-CTA shared memory of the stage.
 // Each lane owns FST_WORDS staging words per bin entry, stored word-major
@@ -268,6 +273,9 @@ struct SmallBox {
 // staging words of a lane (word w of lane l at w * 32 + l)
 enum { FS_E1 = 0, FS_E2, FS_SX1, FS_SY1, FS_SX2, FS_SY2, FS_K1, FS_K2, FS_D1, FS_D2, FS_A, FS_KLO, FS_KHI };
 
+__device__ __forceinline__ void stage_box(const TriSetup& s, const Edges<int>& e, unsigned long long tag, int* wst,
+                                          int lane);
+
 __device__ __forceinline__ void small_box(const TriSetup& s, unsigned long long tag, int px0, int px1, int py0,
                                           int py1, int x0, int y0, int bshift_x, int* wst, int lane, SmallBox& b) {
   const Edges<int> e = make_edges<int>(s, px0, py0);
@@ -286,6 +294,13 @@ __device__ __forceinline__ void small_box(const TriSetup& s, unsigned long long 
   b.mask = mask >> (32 - bw * bh);
   if (b.mask == 0u) return;
   b.place = (((py0 - y0) << bshift_x) + (px0 - x0)) | (bw << 16);
+  stage_box(s, e, tag, wst, lane);
+}
+
+// Staging words of a box of a triangle whose bounding box is below 2^15 in
+// 16.8 units (e: its edges at the box's first pixel).
+__device__ __forceinline__ void stage_box(const TriSetup& s, const Edges<int>& e, unsigned long long tag, int* wst,
+                                          int lane) {
   const float rA = approx_rcp(f32_from_i64(s.A));
   const DepthSetup d = depth_setup(s, rA, tag);
   int* w = wst + lane;
@@ -300,12 +315,9 @@ __device__ __forceinline__ void small_box(const TriSetup& s, unsigned long long 
   w[FS_KHI * 32] = (int)(unsigned)(d.kbase >> 32);
 }
 
-// Depth key of one compacted fragment: descriptor = tile-local pixel index
-// (12 bits) | column in the box << 12 | row << 17 | staging lane << 22.  The
-// same quotient and key as key_min_box.
-__device__ __forceinline__ void fragment_key(const int* wst, unsigned desc, unsigned long long* skey) {
-  const int* w = wst + (desc >> 22);
-  const int rx = (desc >> 12) & 31, ry = (desc >> 17) & 31, idx = desc & 0xFFF;
+// Depth key of one compacted fragment: column rx and row ry of the box staged
+// at w, tile-local pixel index idx.  The same quotient and key as key_min_box.
+__device__ __forceinline__ void fragment_key(const int* w, int rx, int ry, int idx, unsigned long long* skey) {
   // covered: w1, w2 in [0, A] < 2^30, exact in wrapping 32-bit arithmetic
   const int w1 = (int)((unsigned)w[FS_E1 * 32] + (unsigned)rx * (unsigned)w[FS_SX1 * 32] +
                        (unsigned)ry * (unsigned)w[FS_SY1 * 32]);
@@ -330,8 +342,9 @@ __device__ __forceinline__ void fragment_key(const int* wst, unsigned desc, unsi
   if (k < skey[idx]) atomicMin(skey + idx, k);
 }
 
-// Called by every lane of the warp: hands out the warp's covered samples of
-// small boxes FRAG_CAP at a time.  Returns the warp's fragment count.
+// Called by every lane of the warp: hands out the warp's covered samples (a
+// descriptor each: tile-local pixel index (12 bits) | column in the box << 12
+// | row << 17 | staging lane << 22) of small boxes FRAG_CAP at a time.  Returns the warp's fragment count.
 __device__ __forceinline__ unsigned fragment_pass(const SmallBox& b, int bshift_x, int* wst, unsigned long long* skey,
                                                   int lane) {
   if (!__any_sync(FULL_MASK, b.mask != 0u)) return 0u;
@@ -354,10 +367,86 @@ __device__ __forceinline__ unsigned fragment_pass(const SmallBox& b, int bshift_
     }
     __syncwarp();
     const int n = min(FRAG_CAP, m.total - base);
-    for (int k = lane; k < n; k += 32) fragment_key(wst, (unsigned)list[k], skey);
+    for (int k = lane; k < n; k += 32) {
+      const unsigned d = (unsigned)list[k];
+      fragment_key(wst + (d >> 22), (d >> 12) & 31, (d >> 17) & 31, d & 0xFFF, skey);
+    }
     __syncwarp();
   }
   return (unsigned)m.total;
+}
+
+// ------------------------------------------------------- medium boxes
+// A box of more samples than a lane's mask holds, of a triangle whose bounding
+// box is below 2^15 in 16.8 units (128 pixels; 32-bit edge functions).  The
+// lanes stage such triangles like small boxes, and the warp gives their rows
+// out to its lanes: a lane finds the span of covered columns of its row, each
+// edge's end by one division corrected to the exact one, and the rows' covered
+// samples are then given out to consecutive lanes for their depths.  Rows and
+// samples of different triangles fill the warp together, where a warp taking
+// one triangle at a time leaves a third of its lanes idle in each and evaluates
+// edges and remainders in 64 bits.
+//
+// Narrows [lo, hi] to the columns c with w + c s - (1 - tl) >= 0, tl: the
+// edge is top-left (steps s in x and t in y decide it); |w| < 2^31, |s| < 2^23,
+// hi < 64.
+__device__ __forceinline__ void clip_columns(int w, int s, int t, int& lo, int& hi) {
+  const int e = w - 1 + ((s > 0 || (s == 0 && t > 0)) ? 1 : 0);
+  if (s == 0) {
+    if (e < 0) hi = -1;
+    return;
+  }
+  if (s < 0 && e < 0) {
+    hi = -1;
+    return;
+  }
+  if (s > 0 && e >= 0) return;
+  // floor(n / |s|) of n = e (the last covered column) or -e - 1 (the last
+  // column before the first covered one), up to 64
+  const int a = abs(s), n = s < 0 ? e : -e - 1;
+  int q = (int)fminf((float)n * approx_rcp((float)a), 64.0f);
+  const int r = n - q * a;
+  q += r < 0 ? -1 : (r >= a ? 1 : 0);
+  if (s < 0) hi = min(hi, q);
+  else lo = max(lo, q + 1);
+}
+
+// Called by every lane of the warp; rows: the lane's box has this many (0: no
+// medium box); place: tile-local index of its first pixel | box width << 16.
+// Returns the warp's fragment count.
+__device__ __forceinline__ unsigned medium_pass(int rows, int place, int bshift_x, const int* wst,
+                                                unsigned long long* skey, int lane) {
+  if (!__any_sync(FULL_MASK, rows > 0)) return 0u;
+  __syncwarp();  // the staged boxes
+  const MultiSpan mr = warp_prefix(rows, lane);
+  unsigned frags = 0;
+  for (int r0 = 0; r0 < mr.total; r0 += 32) {
+    const int k = min(r0 + lane, mr.total - 1);
+    const int o = pair_owner(mr.incl, k);
+    const int ry = k - __shfl_sync(FULL_MASK, mr.incl - rows, o), op = __shfl_sync(FULL_MASK, place, o);
+    const int* w = wst + o;
+    const int sx1 = w[FS_SX1 * 32], sy1 = w[FS_SY1 * 32], sx2 = w[FS_SX2 * 32], sy2 = w[FS_SY2 * 32];
+    const int w1 = w[FS_E1 * 32] + ry * sy1, w2 = w[FS_E2 * 32] + ry * sy2, w0 = abs(w[FS_A * 32]) - w1 - w2;
+    int lo = 0, hi = r0 + lane < mr.total ? (op >> 16) - 1 : -1;
+    clip_columns(w0, -(sx1 + sx2), -(sy1 + sy2), lo, hi);
+    clip_columns(w1, sx1, sy1, lo, hi);
+    clip_columns(w2, sx2, sy2, lo, hi);
+    const int cnt = max(hi - lo + 1, 0);
+    // the row as its samples need it: tile-local index of its column 0 (12
+    // bits), first covered column (6), row (6), staging lane
+    const unsigned row = (unsigned)((op & 0xFFFF) + (ry << bshift_x)) | (unsigned)(lo & 63) << 12 | (unsigned)ry << 18 |
+                         (unsigned)o << 24;
+    const MultiSpan ms = warp_prefix(cnt, lane);
+    for (int k0 = 0; k0 < ms.total; k0 += 32) {
+      const int j = min(k0 + lane, ms.total - 1);
+      const int rl = pair_owner(ms.incl, j);
+      const unsigned d = __shfl_sync(FULL_MASK, row, rl);
+      const int c = j - __shfl_sync(FULL_MASK, ms.incl - cnt, rl) + (int)(d >> 12 & 63);
+      if (k0 + lane < ms.total) fragment_key(wst + (d >> 24), c, d >> 18 & 63, (int)(d & 0xFFF) + c, skey);
+    }
+    frags += (unsigned)ms.total;
+  }
+  return frags;
 }
 
 // A warp covers a large triangle's box 32 pixels at a time; the ballot of
@@ -593,15 +682,47 @@ __device__ __forceinline__ void shade_vertices(const TileScene& p, int v0, int v
   if (p.rgba_out) p.rgba_out[o] = make_float4(c0 * d, c1 * d, c2 * d, 1.0f);
 }
 
-// Fallback for winners without a record: everything re-read from global
-// memory.  CLIP (near/far clipping on): a winner whose vertices the vertex
+// Lambert from the vertex stage's n . L (and, with vattr, the colours packed
+// beside it: one 16-byte gather a vertex instead of four).
+__device__ __forceinline__ void shade_lambert(const TileScene& p, int v0, int v1, int v2, float b0, float b1, float b2,
+                                              size_t o) {
+  float d, c0 = 0.80f, c1 = 0.75f, c2 = 0.65f;  // material of Listing 1
+  if (p.vattr) {
+    const float4 q0 = __ldg(p.vattr + v0), q1 = __ldg(p.vattr + v1), q2 = __ldg(p.vattr + v2);
+    d = b0 * q0.w + b1 * q1.w + b2 * q2.w;  // (sum b_i n_i) . L, by linearity
+    if (p.color) {
+      c0 = b0 * q0.x + b1 * q1.x + b2 * q2.x;
+      c1 = b0 * q0.y + b1 * q1.y + b2 * q2.y;
+      c2 = b0 * q0.z + b1 * q1.z + b2 * q2.z;
+    }
+  } else {
+    d = b0 * __ldg(p.vdot + v0) + b1 * __ldg(p.vdot + v1) + b2 * __ldg(p.vdot + v2);
+    if (p.color) {
+      const float* q0 = p.color + 3 * (size_t)v0;
+      const float* q1 = p.color + 3 * (size_t)v1;
+      const float* q2 = p.color + 3 * (size_t)v2;
+      c0 = b0 * __ldg(q0) + b1 * __ldg(q1) + b2 * __ldg(q2);
+      c1 = b0 * __ldg(q0 + 1) + b1 * __ldg(q1 + 1) + b2 * __ldg(q2 + 1);
+      c2 = b0 * __ldg(q0 + 2) + b1 * __ldg(q1 + 2) + b2 * __ldg(q2 + 2);
+    }
+  }
+  if (!p.unclamped) d = fmaxf(d, 0.0f);
+  if (p.rgba_out) p.rgba_out[o] = make_float4(c0 * d, c1 * d, c2 * d, 1.0f);
+}
+
+__device__ __forceinline__ int3 tri_indices(const int* __restrict__ tris, unsigned t) {
+  const int* i = tris + 3 * (size_t)t;
+  return make_int3(__ldg(i), __ldg(i + 1), __ldg(i + 2));
+}
+
+// Winners without a record (id: the triangle's indices): everything re-read
+// from global memory, with the arithmetic of a record's.  CLIP (near/far clipping on): a winner whose vertices the vertex
 // stage rejected was clipped, and shades with its clip-space ray weights
 // (perspective-correct by construction); one kernel instance per setting so
 // that the default path carries none of it.
 template <bool PERSP, bool CLIP = false>
-__device__ __forceinline__ void shade_from_global(const TileScene& p, unsigned t, int x, int y, size_t o) {
-  const int v[3] = {__ldg(p.tris + 3 * (size_t)t), __ldg(p.tris + 3 * (size_t)t + 1),
-                    __ldg(p.tris + 3 * (size_t)t + 2)};
+__device__ __forceinline__ void shade_from_global(const TileScene& p, int3 id, int x, int y, size_t o) {
+  const int v[3] = {id.x, id.y, id.z};
   TriSetup s;
   if (!setup_triangle(v[0], v[1], v[2], p.vtx, s)) {
     if (!CLIP || !p.pos) {
@@ -614,11 +735,23 @@ __device__ __forceinline__ void shade_from_global(const TileScene& p, unsigned t
     return;
   }
   const int Px = 256 * x + 128, Py = 256 * y + 128;
-  const long long w1 = (long long)(s.X0 - s.X2) * (Py - s.Y2) - (long long)(s.Y0 - s.Y2) * (Px - s.X2);
-  const long long w2 = (long long)(s.X1 - s.X0) * (Py - s.Y0) - (long long)(s.Y1 - s.Y0) * (Px - s.X0);
   const float rA = approx_rcp(f32_from_i64(s.A));
-  float b1 = f32_from_i64(w1) * rA, b2 = f32_from_i64(w2) * rA, b0 = 1.0f - b1 - b2;
+  float b1, b2;
+  if (s.A < (1LL << 31)) {  // a covered pixel's edge functions lie in [0, A]: exact in 32 bits
+    b1 = (float)edge_fn_wrap32(s.X2, s.Y2, s.X0, s.Y0, Px, Py) * rA;
+    b2 = (float)edge_fn_wrap32(s.X0, s.Y0, s.X1, s.Y1, Px, Py) * rA;
+  } else {
+    const long long w1 = (long long)(s.X0 - s.X2) * (Py - s.Y2) - (long long)(s.Y0 - s.Y2) * (Px - s.X2);
+    const long long w2 = (long long)(s.X1 - s.X0) * (Py - s.Y0) - (long long)(s.Y1 - s.Y0) * (Px - s.X0);
+    b1 = f32_from_i64(w1) * rA;
+    b2 = f32_from_i64(w2) * rA;
+  }
+  float b0 = 1.0f - b1 - b2;
   if (PERSP) perspective_bary(b0, b1, b2, __ldg(p.invw + s.v0), __ldg(p.invw + s.v1), __ldg(p.invw + s.v2));
+  if (p.mode == PIKO_SHADE_LAMBERT && (p.vdot || p.vattr)) {  // as from a record
+    shade_lambert(p, s.v0, s.v1, s.v2, b0, b1, b2, o);
+    return;
+  }
   shade_vertices(p, s.v0, s.v1, s.v2, b0, b1, b2, o);
 }
 
@@ -637,6 +770,16 @@ __device__ __forceinline__ void fill_record(const TileScene& p, const TriSetup& 
     for (int j = 0; j < 3; ++j) iw[j] = __ldg(p.invw + v[j]);
   }
   if (p.mode == PIKO_SHADE_LAMBERT) {
+    if (p.vattr) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const float4 q = __ldg(p.vattr + v[j]);
+        a[j] = q.w;
+        if (!p.color) continue;
+        a[3 + 3 * j] = q.x; a[4 + 3 * j] = q.y; a[5 + 3 * j] = q.z;
+      }
+      return;
+    }
 #pragma unroll
     for (int j = 0; j < 3; ++j) a[j] = __ldg(p.vdot + v[j]);
     if (p.color) {
@@ -691,11 +834,28 @@ __device__ __forceinline__ void process_tile(const TileScene& p, int tile, unsig
   const int x1 = min(x0 + bin_w, p.g.W) - 1, y1 = min(y0 + bin_h, p.g.H) - 1;
   unsigned long long* skey = sm.skey;
   int* wst = sm.sfrag + warp * FRAG_WARP_WORDS;
+  if (p.dkeys) {
+    // the directly rasterized triangles' keys: where the tile has no bin
+    // entries its pixels are shaded elsewhere (piko_direct.cuh), else they are
+    // the tile's starting keys
+    if (beg == end) {
+      __syncthreads();
+      return;
+    }
+    for (int i = tid; i < bin_px; i += nt) {
+      const int x = x0 + (i & (bin_w - 1)), y = y0 + (i >> p.g.bshift_x);
+      const unsigned long long k = x <= x1 && y <= y1 ? __ldcg(p.dkeys + (size_t)y * p.g.W + x) : KEY_EMPTY;
+      if (k != KEY_EMPTY) skey[i] = (k >> 32) << 40 | (unsigned long long)(unsigned)k << p.slot_bits | no_slot;
+    }
+    __syncthreads();
+  }
   for (unsigned c = beg; c < end; c += nt) {
-    const unsigned i = c + tid;
+    // entries are dealt to the warps one by one, so that a short list keeps all of them busy
+    const unsigned i = c + (unsigned)(lane * nwarps + warp);
     bool pushed = false;
     SmallBox sb;
     sb.mask = 0u;
+    int med_rows = 0, med_place = 0;
     if (i < end) {
       unsigned t = __ldg(bin_tris + i) - (unsigned)p.tri_base;
       unsigned slot = (i - beg) < (unsigned)p.nslots ? (i - beg) : no_slot;
@@ -710,7 +870,6 @@ __device__ __forceinline__ void process_tile(const TileScene& p, int tile, unsig
       } else {
         load_setup(p, t, s);
       }
-      if (slot != no_slot) fill_record<PERSP>(p, s, sm.srec + slot * p.rec_stride);
       const int minX = min(s.X0, min(s.X1, s.X2)), maxX = max(s.X0, max(s.X1, s.X2));
       const int minY = min(s.Y0, min(s.Y1, s.Y2)), maxY = max(s.Y0, max(s.Y1, s.Y2));
       int px0, px1, py0, py1;
@@ -719,18 +878,26 @@ __device__ __forceinline__ void process_tile(const TileScene& p, int tile, unsig
       if (px0 <= px1 && py0 <= py1) {
         const int npx = (px1 - px0 + 1) * (py1 - py0 + 1);
         const unsigned long long tag = ((unsigned long long)t << p.slot_bits) | slot;
+        const bool narrow = maxX - minX < 32768 && maxY - minY < 32768;
+        bool covers = true;
         if (STATS) st.tests += npx;
         if (npx <= p.small_px) {
           unsigned f = 0u;
-          if (maxX - minX < 32768 && maxY - minY < 32768) {
+          if (narrow) {
             if (npx <= 32)  // coverage only; the warp's fragment_pass takes the depths
+            {
               small_box(s, tag, px0, px1, py0, py1, x0, y0, p.g.bshift_x, wst, lane, sb);
-            else
+              covers = sb.mask != 0u;
+            } else
               f = raster_thread32(s, tag, px0, px1, py0, py1, x0, y0, p.g.bshift_x, skey);
           } else {
             f = raster_thread64(s, tag, px0, px1, py0, py1, x0, y0, p.g.bshift_x, skey);
           }
           if (STATS) st.frags += f;
+        } else if (narrow) {
+          stage_box(s, make_edges<int>(s, px0, py0), tag, wst, lane);
+          med_rows = py1 - py0 + 1;
+          med_place = (((py0 - y0) << p.g.bshift_x) + (px0 - x0)) | ((px1 - px0 + 1) << 16);
         } else {
           // the ring counter only ever grows; with nt a power of two the ring
           // index stays consistent across its 2^32 wrap
@@ -744,10 +911,13 @@ __device__ __forceinline__ void process_tile(const TileScene& p, int tile, unsig
           e[BG_T * 32] = (int)t; e[BG_SLOT * 32] = (int)slot;
           pushed = true;
         }
+        // a small box without a covered sample needs no record
+        if (slot != no_slot && covers) fill_record<PERSP>(p, s, sm.srec + slot * p.rec_stride);
       }
     }
     {
-      const unsigned f = fragment_pass(sb, p.g.bshift_x, wst, skey, lane);
+      const unsigned f = fragment_pass(sb, p.g.bshift_x, wst, skey, lane) +
+                         medium_pass(med_rows, med_place, p.g.bshift_x, wst, skey, lane);
       if (STATS && lane == 0) st.frags += f;
     }
     // every thread gets the same count of queued large triangles
@@ -797,7 +967,7 @@ __device__ __forceinline__ void process_tile(const TileScene& p, int tile, unsig
     if (slot != no_slot)
       shade_from_record<PERSP>(p, sm.srec + slot * p.rec_stride, x, y, o);
     else
-      shade_from_global<PERSP, CLIP>(p, t, x, y, o);
+      shade_from_global<PERSP, CLIP>(p, tri_indices(p.tris, t), x, y, o);
   }
   __syncthreads();
 }
