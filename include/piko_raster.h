@@ -232,6 +232,12 @@ int piko_raster_backward(piko_raster *h, const piko_scene *scene, const piko_fra
                          const float *dl_drgba, float *dl_dcolor, float *dl_dnormal,
                          float *dl_dlight, void *cuda_stream);
 
+/* The same gradients, stored instead of added: the arrays need no clearing
+ * before the call, and every element is written. */
+int piko_raster_backward_set(piko_raster *h, const piko_scene *scene, const piko_framebuffer *fwd,
+                             const float *dl_drgba, float *dl_dcolor, float *dl_dnormal,
+                             float *dl_dlight, void *cuda_stream);
+
 /* Deferred light pass over a G-buffer written by a GBUFFER forward: for each
  * covered pixel, sum of n_lights point lights (lights: device [n][4] =
  * x, y, z in pixel units, intensity) with

@@ -28,18 +28,17 @@ class _RasterShade(torch.autograd.Function):
                      normal is not None and ctx.needs_input_grad[1],
                      light is not None and ctx.needs_input_grad[2])
         ctx.mark_non_differentiable(fb.key)
+        ctx.set_materialize_grads(False)  # no zero-filled gradient for the key
         return fb.rgba, fb.key
 
     @staticmethod
     def backward(ctx, g_rgba, g_key):
         ds = ctx.scene
         need_c, need_n, need_l = ctx.needs
-        dc = torch.zeros_like(ds.color) if need_c else None
-        dn = torch.zeros_like(ds.normal) if need_n else None
-        dl = torch.zeros_like(ds.light_dir) if need_l else None
-        if g_rgba is not None and (need_c or need_n or need_l):
-            ctx.rasterizer.backward(ds, ctx.fb, g_rgba.contiguous(), dc, dn, dl)
-        return dc, dn, dl, None, None
+        if g_rgba is None or not (need_c or need_n or need_l):
+            return (torch.zeros_like(ds.color) if need_c else None, torch.zeros_like(ds.normal) if need_n else None,
+                    torch.zeros_like(ds.light_dir) if need_l else None, None, None)
+        return (*ctx.rasterizer.gradients(ds, ctx.fb, g_rgba, need_c, need_n, need_l), None, None)
 
 
 def render(rasterizer: Rasterizer, scene: DeviceScene, color: Optional[torch.Tensor] = None,

@@ -28,8 +28,8 @@ int piko_backward_launch(int W, int H, int mode, int unclamped, int T, int V, co
                          const float* vdot, const float4* vattr, const float* color, const float* normal,
                          const float* light,
                          const float* invw, const float* pos, const float* mvp, const unsigned long long* key,
-                         const float* dl_drgba, float4* acc, float* dcolor, float* dnormal, float* dlight, int num_sms,
-                         cudaStream_t s);
+                         const float* dl_drgba, float4* acc, float* dcolor, float* dnormal, float* dlight, int set,
+                         int num_sms, cudaStream_t s);
 
 struct piko_raster {
   int W, H, bin_w, bin_h, schedule;
@@ -706,6 +706,21 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
   }
 }
 
+// The device's address of a host buffer that kernels can write (pinned from
+// its first byte to its last, 16-byte aligned), or NULL.
+static void* mapped_host(void* p, size_t bytes) {
+  cudaPointerAttributes a, z;
+  if (!aligned16(p) || cudaPointerGetAttributes(&a, p) != cudaSuccess ||
+      cudaPointerGetAttributes(&z, static_cast<char*>(p) + bytes - 1) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (a.type != cudaMemoryTypeHost || z.type != cudaMemoryTypeHost || !a.devicePointer ||
+      static_cast<char*>(z.devicePointer) != static_cast<char*>(a.devicePointer) + (bytes - 1))
+    return nullptr;
+  return a.devicePointer;
+}
+
 int piko_raster_forward_host(piko_raster* h, const piko_scene* s, piko_framebuffer* fb, void* cuda_stream) {
   if (!h || !s || !fb) return PIKO_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
@@ -722,10 +737,22 @@ int piko_raster_forward_host(piko_raster* h, const piko_scene* s, piko_framebuff
   if (r == PIKO_OK && s->color) r = grow(h, &h->hs_color, &h->hcap_color, 3 * V, "host-scene colours");
   if (r == PIKO_OK && s->normal) r = grow(h, &h->hs_normal, &h->hcap_normal, 3 * V, "host-scene normals");
   if (r == PIKO_OK) r = grow(h, &h->hs_small, &h->hcap_small, 20, "host-scene matrix and light");
-  if (r == PIKO_OK) r = grow(h, &h->hs_key, &h->hcap_key, P, "host-framebuffer keys");
-  if (r == PIKO_OK && fb->rgba && !gbuf) r = grow(h, &h->hs_rgba, &h->hcap_rgba, P, "host-framebuffer colour");
-  if (r == PIKO_OK && gbuf && fb->gbuf_normal) r = grow(h, &h->hs_gn, &h->hcap_gn, P, "host G-buffer normals");
-  if (r == PIKO_OK && gbuf && fb->gbuf_albedo) r = grow(h, &h->hs_ga, &h->hcap_ga, P, "host G-buffer albedo");
+  // The result is 24 bytes a pixel against a link that takes 187 GB/s whether
+  // a copy engine or kernels fill it (and 204 GB/s inwards), so pinned output
+  // buffers are written by the kernels themselves: the shading then runs
+  // inside the transfer instead of before it.  Pageable ones take a copy, and
+  // so do the mappings that also read the key buffer back.
+  const auto mapped = [&](void* p, long long bytes) {
+    return p && h->schedule <= PIKO_SCHED_HARDWARE ? mapped_host(p, (size_t)(P * bytes)) : nullptr;
+  };
+  void* const m_key = mapped(fb->key, 8);
+  void* const m_rgba = gbuf ? nullptr : mapped(fb->rgba, 16);
+  void* const m_gn = gbuf ? mapped(fb->gbuf_normal, 8) : nullptr;
+  void* const m_ga = gbuf ? mapped(fb->gbuf_albedo, 8) : nullptr;
+  if (r == PIKO_OK && !m_key) r = grow(h, &h->hs_key, &h->hcap_key, P, "host-framebuffer keys");
+  if (r == PIKO_OK && fb->rgba && !gbuf && !m_rgba) r = grow(h, &h->hs_rgba, &h->hcap_rgba, P, "host-framebuffer colour");
+  if (r == PIKO_OK && gbuf && fb->gbuf_normal && !m_gn) r = grow(h, &h->hs_gn, &h->hcap_gn, P, "host G-buffer normals");
+  if (r == PIKO_OK && gbuf && fb->gbuf_albedo && !m_ga) r = grow(h, &h->hs_ga, &h->hcap_ga, P, "host G-buffer albedo");
   if (r != PIKO_OK) return r;
   piko_scene ds = *s;
   ds.pos = reinterpret_cast<const float*>(h->hs_pos);
@@ -755,17 +782,17 @@ int piko_raster_forward_host(piko_raster* h, const piko_scene* s, piko_framebuff
     const cudaError_t e = cudaMemcpyAsync(c.dst, c.src, c.bytes, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "host-to-device copy");
   }
-  dfb.key = reinterpret_cast<uint64_t*>(h->hs_key);
-  dfb.rgba = fb->rgba && !gbuf ? reinterpret_cast<float*>(h->hs_rgba) : nullptr;
-  dfb.gbuf_normal = gbuf && fb->gbuf_normal ? h->hs_gn : nullptr;
-  dfb.gbuf_albedo = gbuf && fb->gbuf_albedo ? h->hs_ga : nullptr;
+  dfb.key = m_key ? static_cast<uint64_t*>(m_key) : reinterpret_cast<uint64_t*>(h->hs_key);
+  if (fb->rgba && !gbuf) dfb.rgba = m_rgba ? static_cast<float*>(m_rgba) : reinterpret_cast<float*>(h->hs_rgba);
+  if (gbuf && fb->gbuf_normal) dfb.gbuf_normal = m_gn ? m_gn : h->hs_gn;
+  if (gbuf && fb->gbuf_albedo) dfb.gbuf_albedo = m_ga ? m_ga : h->hs_ga;
   r = piko_raster_forward(h, &ds, &dfb, cuda_stream);
   if (r != PIKO_OK) return r;
   const Copy out[] = {
-      {fb->key, dfb.key, (size_t)P * 8},
-      {fb->rgba, dfb.rgba, dfb.rgba ? (size_t)P * 16 : 0},
-      {fb->gbuf_normal, dfb.gbuf_normal, dfb.gbuf_normal ? (size_t)P * 8 : 0},
-      {fb->gbuf_albedo, dfb.gbuf_albedo, dfb.gbuf_albedo ? (size_t)P * 8 : 0},
+      {fb->key, dfb.key, m_key ? 0 : (size_t)P * 8},
+      {fb->rgba, dfb.rgba, dfb.rgba && !m_rgba ? (size_t)P * 16 : 0},
+      {fb->gbuf_normal, dfb.gbuf_normal, dfb.gbuf_normal && !m_gn ? (size_t)P * 8 : 0},
+      {fb->gbuf_albedo, dfb.gbuf_albedo, dfb.gbuf_albedo && !m_ga ? (size_t)P * 8 : 0},
   };
   for (const Copy& c : out) {
     if (c.bytes == 0) continue;
@@ -845,8 +872,9 @@ int piko_raster_stats(piko_raster* h, int64_t out[5]) {
   return PIKO_OK;
 }
 
-int piko_raster_backward(piko_raster* h, const piko_scene* s, const piko_framebuffer* fwd, const float* dl_drgba,
-                         float* dl_dcolor, float* dl_dnormal, float* dl_dlight, void* cuda_stream) {
+// set: the gradients are stored instead of added.
+static int backward_pass(piko_raster* h, const piko_scene* s, const piko_framebuffer* fwd, const float* dl_drgba,
+                         float* dl_dcolor, float* dl_dnormal, float* dl_dlight, bool set, void* cuda_stream) {
   if (!h) return PIKO_ERR_INVALID_ARG;
   int r = check_scene(h, s);
   if (r != PIKO_OK) return r;
@@ -859,6 +887,16 @@ int piko_raster_backward(piko_raster* h, const piko_scene* s, const piko_framebu
   if ((r = grow_vertices(h, s->num_vertices)) != PIKO_OK) return r;
   const bool lambert = s->shade_mode == PIKO_SHADE_LAMBERT;
   float* invw = h->perspective ? h->invw : nullptr;
+  if (set) {
+    // arrays that the kernels below do not write
+    const size_t n = 3 * sizeof(float) * (size_t)s->num_vertices;
+    const bool none = s->num_vertices == 0 || s->num_triangles == 0;
+    cudaError_t e = cudaSuccess;
+    if (dl_dcolor && (none || (lambert && !s->color))) e = cudaMemsetAsync(dl_dcolor, 0, n, st);
+    if (e == cudaSuccess && dl_dnormal && (none || !lambert)) e = cudaMemsetAsync(dl_dnormal, 0, n, st);
+    if (e == cudaSuccess && dl_dlight && (none || !lambert)) e = cudaMemsetAsync(dl_dlight, 0, 3 * sizeof(float), st);
+    if (e != cudaSuccess) return cuda_fail(h, e, "gradient clear");
+  }
   if (h->gacc_dirty) {
     const cudaError_t e = cudaMemsetAsync(h->gacc, 0, (size_t)h->vcap * sizeof(float4), st);
     if (e != cudaSuccess) return cuda_fail(h, e, "gradient sums");
@@ -870,15 +908,26 @@ int piko_raster_backward(piko_raster* h, const piko_scene* s, const piko_framebu
   // scene the handle rasterized last
   float4* vattr = packed_attributes(h, s);
   launch_vertex(h->W, h->H, s->num_vertices, s->pos, s->mvp, h->vtx, lambert ? s->normal : nullptr, s->light_dir,
-                lambert ? h->vdot : nullptr, invw, h->num_sms, st, nullptr, nullptr, s->color, vattr);
+                lambert ? h->vdot : nullptr, invw, h->num_sms, st, nullptr, nullptr, s->color, vattr,
+                set && lambert ? dl_dlight : nullptr);
   if (piko_backward_launch(h->W, h->H, s->shade_mode, h->unclamped, s->num_triangles, s->num_vertices, s->tris,
                            h->vtx, h->vdot, vattr, s->color, s->normal, s->light_dir, invw, h->clip ? s->pos : nullptr,
                            s->mvp, reinterpret_cast<const unsigned long long*>(fwd->key), dl_drgba, h->gacc, dl_dcolor,
-                           dl_dnormal, dl_dlight, h->num_sms, st) != 0) {
+                           dl_dnormal, dl_dlight, set ? 1 : 0, h->num_sms, st) != 0) {
     h->gacc_dirty = true;
     return cuda_fail(h, cudaGetLastError(), "backward launch");
   }
   return PIKO_OK;
+}
+
+int piko_raster_backward(piko_raster* h, const piko_scene* s, const piko_framebuffer* fwd, const float* dl_drgba,
+                         float* dl_dcolor, float* dl_dnormal, float* dl_dlight, void* cuda_stream) {
+  return backward_pass(h, s, fwd, dl_drgba, dl_dcolor, dl_dnormal, dl_dlight, false, cuda_stream);
+}
+
+int piko_raster_backward_set(piko_raster* h, const piko_scene* s, const piko_framebuffer* fwd, const float* dl_drgba,
+                             float* dl_dcolor, float* dl_dnormal, float* dl_dlight, void* cuda_stream) {
+  return backward_pass(h, s, fwd, dl_drgba, dl_dcolor, dl_dnormal, dl_dlight, true, cuda_stream);
 }
 
 int piko_raster_deferred_light(piko_raster* h, const piko_framebuffer* gbuf, const float* lights, int n_lights,

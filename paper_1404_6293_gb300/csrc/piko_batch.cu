@@ -43,6 +43,7 @@ struct BatchScene {
   // backward
   const float4* dl;
   float4* acc;  // the gradient sums of the scene's vertices (NULL: no gradients wanted)
+  const float4* attr;  // colour and n . L of the vertices for the backward (Lambert)
 };
 
 struct BatchSync {
@@ -62,10 +63,9 @@ struct BatchParams {
   const int* bin_prefix;
   const int* stat_prefix;  // tiles of static scenes
   const int* dyn_prefix;   // tiles of dynamic scenes
-  const int* btile_prefix;  // backward tiles (BWD_TILE_W x BATCH_BWD_TILE_H) of the tile form's scenes
-  const int* pblock_prefix;  // 8 x 4 pixel blocks of the pixel form's scenes
+  const int* pblock_prefix;  // 16 x 2 pixel blocks (backward)
   int total_pblocks;
-  int total_v, total_t, total_bins, total_static, total_dyn, total_btiles;
+  int total_v, total_t, total_bins, total_static, total_dyn;
   int4* vtx;
   float4* vattr;  // colour and n . L per vertex (Lambert; the colour only where the scene has one)
   float* invw;  // 1 / clip w per vertex (perspective-correct attributes), else NULL
@@ -499,15 +499,15 @@ __global__ void __maxnreg__(PIKO_BATCH_MAXNREG) k_batch_forward(BatchParams b) {
 }
 
 // ------------------------------------------------------------------ backward
-// BWD_TILE_W x BATCH_BWD_TILE_H tiles of every scene, dealt round robin; each tile's gradients are
-// accumulated as in the single-scene backward.
+// 16 x 2 blocks of pixels of every scene; the gradients are accumulated as in
+// the single-scene backward.
 struct BatchBwdParams {
   int n;
   const BatchScene* sc;
-  const int* btile_prefix;  // [n+1] backward tiles per scene (tile form; 0 for a scene of the pixel form)
-  const int* pblock_prefix;  // [n+1] 8 x 4 pixel blocks per scene (pixel form; else 0)
-  int total_btiles, total_pblocks;
+  const int* pblock_prefix;  // [n+1] 16 x 2 pixel blocks per scene
+  int total_pblocks;
   const int4* vtx;
+  float4* vattr;      // colour and n . L per vertex, rewritten here for the first scene of each group
   const float* invw;  // as in BatchParams
   // accumulators (GradAcc) of the finishing pass and the prefix of their chunks
   int ngroups, total_chunks;
@@ -524,58 +524,35 @@ __device__ __forceinline__ void fill_bwd_scene(const BatchBwdParams& b, const Ba
   c.key = d.key_out; c.dl = d.dl; c.acc = d.acc;
 }
 
-// Warp form: each warp takes whole tiles (grid-stride over the batch's
-// tiles), with no CTA barrier; the scene of a tile is found by every lane
-// (uniform loads) and its descriptor kept in the warp's shared slot (in
-// registers it would cost the tile loop its occupancy).
-constexpr int BATCH_BWD_WARPS = BWD_THREADS / 32;
-struct BatchBwdSmem {
-  float stage[BATCH_BWD_WARPS][BWD_VALS][33];
-  BwdScene sc[BATCH_BWD_WARPS];
-};
-template <bool PERSP>
-#ifndef PIKO_BWD_MINB
-#define PIKO_BWD_MINB 3
-#endif
-__global__ void __launch_bounds__(BWD_THREADS, PIKO_BWD_MINB) k_batch_backward(BatchBwdParams b) {
-  extern __shared__ __align__(16) unsigned char bwd_smem_raw[];
-  BatchBwdSmem& sm = *reinterpret_cast<BatchBwdSmem*>(bwd_smem_raw);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nwarps = gridDim.x * BATCH_BWD_WARPS;
-  BwdScene& c = sm.sc[warp];
-  for (int i = blockIdx.x * BATCH_BWD_WARPS + warp; i < b.total_btiles; i += nwarps) {
-    const int s = find_scene(b.btile_prefix, b.n, i);
-    const BatchScene& d = b.sc[s];
-    if (d.acc == nullptr) continue;  // the same for the whole warp
-    __syncwarp();  // the previous tile's reads of c are done
-    if (lane == 0) fill_bwd_scene(b, d, c);
-    __syncwarp();
-    float L0 = 0.f, L1 = 0.f, L2 = 0.f;
-    if (c.mode == PIKO_SHADE_LAMBERT) {
-      L0 = __ldg(c.light); L1 = __ldg(c.light + 1); L2 = __ldg(c.light + 2);
-    }
-    const int lt = i - __ldg(b.btile_prefix + s);
-    const int ntx = (c.W + BWD_TILE_W - 1) / BWD_TILE_W;
-    const int ty = lt / ntx, tx = lt - ty * ntx;
-    backward_warp_tile<PERSP, false, BATCH_BWD_TILE_H>(c, tx * BWD_TILE_W, ty * BATCH_BWD_TILE_H, sm.stage[warp],
-                                                        L0, L1, L2);
+// Colour and n . L of the vertices of each group of Lambert scenes: the
+// attributes may have changed since the forward pass.  One 16-byte gather per
+// vertex then serves a pixel in place of six words (the pixel kernel was at 82%
+// of the L1's throughput with those).
+__global__ void __launch_bounds__(GRAD_CHUNK) k_batch_attributes(BatchBwdParams b) {
+  for (int i = blockIdx.x; i < b.total_chunks; i += gridDim.x) {
+    const int g = find_scene(b.chunk_prefix, b.ngroups, i);
+    const GradAcc& f = b.groups[g];
+    const int v = (i - __ldg(b.chunk_prefix + g)) * GRAD_CHUNK + (int)threadIdx.x;
+    if (!f.normal || v >= f.V) continue;
+    const float *n = f.normal + 3 * (size_t)v, *c = f.color + 3 * (size_t)v;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (f.color) a = make_float4(__ldg(c), __ldg(c + 1), __ldg(c + 2), 0.f);
+    a.w = __ldg(n) * __ldg(f.light) + __ldg(n + 1) * __ldg(f.light + 1) + __ldg(n + 2) * __ldg(f.light + 2);
+    f.attr[v] = a;
   }
 }
-constexpr size_t BATCH_BWD_SMEM = sizeof(BatchBwdSmem);
 
-// Pixel form: a warp takes BATCH_PIX_RUN blocks of 8 x 4 pixels in a row, so
+// A warp takes BATCH_PIX_RUN blocks of 16 x 2 pixels in a row, so
 // that it looks its scene up once for most of them.
 constexpr int BATCH_PIX_RUN = 4;
 template <bool PERSP>
 __global__ void __launch_bounds__(PIX_THREADS, 4) k_batch_backward_pixel(BatchBwdParams b) {
-  __shared__ float sval[PIX_THREADS / 32][BWD_VALS][32];
   __shared__ BwdScene ssc[PIX_THREADS / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int first = (blockIdx.x * (PIX_THREADS / 32) + warp) * BATCH_PIX_RUN;
   if (first >= b.total_pblocks) return;  // the same for the whole warp
   BwdScene& c = ssc[warp];
   int s = find_scene(b.pblock_prefix, b.n, first), held = -1;
-  float L0 = 0.f, L1 = 0.f, L2 = 0.f;
   for (int i = first; i < min(first + BATCH_PIX_RUN, b.total_pblocks); ++i) {
     while (s + 1 < b.n && __ldg(b.pblock_prefix + s + 1) <= i) ++s;
     const BatchScene& d = b.sc[s];
@@ -585,16 +562,11 @@ __global__ void __launch_bounds__(PIX_THREADS, 4) k_batch_backward_pixel(BatchBw
       if (lane == 0) fill_bwd_scene(b, d, c);
       __syncwarp();
       held = s;
-      if (c.mode == PIKO_SHADE_LAMBERT) {
-        L0 = __ldg(c.light); L1 = __ldg(c.light + 1); L2 = __ldg(c.light + 2);
-      }
     }
     const int lt = i - __ldg(b.pblock_prefix + s);
     const int ntx = (c.W + PIX_W - 1) / PIX_W;
     const int ty = lt / ntx, tx = lt - ty * ntx;
-    backward_warp_pixels<PERSP>(c, nullptr, nullptr, tx * PIX_W + (lane & (PIX_W - 1)), ty * PIX_H + lane / PIX_W, sval[warp], L0,
-                                L1, L2);
-    __syncwarp();  // sval is rewritten by the next block
+    backward_warp_pixels<PERSP>(c, nullptr, d.attr, tx * PIX_W + (lane & (PIX_W - 1)), ty * PIX_H + lane / PIX_W);
   }
 }
 
@@ -656,7 +628,7 @@ struct BatchState {
   // host staging (pinned) and the last layout
   void* staging = nullptr;
   size_t staging_cap = 0;
-  size_t desc_bytes = 0;   // of the last layout: scenes, 7 prefix arrays, gradient groups and their prefix
+  size_t desc_bytes = 0;   // of the last layout: scenes, 6 prefix arrays, gradient groups and their prefix
   size_t group_off = 0;    // where the gradient groups start
   cudaEvent_t uploaded = nullptr;
   BatchParams params;
@@ -728,8 +700,8 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   if (!bs) bs = new BatchState();
   if (n < 1 || !scenes || !fbs) { err = "batch needs n >= 1 scenes and framebuffers"; return PIKO_ERR_INVALID_ARG; }
   std::vector<BatchScene> d(n);
-  std::vector<int> pv(n + 1), pt(n + 1), pb(n + 1), ps(n + 1), pd(n + 1), pp(n + 1), pq(n + 1);
-  long long tv = 0, tt = 0, tb = 0, tsd = 0, tdy = 0, tp = 0, tq = 0, tk = 0;
+  std::vector<int> pv(n + 1), pt(n + 1), pb(n + 1), ps(n + 1), pd(n + 1), pq(n + 1);
+  long long tv = 0, tt = 0, tb = 0, tsd = 0, tdy = 0, tq = 0, tk = 0;
   int max_bin_px = 64, max_rec = 0;
   // shading records per tile from the last frame's mean entries per bin
   const int slots_hint = bs ? slots_for_entries(bs->last_entries, (int)(bs->last_bins > 0 ? bs->last_bins : 1)) : 0;
@@ -774,20 +746,16 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
     x.gnorm_out = reinterpret_cast<uint2*>(f.gbuf_normal);
     x.galb_out = reinterpret_cast<uint2*>(f.gbuf_albedo);
     const int ntiles = x.g.nbx * x.g.nby;
-    pv[i] = (int)tv; pt[i] = (int)tt; pb[i] = (int)tb; ps[i] = (int)tsd; pd[i] = (int)tdy; pp[i] = (int)tp; pq[i] = (int)tq;
+    pv[i] = (int)tv; pt[i] = (int)tt; pb[i] = (int)tb; ps[i] = (int)tsd; pd[i] = (int)tdy; pq[i] = (int)tq;
     tv += x.V; tt += x.T; tb += ntiles;
-    if (bwd_pixel_form(x.T, s.width, s.height))
-      tq += (long long)((s.width + PIX_W - 1) / PIX_W) * ((s.height + PIX_H - 1) / PIX_H);
-    else
-      tp += (long long)((s.width + BWD_TILE_W - 1) / BWD_TILE_W) *
-            ((s.height + BATCH_BWD_TILE_H - 1) / BATCH_BWD_TILE_H);
+    tq += (long long)((s.width + PIX_W - 1) / PIX_W) * ((s.height + PIX_H - 1) / PIX_H);
     if (sched == PIKO_SCHED_STATIC) tsd += ntiles;
     else tdy += ntiles;
     if (bw * bh > max_bin_px) max_bin_px = bw * bh;
     if (x.nslots * x.rec_stride > max_rec) max_rec = x.nslots * x.rec_stride;
   }
-  pv[n] = (int)tv; pt[n] = (int)tt; pb[n] = (int)tb; ps[n] = (int)tsd; pd[n] = (int)tdy; pp[n] = (int)tp; pq[n] = (int)tq;
-  if (tv >= (1LL << 31) || tt >= (1LL << 31) || tb >= (1LL << 31) || tp + tq >= (1LL << 31)) {
+  pv[n] = (int)tv; pt[n] = (int)tt; pb[n] = (int)tb; ps[n] = (int)tsd; pd[n] = (int)tdy; pq[n] = (int)tq;
+  if (tv >= (1LL << 31) || tt >= (1LL << 31) || tb >= (1LL << 31) || tq >= (1LL << 31)) {
     err = "batch too large (a total reaches 2^31)";
     return PIKO_ERR_INVALID_ARG;
   }
@@ -833,11 +801,11 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
       return PIKO_ERR_OOM;
     }
   }
-  // descriptors + 7 prefix arrays, uploaded from pinned memory; room after
+  // descriptors + 6 prefix arrays, uploaded from pinned memory; room after
   // them for the backward's gradient groups and their prefix
   const size_t dbytes = sizeof(BatchScene) * n;
   const size_t pbytes = sizeof(int) * (n + 1);
-  const size_t group_off = (dbytes + 7 * pbytes + 15) / 16 * 16;
+  const size_t group_off = (dbytes + 6 * pbytes + 15) / 16 * 16;
   const size_t total = group_off + sizeof(GradAcc) * n + pbytes;
   if (!bs->uploaded && cudaEventCreateWithFlags(&bs->uploaded, cudaEventDisableTiming) != cudaSuccess) {
     err = "cudaEventCreate failed";
@@ -862,8 +830,8 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   }
   char* h = static_cast<char*>(bs->staging);
   std::memcpy(h, d.data(), dbytes);
-  const std::vector<int>* arrays[7] = {&pv, &pt, &pb, &ps, &pd, &pp, &pq};
-  for (int a = 0; a < 7; ++a) std::memcpy(h + dbytes + a * pbytes, arrays[a]->data(), pbytes);
+  const std::vector<int>* arrays[6] = {&pv, &pt, &pb, &ps, &pd, &pq};
+  for (int a = 0; a < 6; ++a) std::memcpy(h + dbytes + a * pbytes, arrays[a]->data(), pbytes);
   if (cudaMemcpyAsync(bs->desc, bs->staging, group_off, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
       cudaEventRecord(bs->uploaded, stream) != cudaSuccess) {
     err = "upload of batch descriptors failed";
@@ -879,11 +847,10 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   b.bin_prefix = reinterpret_cast<const int*>(dd + dbytes + 2 * pbytes);
   b.stat_prefix = reinterpret_cast<const int*>(dd + dbytes + 3 * pbytes);
   b.dyn_prefix = reinterpret_cast<const int*>(dd + dbytes + 4 * pbytes);
-  b.btile_prefix = reinterpret_cast<const int*>(dd + dbytes + 5 * pbytes);
-  b.pblock_prefix = reinterpret_cast<const int*>(dd + dbytes + 6 * pbytes);
+  b.pblock_prefix = reinterpret_cast<const int*>(dd + dbytes + 5 * pbytes);
   b.total_pblocks = (int)tq;
   b.total_v = (int)tv; b.total_t = (int)tt; b.total_bins = (int)tb; b.total_static = (int)tsd;
-  b.total_dyn = (int)tdy; b.total_btiles = (int)tp;
+  b.total_dyn = (int)tdy;
   b.vtx = bs->vtx; b.vattr = bs->vattr; b.invw = persp ? bs->invw : nullptr; b.rect = bs->rect; b.cnt = bs->cnt; b.bin_off = bs->bin_off;
   b.dkeys = bs->dkeys; b.total_dkeys = (unsigned)tk;
   b.cursor = bs->cursor; b.chunk_state = bs->chunk_state; b.bin_tris = bs->bin_tris;
@@ -1006,22 +973,28 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
     const bool lambert = d[i].mode == PIKO_SHADE_LAMBERT;
     GradAcc g;
     g.V = d[i].V;
+    g.set = 0;
     g.normal = lambert ? d[i].normal : nullptr;
     g.light = lambert ? d[i].light : nullptr;
+    g.color = lambert ? d[i].color : nullptr;
+    g.attr = bs->vattr + d[i].vtx_base;
     g.dcolor = dc && (!lambert || d[i].color) ? dc[i] : nullptr;
     g.dnormal = dn && lambert ? dn[i] : nullptr;
     g.dlight = dlt && lambert ? dlt[i] : nullptr;
     d[i].acc = nullptr;
+    d[i].attr = nullptr;
     if (!d[i].dl || d[i].mode == PIKO_SHADE_GBUFFER || g.V == 0 || (!g.dcolor && !g.dnormal && !g.dlight)) continue;
     if (!groups.empty()) {
       const GradAcc& q = groups.back();
-      if (q.V == g.V && q.normal == g.normal && q.light == g.light && q.dcolor == g.dcolor &&
+      if (q.V == g.V && q.normal == g.normal && q.light == g.light && q.color == g.color && q.dcolor == g.dcolor &&
           q.dnormal == g.dnormal && q.dlight == g.dlight) {
         d[i].acc = q.acc;
+        d[i].attr = q.attr;
         continue;
       }
     }
     g.acc = d[i].acc = bs->gacc + acc_used;
+    d[i].attr = g.attr;
     acc_used += g.V;  // at most the batch's vertices
     groups.push_back(g);
     chunk_prefix.push_back(chunk_prefix.back() + (g.V + GRAD_CHUNK - 1) / GRAD_CHUNK);
@@ -1053,53 +1026,26 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
   BatchBwdParams p;
   p.n = n;
   p.sc = bs->params.sc;
-  p.btile_prefix = bs->params.btile_prefix;
-  p.total_btiles = bs->params.total_btiles;
   p.pblock_prefix = bs->params.pblock_prefix;
   p.total_pblocks = bs->params.total_pblocks;
   p.vtx = bs->vtx;
+  p.vattr = bs->vattr;
   p.invw = bs->params.invw;  // the interpolation of the last forward_batch
   p.ngroups = (int)groups.size();
   p.total_chunks = chunk_prefix.back();
   p.groups = reinterpret_cast<const GradAcc*>(static_cast<const char*>(bs->desc) + bs->group_off);
   p.chunk_prefix = reinterpret_cast<const int*>(static_cast<const char*>(bs->desc) + prefix_off);
-  static int per_sm_of[64] = {0};  // the shared-memory opt-in is per device
-  int dev = 0;
-  cudaGetDevice(&dev);
-  int& per_sm = per_sm_of[dev & 63];
-  if (per_sm == 0) {
-    int v = 0;
-    // both instances share the launch bounds and the shared-memory size
-    if (cudaFuncSetAttribute(k_batch_backward<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)BATCH_BWD_SMEM) != cudaSuccess ||
-        cudaFuncSetAttribute(k_batch_backward<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)BATCH_BWD_SMEM) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_batch_backward<false>, BWD_THREADS, BATCH_BWD_SMEM) !=
-            cudaSuccess ||
-        v < 1)
-      v = 1;
-    per_sm = v;
-  }
-  long long blocks = (long long)per_sm * num_sms;
-  const long long need = (p.total_btiles + BATCH_BWD_WARPS - 1) / BATCH_BWD_WARPS;  // a tile per warp
-  if (blocks > need) blocks = need;
-  if (p.total_btiles > 0) {
-    if (bs->persp)
-      k_batch_backward<true><<<(int)blocks, BWD_THREADS, BATCH_BWD_SMEM, stream>>>(p);
-    else
-      k_batch_backward<false><<<(int)blocks, BWD_THREADS, BATCH_BWD_SMEM, stream>>>(p);
-  }
-  if (p.total_pblocks > 0) {
-    const int per_cta = PIX_THREADS / 32 * BATCH_PIX_RUN;
-    const int pblocks = (p.total_pblocks + per_cta - 1) / per_cta;
-    if (bs->persp)
-      k_batch_backward_pixel<true><<<pblocks, PIX_THREADS, 0, stream>>>(p);
-    else
-      k_batch_backward_pixel<false><<<pblocks, PIX_THREADS, 0, stream>>>(p);
-  }
+  const int chunk_blocks = p.total_chunks < 8 * num_sms ? p.total_chunks : 8 * num_sms;
+  k_batch_attributes<<<chunk_blocks, GRAD_CHUNK, 0, stream>>>(p);
+  const int per_cta = PIX_THREADS / 32 * BATCH_PIX_RUN;
+  const int pblocks = (p.total_pblocks + per_cta - 1) / per_cta;
+  if (bs->persp)
+    k_batch_backward_pixel<true><<<pblocks, PIX_THREADS, 0, stream>>>(p);
+  else
+    k_batch_backward_pixel<false><<<pblocks, PIX_THREADS, 0, stream>>>(p);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)
-    e = launch_pdl(k_batch_finish, p.total_chunks < 8 * num_sms ? p.total_chunks : 8 * num_sms, GRAD_CHUNK, 0, stream, p);
+    e = launch_pdl(k_batch_finish, chunk_blocks, GRAD_CHUNK, 0, stream, p);
   if (e != cudaSuccess) {
     bs->gacc_dirty = true;
     err = std::string("batch backward launch: ") + cudaGetErrorString(e);

@@ -23,7 +23,8 @@ __global__ void __launch_bounds__(256) k_vertex(int W, int H, int V, const float
                                                 const float* __restrict__ normal, const float* __restrict__ light,
                                                 float* __restrict__ vdot, float* __restrict__ invw,
                                                 unsigned long long* __restrict__ dkeys, DevStatus* clip_st,
-                                                const float* __restrict__ color, float4* __restrict__ vattr) {
+                                                const float* __restrict__ color, float4* __restrict__ vattr,
+                                                float* zero3) {
   pdl_launch_dependents();  // the count pass may be scheduled; it waits for this grid before reading
   __shared__ float m[16];
   const bool has_m = mvp != nullptr;
@@ -32,6 +33,7 @@ __global__ void __launch_bounds__(256) k_vertex(int W, int H, int V, const float
     __syncthreads();
   }
   if (dkeys) clear_keys(dkeys, (size_t)W * H);
+  if (zero3 && blockIdx.x == 0 && threadIdx.x < 3) zero3[threadIdx.x] = 0.0f;
   if (clip_st && blockIdx.x == 0 && threadIdx.x == 0) clip_st->clip_count = 0u;
   const float fW = (float)W, fH = (float)H;
   float L0 = 0.f, L1 = 0.f, L2 = 0.f;
@@ -62,7 +64,8 @@ __global__ void __launch_bounds__(256) k_vertex(int W, int H, int V, const float
 
 void launch_vertex(int W, int H, int V, const float* pos, const float* mvp, int4* vtx, const float* normal,
                    const float* light, float* vdot, float* invw, int num_sms, cudaStream_t s,
-                   unsigned long long* dkeys, DevStatus* clip_st, const float* color, float4* vattr) {
+                   unsigned long long* dkeys, DevStatus* clip_st, const float* color, float4* vattr,
+                   float* zero3) {
   if (V <= 0) return;
   // one vertex per thread: every load is in flight at once; at least a wave
   // of CTAs when there are keys to clear
@@ -70,10 +73,10 @@ void launch_vertex(int W, int H, int V, const float* pos, const float* mvp, int4
   if (dkeys && blocks < 8 * num_sms) blocks = 8 * num_sms;
   if (invw)
     k_vertex<true><<<blocks, 256, 0, s>>>(W, H, V, reinterpret_cast<const float4*>(pos), mvp, vtx, normal, light, vdot,
-                                          invw, dkeys, clip_st, color, vattr);
+                                          invw, dkeys, clip_st, color, vattr, zero3);
   else
     k_vertex<false><<<blocks, 256, 0, s>>>(W, H, V, reinterpret_cast<const float4*>(pos), mvp, vtx, normal, light,
-                                           vdot, nullptr, dkeys, clip_st, color, vattr);
+                                           vdot, nullptr, dkeys, clip_st, color, vattr, zero3);
 }
 
 // ======================================================================

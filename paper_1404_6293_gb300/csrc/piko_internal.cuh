@@ -384,11 +384,12 @@ struct DirectRaster {
 // interpolate to the same value).
 // dkeys (optional): W * H keys of the count pass's direct rasterization, set
 // to KEY_EMPTY here; clip_st (optional): its clip_count is set to 0; vattr
-// (optional, with vdot): takes each vertex's colour and n . L in vdot's place.
+// (optional, with vdot): takes each vertex's colour and n . L in vdot's place;
+// zero3 (optional): three floats set to 0.
 void launch_vertex(int W, int H, int V, const float* pos, const float* mvp, int4* vtx, const float* normal,
                    const float* light, float* vdot, float* invw, int num_sms, cudaStream_t s,
                    unsigned long long* dkeys = nullptr, DevStatus* clip_st = nullptr, const float* color = nullptr,
-                   float4* vattr = nullptr);
+                   float4* vattr = nullptr, float* zero3 = nullptr);
 // Count pass and scan (two launches): bin_count holds 2 * nbins counters
 // (single-bin and multi-bin entries), zero between frames; the scan turns
 // them into CSR offsets and scatter cursors (capacity: entries the bin lists

@@ -850,7 +850,9 @@ __device__ __forceinline__ void process_tile(const TileScene& p, int tile, unsig
     __syncthreads();
   }
   for (unsigned c = beg; c < end; c += nt) {
-    // entries are dealt to the warps one by one, so that a short list keeps all of them busy
+    // entries are dealt to the warps one by one, so that a short list keeps
+    // all of them busy (packed 16 or 32 to a warp, a 256x256 frame of 1,000
+    // triangles took 44 and 55 us against 34)
     const unsigned i = c + (unsigned)(lane * nwarps + warp);
     bool pushed = false;
     SmallBox sb;

@@ -337,3 +337,16 @@ class Rasterizer:
         self._check(self.lib.piko_raster_backward(self._h, C.byref(cs), C.byref(cf), _ptr(g), _ptr(dcolor),
                                                   _ptr(dnormal), _ptr(dlight), self._stream(stream)))
         return dcolor, dnormal, dlight
+
+    def gradients(self, scene: DeviceScene, fb: Framebuffer, dl_drgba: torch.Tensor, color=True, normal=True,
+                  light=True, stream=None):
+        """The gradients of ``backward`` in new tensors (None for those not
+        asked for), which the kernels write without a clear before them."""
+        dc = torch.empty_like(scene.color) if color else None
+        dn = torch.empty_like(scene.normal) if normal else None
+        dl = torch.empty_like(scene.light_dir) if light else None
+        cs, cf = scene.c_struct(), fb.c_struct()
+        g = dl_drgba.contiguous()
+        self._check(self.lib.piko_raster_backward_set(self._h, C.byref(cs), C.byref(cf), _ptr(g), _ptr(dc), _ptr(dn),
+                                                      _ptr(dl), self._stream(stream)))
+        return dc, dn, dl
