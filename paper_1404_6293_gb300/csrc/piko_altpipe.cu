@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(ALT_THREADS) k_alt_shade_pixels(const __grid_c
       continue;
     }
     const int y = (int)(o / W), x = (int)(o - (long long)y * W);
-    shade_from_global<PERSP, true>(p.sc, tri_indices(p.sc.tris, (unsigned)k), x, y, (size_t)o);
+    shade_winner<PERSP, true>(p.sc, tri_indices(p.sc.tris, (unsigned)k), x, y, (size_t)o);
   }
 }
 
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(ALT_THREADS) k_frag_shade(const __grid_constan
        i += (unsigned long long)gridDim.x * blockDim.x) {
     const unsigned o = p.frag_pix[i];
     const int y = (int)(o / (unsigned)W), x = (int)(o - (unsigned)y * (unsigned)W);
-    shade_from_global<PERSP, true>(fs, tri_indices(fs.tris, (unsigned)p.frag_key[i]), x, y, (size_t)i);
+    shade_winner<PERSP, true>(fs, tri_indices(fs.tris, (unsigned)p.frag_key[i]), x, y, (size_t)i);
   }
 }
 
@@ -267,7 +267,7 @@ cudaError_t alt_stage(const AltInputs& in, int stage, bool persp, int num_sms, c
   sc.g.W = in.W; sc.g.H = in.H;
   sc.g.bshift_x = sc.g.bshift_y = 0; sc.g.nbx = sc.g.nby = 0;
   sc.mode = in.mode; sc.unclamped = in.unclamped; sc.small_px = 0;
-  sc.slot_bits = 0; sc.nslots = 0; sc.rec_stride = 0; sc.tri_base = 0;
+  sc.tri_base = 0;
   sc.tris = in.tris; sc.vtx = in.vtx; sc.color = in.color; sc.normal = in.normal; sc.light = in.light;
   sc.vdot = nullptr; sc.vattr = nullptr; sc.invw = persp ? in.invw : nullptr;
   sc.T = in.T; sc.clip_tris = in.clip_tris; sc.clip_orig = in.clip_orig;

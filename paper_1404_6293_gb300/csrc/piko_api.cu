@@ -18,7 +18,6 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
 int batch_launch_forward(BatchState* bs, DevStatus* st, bool persistent, cudaStream_t stream, std::string& err,
                          long long wait_budget, int withhold);
 long long batch_capacity(const BatchState* bs);
-void batch_note_entries(BatchState* bs, long long entries);
 int batch_grow_entries(BatchState* bs, long long need, std::string& err);
 int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const piko_framebuffer* fbs,
                           const float* const* dl, float* const* dc, float* const* dn, float* const* dlt, int num_sms,
@@ -99,11 +98,9 @@ struct piko_raster {
   long long hcap_pos = 0, hcap_tris = 0, hcap_color = 0, hcap_normal = 0, hcap_small = 0, hcap_key = 0,
             hcap_rgba = 0, hcap_gn = 0, hcap_ga = 0;
   DevStatus* status = nullptr;
-  unsigned long long* h_needed = nullptr;  // pinned, written by the scan (ScanReport): bin entries needed, those of
-                                           // them in the lists, clipped sub-triangles, the report's tag
+  unsigned long long* h_needed = nullptr;  // pinned, written by the scan (ScanReport): bin entries needed,
+                                           // clipped sub-triangles, the report's tag
   unsigned long long report_tag = 0;
-  long long last_entries = 0;              // bin entries of the last frame read back (0: none yet)
-  int last_tris = -1;                      // triangles of that frame
   cudaStream_t last_stream = nullptr;
   std::string err;
 };
@@ -208,7 +205,7 @@ piko_raster* piko_raster_create(int width, int height, int bin_w, int bin_h, int
             cudaMemset(h->chunk_state, 0, sizeof(unsigned long long) * scan_chunks(h->nbins)) == cudaSuccess &&
             cudaMalloc(&h->status, sizeof(DevStatus)) == cudaSuccess &&
             cudaMalloc(&h->heavy, sizeof(uint2) * HEAVY_LIST_CAP) == cudaSuccess &&
-            cudaMallocHost(&h->h_needed, 4 * sizeof(unsigned long long)) == cudaSuccess &&
+            cudaMallocHost(&h->h_needed, 3 * sizeof(unsigned long long)) == cudaSuccess &&
             cudaMallocHost(&h->h_frags, sizeof(unsigned)) == cudaSuccess &&
             cudaMallocHost(&h->h_clips, sizeof(unsigned)) == cudaSuccess &&
             cudaMemset(h->bin_count, 0, sizeof(unsigned) * 2 * h->nbins) == cudaSuccess &&
@@ -219,7 +216,7 @@ piko_raster* piko_raster_create(int width, int height, int bin_w, int bin_h, int
     piko_raster_destroy(h);
     return nullptr;
   }
-  memset(h->h_needed, 0, 4 * sizeof(unsigned long long));
+  memset(h->h_needed, 0, 3 * sizeof(unsigned long long));
   return h;
 }
 
@@ -412,7 +409,7 @@ static int check_scene(piko_raster* h, const piko_scene* s) {
 // h_needed.  The scan writes it to host memory itself, so the kernels launched
 // behind the scan keep running meanwhile.  Ends with the stream at the latest.
 static int wait_report(piko_raster* h, cudaStream_t st) {
-  const auto arrived = [&] { return __atomic_load_n(h->h_needed + 3, __ATOMIC_ACQUIRE) == h->report_tag; };
+  const auto arrived = [&] { return __atomic_load_n(h->h_needed + 2, __ATOMIC_ACQUIRE) == h->report_tag; };
   for (unsigned spin = 1; !arrived(); ++spin) {
     if (spin & 2047u) continue;
     const cudaError_t e = cudaStreamQuery(st);
@@ -547,8 +544,6 @@ static int scatter_and_process(piko_raster* h, const piko_scene* s, piko_framebu
   ProcessParams p;
   p.g = h->g;
   p.ntiles = h->nbins;
-  // records sized from the last bin-list total read back
-  p.slots_hint = slots_for_entries(h->last_entries, h->nbins);
   p.schedule = h->schedule;
   p.small_px = h->small_px;
   p.mode = s->shade_mode;
@@ -618,7 +613,7 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
   const bool ev = h->use_stage_ev;
   h->use_stage_ev = false;
   if (ev) cudaEventRecord(h->stage_ev[0], st);
-  if (h->stats) cudaMemsetAsync(&h->status->tests, 0, 4 * sizeof(unsigned long long), st);
+  if (h->stats) cudaMemsetAsync(&h->status->tests, 0, 3 * sizeof(unsigned long long), st);
   float4* vattr = packed_attributes(h, s);
   DirectRaster direct;
   direct.keys = direct_keys(h, T, V, st);
@@ -627,15 +622,12 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
                 lambert ? h->vdot : nullptr, h->perspective ? h->invw : nullptr, h->num_sms, st, direct.keys,
                 h->clip ? h->status : nullptr, s->color, vattr);
   const bool other = h->schedule == PIKO_SCHED_FUSED || h->schedule == PIKO_SCHED_UNFUSED;
-  // With the capacity check the host has to see the bin-list size.  On a
-  // handle's first frame, or one of another triangle count, it waits for it
-  // before scattering, as the lists' size also sizes the Process stage's
-  // records; from then on the scatter and Process kernels are launched behind
-  // the scan, with the last size (they skip a frame whose lists overflowed),
-  // and the host reads the scan's report while they run.
+  // With the capacity check the host has to see the sizes of the bin lists and
+  // of the clip pass's list: it reads them from the scan's report while the
+  // scatter and Process kernels, launched behind the scan, run; these skip a
+  // frame whose lists overflowed, and the host then repeats it with larger ones.
   const bool check = h->check_capacity != 0;
-  const bool ahead = check && !other && h->last_entries > 0 && h->last_tris == T;
-  if (h->clip && (r = clip_pass(h, s, st, check && !ahead, V > 0)) != PIKO_OK) return r;
+  if (h->clip && (r = clip_pass(h, s, st, check && other, V > 0)) != PIKO_OK) return r;
   if (ev) cudaEventRecord(h->stage_ev[1], st);
   if (other) return forward_other_mapping(h, s, fb, st, ev);
   bool clip_grown = false, bins_grown = false;
@@ -668,41 +660,29 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
                   h->chunk_state, scan_epoch, st, h->wait_budget, h->withhold, &report);
       if (ev) cudaEventRecord(h->stage_ev[3], st);
     }
-    bool fits = true;
-    for (int step = 0; step < 2; ++step) {
-      // ahead: launch, then look at the report; else the other way round
-      if ((step == 0) == ahead || !check) {
-        if ((r = scatter_and_process(h, s, fb, st, ev, direct, vattr, clip_tris, clip_cap)) != PIKO_OK) return r;
-        if (!check) return PIKO_OK;
-        continue;
-      }
-      if ((r = wait_report(h, st)) != PIKO_OK) return r;
-      const long long need = (long long)h->h_needed[0], clips = (long long)h->h_needed[2];
-      if (h->clip && clips > ccap) {
-        if (clip_grown) return fail(h, PIKO_ERR_OVERFLOW, "clipped triangle list too large");
-        clip_grown = true;
-        const long long want = clips + clips / 8 + 1024;
-        if ((r = grow(h, &h->clip_tris, &h->ccap_tris, 3 * want, "clipped triangles")) != PIKO_OK ||
-            (r = grow(h, &h->clip_orig, &h->ccap_orig, want, "clipped triangle indices")) != PIKO_OK)
-          return r;
-        fits = false;
-      } else if (need > h->ecap) {
-        if (bins_grown || need > 0xFFFFFFF0LL) return fail(h, PIKO_ERR_OVERFLOW, "bin lists too large");
-        bins_grown = true;
-        if ((r = grow(h, &h->bin_tris, &h->ecap, need, "bin lists")) != PIKO_OK) return r;
-        fits = false;
-      }
-      if (!fits) {
-        // the failed pass recorded an overflow and zeroed the counts: clear and count again
-        const cudaError_t e = cudaMemsetAsync(h->status, 0, sizeof(unsigned) * 2, st);
-        if (e != cudaSuccess) return cuda_fail(h, e, "status clear");
-        if (h->clip && clips > ccap && (r = clip_pass(h, s, st, false, false)) != PIKO_OK) return r;
-        break;
-      }
-      h->last_entries = h->h_needed[1] > 0 ? (long long)h->h_needed[1] : 1;
-      h->last_tris = T;
+    if ((r = scatter_and_process(h, s, fb, st, ev, direct, vattr, clip_tris, clip_cap)) != PIKO_OK) return r;
+    if (!check) return PIKO_OK;
+    if ((r = wait_report(h, st)) != PIKO_OK) return r;
+    const long long need = (long long)h->h_needed[0], clips = (long long)h->h_needed[1];
+    const bool clip_more = h->clip && clips > ccap;
+    if (clip_more) {
+      if (clip_grown) return fail(h, PIKO_ERR_OVERFLOW, "clipped triangle list too large");
+      clip_grown = true;
+      const long long want = clips + clips / 8 + 1024;
+      if ((r = grow(h, &h->clip_tris, &h->ccap_tris, 3 * want, "clipped triangles")) != PIKO_OK ||
+          (r = grow(h, &h->clip_orig, &h->ccap_orig, want, "clipped triangle indices")) != PIKO_OK)
+        return r;
+    } else if (need > h->ecap) {
+      if (bins_grown || need > 0xFFFFFFF0LL) return fail(h, PIKO_ERR_OVERFLOW, "bin lists too large");
+      bins_grown = true;
+      if ((r = grow(h, &h->bin_tris, &h->ecap, need, "bin lists")) != PIKO_OK) return r;
+    } else {
+      return PIKO_OK;
     }
-    if (fits) return PIKO_OK;
+    // the failed pass recorded an overflow and zeroed the counts: clear and count again
+    const cudaError_t e = cudaMemsetAsync(h->status, 0, sizeof(unsigned) * 2, st);
+    if (e != cudaSuccess) return cuda_fail(h, e, "status clear");
+    if (clip_more && (r = clip_pass(h, s, st, false, false)) != PIKO_OK) return r;
   }
 }
 
@@ -818,12 +798,11 @@ int piko_raster_forward_batch(piko_raster* h, const piko_scene* scenes, int n, p
                                   h->withhold)) != PIKO_OK)
       return r;
     if (!h->check_capacity) return PIKO_OK;
-    cudaError_t e = cudaMemcpyAsync(h->h_needed, &h->status->needed, 2 * sizeof(unsigned long long),
+    cudaError_t e = cudaMemcpyAsync(h->h_needed, &h->status->needed, sizeof(unsigned long long),
                                     cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(h, e, "batch bin-list size read-back");
     const long long need = (long long)*h->h_needed;
-    batch_note_entries(h->batch, h->h_needed[1] > 0 ? (long long)h->h_needed[1] : 1);
     if (need <= batch_capacity(h->batch)) return PIKO_OK;
     if (attempt > 0 || need > 0xFFFFFFF0LL) return fail(h, PIKO_ERR_OVERFLOW, "batch bin lists too large");
     if ((r = batch_grow_entries(h->batch, need, h->err)) != PIKO_OK) return r;

@@ -28,7 +28,6 @@ struct BatchScene {
   int vtx_base, tri_base, bin_base;
   int direct;         // small triangles are rasterized by the count pass (piko_direct.cuh)
   unsigned key_base;  // into the direct keys
-  int slot_bits, nslots, rec_stride;
   int unclamped;  // Lambert without the clamp (the handle's option)
   const float4* pos;
   const int* tris;
@@ -374,9 +373,6 @@ __device__ void load_tile_scene(const BatchParams& b, int s, TileScene& t) {
   t.mode = d.mode;
   t.unclamped = d.unclamped;
   t.small_px = 32;
-  t.slot_bits = d.slot_bits;
-  t.nslots = d.nslots;
-  t.rec_stride = d.rec_stride;
   t.tri_base = d.tri_base;
   t.tris = d.tris;
   t.vtx = b.vtx + d.vtx_base;
@@ -470,7 +466,6 @@ __global__ void __maxnreg__(PIKO_BATCH_MAXNREG) k_batch_forward(BatchParams b) {
   sm.skey = smem;
   sm.sbig = reinterpret_cast<int*>(smem + b.max_bin_px);
   sm.sfrag = sm.sbig + blockDim.x;
-  sm.srec = sm.sfrag + (blockDim.x >> 5) * FRAG_WARP_WORDS;
   sm.s_nbig = &s_nbig;
   if (cta_should_stop(b.st)) return;
   if (b.phases & PH_VERTEX) {
@@ -637,8 +632,6 @@ struct BatchState {
   int grid = 0;
   int n = 0;
   int persp = 0;               // the layout's attribute interpolation (perspective-correct or not)
-  long long last_entries = 0;  // bin entries of the last frame read back (sizes the shading records)
-  long long last_bins = 0;     // bins of that frame
 };
 
 namespace {
@@ -702,9 +695,7 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   std::vector<BatchScene> d(n);
   std::vector<int> pv(n + 1), pt(n + 1), pb(n + 1), ps(n + 1), pd(n + 1), pq(n + 1);
   long long tv = 0, tt = 0, tb = 0, tsd = 0, tdy = 0, tq = 0, tk = 0;
-  int max_bin_px = 64, max_rec = 0;
-  // shading records per tile from the last frame's mean entries per bin
-  const int slots_hint = bs ? slots_for_entries(bs->last_entries, (int)(bs->last_bins > 0 ? bs->last_bins : 1)) : 0;
+  int max_bin_px = 64;
   for (int i = 0; i < n; ++i) {
     const piko_scene& s = scenes[i];
     const piko_framebuffer& f = fbs[i];
@@ -736,8 +727,6 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
       x.key_base = (unsigned)tk;
       tk += px;
     }
-    tile_layout(s.num_triangles, bw * bh, s.shade_mode, s.color != nullptr, persp != 0, 255, x.slot_bits, x.nslots,
-                x.rec_stride, slots_hint);
     x.unclamped = unclamped;
     x.pos = reinterpret_cast<const float4*>(s.pos);
     x.tris = s.tris; x.mvp = s.mvp; x.color = s.color; x.normal = s.normal; x.light = s.light_dir;
@@ -752,7 +741,6 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
     if (sched == PIKO_SCHED_STATIC) tsd += ntiles;
     else tdy += ntiles;
     if (bw * bh > max_bin_px) max_bin_px = bw * bh;
-    if (x.nslots * x.rec_stride > max_rec) max_rec = x.nslots * x.rec_stride;
   }
   pv[n] = (int)tv; pt[n] = (int)tt; pb[n] = (int)tb; ps[n] = (int)tsd; pd[n] = (int)tdy; pq[n] = (int)tq;
   if (tv >= (1LL << 31) || tt >= (1LL << 31) || tb >= (1LL << 31) || tq >= (1LL << 31)) {
@@ -856,7 +844,7 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   b.cursor = bs->cursor; b.chunk_state = bs->chunk_state; b.bin_tris = bs->bin_tris;
   b.capacity = (unsigned long long)bs->ecap; b.sync = bs->sync;
   b.max_bin_px = max_bin_px;
-  bs->smem = tile_smem_bytes(max_bin_px, BATCH_THREADS, 1, 0) + (size_t)max_rec * 4;
+  bs->smem = tile_smem_bytes(max_bin_px, BATCH_THREADS);
   const auto kf = persp ? k_batch_forward<true> : k_batch_forward<false>;
   if (bs->smem > 48 * 1024 &&
       cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bs->smem) != cudaSuccess) {
@@ -931,12 +919,6 @@ int batch_launch_forward(BatchState* bs, DevStatus* st, bool persistent, cudaStr
 }
 
 long long batch_capacity(const BatchState* bs) { return bs ? bs->ecap : 0; }
-
-void batch_note_entries(BatchState* bs, long long entries) {
-  if (!bs) return;
-  bs->last_entries = entries;
-  bs->last_bins = bs->params.total_bins;
-}
 
 int batch_grow_entries(BatchState* bs, long long need, std::string& err) {
   return grow_dev(&bs->bin_tris, &bs->ecap, need, false, err);

@@ -3,8 +3,8 @@
 //
 // The count pass of AssignBin holds a triangle's snapped vertices in
 // registers.  For a triangle whose box is a few pixels, binning it (a
-// rectangle, a list entry, a second gather of its indices and vertices, a
-// shading record) costs several times the work of rasterizing it, so the pass
+// rectangle, a list entry, a second gather of its indices and vertices) costs
+// several times the work of rasterizing it, so the pass
 // takes its samples right there: a 64-bit atomic minimum per covered sample on
 // one key per pixel in global memory (depth << 32 | triangle; the minimum is
 // the same in any order).  Larger triangles are binned as before, and the
@@ -115,14 +115,14 @@ __device__ __forceinline__ bool direct_triangle(int4 p0, int4 p1, int4 p2, unsig
 // ---------------------------------------------------------------- shading
 // Colour and key of pixel (x, y), whose winner (indices id, key k) was
 // rasterized directly: its snapped extents are below 2^15, so areas and edge
-// functions are exact in 32 bits.  The arithmetic is a shading record's.
+// functions are exact in 32 bits.
 // CLIP: a winner whose vertices the vertex stage rejected was clipped.
 template <bool PERSP, bool CLIP>
 __device__ __forceinline__ void shade_direct_pixel(const TileScene& p, int3 id, int x, int y, size_t o) {
   const int4 p0 = __ldg(p.vtx + id.x);
   int4 p1 = __ldg(p.vtx + id.y), p2 = __ldg(p.vtx + id.z);
   if (CLIP && !(p0.w & p1.w & p2.w)) {
-    shade_from_global<PERSP, true>(p, id, x, y, o);
+    shade_winner<PERSP, true>(p, id, x, y, o);
     return;
   }
   int A = (p1.x - p0.x) * (p2.y - p0.y) - (p2.x - p0.x) * (p1.y - p0.y);

@@ -49,7 +49,6 @@ struct DevStatus {
   unsigned int flags;           // bit c set when PIKO_ERR c was recorded
   unsigned int first_code;      // first PIKO_ERR_* recorded (0 = none)
   unsigned long long needed;    // bin entries the last scan required
-  unsigned long long listed;    // those of them in the lists (the rest: direct_entries; read back together with needed)
   unsigned int queue_head;      // tile counter of the dynamic schedule
   unsigned int scan_ticket;     // next chunk number of the scan (reset by its last chunk)
   unsigned int frag_count;      // fragments emitted by the unfused pipeline's rasterizer
@@ -326,15 +325,6 @@ __device__ __forceinline__ void clip_ray_weights(const float4* pos, const float*
 }
 
 // --------------------------------------------------------------- kernels
-// Records wanted for a scene whose bin lists hold `entries` entries over
-// `tiles` tiles: 1.4 x the mean, in multiples of 32 (1.4 x covers the
-// spread of entry counts between tiles of the measured workloads).
-inline int slots_for_entries(long long entries, int tiles) {
-  if (entries <= 0 || tiles <= 0) return 0;
-  const long long want = (14 * entries / tiles + 5 * 32) / (10 * 32) * 32;  // round(1.4 mean / 32) * 32
-  return (int)(want < 32 ? 32 : (want > 4096 ? 4096 : want));
-}
-
 struct ProcessParams {
   RasterGeom g;
   int ntiles;
@@ -342,12 +332,8 @@ struct ProcessParams {
   int small_px;
   int mode;
   int unclamped;
-  int slots_hint;  // shading records per tile wanted (0: the largest the key encoding allows)
   int stats;
   int num_triangles;
-  int slot_bits;   // set by launch_process: bits of the record slot below the triangle index
-  int nslots;      // shared-memory records per tile
-  int rec_stride;  // 32-bit words per record
   const int* tris;
   const int4* vtx;
   const float* color;

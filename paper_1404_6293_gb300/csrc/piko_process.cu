@@ -14,9 +14,6 @@ TileScene scene_of(const ProcessParams& p) {
   sc.mode = p.mode;
   sc.unclamped = p.unclamped;
   sc.small_px = p.small_px;
-  sc.slot_bits = p.slot_bits;
-  sc.nslots = p.nslots;
-  sc.rec_stride = p.rec_stride;
   sc.tri_base = 0;
   sc.tris = p.tris;
   sc.vtx = p.vtx;
@@ -67,7 +64,6 @@ __global__ void __maxnreg__(PIKO_PROCESS_MAXNREG) k_process(const __grid_constan
   sm.skey = smem;
   sm.sbig = reinterpret_cast<int*>(smem + bin_px);
   sm.sfrag = sm.sbig + nt;
-  sm.srec = sm.sfrag + (nt >> 5) * FRAG_WARP_WORDS;
   sm.s_nbig = &s_nbig;
   const TileScene& sc = pl.sc;
   for (int i = tid; i < bin_px; i += nt) sm.skey[i] = KEY_EMPTY;
@@ -132,14 +128,8 @@ __global__ void __maxnreg__(PIKO_PROCESS_MAXNREG) k_process(const __grid_constan
 }
 
 // ---------------------------------------------------------------- host side
-static void layout(ProcessParams& p, int threads) {
-  (void)threads;
-  tile_layout(p.num_triangles, 1 << (p.g.bshift_x + p.g.bshift_y), p.mode, p.color != nullptr, p.invw != nullptr, 511,
-              p.slot_bits, p.nslots, p.rec_stride, p.slots_hint);
-}
-
 static size_t smem_bytes(const ProcessParams& p, int threads) {
-  return tile_smem_bytes(1 << (p.g.bshift_x + p.g.bshift_y), threads, p.nslots, p.rec_stride);
+  return tile_smem_bytes(1 << (p.g.bshift_x + p.g.bshift_y), threads);
 }
 
 using ProcessKernel = void (*)(ProcessLaunch);
@@ -162,9 +152,7 @@ static ProcessKernel process_kernel(const ProcessParams& p) {
   return p.clip_tris ? process_kernel_clip<true>(p) : process_kernel_clip<false>(p);
 }
 
-cudaError_t process_occupancy(const ProcessParams& p0, int threads, int* blocks_per_sm) {
-  ProcessParams p = p0;
-  layout(p, threads);
+cudaError_t process_occupancy(const ProcessParams& p, int threads, int* blocks_per_sm) {
   const size_t smem = smem_bytes(p, threads);
   const ProcessKernel k = process_kernel(p);
   if (smem > 48 * 1024) {
@@ -174,9 +162,7 @@ cudaError_t process_occupancy(const ProcessParams& p0, int threads, int* blocks_
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem);
 }
 
-cudaError_t launch_process(const ProcessParams& p0, int threads, int grid, cudaStream_t s) {
-  ProcessParams p = p0;
-  layout(p, threads);
+cudaError_t launch_process(const ProcessParams& p, int threads, int grid, cudaStream_t s) {
   const size_t smem = smem_bytes(p, threads);
   const ProcessKernel k = process_kernel(p);
   if (smem > 48 * 1024) {

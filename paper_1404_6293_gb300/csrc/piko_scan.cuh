@@ -63,9 +63,9 @@ __device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned l
 }
 
 // What the host reads of a scan without waiting for the stream: pinned words
-// written by the scan itself (needed, listed, clipped sub-triangles, then tag).
+// written by the scan itself (needed, clipped sub-triangles, then tag).
 struct ScanReport {
-  unsigned long long* host = nullptr;  // 4 words (NULL: no report)
+  unsigned long long* host = nullptr;  // 3 words (NULL: no report)
   unsigned long long tag = 0;          // differs between consecutive reports of a handle
 };
 
@@ -171,16 +171,14 @@ __device__ __forceinline__ void scan_chunk(int chunk, int nchunks, int nbins, un
     const bool ok = total <= capacity;
     if (ok) bin_off[nbins] = (unsigned)listed;
     st->needed = total;
-    st->listed = listed;
     *queue_to_reset = 0u;
     if (!ok) record_error(st, PIKO_ERR_OVERFLOW);
     if (report.host) {
       volatile unsigned long long* r = report.host;
       r[0] = total;
-      r[1] = listed;
-      r[2] = *reinterpret_cast<volatile unsigned*>(&st->clip_count);
+      r[1] = *reinterpret_cast<volatile unsigned*>(&st->clip_count);
       __threadfence_system();
-      r[3] = report.tag;
+      r[2] = report.tag;
     }
   }
 }

@@ -7,20 +7,21 @@
 // buffer in shared memory (the on-chip depth buffer Sec. 5.2.4 names).
 //
 // Per tile:
-//  1. each thread takes one bin entry, re-derives the triangle from the
-//     snapped vertices and stores what shading needs (edge coordinates, 1/A
-//     and the vertex attributes) in a shared-memory record.  A small box
-//     inside the tile is walked by the thread for coverage only, and the
-//     warp then shares out the covered samples of all its small boxes for
-//     their depths (fragment_pass); larger boxes of triangles up to 128
-//     pixels a side are shared out by rows and samples (medium_pass); larger
-//     triangles go to a queue that whole warps rasterize one at a time;
+//  1. each thread takes one bin entry and re-derives the triangle from the
+//     snapped vertices.  A small box inside the tile is walked by the thread
+//     for coverage only, and the warp then shares out the covered samples of
+//     all its small boxes for their depths (fragment_pass); larger boxes of
+//     triangles up to 128 pixels a side are shared out by rows and samples
+//     (medium_pass); larger triangles go to a queue that whole warps rasterize
+//     one at a time;
 //  2. every covered sample does a 64-bit atomic minimum on the tile's key,
-//     key = depth << 40 | triangle << slot_bits | record slot: ordered by
-//     (depth, triangle) exactly like depth << 32 | triangle, since a
-//     triangle has one record per tile;
-//  3. one thread per pixel shades the winner from its record and writes the
-//     key (as depth << 32 | triangle) and the colour, rows contiguous.
+//     depth << 32 | triangle;
+//  3. one thread per pixel shades the winner from the scene's vertices and
+//     writes the key and the colour, rows contiguous.  (Attributes kept in
+//     shared-memory records per entry made the same colours from fewer
+//     gathers, but were filled for entries that win nothing, grew the kernel
+//     past the instruction cache and took a sixth more of a 1920x1080 G-buffer
+//     frame's time; elsewhere the two were equal.)
 #pragma once
 
 #include <cuda_fp16.h>
@@ -34,7 +35,6 @@ namespace piko {
 struct TileScene {
   RasterGeom g;
   int mode, unclamped, small_px;
-  int slot_bits, nslots, rec_stride;
   int tri_base;
   const int* tris;
   const int4* vtx;
@@ -70,39 +70,24 @@ TileScene scene_of(const ProcessParams& p);  // piko_process.cu
 //    fragment_pass (FS_* words);
 //  - a large triangle queued for the warps: its snapped vertices, depths and
 //    area as set up by the lane that met it (so that the warp re-reads
-//    nothing from global memory), then its triangle index and record slot
-//    (BG_* words).
+//    nothing from global memory), then its triangle index (BG_* words).
 // After the staging words, each warp has a list of up to FRAG_CAP fragment
 // descriptors.  The queue of large triangles holds the thread index of each.
 constexpr int FST_WORDS = 13;
 constexpr int FRAG_CAP = 128;
 constexpr int FRAG_WARP_WORDS = FST_WORDS * 32 + FRAG_CAP;
-enum { BG_X0 = 0, BG_Y0, BG_X1, BG_Y1, BG_X2, BG_Y2, BG_Z0, BG_Z1, BG_Z2, BG_ALO, BG_AHI, BG_T, BG_SLOT };
+enum { BG_X0 = 0, BG_Y0, BG_X1, BG_Y1, BG_X2, BG_Y2, BG_Z0, BG_Z1, BG_Z2, BG_ALO, BG_AHI, BG_T };
 
 struct TileSmem {
   unsigned long long* skey;  // [bin_px], all KEY_EMPTY between tiles
   int* sbig;                 // [nt] ring of the threads whose large triangles are queued
   int* sfrag;                // [nt / 32][FRAG_WARP_WORDS]
-  int* srec;                 // [nslots][rec_stride]
   unsigned* s_nbig;          // grows monotonically
 };
 
 struct TileStats {
   unsigned long long tests, frags, shaded;
 };
-
-// record words: 0..5 X0 Y0 X1 Y1 X2 Y2 (oriented), 6 = 1/A (float), then the
-// attributes, then (perspective-correct attributes only) 1/w of the three
-// vertices
-constexpr int R_RA = 6;
-constexpr int R_ATTR = 7;
-
-__host__ __device__ __forceinline__ int rec_attr_count(int mode, bool has_color) {
-  if (mode == PIKO_SHADE_GOURAUD) return 9;              // c0 c1 c2
-  if (mode == PIKO_SHADE_LAMBERT) return has_color ? 12 : 3;  // d0 d1 d2 (n_i . L) [+ c0 c1 c2]
-  return 18;                                             // n0 n1 n2 c0 c1 c2
-}
-
 
 // ---------------------------------------------------------------- raster
 // Large boxes of at least this many pixels in a tile are walked by row spans
@@ -139,7 +124,7 @@ __device__ __forceinline__ Edges<I> make_edges(const TriSetup& s, int px, int py
 }
 
 __device__ __forceinline__ void key_store(unsigned long long* skey, int idx, unsigned z, unsigned long long tag) {
-  const unsigned long long k = ((unsigned long long)z << 40) | tag;
+  const unsigned long long k = ((unsigned long long)z << 32) | tag;
   if (k < skey[idx]) atomicMin(skey + idx, k);
 }
 
@@ -168,7 +153,7 @@ __device__ __forceinline__ void key_min_mid(unsigned long long* skey, int idx, i
 //    wrapping arithmetic gives r exactly;
 //  - otherwise r is formed in 64 bits and the estimate is within 16 of q.
 // The choice is per entry, so a warp rarely splits between the two forms.
-// The key is Z0 << 40 | tag plus q << 40 (Z0 + q stays in [0, 2^24)).
+// The key is Z0 << 32 | triangle plus q << 32 (Z0 + q stays in [0, 2^24)).
 struct DepthSetup {
   int d1, d2, A;
   float k1, k2;
@@ -183,7 +168,7 @@ __device__ __forceinline__ DepthSetup depth_setup(const TriSetup& s, float rA, u
   d.A = (int)s.A;
   d.k1 = rA * (float)d.d1;
   d.k2 = rA * (float)d.d2;
-  d.kbase = ((unsigned long long)(unsigned)s.Z0 << 40) | tag;
+  d.kbase = ((unsigned long long)(unsigned)s.Z0 << 32) | tag;
   d.fast = s.A < (1LL << 27) && abs(d.d1) + abs(d.d2) < (1 << 22);
   return d;
 }
@@ -199,7 +184,7 @@ __device__ __forceinline__ void key_min_box(unsigned long long* skey, int idx, i
     for (int it = 0; r < 0 && it < DIV_FIX_LIMIT; ++it) { --q; r += d.A; }
     for (int it = 0; r >= d.A && it < DIV_FIX_LIMIT; ++it) { ++q; r -= d.A; }
   }
-  const unsigned long long k = d.kbase + ((unsigned long long)(long long)q << 40);
+  const unsigned long long k = d.kbase + ((unsigned long long)(long long)q << 32);
   if (k < skey[idx]) atomicMin(skey + idx, k);
 }
 
@@ -336,8 +321,7 @@ __device__ __forceinline__ void fragment_key(const int* w, int rx, int ry, int i
     for (int it = 0; r < 0 && it < DIV_FIX_LIMIT; ++it) { --q; r += A; }
     for (int it = 0; r >= A && it < DIV_FIX_LIMIT; ++it) { ++q; r -= A; }
   }
-  // the depth field starts at bit 40: q moves the high word by q << 8
-  const unsigned hi = (unsigned)w[FS_KHI * 32] + ((unsigned)q << 8);
+  const unsigned hi = (unsigned)w[FS_KHI * 32] + (unsigned)q;
   const unsigned long long k = ((unsigned long long)hi << 32) | (unsigned)w[FS_KLO * 32];
   if (k < skey[idx]) atomicMin(skey + idx, k);
 }
@@ -587,68 +571,6 @@ __device__ __forceinline__ void write_empty(const TileScene& p, size_t o) {
   }
 }
 
-// Barycentrics of pixel (x, y) from a record: exact edge functions times
-// 1/A.  The record stores 1/A negated when A >= 2^31; below that the pixel's
-// edge functions (in [0, A], the pixel being covered) are exact in wrapping
-// 32-bit arithmetic.
-__device__ __forceinline__ void rec_bary(const int* r, int x, int y, float& b0, float& b1, float& b2) {
-  const int Px = 256 * x + 128, Py = 256 * y + 128;
-  const int X0 = r[0], Y0 = r[1], X1 = r[2], Y1 = r[3], X2 = r[4], Y2 = r[5];
-  const float rAs = __int_as_float(r[R_RA]);
-  if (rAs > 0.0f) {
-    b1 = (float)edge_fn_wrap32(X2, Y2, X0, Y0, Px, Py) * rAs;
-    b2 = (float)edge_fn_wrap32(X0, Y0, X1, Y1, Px, Py) * rAs;
-  } else {
-    // exact edge functions from 32-bit differences (each below 2^24) widened once
-    const long long w1 = (long long)(X0 - X2) * (Py - Y2) - (long long)(Y0 - Y2) * (Px - X2);
-    const long long w2 = (long long)(X1 - X0) * (Py - Y0) - (long long)(Y1 - Y0) * (Px - X0);
-    b1 = f32_from_i64(w1) * -rAs;
-    b2 = f32_from_i64(w2) * -rAs;
-  }
-  b0 = 1.0f - b1 - b2;
-}
-
-// PERSP: perspective-correct barycentrics (the record holds the vertices' 1/w)
-template <bool PERSP>
-__device__ __forceinline__ void shade_from_record(const TileScene& p, const int* r, int x, int y, size_t o) {
-  float b0, b1, b2;
-  rec_bary(r, x, y, b0, b1, b2);
-  const float* a = reinterpret_cast<const float*>(r + R_ATTR);
-  if (PERSP) {
-    const float* iw = a + rec_attr_count(p.mode, p.color != nullptr);
-    perspective_bary(b0, b1, b2, iw[0], iw[1], iw[2]);
-  }
-  if (p.mode == PIKO_SHADE_GOURAUD) {
-    if (p.rgba_out)
-      p.rgba_out[o] = make_float4(b0 * a[0] + b1 * a[3] + b2 * a[6], b0 * a[1] + b1 * a[4] + b2 * a[7],
-                                  b0 * a[2] + b1 * a[5] + b2 * a[8], 1.0f);
-    return;
-  }
-  if (p.mode == PIKO_SHADE_LAMBERT) {
-    float d = b0 * a[0] + b1 * a[1] + b2 * a[2];  // (sum b_i n_i) . L, by linearity
-    if (!p.unclamped) d = fmaxf(d, 0.0f);
-    float c0 = 0.80f, c1 = 0.75f, c2 = 0.65f;      // material of Listing 1
-    if (p.color) {
-      c0 = b0 * a[3] + b1 * a[6] + b2 * a[9];
-      c1 = b0 * a[4] + b1 * a[7] + b2 * a[10];
-      c2 = b0 * a[5] + b1 * a[8] + b2 * a[11];
-    }
-    if (p.rgba_out) p.rgba_out[o] = make_float4(c0 * d, c1 * d, c2 * d, 1.0f);
-    return;
-  }
-  const float nx = b0 * a[0] + b1 * a[3] + b2 * a[6];
-  const float ny = b0 * a[1] + b1 * a[4] + b2 * a[7];
-  const float nz = b0 * a[2] + b1 * a[5] + b2 * a[8];
-  float c0 = 0.80f, c1 = 0.75f, c2 = 0.65f;
-  if (p.color) {
-    c0 = b0 * a[9] + b1 * a[12] + b2 * a[15];
-    c1 = b0 * a[10] + b1 * a[13] + b2 * a[16];
-    c2 = b0 * a[11] + b1 * a[14] + b2 * a[17];
-  }
-  p.gnorm_out[o] = pack_half4(nx, ny, nz, 0.0f);
-  p.galb_out[o] = pack_half4(c0, c1, c2, 1.0f);
-}
-
 // Attributes of a winner with barycentrics (b0, b1, b2) over vertices
 // (v0, v1, v2), read from global memory, shaded and written at o.
 __device__ __forceinline__ void shade_vertices(const TileScene& p, int v0, int v1, int v2, float b0, float b1,
@@ -715,13 +637,13 @@ __device__ __forceinline__ int3 tri_indices(const int* __restrict__ tris, unsign
   return make_int3(__ldg(i), __ldg(i + 1), __ldg(i + 2));
 }
 
-// Winners without a record (id: the triangle's indices): everything re-read
-// from global memory, with the arithmetic of a record's.  CLIP (near/far clipping on): a winner whose vertices the vertex
-// stage rejected was clipped, and shades with its clip-space ray weights
+// Colour of a winner (id: the triangle's indices) at pixel (x, y), written at
+// o.  CLIP (near/far clipping on): a winner whose vertices the vertex stage
+// rejected was clipped, and shades with its clip-space ray weights
 // (perspective-correct by construction); one kernel instance per setting so
 // that the default path carries none of it.
 template <bool PERSP, bool CLIP = false>
-__device__ __forceinline__ void shade_from_global(const TileScene& p, int3 id, int x, int y, size_t o) {
+__device__ __forceinline__ void shade_winner(const TileScene& p, int3 id, int x, int y, size_t o) {
   const int v[3] = {id.x, id.y, id.z};
   TriSetup s;
   if (!setup_triangle(v[0], v[1], v[2], p.vtx, s)) {
@@ -748,64 +670,11 @@ __device__ __forceinline__ void shade_from_global(const TileScene& p, int3 id, i
   }
   float b0 = 1.0f - b1 - b2;
   if (PERSP) perspective_bary(b0, b1, b2, __ldg(p.invw + s.v0), __ldg(p.invw + s.v1), __ldg(p.invw + s.v2));
-  if (p.mode == PIKO_SHADE_LAMBERT && (p.vdot || p.vattr)) {  // as from a record
+  if (p.mode == PIKO_SHADE_LAMBERT && (p.vdot || p.vattr)) {
     shade_lambert(p, s.v0, s.v1, s.v2, b0, b1, b2, o);
     return;
   }
   shade_vertices(p, s.v0, s.v1, s.v2, b0, b1, b2, o);
-}
-
-// Fills the shared-memory record of one bin entry (PERSP: with 1/w).
-template <bool PERSP>
-__device__ __forceinline__ void fill_record(const TileScene& p, const TriSetup& s, int* r) {
-  r[0] = s.X0; r[1] = s.Y0; r[2] = s.X1; r[3] = s.Y1; r[4] = s.X2; r[5] = s.Y2;
-  // 1/A, negated when A >= 2^31 (rec_bary then takes the 64-bit form)
-  const float rA = approx_rcp(f32_from_i64(s.A));
-  r[R_RA] = __float_as_int(s.A < (1LL << 31) ? rA : -rA);
-  float* a = reinterpret_cast<float*>(r + R_ATTR);
-  const int v[3] = {s.v0, s.v1, s.v2};
-  if (PERSP) {
-    float* iw = a + rec_attr_count(p.mode, p.color != nullptr);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) iw[j] = __ldg(p.invw + v[j]);
-  }
-  if (p.mode == PIKO_SHADE_LAMBERT) {
-    if (p.vattr) {
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const float4 q = __ldg(p.vattr + v[j]);
-        a[j] = q.w;
-        if (!p.color) continue;
-        a[3 + 3 * j] = q.x; a[4 + 3 * j] = q.y; a[5 + 3 * j] = q.z;
-      }
-      return;
-    }
-#pragma unroll
-    for (int j = 0; j < 3; ++j) a[j] = __ldg(p.vdot + v[j]);
-    if (p.color) {
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const float* c = p.color + 3 * (size_t)v[j];
-        a[3 + 3 * j] = __ldg(c); a[4 + 3 * j] = __ldg(c + 1); a[5 + 3 * j] = __ldg(c + 2);
-      }
-    }
-    return;
-  }
-  const int coff = p.mode == PIKO_SHADE_GOURAUD ? 0 : 9;
-  if (p.mode == PIKO_SHADE_GBUFFER) {
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const float* n = p.normal + 3 * (size_t)v[j];
-      a[3 * j] = __ldg(n); a[3 * j + 1] = __ldg(n + 1); a[3 * j + 2] = __ldg(n + 2);
-    }
-  }
-  if (p.color) {
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const float* c = p.color + 3 * (size_t)v[j];
-      a[coff + 3 * j] = __ldg(c); a[coff + 3 * j + 1] = __ldg(c + 1); a[coff + 3 * j + 2] = __ldg(c + 2);
-    }
-  }
 }
 
 // t is the scene-local triangle index
@@ -828,7 +697,6 @@ __device__ __forceinline__ void process_tile(const TileScene& p, int tile, unsig
   const int nt = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = nt >> 5;
   const int bin_w = 1 << p.g.bshift_x, bin_h = 1 << p.g.bshift_y;
   const int bin_px = bin_w * bin_h;
-  const unsigned no_slot = (1u << p.slot_bits) - 1u;
   const int tx = tile % p.g.nbx, ty = tile / p.g.nbx;
   const int x0 = tx << p.g.bshift_x, y0 = ty << p.g.bshift_y;
   const int x1 = min(x0 + bin_w, p.g.W) - 1, y1 = min(y0 + bin_h, p.g.H) - 1;
@@ -845,7 +713,7 @@ __device__ __forceinline__ void process_tile(const TileScene& p, int tile, unsig
     for (int i = tid; i < bin_px; i += nt) {
       const int x = x0 + (i & (bin_w - 1)), y = y0 + (i >> p.g.bshift_x);
       const unsigned long long k = x <= x1 && y <= y1 ? __ldcg(p.dkeys + (size_t)y * p.g.W + x) : KEY_EMPTY;
-      if (k != KEY_EMPTY) skey[i] = (k >> 32) << 40 | (unsigned long long)(unsigned)k << p.slot_bits | no_slot;
+      if (k != KEY_EMPTY) skey[i] = k;
     }
     __syncthreads();
   }
@@ -860,15 +728,12 @@ __device__ __forceinline__ void process_tile(const TileScene& p, int tile, unsig
     int med_rows = 0, med_place = 0;
     if (i < end) {
       unsigned t = __ldg(bin_tris + i) - (unsigned)p.tri_base;
-      unsigned slot = (i - beg) < (unsigned)p.nslots ? (i - beg) : no_slot;
       TriSetup s;
       if (CLIP && t >= (unsigned)p.T) {
-        // a clipped sub-triangle: its points, the key of its triangle, no
-        // record (the winner shades from its triangle's clip coordinates)
+        // a clipped sub-triangle: its points, and the key of its triangle
         const int4* c = p.clip_tris + 3 * (size_t)(t - (unsigned)p.T);
         setup_points(__ldg(c), __ldg(c + 1), __ldg(c + 2), s);
         t = __ldg(p.clip_orig + (t - (unsigned)p.T));
-        slot = no_slot;
       } else {
         load_setup(p, t, s);
       }
@@ -879,18 +744,15 @@ __device__ __forceinline__ void process_tile(const TileScene& p, int tile, unsig
       centre_range(minY, maxY, y0, y1, py0, py1);
       if (px0 <= px1 && py0 <= py1) {
         const int npx = (px1 - px0 + 1) * (py1 - py0 + 1);
-        const unsigned long long tag = ((unsigned long long)t << p.slot_bits) | slot;
+        const unsigned long long tag = t;
         const bool narrow = maxX - minX < 32768 && maxY - minY < 32768;
-        bool covers = true;
         if (STATS) st.tests += npx;
         if (npx <= p.small_px) {
           unsigned f = 0u;
           if (narrow) {
             if (npx <= 32)  // coverage only; the warp's fragment_pass takes the depths
-            {
               small_box(s, tag, px0, px1, py0, py1, x0, y0, p.g.bshift_x, wst, lane, sb);
-              covers = sb.mask != 0u;
-            } else
+            else
               f = raster_thread32(s, tag, px0, px1, py0, py1, x0, y0, p.g.bshift_x, skey);
           } else {
             f = raster_thread64(s, tag, px0, px1, py0, py1, x0, y0, p.g.bshift_x, skey);
@@ -910,11 +772,9 @@ __device__ __forceinline__ void process_tile(const TileScene& p, int tile, unsig
           e[BG_X2 * 32] = s.X2; e[BG_Y2 * 32] = s.Y2;
           e[BG_Z0 * 32] = s.Z0; e[BG_Z1 * 32] = s.Z1; e[BG_Z2 * 32] = s.Z2;
           e[BG_ALO * 32] = (int)(unsigned)(s.A & 0xFFFFFFFFll); e[BG_AHI * 32] = (int)(s.A >> 32);
-          e[BG_T * 32] = (int)t; e[BG_SLOT * 32] = (int)slot;
+          e[BG_T * 32] = (int)t;
           pushed = true;
         }
-        // a small box without a covered sample needs no record
-        if (slot != no_slot && covers) fill_record<PERSP>(p, s, sm.srec + slot * p.rec_stride);
       }
     }
     {
@@ -934,11 +794,11 @@ __device__ __forceinline__ void process_tile(const TileScene& p, int tile, unsig
         s.Z0 = e[BG_Z0 * 32]; s.Z1 = e[BG_Z1 * 32]; s.Z2 = e[BG_Z2 * 32];
         s.A = (long long)(((unsigned long long)(unsigned)e[BG_AHI * 32] << 32) | (unsigned)e[BG_ALO * 32]);
         s.v0 = s.v1 = s.v2 = 0;  // not needed to rasterize
-        const unsigned t = (unsigned)e[BG_T * 32], slot = (unsigned)e[BG_SLOT * 32];
+        const unsigned t = (unsigned)e[BG_T * 32];
         int px0, px1, py0, py1;
         centre_range(min(s.X0, min(s.X1, s.X2)), max(s.X0, max(s.X1, s.X2)), x0, x1, px0, px1);
         centre_range(min(s.Y0, min(s.Y1, s.Y2)), max(s.Y0, max(s.Y1, s.Y2)), y0, y1, py0, py1);
-        const unsigned long long tag = ((unsigned long long)t << p.slot_bits) | slot;
+        const unsigned long long tag = t;
         const unsigned f = (px1 - px0 + 1) * (py1 - py0 + 1) >= PIKO_SPAN_MIN_PX
                                ? raster_warp_spans(s, tag, px0, px1, py0, py1, x0, y0, p.g.bshift_x, skey, lane)
                                : raster_warp(s, tag, px0, px1, py0, py1, x0, y0, p.g.bshift_x, skey, lane);
@@ -948,55 +808,41 @@ __device__ __forceinline__ void process_tile(const TileScene& p, int tile, unsig
       __syncthreads();
     }
   }
-  // shade, write, and leave the key tile cleared for the next tile
-  for (int i = tid; i < bin_px; i += nt) {
-    const unsigned long long k = skey[i];
-    skey[i] = KEY_EMPTY;
-    const int x = x0 + (i & (bin_w - 1)), y = y0 + (i >> p.g.bshift_x);
-    if (x > x1 || y > y1) continue;
-    const size_t o = (size_t)y * p.g.W + x;
-    if (k == KEY_EMPTY) {
-      p.key_out[o] = KEY_EMPTY;
-      write_empty(p, o);
-      continue;
+  // shade, write, and leave the key tile cleared for the next tile; the
+  // indices of a thread's next winner are loaded before it shades one
+  auto take = [&](int i) {
+    unsigned long long k = KEY_EMPTY;
+    if (i < bin_px) {
+      k = skey[i];
+      skey[i] = KEY_EMPTY;
     }
-    const unsigned z = (unsigned)(k >> 40);
-    // the triangle field sits between the slot and the depth: 40 - slot_bits wide
-    const unsigned t = (unsigned)((k >> p.slot_bits) & ((1ull << (40 - p.slot_bits)) - 1ull));
-    const unsigned slot = (unsigned)(k & no_slot);
-    p.key_out[o] = ((unsigned long long)z << 32) | t;
-    if (STATS) ++st.shaded;
-    if (slot != no_slot)
-      shade_from_record<PERSP>(p, sm.srec + slot * p.rec_stride, x, y, o);
-    else
-      shade_from_global<PERSP, CLIP>(p, tri_indices(p.tris, t), x, y, o);
+    return k;
+  };
+  unsigned long long k = take(tid);
+  int3 id = make_int3(0, 0, 0), idn = id;
+  if (k != KEY_EMPTY) id = tri_indices(p.tris, (unsigned)k);
+  for (int i = tid; i < bin_px; i += nt) {
+    const unsigned long long kn = take(i + nt);
+    if (kn != KEY_EMPTY) idn = tri_indices(p.tris, (unsigned)kn);
+    const int x = x0 + (i & (bin_w - 1)), y = y0 + (i >> p.g.bshift_x);
+    if (x <= x1 && y <= y1) {
+      const size_t o = (size_t)y * p.g.W + x;
+      p.key_out[o] = k;
+      if (k == KEY_EMPTY) {
+        write_empty(p, o);
+      } else {
+        if (STATS) ++st.shaded;
+        shade_winner<PERSP, CLIP>(p, id, x, y, o);
+      }
+    }
+    k = kn;
+    id = idn;
   }
   __syncthreads();
 }
 
-// Record layout of a scene: slot bits below the triangle index (2^id_bits > T,
-// so no key equals the all-ones empty key), records per tile and words per
-// record (odd, so that distinct records fall in distinct banks).  want_slots
-// (0: as many as allowed) sizes the record area: shared memory taken by
-// records is taken from L1, which serves the kernel's gathers, so records
-// are sized for the tiles' typical entry count rather than the largest.
-// persp adds the three vertices' 1/w (perspective-correct attributes).
-inline void tile_layout(int num_triangles, int bin_px, int mode, bool has_color, bool persp, int max_slots,
-                        int& slot_bits, int& nslots, int& rec_stride, int want_slots = 0) {
-  int id_bits = 1;
-  while (id_bits < 32 && (1LL << id_bits) <= (long long)num_triangles) ++id_bits;
-  slot_bits = 40 - id_bits < 16 ? 40 - id_bits : 16;
-  int want = bin_px <= 256 ? 255 : max_slots;
-  if (want_slots > 0 && want_slots < want) want = want_slots;
-  const int cap = (1 << slot_bits) - 1;
-  nslots = want < cap ? want : cap;
-  rec_stride = R_ATTR + rec_attr_count(mode, has_color) + (persp ? 3 : 0);
-  if ((rec_stride & 1) == 0) ++rec_stride;
-}
-
-inline size_t tile_smem_bytes(int bin_px, int threads, int nslots, int rec_stride) {
-  return (size_t)bin_px * 8 + (size_t)threads * 4 + (size_t)(threads / 32) * FRAG_WARP_WORDS * 4 +
-         (size_t)nslots * rec_stride * 4;
+inline size_t tile_smem_bytes(int bin_px, int threads) {
+  return (size_t)bin_px * 8 + (size_t)threads * 4 + (size_t)(threads / 32) * FRAG_WARP_WORDS * 4;
 }
 
 }  // namespace piko
