@@ -74,6 +74,7 @@ struct piko_raster {
   unsigned heavy_epoch = 0;
   unsigned long long* dkeys = nullptr;  // a key per pixel of directly rasterized triangles (piko_direct.cuh)
   long long dkcap = 0;
+  unsigned* busy = nullptr;             // tiles with bin entries, of a frame with direct keys
   // fragment buffers of the unfused pipeline (PIKO_SCHED_UNFUSED)
   unsigned* frag_pix = nullptr;
   unsigned long long* frag_key = nullptr;
@@ -204,6 +205,7 @@ piko_raster* piko_raster_create(int width, int height, int bin_w, int bin_h, int
             cudaMalloc(&h->chunk_state, sizeof(unsigned long long) * scan_chunks(h->nbins)) == cudaSuccess &&
             cudaMemset(h->chunk_state, 0, sizeof(unsigned long long) * scan_chunks(h->nbins)) == cudaSuccess &&
             cudaMalloc(&h->status, sizeof(DevStatus)) == cudaSuccess &&
+            cudaMalloc(&h->busy, sizeof(unsigned) * h->nbins) == cudaSuccess &&
             cudaMalloc(&h->heavy, sizeof(uint2) * HEAVY_LIST_CAP) == cudaSuccess &&
             cudaMallocHost(&h->h_needed, 3 * sizeof(unsigned long long)) == cudaSuccess &&
             cudaMallocHost(&h->h_frags, sizeof(unsigned)) == cudaSuccess &&
@@ -232,6 +234,7 @@ void piko_raster_destroy(piko_raster* h) {
   cudaFree(h->bin_tris);
   cudaFree(h->heavy);
   cudaFree(h->dkeys);
+  cudaFree(h->busy);
   cudaFree(h->frag_pix);
   cudaFree(h->frag_key);
   cudaFree(h->frag_rgba);
@@ -565,6 +568,7 @@ static int scatter_and_process(piko_raster* h, const piko_scene* s, piko_framebu
   p.bin_off = h->bin_off;
   p.bin_tris = h->bin_tris;
   p.dkeys = direct.keys;
+  p.busy = direct.busy;
   p.key_out = reinterpret_cast<unsigned long long*>(fb->key);
   p.rgba_out = reinterpret_cast<float4*>(fb->rgba);
   p.gnorm_out = reinterpret_cast<uint2*>(fb->gbuf_normal);
@@ -617,6 +621,7 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
   float4* vattr = packed_attributes(h, s);
   DirectRaster direct;
   direct.keys = direct_keys(h, T, V, st);
+  direct.busy = direct.keys ? h->busy : nullptr;
   direct.max_px = h->small_px < DIRECT_MAX_PX ? h->small_px : DIRECT_MAX_PX;
   launch_vertex(h->W, h->H, V, s->pos, s->mvp, h->vtx, lambert ? s->normal : nullptr, s->light_dir,
                 lambert ? h->vdot : nullptr, h->perspective ? h->invw : nullptr, h->num_sms, st, direct.keys,
@@ -657,7 +662,7 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
                          clip_tris, clip_cap, h->exact_bins, h->heavy, heavy_cap(h), heavy_epoch, direct);
       if (ev) cudaEventRecord(h->stage_ev[2], st);
       launch_scan(h->nbins, h->bin_count, h->bin_off, h->cursor, (unsigned long long)h->ecap, h->status,
-                  h->chunk_state, scan_epoch, st, h->wait_budget, h->withhold, &report);
+                  h->chunk_state, scan_epoch, st, h->wait_budget, h->withhold, &report, direct.busy);
       if (ev) cudaEventRecord(h->stage_ev[3], st);
     }
     if ((r = scatter_and_process(h, s, fb, st, ev, direct, vattr, clip_tris, clip_cap)) != PIKO_OK) return r;

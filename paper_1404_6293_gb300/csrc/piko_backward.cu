@@ -14,7 +14,7 @@ struct BackwardParams {
 
 // A warp per 16 x 2 pixels.
 template <bool PERSP>
-__global__ void __launch_bounds__(PIX_THREADS, 4) k_backward_pixel(const __grid_constant__ BackwardParams p) {
+__global__ void __launch_bounds__(PIX_THREADS, 5) k_backward_pixel(const __grid_constant__ BackwardParams p) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tile = blockIdx.x * (PIX_THREADS / 32) + warp;
   if (tile >= p.ntiles) return;  // the same for the whole warp

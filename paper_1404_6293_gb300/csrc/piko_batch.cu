@@ -210,14 +210,13 @@ __device__ __forceinline__ LaneBins lane_setup(const BatchParams& b, int t, int 
   r.nbx = d.g.nbx;
   r.bin_base = d.bin_base;
   const int tl = t - d.tri_base;
-  const int ia = __ldg(d.tris + 3 * (size_t)tl), ib = __ldg(d.tris + 3 * (size_t)tl + 1),
-            ic = __ldg(d.tris + 3 * (size_t)tl + 2);
-  if ((unsigned)ia >= (unsigned)d.V || (unsigned)ib >= (unsigned)d.V || (unsigned)ic >= (unsigned)d.V) {
+  const int3 id = tri_indices(d.tris, (unsigned)tl);
+  if ((unsigned)id.x >= (unsigned)d.V || (unsigned)id.y >= (unsigned)d.V || (unsigned)id.z >= (unsigned)d.V) {
     record_error(b.st, PIKO_ERR_BAD_INDEX);
     return r;
   }
   const int4* vtx = b.vtx + d.vtx_base;
-  const int4 p0 = __ldg(vtx + ia), p1 = __ldg(vtx + ib), p2 = __ldg(vtx + ic);
+  const int4 p0 = __ldg(vtx + id.x), p1 = __ldg(vtx + id.y), p2 = __ldg(vtx + id.z);
   if (!(p0.w & p1.w & p2.w)) return r;
   const int minx = min(p0.x, min(p1.x, p2.x)), maxx = max(p0.x, max(p1.x, p2.x));
   const int miny = min(p0.y, min(p1.y, p2.y)), maxy = max(p0.y, max(p1.y, p2.y));
@@ -524,8 +523,12 @@ __device__ __forceinline__ void fill_bwd_scene(const BatchBwdParams& b, const Ba
 // vertex then serves a pixel in place of six words (the pixel kernel was at 82%
 // of the L1's throughput with those).
 __global__ void __launch_bounds__(GRAD_CHUNK) k_batch_attributes(BatchBwdParams b) {
-  for (int i = blockIdx.x; i < b.total_chunks; i += gridDim.x) {
-    const int g = find_scene(b.chunk_prefix, b.ngroups, i);
+  // chunks in a row per CTA, so that it looks its group up once
+  const int per = (b.total_chunks + (int)gridDim.x - 1) / (int)gridDim.x, first = (int)blockIdx.x * per;
+  if (first >= b.total_chunks) return;
+  int g = find_scene(b.chunk_prefix, b.ngroups, first);
+  for (int i = first; i < min(first + per, b.total_chunks); ++i) {
+    while (__ldg(b.chunk_prefix + g + 1) <= i) ++g;
     const GradAcc& f = b.groups[g];
     const int v = (i - __ldg(b.chunk_prefix + g)) * GRAD_CHUNK + (int)threadIdx.x;
     if (!f.normal || v >= f.V) continue;
@@ -539,7 +542,7 @@ __global__ void __launch_bounds__(GRAD_CHUNK) k_batch_attributes(BatchBwdParams 
 
 // A warp takes BATCH_PIX_RUN blocks of 16 x 2 pixels in a row, so
 // that it looks its scene up once for most of them.
-constexpr int BATCH_PIX_RUN = 4;
+constexpr int BATCH_PIX_RUN = 8;
 template <bool PERSP>
 __global__ void __launch_bounds__(PIX_THREADS, 4) k_batch_backward_pixel(BatchBwdParams b) {
   __shared__ BwdScene ssc[PIX_THREADS / 32];
@@ -569,8 +572,11 @@ __global__ void __launch_bounds__(PIX_THREADS, 4) k_batch_backward_pixel(BatchBw
 __global__ void __launch_bounds__(GRAD_CHUNK) k_batch_finish(BatchBwdParams b) {
   __shared__ GradFinishSmem sm;
   pdl_wait();  // the accumulators
-  for (int i = blockIdx.x; i < b.total_chunks; i += gridDim.x) {
-    const int g = find_scene(b.chunk_prefix, b.ngroups, i);
+  const int per = (b.total_chunks + (int)gridDim.x - 1) / (int)gridDim.x, first = (int)blockIdx.x * per;
+  if (first >= b.total_chunks) return;
+  int g = find_scene(b.chunk_prefix, b.ngroups, first);
+  for (int i = first; i < min(first + per, b.total_chunks); ++i) {
+    while (__ldg(b.chunk_prefix + g + 1) <= i) ++g;
     grad_finish_chunk(b.groups[g], i - __ldg(b.chunk_prefix + g), sm);
   }
 }

@@ -160,39 +160,45 @@ __device__ __forceinline__ void backward_warp_pixels(const BwdScene& sc, const f
   }
   pdl_wait();  // snapped vertices and light terms
   pdl_launch_dependents();
-  TriSetup s;
-  s.v0 = s.v1 = s.v2 = 0;
+  if (hit)
+    hit = (unsigned)ia < (unsigned)sc.V && (unsigned)ib < (unsigned)sc.V && (unsigned)ic < (unsigned)sc.V;
+  int4 p0 = make_int4(0, 0, 0, 0), p1 = p0, p2 = p0;
+  long long A = 0;
   bool clipped = false;
   if (hit) {
-    const bool in_range = ia >= 0 && ia < sc.V && ib >= 0 && ib < sc.V && ic >= 0 && ic < sc.V;
-    hit = in_range && setup_triangle(ia, ib, ic, sc.vtx, s);
-    if (!hit && in_range && sc.pos) {  // a winner the vertex stage rejected was clipped
-      clipped = hit = true;
-      s.v0 = ia; s.v1 = ib; s.v2 = ic;
+    p0 = __ldg(sc.vtx + ia); p1 = __ldg(sc.vtx + ib); p2 = __ldg(sc.vtx + ic);
+    // twice the area: negative, like the edge functions below, for a triangle
+    // wound the other way
+    A = (long long)(p1.x - p0.x) * (p2.y - p0.y) - (long long)(p2.x - p0.x) * (p1.y - p0.y);
+    if (A == 0 || !(p0.w & p1.w & p2.w)) {  // a winner the vertex stage rejected was clipped
+      clipped = sc.pos != nullptr;
+      hit = clipped;
     }
   }
+  if (!__any_sync(FULL_MASK, hit)) return;
   if (!hit) t = BWD_NONE;
   float v[BWD_VALS];
 #pragma unroll
   for (int q = 0; q < BWD_VALS; ++q) v[q] = 0.f;
   if (hit) {
-    const int vid[3] = {s.v0, s.v1, s.v2};
+    const int vid[3] = {ia, ib, ic};
     float b[3];
     if (clipped) {
       clip_ray_weights(sc.pos, sc.mvp, sc.W, sc.H, vid, x, y, b[0], b[1], b[2]);
     } else {
-      const float rA = __frcp_rn(f32_from_i64(s.A));
-      if (s.A < (1LL << 31)) {  // the covered pixel's edge functions lie in [0, A]: exact in 32 bits
-        const int Px = 256 * x + 128, Py = 256 * y + 128;
-        const int w1 = edge_fn_wrap32(s.X2, s.Y2, s.X0, s.Y0, Px, Py), w2 = edge_fn_wrap32(s.X0, s.Y0, s.X1, s.Y1, Px, Py);
-        b[0] = (float)((int)s.A - w1 - w2) * rA;
+      const int dx1 = p0.x - p2.x, dy1 = p0.y - p2.y, dx2 = p1.x - p0.x, dy2 = p1.y - p0.y;
+      const int ux = 256 * x + 128 - p0.x, uy = 256 * y + 128 - p0.y;
+      if (A == (long long)(int)A) {  // the covered pixel's edge functions lie in [0, A]: exact in 32 bits
+        const float rA = __frcp_rn((float)(int)A);
+        const int w1 = (int)((unsigned)dx1 * (unsigned)uy - (unsigned)dy1 * (unsigned)ux);
+        const int w2 = (int)((unsigned)dx2 * (unsigned)uy - (unsigned)dy2 * (unsigned)ux);
+        b[0] = (float)((int)A - w1 - w2) * rA;
         b[1] = (float)w1 * rA;
         b[2] = (float)w2 * rA;
       } else {
-        const long long Px = 256LL * x + 128, Py = 256LL * y + 128;
-        const long long w1 = (long long)(s.X0 - s.X2) * (Py - s.Y2) - (long long)(s.Y0 - s.Y2) * (Px - s.X2);
-        const long long w2 = (long long)(s.X1 - s.X0) * (Py - s.Y0) - (long long)(s.Y1 - s.Y0) * (Px - s.X0);
-        b[0] = f32_from_i64(s.A - w1 - w2) * rA;
+        const float rA = __frcp_rn(f32_from_i64(A));
+        const long long w1 = (long long)dx1 * uy - (long long)dy1 * ux, w2 = (long long)dx2 * uy - (long long)dy2 * ux;
+        b[0] = f32_from_i64(A - w1 - w2) * rA;
         b[1] = f32_from_i64(w1) * rA;
         b[2] = f32_from_i64(w2) * rA;
       }
@@ -242,7 +248,7 @@ __device__ __forceinline__ void backward_warp_pixels(const BwdScene& sc, const f
   const int end = after ? __ffs(after) - 1 : 32;        // one past this lane's run
 #pragma unroll
   for (int o = 1; o < PIX_W; o <<= 1) {
-    const bool add = lane + o < end;
+    const bool add = hit && lane + o < end;
     if (!__any_sync(FULL_MASK, add)) break;
 #pragma unroll
     for (int q = 0; q < BWD_VALS; ++q) {
@@ -251,9 +257,9 @@ __device__ __forceinline__ void backward_warp_pixels(const BwdScene& sc, const f
     }
   }
   if (hit && ((heads >> lane) & 1u)) {
-    grad_add(sc.acc + s.v0, v[0], v[3], v[6], v[9]);
-    grad_add(sc.acc + s.v1, v[1], v[4], v[7], v[10]);
-    grad_add(sc.acc + s.v2, v[2], v[5], v[8], v[11]);
+    grad_add(sc.acc + ia, v[0], v[3], v[6], v[9]);
+    grad_add(sc.acc + ib, v[1], v[4], v[7], v[10]);
+    grad_add(sc.acc + ic, v[2], v[5], v[8], v[11]);
   }
 }
 

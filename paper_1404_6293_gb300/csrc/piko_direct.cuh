@@ -119,27 +119,17 @@ __device__ __forceinline__ bool direct_triangle(int4 p0, int4 p1, int4 p2, unsig
 // CLIP: a winner whose vertices the vertex stage rejected was clipped.
 template <bool PERSP, bool CLIP>
 __device__ __forceinline__ void shade_direct_pixel(const TileScene& p, int3 id, int x, int y, size_t o) {
-  const int4 p0 = __ldg(p.vtx + id.x);
-  int4 p1 = __ldg(p.vtx + id.y), p2 = __ldg(p.vtx + id.z);
+  const int4 p0 = __ldg(p.vtx + id.x), p1 = __ldg(p.vtx + id.y), p2 = __ldg(p.vtx + id.z);
   if (CLIP && !(p0.w & p1.w & p2.w)) {
     shade_winner<PERSP, true>(p, id, x, y, o);
     return;
   }
-  int A = (p1.x - p0.x) * (p2.y - p0.y) - (p2.x - p0.x) * (p1.y - p0.y);
-  if (A < 0) {
-    A = -A;
-    const int4 q = p1;
-    p1 = p2;
-    p2 = q;
-    const int i = id.y;
-    id.y = id.z;
-    id.z = i;
-  }
-  const float rA = approx_rcp((float)A);
-  const int Px = 256 * x + 128, Py = 256 * y + 128;
-  float b1 = (float)edge_fn_wrap32(p2.x, p2.y, p0.x, p0.y, Px, Py) * rA;
-  float b2 = (float)edge_fn_wrap32(p0.x, p0.y, p1.x, p1.y, Px, Py) * rA;
-  float b0 = 1.0f - b1 - b2;
+  // edges 2->0 and 0->1 and the area, all negative for a triangle wound the
+  // other way: the signs cancel in the weights of vertices 1 and 2
+  const int dx1 = p0.x - p2.x, dy1 = p0.y - p2.y, dx2 = p1.x - p0.x, dy2 = p1.y - p0.y;
+  const int u = 256 * x + 128 - p0.x, v = 256 * y + 128 - p0.y;
+  const float rA = __fdividef(1.0f, (float)(dx1 * dy2 - dx2 * dy1));
+  float b1 = (float)(dx1 * v - dy1 * u) * rA, b2 = (float)(dx2 * v - dy2 * u) * rA, b0 = 1.0f - b1 - b2;
   if (PERSP) perspective_bary(b0, b1, b2, __ldg(p.invw + id.x), __ldg(p.invw + id.y), __ldg(p.invw + id.z));
   if (p.mode == PIKO_SHADE_LAMBERT)
     shade_lambert(p, id.x, id.y, id.z, b0, b1, b2, o);

@@ -349,7 +349,8 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan(int nbins, unsigned* __re
                                                        unsigned* __restrict__ bin_off, unsigned* __restrict__ cursor,
                                                        unsigned long long capacity, DevStatus* st,
                                                        unsigned long long* __restrict__ chunk_state, unsigned epoch,
-                                                       long long wait_budget, int withhold, ScanReport report) {
+                                                       long long wait_budget, int withhold, ScanReport report,
+                                                       unsigned* __restrict__ busy) {
   __shared__ ScanSmem sm;
   pdl_wait();  // counts and the ticket reset of the count pass
   pdl_launch_dependents();
@@ -359,7 +360,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan(int nbins, unsigned* __re
   const int nchunks = (nbins + SCAN_CHUNK - 1) / SCAN_CHUNK;
   if (chunk >= nchunks) return;  // only with a corrupted ticket; the count pass resets it every frame
   scan_chunk(chunk, nchunks, nbins, cnt, bin_off, cursor, capacity, st, chunk_state, epoch, sm, &st->queue_head,
-             wait_budget, withhold, report);
+             wait_budget, withhold, report, busy);
   // one CTA per chunk: every ticket was taken before the last chunk's
   // look-back ended, so the last chunk may reset the ticket
   if (chunk == nchunks - 1 && threadIdx.x == 0) st->scan_ticket = 0u;
@@ -541,7 +542,8 @@ __global__ void __launch_bounds__(256, EXACT || DIRECT ? 4 : 8) k_setup_count(Ra
   // the vertex stage does not touch the status word, and everything before
   // it has completed (it is launched without the early-start attribute)
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    st->scan_ticket = 0u;  // the scan runs after this kernel
+    st->scan_ticket = 0u;  // the scan runs after this kernel (or in its last CTA)
+    st->busy_n = 0u;
     // the other parity's heavy counter is the next count pass's: nothing reads it until then
     st->heavy_n[(heavy_epoch + 1u) & 1u] = 0u;
   }
@@ -605,7 +607,7 @@ __global__ void __launch_bounds__(256, EXACT || DIRECT ? 4 : 8) k_setup_count(Ra
       __threadfence();
       if (threadIdx.x == 0) st->count_done = 0u;  // for the next frame
       scan_chunk(0, 1, nbins, cnt, fs.bin_off, fs.cursor, fs.capacity, st, fs.chunk_state, fs.epoch, scan_sm,
-                 &st->queue_head, WAIT_BUDGET_CYCLES, 0, fs.report);
+                 &st->queue_head, WAIT_BUDGET_CYCLES, 0, fs.report, direct.busy);
     }
   }
 }
@@ -671,9 +673,9 @@ bool launch_count_and_scan(const RasterGeom& g, int T, const int* tris, int V, c
 
 void launch_scan(int nbins, unsigned* bin_count, unsigned* bin_off, unsigned* cursor, unsigned long long capacity,
                  DevStatus* st, unsigned long long* chunk_state, unsigned epoch, cudaStream_t s, long long wait_budget,
-                 int withhold, const ScanReport* report) {
+                 int withhold, const ScanReport* report, unsigned* busy) {
   launch_pdl(k_scan, scan_chunks(nbins), SCAN_THREADS, 0, s, nbins, bin_count, bin_off, cursor, capacity, st,
-             chunk_state, epoch, wait_budget, withhold, report ? *report : ScanReport());
+             chunk_state, epoch, wait_budget, withhold, report ? *report : ScanReport(), busy);
 }
 
 // ======================================================================
@@ -845,39 +847,44 @@ __global__ void __launch_bounds__(256, CLIP ? 4 : 5) k_scatter_shade(const __gri
     return;
   }
   const int lane = threadIdx.x & 31;
-  const int per_row = (g.W + SHADE_W - 1) / SHADE_W, blocks = per_row * ((g.H + SHADE_H - 1) / SHADE_H);
-  const int step = ((int)gridDim.x - a.scatter_blocks) * 8;
-  // a lane's pixel of block b (past the framebuffer: nothing), and its key,
-  // EMPTY where the block is the Process stage's (mine false).  Bins are at
-  // least 8 x 8 pixels, so a block lies in one.
+  const int per_row = (g.W + SHADE_W - 1) / SHADE_W, rows = (g.H + SHADE_H - 1) / SHADE_H;
+  // a warp's blocks lie `step` apart in row-major order: sx along x, sy along y
+  const int step = ((int)gridDim.x - a.scatter_blocks) * 8, sy = step / per_row, sx = step - sy * per_row;
+  // a lane's pixel of the block in column bx and row by (past the framebuffer:
+  // nothing), and its key, EMPTY where the block is the Process stage's (mine
+  // false).  Bins are at least 8 x 8 pixels, so a block lies in one.
   struct Block {
     int x, y;
     unsigned long long k;
     bool mine;
   };
-  auto load = [&](int b) {
+  int b = ((int)blockIdx.x - a.scatter_blocks) * 8 + (int)(threadIdx.x >> 5);
+  int by = b / per_row, bx = b - by * per_row;  // of the block to load next
+  auto load = [&]() {
     Block r;
     r.mine = false;
     r.k = KEY_EMPTY;
-    r.x = r.y = 0;
-    if (b < blocks) {
-      const int by = b / per_row, x0 = (b - by * per_row) * SHADE_W, y0 = by * SHADE_H;
-      const int bin = (y0 >> g.bshift_y) * g.nbx + (x0 >> g.bshift_x);
-      r.x = x0 + (lane & (SHADE_W - 1));
-      r.y = y0 + lane / SHADE_W;
+    r.x = bx * SHADE_W + (lane & (SHADE_W - 1));
+    r.y = by * SHADE_H + lane / SHADE_W;
+    if (by < rows) {
+      const int bin = ((by * SHADE_H) >> g.bshift_y) * g.nbx + ((bx * SHADE_W) >> g.bshift_x);
       r.k = direct_key(sc, r.x, r.y);
       r.mine = __ldg(a.bin_off + bin) == __ldg(a.bin_off + bin + 1);
+      bx += sx;
+      by += sy;
+      if (bx >= per_row) {
+        bx -= per_row;
+        ++by;
+      }
     }
     return r;
   };
-  int b = ((int)blockIdx.x - a.scatter_blocks) * 8 + (int)(threadIdx.x >> 5);
-  Block cur = load(b), next = load(b < blocks - step ? b + step : blocks);
+  Block cur = load(), next = load();
   int3 id = make_int3(0, 0, 0), idn = id;
   if (cur.k != KEY_EMPTY) id = tri_indices(sc.tris, (unsigned)cur.k);
-  while (b < blocks) {
+  while (cur.y - lane / SHADE_W < g.H) {  // the same for the whole warp
     if (next.k != KEY_EMPTY) idn = tri_indices(sc.tris, (unsigned)next.k);
-    b = b < blocks - step ? b + step : blocks;
-    const Block after = load(b < blocks - step ? b + step : blocks);
+    const Block after = load();
     if (cur.mine) shade_direct_block<PERSP, CLIP>(sc, cur.k, id, cur.x, cur.y);
     cur = next;
     next = after;

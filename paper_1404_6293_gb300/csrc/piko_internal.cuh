@@ -59,6 +59,7 @@ struct DevStatus {
   unsigned long long binned;    // triangles that reached at least one bin
   unsigned int heavy_n[2];      // chunks in the heavy-triangle list of AssignBin, by count-pass parity
   unsigned int count_done;      // count-pass CTAs finished (its last CTA scans small frames; then 0 again)
+  unsigned int busy_n;          // bins with entries (listed by the scan of a frame with direct keys; 0 before it)
   unsigned long long direct_entries;  // bin entries of the triangles the count pass rasterized itself (0 after the scan)
 };
 
@@ -220,7 +221,7 @@ __device__ __forceinline__ long long floor_div_est128(__int128 n, long long A, f
 }
 
 
-// Approximate 1/a (a >= 1): only ever used as an estimate that integer
+// Approximate 1/a (|a| >= 1): only ever used as an estimate that integer
 // arithmetic corrects, or for float barycentrics.
 __device__ __forceinline__ float approx_rcp(float a) { return __fdividef(1.0f, a); }
 
@@ -349,6 +350,7 @@ struct ProcessParams {
   const unsigned* bin_off;
   const unsigned* bin_tris;
   const unsigned long long* dkeys;  // keys of the count pass's direct rasterization (NULL: none)
+  const unsigned* busy;  // with dkeys: the st->busy_n tiles that have entries; only these are processed
   unsigned long long* key_out;
   float4* rgba_out;
   uint2* gnorm_out;  // binary16 x4
@@ -363,6 +365,7 @@ struct DirectRaster {
   unsigned long long* keys = nullptr;  // W * H keys, KEY_EMPTY before the pass (NULL: every triangle is binned)
   int max_px = 0;                      // largest box taken, in pixels
   const unsigned* clip_orig = nullptr; // triangle of each clipped sub-triangle
+  unsigned* busy = nullptr;            // nbins words: the scan lists the bins with entries there
 };
 
 // Vertex stage.  If vdot is not NULL it also stores n_v . L per vertex (the
@@ -418,7 +421,8 @@ void launch_clip(int W, int H, int T, const int* tris, int V, const float* pos, 
 // test hook bits (piko_scan.cuh).
 void launch_scan(int nbins, unsigned* bin_count, unsigned* bin_off, unsigned* cursor, unsigned long long capacity,
                  DevStatus* st, unsigned long long* chunk_state, unsigned epoch, cudaStream_t s,
-                 long long wait_budget = 40000000, int withhold = 0, const ScanReport* report = nullptr);
+                 long long wait_budget = 40000000, int withhold = 0, const ScanReport* report = nullptr,
+                 unsigned* busy = nullptr);
 int scan_chunks(int nbins);
 void launch_scatter(const RasterGeom& g, int T, const BinRect* rect, const unsigned* bin_off, unsigned* cursor,
                     unsigned* bin_tris, unsigned long long capacity, DevStatus* st, int num_sms, cudaStream_t s,

@@ -231,6 +231,7 @@ extern "C" int piko_raster_forward_noalloc(const piko_scene* s, piko_framebuffer
   p.mvp = s->mvp;
   p.bin_off = bin_off;
   p.bin_tris = bin_tris;
+  p.busy = nullptr;
   p.dkeys = nullptr;  // every triangle is binned: the array has no room for a key per pixel
   p.key_out = reinterpret_cast<unsigned long long*>(fb->key);
   p.rgba_out = reinterpret_cast<float4*>(fb->rgba);

@@ -66,17 +66,26 @@ __global__ void __maxnreg__(PIKO_PROCESS_MAXNREG) k_process(const __grid_constan
   sm.sfrag = sm.sbig + nt;
   sm.s_nbig = &s_nbig;
   const TileScene& sc = pl.sc;
-  for (int i = tid; i < bin_px; i += nt) sm.skey[i] = KEY_EMPTY;
+  auto clear_keys = [&] {
+    for (int i = tid; i < bin_px; i += nt) sm.skey[i] = KEY_EMPTY;
+  };
+  if (!p.busy) clear_keys();
   pdl_wait();  // bin lists and status of the scatter pass
-  // the first tile's range is loaded before the status word is tested, so
-  // that the two global round trips overlap (static and hardware schedules)
-  unsigned nbeg = 0u, nend = 0u;
-  if (SCHED != PIKO_SCHED_DYNAMIC && (int)blockIdx.x < p.ntiles) {
-    nbeg = __ldg(p.bin_off + blockIdx.x);
-    nend = __ldg(p.bin_off + blockIdx.x + 1);
-  }
-  if (p.st->flags & STATUS_SKIP_MASK) return;
+  // with direct keys the tiles without entries are shaded already: a frame of
+  // tiny triangles ends here after one look at the list's length
+  const int ntiles = p.busy ? (int)min(__ldcg(&p.st->busy_n), (unsigned)p.ntiles) : p.ntiles;
   constexpr bool dynamic = SCHED == PIKO_SCHED_DYNAMIC;
+  if ((p.st->flags & STATUS_SKIP_MASK) || (!dynamic && (int)blockIdx.x >= ntiles) || ntiles == 0) return;
+  auto tile_at = [&](int i) { return p.busy ? (int)__ldg(p.busy + i) : i; };
+  // the first tile's range (static and hardware schedules)
+  int tile = 0;
+  unsigned nbeg = 0u, nend = 0u;
+  if (!dynamic) {
+    tile = tile_at(blockIdx.x);
+    nbeg = __ldg(p.bin_off + tile);
+    nend = __ldg(p.bin_off + tile + 1);
+  }
+  if (p.busy) clear_keys();
   if (tid == 0) {
     s_nbig = 0u;
     if (dynamic) s_tile[0] = (int)atomicAdd(&p.st->queue_head, 1u);
@@ -84,34 +93,26 @@ __global__ void __maxnreg__(PIKO_PROCESS_MAXNREG) k_process(const __grid_constan
   __syncthreads();
   unsigned big_base = 0u;
   TileStats st = {0ull, 0ull, 0ull};
-  for (int iter = 0;; ++iter) {
-    int tile;
-    if (SCHED == PIKO_SCHED_HARDWARE) {
-      if (iter > 0) break;
-      tile = blockIdx.x;
-    } else if (SCHED == PIKO_SCHED_STATIC) {
-      tile = blockIdx.x + iter * gridDim.x;
-    } else {
-      tile = s_tile[iter & 1];
-      // fetch the next tile now; it is read after the tile's closing barrier
-      if (tid == 0 && tile < p.ntiles) s_tile[(iter + 1) & 1] = (int)atomicAdd(&p.st->queue_head, 1u);
-    }
-    if (tile >= p.ntiles) break;
-    unsigned beg, end;
-    if (SCHED == PIKO_SCHED_DYNAMIC) {
+  int at = dynamic ? s_tile[0] : (int)blockIdx.x;
+  for (int iter = 0; at < ntiles; ++iter) {
+    unsigned beg = nbeg, end = nend;
+    int next_tile = 0;
+    if (dynamic) {
+      tile = tile_at(at);
       beg = __ldg(p.bin_off + tile);
       end = __ldg(p.bin_off + tile + 1);
-    } else {
-      beg = nbeg;
-      end = nend;
+      // fetch the next tile now; it is read after the tile's closing barrier
+      if (tid == 0) s_tile[(iter + 1) & 1] = (int)atomicAdd(&p.st->queue_head, 1u);
+    } else if (SCHED == PIKO_SCHED_STATIC && at + (int)gridDim.x < ntiles) {
       // the static schedule's next tile is known: its range loads during this one
-      const int next = tile + (int)gridDim.x;
-      if (SCHED == PIKO_SCHED_STATIC && next < p.ntiles) {
-        nbeg = __ldg(p.bin_off + next);
-        nend = __ldg(p.bin_off + next + 1);
-      }
+      next_tile = tile_at(at + (int)gridDim.x);
+      nbeg = __ldg(p.bin_off + next_tile);
+      nend = __ldg(p.bin_off + next_tile + 1);
     }
     process_tile<STATS, PERSP, CLIP>(sc, tile, beg, end, p.bin_tris, sm, big_base, st);
+    if (SCHED == PIKO_SCHED_HARDWARE) break;
+    tile = next_tile;
+    at = dynamic ? s_tile[(iter + 1) & 1] : at + (int)gridDim.x;
   }
   if (STATS) {  // one atomic per warp: same-address atomics from every thread serialise
     for (int o = 16; o > 0; o >>= 1) {

@@ -77,7 +77,8 @@ __device__ __forceinline__ void scan_chunk(int chunk, int nchunks, int nbins, un
                                            unsigned long long capacity, DevStatus* st,
                                            unsigned long long* __restrict__ chunk_state, unsigned epoch, ScanSmem& sm,
                                            unsigned* queue_to_reset, long long wait_budget = WAIT_BUDGET_CYCLES,
-                                           int withhold = 0, ScanReport report = ScanReport()) {
+                                           int withhold = 0, ScanReport report = ScanReport(),
+                                           unsigned* __restrict__ busy = nullptr) {
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
   const unsigned long long tag = (unsigned long long)(epoch & 0xFFFFu) << 46;
   unsigned* __restrict__ multi = cnt + nbins;
@@ -141,6 +142,18 @@ __device__ __forceinline__ void scan_chunk(int chunk, int nchunks, int nbins, un
     of[j] = (unsigned)run;
     cu[j] = (unsigned)(run + sg[j]);
     run += (unsigned long long)sg[j] + mu[j];
+  }
+  if (busy) {  // the bins with entries, in any order
+    int n = 0;
+#pragma unroll
+    for (int j = 0; j < SCAN_PER; ++j) n += sg[j] + mu[j] != 0u;
+    const MultiSpan m = warp_prefix(n, lane);
+    unsigned at = 0u;
+    if (lane == 0 && m.total > 0) at = atomicAdd(&st->busy_n, (unsigned)m.total);
+    at = __shfl_sync(FULL_MASK, at, 0) + (unsigned)(m.incl - n);
+#pragma unroll
+    for (int j = 0; j < SCAN_PER; ++j)
+      if (sg[j] + mu[j] != 0u) busy[at++] = (unsigned)(b0 + j);
   }
   if (vec && b0 + SCAN_PER <= nbins) {
     reinterpret_cast<uint4*>(bin_off + b0)[0] = make_uint4(of[0], of[1], of[2], of[3]);
