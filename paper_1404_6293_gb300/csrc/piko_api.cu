@@ -59,7 +59,8 @@ struct piko_raster {
   float* vdot = nullptr;    // n . L, for Lambert without colours
   float* invw = nullptr;    // 1 / clip w, with perspective-correct attributes
   bool gacc_dirty = false;  // gacc is not zero: new, or a backward launch failed
-  BinRect* rect = nullptr;
+  BinRect* rect = nullptr;         // per triangle, then (marks) a byte per 32 triangles: one allocation of tcap triangles
+  unsigned char* marks = nullptr;  // (DirectRaster)
   long long tcap = 0;
   unsigned* bin_count = nullptr;  // 2 * nbins, zero between frames
   unsigned* bin_off = nullptr;    // nbins + 1
@@ -170,6 +171,19 @@ int grow_vertices(piko_raster* h, long long need) {
   h->invw = h->vdot + cap;
   h->gacc_dirty = true;
   h->vcap = cap;
+  return PIKO_OK;
+}
+
+// The per-triangle rectangles and the marks behind them.
+int grow_triangles(piko_raster* h, long long need) {
+  if (need <= h->tcap) return PIKO_OK;
+  const long long words = need + need / 256 + 64;  // a BinRect is 8 bytes: room for 8 marks each
+  long long cap = 0;
+  h->tcap = 0;
+  const int r = grow(h, &h->rect, &cap, words, "bin rectangles");
+  if (r != PIKO_OK) return r;
+  h->tcap = (cap - 16) / 257 * 256;  // 256 rectangles and their 8 marks take 257 words
+  h->marks = reinterpret_cast<unsigned char*>(h->rect + h->tcap);
   return PIKO_OK;
 }
 
@@ -357,7 +371,7 @@ int piko_raster_reserve(piko_raster* h, int64_t max_vertices, int64_t max_triang
     return fail(h, PIKO_ERR_INVALID_ARG, "reserve sizes out of range");
   int r;
   if ((r = grow_vertices(h, max_vertices)) != PIKO_OK) return r;
-  if ((r = grow(h, &h->rect, &h->tcap, max_triangles, "bin rectangles")) != PIKO_OK) return r;
+  if ((r = grow_triangles(h, max_triangles)) != PIKO_OK) return r;
   if ((r = grow(h, &h->bin_tris, &h->ecap, max_bin_entries, "bin lists")) != PIKO_OK) return r;
   // keys of direct rasterization, if such scenes can take it (else, or without
   // the memory, every triangle is binned)
@@ -576,7 +590,8 @@ static int scatter_and_process(piko_raster* h, const piko_scene* s, piko_framebu
   p.st = h->status;
   if (direct.keys) {
     const cudaError_t e = launch_scatter_shade(p, h->rect, h->cursor, h->bin_tris, (unsigned long long)h->ecap,
-                                               h->num_sms, st, clip_cap, h->heavy, heavy_cap(h), h->heavy_epoch);
+                                               h->num_sms, st, clip_cap, h->heavy, heavy_cap(h), h->heavy_epoch,
+                                               direct.marks);
     if (e != cudaSuccess) return cuda_fail(h, e, "scatter launch");
   } else {
     launch_scatter(h->g, T, h->rect, h->bin_off, h->cursor, h->bin_tris, (unsigned long long)h->ecap, h->status,
@@ -610,7 +625,7 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
   const int V = s->num_vertices, T = s->num_triangles;
   if ((r = grow_vertices(h, V)) != PIKO_OK) return r;
   const bool lambert = s->shade_mode == PIKO_SHADE_LAMBERT;
-  if ((r = grow(h, &h->rect, &h->tcap, T, "bin rectangles")) != PIKO_OK) return r;
+  if ((r = grow_triangles(h, T)) != PIKO_OK) return r;
   if (h->ecap == 0 && (r = grow(h, &h->bin_tris, &h->ecap, (long long)T * 2 + 4096, "bin lists")) != PIKO_OK)
     return r;
 
@@ -641,8 +656,9 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
     const int4* clip_tris = h->clip ? h->clip_tris : nullptr;
     const long long ccap = h->ccap_tris / 3 < h->ccap_orig ? h->ccap_tris / 3 : h->ccap_orig;
     const unsigned clip_cap = h->clip ? (unsigned)ccap : 0u;
-    if (clip_cap && (r = grow(h, &h->rect, &h->tcap, (long long)T + clip_cap, "bin rectangles")) != PIKO_OK) return r;
+    if (clip_cap && (r = grow_triangles(h, (long long)T + clip_cap)) != PIKO_OK) return r;
     direct.clip_orig = h->clip ? h->clip_orig : nullptr;
+    direct.marks = h->marks;
     // a frame of one scan chunk of bins is scanned by the count pass's last
     // CTA (one launch fewer on the chain); larger frames take the scan kernel
     // (with stage events on, the count and scan launches stay apart)
@@ -799,8 +815,9 @@ int piko_raster_forward_batch(piko_raster* h, const piko_scene* scenes, int n, p
                         h->unclamped, h->perspective, st, h->err);
   if (r != PIKO_OK) return r;
   for (int attempt = 0;; ++attempt) {
-    if ((r = batch_launch_forward(h->batch, h->status, h->batch_launch == 0, st, h->err, h->wait_budget,
-                                  h->withhold)) != PIKO_OK)
+    if ((r = batch_launch_forward(h->batch, h->status,
+                                  h->batch_launch == 0 && (h->withhold & TEST_WITHHOLD_BARRIER), st, h->err,
+                                  h->wait_budget, h->withhold)) != PIKO_OK)
       return r;
     if (!h->check_capacity) return PIKO_OK;
     cudaError_t e = cudaMemcpyAsync(h->h_needed, &h->status->needed, sizeof(unsigned long long),

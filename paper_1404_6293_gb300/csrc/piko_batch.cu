@@ -4,10 +4,10 @@
 // triangles, bins and tiles of scene s follow those of scenes 0..s-1, and a
 // work item finds its scene by binary search over the prefix counts.  The
 // phases are those of the single-scene forward (vertex stage, setup and
-// counts, scan, scatter, Process); by default they run in one persistent
-// cooperative launch whose CTAs meet at grid barriers between phases.  The
-// Piko paper's runtime is multi-kernel and names a persistent kernel as the
-// alternative it did not take (Sec. 5); the per-scene bin size and schedule
+// counts, scan, scatter, Process), a launch each, or one persistent cooperative
+// launch whose CTAs meet at grid barriers between phases.  The Piko paper's
+// runtime is multi-kernel and names a persistent kernel as the alternative it
+// did not take (Sec. 5); the per-scene bin size and schedule
 // are the knobs its Sec. 7.2 explores by hand.
 //
 // Every wait (grid barrier, scan look-back) is bounded by a clock budget;
@@ -52,8 +52,6 @@ struct BatchSync {
   unsigned pad;
 };
 
-enum : int { PH_VERTEX = 1, PH_COUNT = 2, PH_SCAN = 4, PH_SCATTER = 8, PH_PROCESS = 16 };
-
 struct BatchParams {
   int n;
   const BatchScene* sc;    // [n]
@@ -69,6 +67,7 @@ struct BatchParams {
   float4* vattr;  // colour and n . L per vertex (Lambert; the colour only where the scene has one)
   float* invw;  // 1 / clip w per vertex (perspective-correct attributes), else NULL
   BinRect* rect;
+  unsigned char* marks;  // a byte per 32 triangles: 1 where some of them have bin entries (else their rects are not written)
   unsigned long long* dkeys;  // a key per pixel of the scenes with direct rasterization
   unsigned total_dkeys;
   unsigned* cnt;  // 2 * total_bins, zero between frames
@@ -80,8 +79,6 @@ struct BatchParams {
   unsigned long long capacity;
   DevStatus* st;
   BatchSync* sync;
-  int phases;      // PH_* to run in this launch
-  int persistent;  // grid barriers between phases
   int max_bin_px;
   long long wait_budget;  // clock cycles a device-side wait may take before PIKO_ERR_TIMEOUT
   int withhold;           // test hooks: TEST_WITHHOLD_* bits (piko_scan.cuh)
@@ -280,10 +277,9 @@ __device__ void phase_count(const BatchParams& b) {
     const int t = base + lane;
     const LaneBins r = lane_setup(b, t, lane);
     dentries += r.dentries;
-    if (!__any_sync(FULL_MASK, r.valid)) {  // nothing to bin
-      if (t < b.total_t) b.rect[t] = BinRect{0xFFFFFFFFu, 0u};
-      continue;
-    }
+    const bool any = __any_sync(FULL_MASK, r.valid);
+    if (lane == 0) b.marks[base >> 5] = any ? 1 : 0;
+    if (!any) continue;  // nothing to bin
     const unsigned bin = r.single ? (unsigned)(r.bin_base + r.by0 * r.nbx + r.bx0) : 0xFFFFFFFFu;
     const unsigned grp = __match_any_sync(FULL_MASK, bin);
     const int leader = __ffs(grp) - 1;
@@ -329,34 +325,44 @@ __device__ void phase_scan(const BatchParams& b, ScanSmem& sm) {
   }
 }
 
-__device__ void phase_scatter(const BatchParams& b) {
-  const int lane = threadIdx.x & 31;
-  const int warps_total = gridDim.x * (blockDim.x >> 5);
-  for (int base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; base < b.total_t;
-       base += warps_total * 32) {
-    const int t = base + lane;
-    LaneBins r = no_bins();
-    if (t < b.total_t) {
-      const BinRect q = b.rect[t];
-      if (q.lo != 0xFFFFFFFFu) {
-        const BatchScene& d = b.sc[find_scene_lane(b.tri_prefix, b.n, base, t)];
-        r.valid = true;
-        r.nbx = d.g.nbx;
-        r.bin_base = d.bin_base;
-        if (q.lo & 0x8000u) {
-          r.single = true;
-          const int gbin = d.bin_base + (int)(q.lo >> 16) * d.g.nbx + (int)(q.lo & 0x7FFFu);
-          const unsigned pos = __ldg(b.bin_off + gbin) + q.hi;
-          if (pos < b.capacity) b.bin_tris[pos] = (unsigned)t;
-        } else {
-          r.bx0 = q.lo & 0xFFFF; r.by0 = q.lo >> 16; r.bx1 = q.hi & 0xFFFF; r.by1 = q.hi >> 16;
-        }
+// Bin entries of the 32 triangles from base on.
+__device__ __forceinline__ void scatter_triangles(const BatchParams& b, int base, int lane) {
+  const int t = base + lane;
+  LaneBins r = no_bins();
+  if (t < b.total_t) {
+    const BinRect q = b.rect[t];
+    if (q.lo != 0xFFFFFFFFu) {
+      const BatchScene& d = b.sc[find_scene_lane(b.tri_prefix, b.n, base, t)];
+      r.valid = true;
+      r.nbx = d.g.nbx;
+      r.bin_base = d.bin_base;
+      if (q.lo & 0x8000u) {
+        r.single = true;
+        const int gbin = d.bin_base + (int)(q.lo >> 16) * d.g.nbx + (int)(q.lo & 0x7FFFu);
+        const unsigned pos = __ldg(b.bin_off + gbin) + q.hi;
+        if (pos < b.capacity) b.bin_tris[pos] = (unsigned)t;
+      } else {
+        r.bx0 = q.lo & 0xFFFF; r.by0 = q.lo >> 16; r.bx1 = q.hi & 0xFFFF; r.by1 = q.hi >> 16;
       }
     }
-    for_multi_pairs(r, lane, [&](int owner, int gbin) {
-      const unsigned pos = atomicAdd(b.cursor + gbin, 1u);
-      if (pos < b.capacity) b.bin_tris[pos] = (unsigned)(base + owner);
-    });
+  }
+  for_multi_pairs(r, lane, [&](int owner, int gbin) {
+    const unsigned pos = atomicAdd(b.cursor + gbin, 1u);
+    if (pos < b.capacity) b.bin_tris[pos] = (unsigned)(base + owner);
+  });
+}
+
+__device__ void phase_scatter(const BatchParams& b) {
+  const int lane = threadIdx.x & 31;
+  const int step = gridDim.x * (blockDim.x >> 5) * 32;
+  // the marks of the warp's next 32 batches of triangles in one load; unmarked ones are skipped
+  for (long long base0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; base0 < b.total_t;
+       base0 += 32LL * step) {
+    const long long mine = base0 + (long long)lane * step;
+    for (unsigned m = __ballot_sync(FULL_MASK, mine < b.total_t && __ldcg(b.marks + (mine >> 5)) != 0); m != 0u;
+         m &= m - 1u) {
+      scatter_triangles(b, (int)(base0 + (long long)(__ffs(m) - 1) * step), lane);
+    }
   }
 }
 
@@ -454,42 +460,76 @@ __device__ void phase_process(const BatchParams& b, ProcessShared& ps, const Til
 #endif
 constexpr int BATCH_THREADS = PIKO_BATCH_THREADS;  // CTA size of the persistent batch kernel
 
-// PERSP: perspective-correct attributes; one instance per setting
-template <bool PERSP>
-__global__ void __maxnreg__(PIKO_BATCH_MAXNREG) k_batch_forward(BatchParams b) {
-  extern __shared__ __align__(16) unsigned long long smem[];
-  __shared__ ScanSmem scan_sm;
-  __shared__ ProcessShared ps;
-  __shared__ unsigned s_nbig;
+struct BatchSmem {
+  ProcessShared ps;
+  unsigned nbig;
+};
+__device__ __forceinline__ TileSmem batch_tile_smem(const BatchParams& b, unsigned long long* smem, BatchSmem& bs) {
   TileSmem sm;
   sm.skey = smem;
   sm.sbig = reinterpret_cast<int*>(smem + b.max_bin_px);
   sm.sfrag = sm.sbig + blockDim.x;
-  sm.s_nbig = &s_nbig;
+  sm.s_nbig = &bs.nbig;
+  return sm;
+}
+
+// All phases in one cooperative launch.  PERSP: perspective-correct attributes;
+// one instance per setting
+template <bool PERSP>
+__global__ void __maxnreg__(PIKO_BATCH_MAXNREG) k_batch_forward(BatchParams b) {
+  extern __shared__ __align__(16) unsigned long long smem[];
+  __shared__ ScanSmem scan_sm;
+  __shared__ BatchSmem bsm;
+  const TileSmem sm = batch_tile_smem(b, smem, bsm);
   if (cta_should_stop(b.st)) return;
-  if (b.phases & PH_VERTEX) {
-    phase_vertex<PERSP>(b);
-    const bool skip = (b.withhold & TEST_WITHHOLD_BARRIER) && blockIdx.x == 0;
-    if (b.persistent && !grid_barrier(b.sync, b.st, b.wait_budget, skip)) return;
-  }
-  if (b.phases & PH_COUNT) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) b.st->scan_ticket = 0u;  // the scan runs after a barrier
-    phase_count(b);
-    if (b.persistent && !grid_barrier(b.sync, b.st, b.wait_budget)) return;
-  }
-  if (b.phases & PH_SCAN) {
-    phase_scan(b, scan_sm);
-    if (b.persistent && !grid_barrier(b.sync, b.st, b.wait_budget)) return;
-  }
-  if (b.phases & PH_SCATTER) {
-    if (cta_should_stop(b.st)) return;
-    phase_scatter(b);
-    if (b.persistent && !grid_barrier(b.sync, b.st, b.wait_budget)) return;
-  }
-  if (b.phases & PH_PROCESS) {
-    if (cta_should_stop(b.st)) return;
-    phase_process<PERSP>(b, ps, sm);
-  }
+  phase_vertex<PERSP>(b);
+  const bool skip = (b.withhold & TEST_WITHHOLD_BARRIER) && blockIdx.x == 0;
+  if (!grid_barrier(b.sync, b.st, b.wait_budget, skip)) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) b.st->scan_ticket = 0u;  // the scan runs after a barrier
+  phase_count(b);
+  if (!grid_barrier(b.sync, b.st, b.wait_budget)) return;
+  phase_scan(b, scan_sm);
+  if (!grid_barrier(b.sync, b.st, b.wait_budget)) return;
+  if (cta_should_stop(b.st)) return;
+  phase_scatter(b);
+  if (!grid_barrier(b.sync, b.st, b.wait_budget)) return;
+  if (cta_should_stop(b.st)) return;
+  phase_process<PERSP>(b, bsm.ps, sm);
+}
+
+// One launch per phase (the default), each with the registers and threads that suit it: in
+// the persistent kernel every phase runs at the Process stage's 64 registers,
+// with half the warps that the gathers of the first ones want in flight.
+template <bool PERSP>
+__global__ void __launch_bounds__(256, 8) k_batch_vertex(BatchParams b) {
+  pdl_launch_dependents();
+  if (!cta_should_stop(b.st)) phase_vertex<PERSP>(b);
+}
+__global__ void __launch_bounds__(256, 4) k_batch_count(BatchParams b) {
+  pdl_wait();
+  pdl_launch_dependents();
+  if (cta_should_stop(b.st)) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) b.st->scan_ticket = 0u;  // the scan runs after this kernel
+  phase_count(b);
+}
+__global__ void __launch_bounds__(BATCH_THREADS) k_batch_scan(BatchParams b) {
+  __shared__ ScanSmem scan_sm;
+  pdl_wait();
+  pdl_launch_dependents();
+  if (!cta_should_stop(b.st)) phase_scan(b, scan_sm);
+}
+__global__ void __launch_bounds__(256, 6) k_batch_scatter(BatchParams b) {
+  pdl_wait();
+  pdl_launch_dependents();
+  if (!cta_should_stop(b.st)) phase_scatter(b);
+}
+template <bool PERSP>
+__global__ void __maxnreg__(PIKO_BATCH_MAXNREG) k_batch_process(BatchParams b) {
+  extern __shared__ __align__(16) unsigned long long smem[];
+  __shared__ BatchSmem bsm;
+  const TileSmem sm = batch_tile_smem(b, smem, bsm);
+  pdl_wait();
+  if (!cta_should_stop(b.st)) phase_process<PERSP>(b, bsm.ps, sm);
 }
 
 // ------------------------------------------------------------------ backward
@@ -619,6 +659,8 @@ struct BatchState {
   long long bcap = 0;  // bins
   unsigned* bin_tris = nullptr;
   long long ecap = 0;
+  unsigned char* marks = nullptr;
+  long long mcap = 0;
   unsigned long long* dkeys = nullptr;  // keys of direct rasterization
   long long dkcap = 0;
   float4* gacc = nullptr;  // gradient sums, zero between calls
@@ -636,6 +678,7 @@ struct BatchState {
   std::vector<BatchScene> host_desc;  // the uploaded descriptors
   size_t smem = 0;
   int grid = 0;
+  int num_sms = 0;
   int n = 0;
   int persp = 0;               // the layout's attribute interpolation (perspective-correct or not)
 };
@@ -684,6 +727,7 @@ void batch_state_free(BatchState* bs) {
   cudaFree(bs->bin_tris);
   cudaFree(bs->gacc);
   cudaFree(bs->dkeys);
+  cudaFree(bs->marks);
   cudaFree(bs->sync);
   if (bs->staging) cudaFreeHost(bs->staging);
   if (bs->uploaded) cudaEventDestroy(bs->uploaded);
@@ -759,6 +803,7 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   if ((r = grow_dev(&bs->vattr, &bs->dcap, tv, false, err)) != PIKO_OK) return r;
   if (persp && (r = grow_dev(&bs->invw, &bs->icap, tv, false, err)) != PIKO_OK) return r;
   if ((r = grow_dev(&bs->rect, &bs->tcap, tt, false, err)) != PIKO_OK) return r;
+  if ((r = grow_dev(&bs->marks, &bs->mcap, (tt + 31) / 32, false, err)) != PIKO_OK) return r;
   // here and not in the backward call, which may be recorded into a graph
   if (tv > bs->gcap) bs->gacc_dirty = true;
   if ((r = grow_dev(&bs->gacc, &bs->gcap, tv, false, err)) != PIKO_OK) return r;
@@ -845,15 +890,17 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   b.total_pblocks = (int)tq;
   b.total_v = (int)tv; b.total_t = (int)tt; b.total_bins = (int)tb; b.total_static = (int)tsd;
   b.total_dyn = (int)tdy;
-  b.vtx = bs->vtx; b.vattr = bs->vattr; b.invw = persp ? bs->invw : nullptr; b.rect = bs->rect; b.cnt = bs->cnt; b.bin_off = bs->bin_off;
+  b.vtx = bs->vtx; b.vattr = bs->vattr; b.invw = persp ? bs->invw : nullptr; b.rect = bs->rect; b.marks = bs->marks; b.cnt = bs->cnt; b.bin_off = bs->bin_off;
   b.dkeys = bs->dkeys; b.total_dkeys = (unsigned)tk;
   b.cursor = bs->cursor; b.chunk_state = bs->chunk_state; b.bin_tris = bs->bin_tris;
   b.capacity = (unsigned long long)bs->ecap; b.sync = bs->sync;
   b.max_bin_px = max_bin_px;
   bs->smem = tile_smem_bytes(max_bin_px, BATCH_THREADS);
   const auto kf = persp ? k_batch_forward<true> : k_batch_forward<false>;
+  const auto kp = persp ? k_batch_process<true> : k_batch_process<false>;
   if (bs->smem > 48 * 1024 &&
-      cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bs->smem) != cudaSuccess) {
+      (cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bs->smem) != cudaSuccess ||
+       cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bs->smem) != cudaSuccess)) {
     err = "batch shared memory request refused";
     return PIKO_ERR_CUDA;
   }
@@ -865,6 +912,7 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
     return PIKO_ERR_CUDA;
   }
   bs->grid = per_sm * num_sms;
+  bs->num_sms = num_sms;
   bs->desc_bytes = total;
   bs->group_off = group_off;
   bs->n = n;
@@ -873,7 +921,10 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   return PIKO_OK;
 }
 
-// Launches the forward phases; persistent = one cooperative launch.
+// Launches the forward phases, a launch each; persistent: all in one
+// cooperative launch, the form whose grid barriers have a test hook.  (The
+// separate launches are faster at every size: 49 against 62 us for three scenes
+// of 5,000 triangles at most, 407 against 455 for 32 of up to 100,000.)
 int batch_launch_forward(BatchState* bs, DevStatus* st, bool persistent, cudaStream_t stream, std::string& err,
                          long long wait_budget, int withhold) {
   BatchParams b = bs->params;
@@ -888,8 +939,6 @@ int batch_launch_forward(BatchState* bs, DevStatus* st, bool persistent, cudaStr
     return PIKO_ERR_CUDA;
   }
   if (persistent) {
-    b.phases = PH_VERTEX | PH_COUNT | PH_SCAN | PH_SCATTER | PH_PROCESS;
-    b.persistent = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(bs->grid);
     cfg.blockDim = dim3(BATCH_THREADS);
@@ -907,16 +956,25 @@ int batch_launch_forward(BatchState* bs, DevStatus* st, bool persistent, cudaStr
     }
     return PIKO_OK;
   }
-  b.persistent = 0;
-  const int phases[5] = {PH_VERTEX, PH_COUNT, PH_SCAN, PH_SCATTER, PH_PROCESS};
-  for (int k = 0; k < 5; ++k) {
-    b.phases = phases[k];
-    if (bs->persp)
-      k_batch_forward<true><<<bs->grid, BATCH_THREADS, bs->smem, stream>>>(b);
-    else
-      k_batch_forward<false><<<bs->grid, BATCH_THREADS, bs->smem, stream>>>(b);
-  }
-  const cudaError_t e = cudaGetLastError();
+  auto blocks_of = [&](long long items, int per_sm) {
+    const long long need = (items + 255) / 256, wave = (long long)per_sm * bs->num_sms;
+    return (int)(need < 1 ? 1 : (need < wave ? need : wave));
+  };
+  const long long clear = (long long)b.total_dkeys / 4;
+  const int vblocks = blocks_of(b.total_v > clear ? b.total_v : clear, 8);
+  cudaError_t e = cudaSuccess;
+  if (bs->persp)
+    k_batch_vertex<true><<<vblocks, 256, 0, stream>>>(b);
+  else
+    k_batch_vertex<false><<<vblocks, 256, 0, stream>>>(b);
+  if ((e = cudaGetLastError()) == cudaSuccess)
+    e = launch_pdl(k_batch_count, blocks_of(b.total_t, 4), 256, 0, stream, b);
+  const int chunks = (b.total_bins + BATCH_THREADS * SCAN_PER - 1) / (BATCH_THREADS * SCAN_PER);
+  if (e == cudaSuccess)
+    e = launch_pdl(k_batch_scan, chunks < bs->grid ? (chunks < 1 ? 1 : chunks) : bs->grid, BATCH_THREADS, 0, stream, b);
+  if (e == cudaSuccess) e = launch_pdl(k_batch_scatter, blocks_of(b.total_t, 6), 256, 0, stream, b);
+  if (e == cudaSuccess)
+    e = launch_pdl(bs->persp ? k_batch_process<true> : k_batch_process<false>, bs->grid, BATCH_THREADS, bs->smem, stream, b);
   if (e != cudaSuccess) {
     err = std::string("batch launch: ") + cudaGetErrorString(e);
     return PIKO_ERR_CUDA;

@@ -439,9 +439,10 @@ __device__ __forceinline__ void count_batch(const RasterGeom& g, int T, int t, c
       }
     }
   }
-  if (DIRECT && !__any_sync(FULL_MASK, valid)) {  // nothing to bin
-    if (t < T) rect[t] = BinRect{RECT_CULLED, 0u};
-    return;
+  if (DIRECT) {
+    const bool any = __any_sync(FULL_MASK, valid);
+    if (lane == 0) direct.marks[t >> 5] = any ? 1 : 0;  // (a warp's batch starts at a multiple of 32)
+    if (!any) return;  // nothing to bin
   }
   if (stats) {
     const unsigned nv = __popc(__ballot_sync(FULL_MASK, valid));
@@ -747,15 +748,16 @@ __device__ __forceinline__ unsigned single_pos(const RasterGeom& g, BinRect r, c
   return __ldg(bin_off + bin) + r.hi;
 }
 
-// The pass of CTA `block` of nblocks.
-template <bool EXACT>
+// The pass of CTA `block` of nblocks.  MARKS: only batches of 32 triangles with
+// a mark have rectangles.
+template <bool EXACT, bool MARKS>
 __device__ __forceinline__ void scatter_cta(const RasterGeom& g, int T, const BinRect* __restrict__ rect,
                                             const unsigned* __restrict__ bin_off, unsigned* __restrict__ cursor,
                                             unsigned* __restrict__ bin_tris, unsigned long long capacity,
                                             const DevStatus* st, const int4* __restrict__ clip_tris, unsigned clip_cap,
                                             const int* __restrict__ tris, int V, const int4* __restrict__ vtx,
                                             const uint2* __restrict__ heavy, unsigned heavy_cap, unsigned heavy_epoch,
-                                            int block, int nblocks) {
+                                            const unsigned char* __restrict__ marks, int block, int nblocks) {
   const int T_in = T;
   T = frame_triangles(T, clip_tris, clip_cap, st);
   // the heavy list's length is loaded now and used after the per-warp work
@@ -764,10 +766,9 @@ __device__ __forceinline__ void scatter_cta(const RasterGeom& g, int T, const Bi
   const int step = nblocks * (blockDim.x >> 5) * 32;
   BinRect none;
   none.lo = RECT_CULLED; none.hi = 0u;
-  // two batches per iteration, loads first
-  for (int base = (block * (blockDim.x >> 5) + wib) * 32; base < T; base += 2 * step) {
-    const int baseB = base + step;
-    const bool hasB = baseB < T;
+  // two batches at a time, loads first; baseB < 0: none
+  auto two = [&](int base, int baseB) {
+    const bool hasB = baseB >= 0;
     const BinRect ra = base + lane < T ? rect[base + lane] : none;
     const BinRect rb = hasB && baseB + lane < T ? rect[baseB + lane] : none;
     const unsigned pa = single_pos(g, ra, bin_off), pb = single_pos(g, rb, bin_off);
@@ -778,6 +779,23 @@ __device__ __forceinline__ void scatter_cta(const RasterGeom& g, int T, const Bi
     }
     scatter_batch<EXACT>(g, base, ra, pa, cursor, bin_tris, capacity, lane, oa);
     if (hasB) scatter_batch<EXACT>(g, baseB, rb, pb, cursor, bin_tris, capacity, lane, ob);
+  };
+  const int warp0 = (block * (blockDim.x >> 5) + wib) * 32;
+  if (MARKS) {
+    // the marks of the warp's next 32 batches in one load; unmarked ones are skipped
+    for (long long base = warp0; base < T; base += 32LL * step) {
+      const long long mine = base + (long long)lane * step;
+      unsigned m = __ballot_sync(FULL_MASK, mine < T && __ldg(marks + (mine >> 5)) != 0);
+      while (m != 0u) {
+        const int first = __ffs(m) - 1;
+        m &= m - 1u;
+        const int second = m ? __ffs(m) - 1 : -1;
+        m &= m - 1u;
+        two((int)(base + (long long)first * step), second >= 0 ? (int)(base + (long long)second * step) : -1);
+      }
+    }
+  } else {
+    for (int base = warp0; base < T; base += 2 * step) two(base, base + step < T ? base + step : -1);
   }
   // the heavy list's chunks, one per CTA step, a pair per thread
   for (unsigned e = block; e < nheavy; e += nblocks) {
@@ -812,8 +830,8 @@ __global__ void __launch_bounds__(256, EXACT ? 4 : 8) k_scatter(RasterGeom g, in
   pdl_wait();  // offsets, cursors and the status of the scan
   pdl_launch_dependents();
   if (st->flags & STATUS_SKIP_MASK) return;
-  scatter_cta<EXACT>(g, T, rect, bin_off, cursor, bin_tris, capacity, st, clip_tris, clip_cap, tris, V, vtx, heavy,
-                     heavy_cap, heavy_epoch, blockIdx.x, gridDim.x);
+  scatter_cta<EXACT, false>(g, T, rect, bin_off, cursor, bin_tris, capacity, st, clip_tris, clip_cap, tris, V, vtx,
+                            heavy, heavy_cap, heavy_epoch, nullptr, blockIdx.x, gridDim.x);
 }
 
 // A frame with direct keys: the first scatter_blocks CTAs scatter, the others
@@ -832,6 +850,7 @@ struct ScatterShade {
   unsigned clip_cap;
   const uint2* heavy;
   unsigned heavy_cap, heavy_epoch;
+  const unsigned char* marks;
   int scatter_blocks;
 };
 template <bool PERSP, bool CLIP>
@@ -842,8 +861,9 @@ __global__ void __launch_bounds__(256, CLIP ? 4 : 5) k_scatter_shade(const __gri
   const TileScene& sc = a.sc;
   const RasterGeom& g = sc.g;
   if ((int)blockIdx.x < a.scatter_blocks) {
-    scatter_cta<false>(g, sc.T, a.rect, a.bin_off, a.cursor, a.bin_tris, a.capacity, a.st, sc.clip_tris, a.clip_cap,
-                       nullptr, 0, nullptr, a.heavy, a.heavy_cap, a.heavy_epoch, blockIdx.x, a.scatter_blocks);
+    scatter_cta<false, true>(g, sc.T, a.rect, a.bin_off, a.cursor, a.bin_tris, a.capacity, a.st, sc.clip_tris,
+                             a.clip_cap, nullptr, 0, nullptr, a.heavy, a.heavy_cap, a.heavy_epoch, a.marks, blockIdx.x,
+                             a.scatter_blocks);
     return;
   }
   const int lane = threadIdx.x & 31;
@@ -908,7 +928,8 @@ void launch_scatter(const RasterGeom& g, int T, const BinRect* rect, const unsig
 
 cudaError_t launch_scatter_shade(const ProcessParams& p, const BinRect* rect, unsigned* cursor, unsigned* bin_tris,
                                  unsigned long long capacity, int num_sms, cudaStream_t s, unsigned clip_cap,
-                                 const uint2* heavy, unsigned heavy_cap, unsigned heavy_epoch) {
+                                 const uint2* heavy, unsigned heavy_cap, unsigned heavy_epoch,
+                                 const unsigned char* marks) {
   const long long TT = (long long)p.num_triangles + (p.clip_tris ? clip_cap : 0u);
   const long long need = ((TT + 31) / 32 + 7) / 8;
   ScatterShade a;
@@ -916,7 +937,9 @@ cudaError_t launch_scatter_shade(const ProcessParams& p, const BinRect* rect, un
   a.rect = rect; a.bin_off = p.bin_off; a.cursor = cursor; a.bin_tris = bin_tris; a.capacity = capacity; a.st = p.st;
   a.clip_cap = clip_cap;
   a.heavy = heavy_cap ? heavy : nullptr; a.heavy_cap = heavy_cap; a.heavy_epoch = heavy_epoch;
-  a.scatter_blocks = (int)(need < 6LL * num_sms ? need : 6LL * num_sms);
+  a.marks = marks;
+  // two CTAs of scattering warps per SM: a warp looks at 32 batches with one load
+  a.scatter_blocks = (int)(need < 2LL * num_sms ? need : 2LL * num_sms);
   const long long warps = (long long)((p.g.W + SHADE_W - 1) / SHADE_W) * ((p.g.H + SHADE_H - 1) / SHADE_H);
   const bool clip = p.clip_tris != nullptr;
   const auto kernel = p.invw ? (clip ? k_scatter_shade<true, true> : k_scatter_shade<true, false>)

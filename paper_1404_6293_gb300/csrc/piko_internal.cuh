@@ -365,6 +365,8 @@ struct DirectRaster {
   unsigned long long* keys = nullptr;  // W * H keys, KEY_EMPTY before the pass (NULL: every triangle is binned)
   int max_px = 0;                      // largest box taken, in pixels
   const unsigned* clip_orig = nullptr; // triangle of each clipped sub-triangle
+  unsigned char* marks = nullptr;      // a byte per 32 triangles: 1 where some of them got bin entries, 0 where none
+                                       // did (their rectangles are then not written)
   unsigned* busy = nullptr;            // nbins words: the scan lists the bins with entries there
 };
 
@@ -434,7 +436,8 @@ cudaError_t launch_process(const ProcessParams& p, int threads, int grid, cudaSt
 // shading of the tiles without bin entries, in one launch.
 cudaError_t launch_scatter_shade(const ProcessParams& p, const BinRect* rect, unsigned* cursor, unsigned* bin_tris,
                                  unsigned long long capacity, int num_sms, cudaStream_t s, unsigned clip_cap,
-                                 const uint2* heavy, unsigned heavy_cap, unsigned heavy_epoch);
+                                 const uint2* heavy, unsigned heavy_cap, unsigned heavy_epoch,
+                                 const unsigned char* marks);
 cudaError_t process_occupancy(const ProcessParams& p, int threads, int* blocks_per_sm);
 
 // Boxes (pixels of a triangle's bounding box inside a tile) up to this size
