@@ -33,9 +33,16 @@ __device__ __forceinline__ void clear_keys(unsigned long long* keys, size_t n) {
   if ((n & 1) && first == 0) keys[n - 1] = KEY_EMPTY;
 }
 
-// A scene whose triangles are small on average: fewer than 16 pixels of the
-// framebuffer for each.
-inline bool direct_scene(long long T, long long V, int W, int H) { return V > 0 && 16 * T >= (long long)W * H; }
+// Scenes worth it: triangles small on average, fewer than 16 pixels of the
+// framebuffer for each in a mesh, whose triangles share vertices and are of
+// similar size, and fewer than 4 in a soup of separate triangles, where large
+// ones among them leave every tile with both kinds to merge and a pixel's
+// vertices are shared with none of its neighbours'.  (Terrain at 7 pixels a
+// triangle: 41 us with the line at 16, 49 at 4; a power-law soup at 4.1 pixels
+// a triangle: 265 and 250 us.)
+inline bool direct_scene(long long T, long long V, int W, int H) {
+  return V > 0 && (V < 2 * T ? 16 : 4) * T >= (long long)W * H;
+}
 
 // A triangle of at most 128 pixels a side (its snapped extents below 2^15, so
 // that areas and edge functions are exact in 32 bits) whose box, clipped to

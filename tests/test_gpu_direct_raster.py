@@ -80,7 +80,7 @@ _LIMITS = [(32, 1), (33, 1), (1, 32), (1, 33), (8, 4), (4, 8), (16, 2), (11, 3),
 @pytest.mark.parametrize("size", [(131, 137), (150, 70)])
 def test_boxes_at_the_limits(bins, size):
     W, H = size
-    copies = -(-W * H // (16 * len(_LIMITS))) + 1  # enough triangles for the direct route
+    copies = -(-W * H // (4 * len(_LIMITS))) + 1  # enough triangles for the direct route
     _check(_triangles(W, H, _LIMITS, 7 * bins + W, copies), bins, "dynamic").close()
 
 
@@ -148,7 +148,7 @@ def test_batch_of_all_routes(check):
     from paper_1404_6293_gb300 import _lib as L
     from paper_1404_6293_gb300.raster import DeviceScene, Rasterizer
     scenes = [S.heightfield(100, 75, 60, 50, seed=1, with_color=True), S.random_triangles(90, 60, 40, 30.0, seed=2),
-              S.random_triangles(33, 200, 2000, 4.0, seed=3), _triangles(131, 137, _LIMITS, 4, 70),
+              S.random_triangles(33, 200, 2000, 4.0, seed=3), _triangles(131, 137, _LIMITS, 4, 230),
               S.power_law_triangles(120, 90, 2000, seed=5)]
     r = Rasterizer(100, 75, 16, 16, "static")
     ds = [DeviceScene.from_host(s) for s in scenes]
