@@ -497,6 +497,21 @@ def size_and_count(r, ds, fb):
     return stats, int((fb.key != -1).sum().item())
 
 
+def small_triangle_frame(scene) -> bool:
+    """Whether the library rasterizes the scene's small triangles in the count
+    pass and shades tiles without bin entries in the scatter launch
+    (direct_scene in csrc/piko_direct.cuh)."""
+    V, T = scene.num_vertices, scene.num_triangles
+    return V > 0 and (16 if V < 2 * T else 4) * T >= scene.width * scene.height
+
+
+def process_stage_ms(scene, stage_ms) -> float:
+    """Time of the stages that share the Process stage's work: Process alone,
+    or with the count and scatter launches in a frame of small triangles."""
+    mean = stage_ms.mean(axis=0)
+    return float(mean[1] + mean[3] + mean[4]) if small_triangle_frame(scene) else float(mean[4])
+
+
 def process_roofline(ctx, scene, stats, proc_ms, clk, traffic=None) -> dict:
     """Roofline of the Process kernel: algorithmic bytes (4 B per bin entry,
     12 B of indices per binned triangle, 16 B per snapped vertex, 12 B per
@@ -520,7 +535,8 @@ def process_roofline(ctx, scene, stats, proc_ms, clk, traffic=None) -> dict:
         achieved = bytes_proc / (proc_ms * 1e-3) / 1e9
         roof = {"bound": "hbm", "achieved": achieved, "peak": ctx.hbm, "unit": "GB/s", "frac": achieved / ctx.hbm,
                 "traffic": traffic, "peak_note": "of measured (MEASURED_PEAKS.json hbm_gbs)"}
-    roof.update({"kernel": "k_process", "kernel_ms": proc_ms, "algorithmic_bytes": bytes_proc,
+    roof.update({"kernel": "k_setup_count + k_scatter_shade + k_process" if small_triangle_frame(scene) else "k_process",
+                 "kernel_ms": proc_ms, "algorithmic_bytes": bytes_proc,
                  "algorithmic_ops": ops_proc, "t_hbm_us": t_hbm * 1e6, "t_alu_us": t_alu * 1e6,
                  "sm_mhz_used": ctx.f_mhz(clk),
                  "frac_at_2070mhz": max(t_hbm, ops_proc / (ctx.n_sm * 128 * 2070e6)) / (proc_ms * 1e-3)})
@@ -636,7 +652,7 @@ def run_ours(args):
     ms = max_over_ranks(float(np.sum(step_ms) / K), dist, "cuda")
     value = job_throughput(T, world, ms)
     shaded_gfrag = job_throughput(covered, world, ms, 1e9)
-    proc_ms = float(stage_ms[:, 4].mean())
+    proc_ms = process_stage_ms(scene, stage_ms)
     roof = process_roofline(ctx, scene, stats, proc_ms, clk, headline_traffic(args))
     roof["forward_frac"] = max(roof["t_hbm_us"], roof["t_alu_us"]) * 1e-3 / ms
 
@@ -843,7 +859,7 @@ def measure_random256(args, ctx) -> dict:
     if r.status()[0] != 0:
         raise RuntimeError("status error in the 256x256 loop")
     ms = sum(step_ms) / K
-    proc_ms = float(stage_ms[:, 4].mean())
+    proc_ms = process_stage_ms(scene, stage_ms)
     rec = {"workload": "random triangles 256x256, 1,000 triangles of 40-px radius, Gouraud, 16x16 bins, static",
            "value": scene.num_triangles / (ms * 1e-3) / 1e6, "unit": UNIT, "ms_per_step": ms,
            "shaded_gfrag_s": covered / (ms * 1e-3) / 1e9,
@@ -892,7 +908,7 @@ def measure_reyes(args, ctx) -> dict:
         runs[(bins, sched)] = (sum(step_ms) / K, stage_ms, stats, covered, clk)
         r.close()
     ms, stage_ms, stats, covered, clk = runs[(32, "dynamic")]
-    proc_ms = float(stage_ms[:, 4].mean())
+    proc_ms = process_stage_ms(scene, stage_ms)
     rec = {"workload": f"Reyes Sample: {scene.num_triangles} micropolygon triangles (256 bicubic patches diced to "
                        "~0.5-px quads), 1024x768, Lambert, 32x32 bins, dynamic",
            "value": scene.num_triangles / (ms * 1e-3) / 1e6, "unit": UNIT, "ms_per_step": ms,
@@ -1086,12 +1102,12 @@ def measure_sphere(args, ctx) -> dict:
                   "backward_batch (16x16 bins, dynamic), each replayed from its own CUDA graph",
            "forward_ms": float(fwd.mean()), "loss_gradient_ms": float(lossg.mean()),
            "backward_ms": float(bwd.mean()), "covered_pixels": covered,
-           "roofline": {"kernel": "k_batch_backward (64 views, with the gradient arrays' zeroing)", "bound": "hbm",
+           "roofline": {"kernel": "k_batch_backward_pixel (64 views, with the gradient arrays' zeroing)", "bound": "hbm",
                         "achieved": bw_bytes / bt / 1e9, "peak": ctx.hbm, "unit": "GB/s",
                         "frac": bw_bytes / bt / 1e9 / ctx.hbm, "traffic": None,
                         "bytes": "24 B per pixel (key, dL/dRGBA) + 40 B per vertex read + 24 B per vertex per view "
                                  "of gradient updates"},
-           "clocks": clk, "gpu_launches": 2 * K,
+           "clocks": clk, "gpu_launches": 8 * K,  # five forward phases; attributes, pixels and finish of the backward
            "parity": "keys bit-exact, colour <= 1e-5, gradients <= 1e-4 rel vs the oracle on every view "
                      "(tests/test_gpu_full_size.py)"}
     if not args.no_cpu_baseline:
@@ -1180,7 +1196,7 @@ def measure_batch(args, ctx) -> dict:
         for i in range(n):
             handles[(host[i].width, host[i].height)].backward(ds[i], fbs_p[i], gviews[i], dcv_p[i], dnv_p[i], dlv_p[i])
 
-    # ---- batched: autotuned knobs, one persistent launch per pass, graph-captured
+    # ---- batched: autotuned knobs, a launch per phase, graph-captured
     t0 = time.perf_counter()
     if args.batch_bins:
         bins, scheds = [(args.batch_bins, args.batch_bins)] * n, [args.batch_schedule] * n
@@ -1267,8 +1283,7 @@ def measure_batch(args, ctx) -> dict:
                      "how": "per-scene piko_raster_forward then piko_raster_backward, 16x16 static"},
            "batched": {"value": T / (ms_batch * 1e-3) / 1e6, "ms_per_step": ms_batch,
                        "forward_ms": f_ms, "loss_gradient_ms": l_ms, "backward_ms": b_ms,
-                       "how": ("forward_batch (one persistent cooperative launch)" if args.batch_launch ==
-                               "persistent" else "forward_batch (one launch per phase)") + ", the loss gradient "
+                       "how": "forward_batch (one launch per phase), the loss gradient "
                               "(one elementwise torch op) and backward_batch (with the gradient arrays' zeroing), "
                               "each replayed from its own CUDA graph",
                        "autotune_s": tune_s, "static_scenes": n_static,
@@ -1279,7 +1294,7 @@ def measure_batch(args, ctx) -> dict:
                                     "uniform_forward_ms": {f"{u['bin'][0]}x{u['bin'][1]} {u['schedule']}": u["ms"]
                                                            for u in tune_report["uniform"]}}},
            "speedup_batched_over_plain": ms_plain / ms_batch,
-           "roofline": {"kernel": "k_batch_backward (with the gradient arrays' zeroing)", "bound": "hbm",
+           "roofline": {"kernel": "k_batch_backward_pixel (with the gradient arrays' zeroing)", "bound": "hbm",
                         "achieved": bw_bytes / (b_ms * 1e-3) / 1e9, "peak": ctx.hbm, "unit": "GB/s",
                         "frac": bw_bytes / (b_ms * 1e-3) / 1e9 / ctx.hbm, "traffic": None,
                         "algorithmic_bytes": bw_bytes},
@@ -1287,8 +1302,8 @@ def measure_batch(args, ctx) -> dict:
                       "grad_scale": gscale,
                       "oracle": "every scene's keys bit-exact and colour <= 1e-5 vs the oracle "
                                 "(tests/test_gpu_full_size.py)"},
-           "clocks": clk, "gpu_launches": (2 if args.batch_launch == "persistent" else 6) * args.steps,
-           "gpu_launches_plain": sum(forward_launches(s.width, s.height, 16, 16) + 2 for s in host) * args.steps}
+           "clocks": clk, "gpu_launches": 8 * args.steps,
+           "gpu_launches_plain": sum(forward_launches(s.width, s.height, 16, 16) + 3 for s in host) * args.steps}
     if not args.no_cpu_baseline:
         import oracle
         hc = host_cpu()
@@ -1365,7 +1380,7 @@ def main():
                     "instead of the autotuner's choice (0: autotune)")
     ap.add_argument("--batch-schedule", default="dynamic", choices=["static", "dynamic"])
     ap.add_argument("--batch-launch", default="persistent", choices=["persistent", "per-phase"],
-                    help="batch workload: one cooperative launch, or one launch per phase (for launch lists)")
+                    help="batch workload: the library's choice, or always one launch per phase (now the same)")
     ap.add_argument("--workload", default="heightfield",
                     choices=["heightfield", "random256", "deferred", "sphere", "batch", "reyes"],
                     help="heightfield: the headline line (with every other configuration under 'configs'); "

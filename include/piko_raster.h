@@ -88,14 +88,18 @@ extern "C" {
                                        fewer bins than twice the GPU's SMs                  */
 #define PIKO_OPT_UNCLAMPED 2        /* 1: Lambert without the max(0, .) clamp,
                                        rgb = albedo * (n . L); default 0 (clamped)         */
-#define PIKO_OPT_CHECK_CAPACITY 3   /* 1 (default): forward reads the bin-list size back
-                                       after the scan (one host sync) and grows scratch
-                                       before scattering; 0: no sync, overflow is reported
-                                       as PIKO_ERR_OVERFLOW by piko_raster_status          */
+#define PIKO_OPT_CHECK_CAPACITY 3   /* 1 (default): forward launches the whole frame, then
+                                       waits until the scan has reported the bin-list size
+                                       (the later kernels still run) and, if the lists were
+                                       too small, grows them and repeats the frame; 0: no
+                                       wait, overflow is reported as PIKO_ERR_OVERFLOW by
+                                       piko_raster_status                                  */
 #define PIKO_OPT_SCHEDULE 4         /* change the schedule (PIKO_SCHED_*)                   */
 #define PIKO_OPT_SMALL_TRI_PIXELS 5 /* triangles whose box inside a tile has at most this
                                        many pixels are rasterized by one thread; larger ones
-                                       by a whole warp (default 32)                         */
+                                       are shared out over a warp (default 32).  In frames of
+                                       small triangles those whose whole box is that small
+                                       (32 at most) never reach a tile; 0: all do            */
 #define PIKO_OPT_STATS 6            /* 1: the Process stage also counts its work (see
                                        piko_raster_stats); default 0                        */
 #define PIKO_OPT_BATCH_LAUNCH 7     /* how piko_raster_forward_batch launches its phases:
@@ -253,12 +257,10 @@ int piko_raster_deferred_light(piko_raster *h, const piko_framebuffer *gbuf, con
 
 /* Many scenes in one pass (scenes with uneven triangle counts and
  * resolutions, or many views of one mesh): vertex stage, setup and counts,
- * scan, scatter and Process for all n scenes run as one persistent
- * cooperative launch whose CTAs meet at grid barriers between the phases
- * (PIKO_OPT_BATCH_LAUNCH = 1: one launch per phase instead).  The paper's
- * runtime is multi-kernel (Sec. 5, Sec. 6) and names a persistent kernel as
- * the alternative; scenes, bins and tiles of all scenes share one index
- * space here.
+ * scan, scatter and Process for all n scenes run as one launch each.  The
+ * paper's runtime is multi-kernel (Sec. 5, Sec. 6) and names a persistent
+ * kernel as the alternative; scenes, bins and tiles of all scenes share one
+ * index space here.
  *  scenes, fbs  host arrays of n descriptors (their pointers are device
  *               memory); each scene has its own width and height
  *               (1..32767) and shading mode, and writes its own framebuffer.
@@ -269,9 +271,7 @@ int piko_raster_deferred_light(piko_raster *h, const piko_framebuffer *gbuf, con
  *               (taken from a shared queue after the static tiles; HARDWARE
  *               is treated as DYNAMIC), or NULL for the handle's schedule.
  * Keys are bit-identical to n piko_raster_forward calls with the same bin
- * sizes; colours agree with them within float32 rounding (a winner is
- * shaded from its tile's shared-memory record or, past the records a tile
- * holds, from global memory).  With PIKO_OPT_CHECK_CAPACITY = 1 the call waits for the
+ * sizes; colours agree with them within float32 rounding.  With PIKO_OPT_CHECK_CAPACITY = 1 the call waits for the
  * launch, and relaunches once with larger bin lists if they overflowed; with
  * 0 it never waits (so it can be captured in a CUDA graph after a first call
  * with the same scenes, or piko_raster_reserve, has sized the scratch) and
@@ -283,7 +283,7 @@ int piko_raster_forward_batch(piko_raster *h, const piko_scene *scenes, int n, p
                               const int32_t *bin_sizes, const int32_t *schedules, void *cuda_stream);
 
 /* Gradients for all scenes of the last piko_raster_forward_batch on this
- * handle (same scenes, same order), in one launch: dl_drgba, dl_dcolor,
+ * handle (same scenes, same order): dl_drgba, dl_dcolor,
  * dl_dnormal and dl_dlight are host arrays of n device pointers (entries
  * may be NULL to skip that output for a scene); semantics per scene as in
  * piko_raster_backward (accumulated, visibility fixed by fbs[i].key). */

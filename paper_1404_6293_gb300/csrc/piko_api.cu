@@ -27,8 +27,13 @@ int piko_backward_launch(int W, int H, int mode, int unclamped, int T, int V, co
                          const float* vdot, const float4* vattr, const float* color, const float* normal,
                          const float* light,
                          const float* invw, const float* pos, const float* mvp, const unsigned long long* key,
-                         const float* dl_drgba, float4* acc, float* dcolor, float* dnormal, float* dlight, int set,
-                         int num_sms, cudaStream_t s);
+                         const float* dl_drgba, float4* acc, long long acc_room, float* dcolor, float* dnormal,
+                         float* dlight, int set, int num_sms, cudaStream_t s);
+
+// Gradient accumulators of a handle beyond one per vertex: copies for scenes of
+// few vertices and many pixels, three at most (1 MB at most).  Not more, as an
+// allocation past a megabyte costs a first frame 75 us more than one below.
+inline long long gacc_extra(long long vertices) { return 3 * vertices < 65536 ? 3 * vertices : 65536; }
 
 struct piko_raster {
   int W, H, bin_w, bin_h, schedule;
@@ -55,7 +60,7 @@ struct piko_raster {
   long long vcap = 0;
   int4* vtx = nullptr;      // snapped position
   float4* vattr = nullptr;  // colour and n . L, for Lambert with colours
-  float4* gacc = nullptr;   // gradient sums, zero between calls
+  float4* gacc = nullptr;   // gradient sums, zero between calls; gacc_extra(vcap) more of them for copies
   float* vdot = nullptr;    // n . L, for Lambert without colours
   float* invw = nullptr;    // 1 / clip w, with perspective-correct attributes
   bool gacc_dirty = false;  // gacc is not zero: new, or a backward launch failed
@@ -155,19 +160,26 @@ int grow_vertices(piko_raster* h, long long need) {
   long long cap = 0;
   h->vcap = 0;
   const long long per_vertex = sizeof(int4) + 2 * sizeof(float4) + 2 * sizeof(float);
+  // a quarter more than needed, so that slowly growing scenes do not allocate each time
+  cap = (need + need / 4 + 255) / 256 * 256;
   long long bytes = 0;
   h->vertex_block = nullptr;
-  const int r = grow(h, &block, &bytes, need * per_vertex, "vertex buffer");
-  if (r != PIKO_OK) {
-    h->vertex_block = block;
-    return r;
+  if (block) {
+    const cudaError_t e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) return cuda_fail(h, e, "cudaDeviceSynchronize");
+    cudaFree(block);
+    block = nullptr;
   }
-  cap = bytes / per_vertex / 4 * 4;
+  bytes = cap * per_vertex + gacc_extra(cap) * (long long)sizeof(float4);
+  if (cudaMalloc(reinterpret_cast<void**>(&block), (size_t)bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(h, PIKO_ERR_OOM, "cudaMalloc of vertex buffer failed");
+  }
   h->vertex_block = block;
   h->vtx = reinterpret_cast<int4*>(block);
   h->vattr = reinterpret_cast<float4*>(h->vtx + cap);
   h->gacc = h->vattr + cap;
-  h->vdot = reinterpret_cast<float*>(h->gacc + cap);
+  h->vdot = reinterpret_cast<float*>(h->gacc + cap + gacc_extra(cap));
   h->invw = h->vdot + cap;
   h->gacc_dirty = true;
   h->vcap = cap;
@@ -625,7 +637,7 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
   const int V = s->num_vertices, T = s->num_triangles;
   if ((r = grow_vertices(h, V)) != PIKO_OK) return r;
   const bool lambert = s->shade_mode == PIKO_SHADE_LAMBERT;
-  if ((r = grow_triangles(h, T)) != PIKO_OK) return r;
+  if (!h->clip && (r = grow_triangles(h, T)) != PIKO_OK) return r;  // (with clipping: once its list is sized, below)
   if (h->ecap == 0 && (r = grow(h, &h->bin_tris, &h->ecap, (long long)T * 2 + 4096, "bin lists")) != PIKO_OK)
     return r;
 
@@ -656,7 +668,7 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
     const int4* clip_tris = h->clip ? h->clip_tris : nullptr;
     const long long ccap = h->ccap_tris / 3 < h->ccap_orig ? h->ccap_tris / 3 : h->ccap_orig;
     const unsigned clip_cap = h->clip ? (unsigned)ccap : 0u;
-    if (clip_cap && (r = grow_triangles(h, (long long)T + clip_cap)) != PIKO_OK) return r;
+    if (h->clip && (r = grow_triangles(h, (long long)T + clip_cap)) != PIKO_OK) return r;
     direct.clip_orig = h->clip ? h->clip_orig : nullptr;
     direct.marks = h->marks;
     // a frame of one scan chunk of bins is scanned by the count pass's last
@@ -899,7 +911,7 @@ static int backward_pass(piko_raster* h, const piko_scene* s, const piko_framebu
     if (e != cudaSuccess) return cuda_fail(h, e, "gradient clear");
   }
   if (h->gacc_dirty) {
-    const cudaError_t e = cudaMemsetAsync(h->gacc, 0, (size_t)h->vcap * sizeof(float4), st);
+    const cudaError_t e = cudaMemsetAsync(h->gacc, 0, (size_t)(h->vcap + gacc_extra(h->vcap)) * sizeof(float4), st);
     if (e != cudaSuccess) return cuda_fail(h, e, "gradient sums");
     // a captured clear has not run
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -913,8 +925,8 @@ static int backward_pass(piko_raster* h, const piko_scene* s, const piko_framebu
                 set && lambert ? dl_dlight : nullptr);
   if (piko_backward_launch(h->W, h->H, s->shade_mode, h->unclamped, s->num_triangles, s->num_vertices, s->tris,
                            h->vtx, h->vdot, vattr, s->color, s->normal, s->light_dir, invw, h->clip ? s->pos : nullptr,
-                           s->mvp, reinterpret_cast<const unsigned long long*>(fwd->key), dl_drgba, h->gacc, dl_dcolor,
-                           dl_dnormal, dl_dlight, set ? 1 : 0, h->num_sms, st) != 0) {
+                           s->mvp, reinterpret_cast<const unsigned long long*>(fwd->key), dl_drgba, h->gacc,
+                           h->vcap + gacc_extra(h->vcap), dl_dcolor, dl_dnormal, dl_dlight, set ? 1 : 0, h->num_sms, st) != 0) {
     h->gacc_dirty = true;
     return cuda_fail(h, cudaGetLastError(), "backward launch");
   }

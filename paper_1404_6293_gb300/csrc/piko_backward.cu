@@ -19,7 +19,8 @@ __global__ void __launch_bounds__(PIX_THREADS, 5) k_backward_pixel(const __grid_
   const int tile = blockIdx.x * (PIX_THREADS / 32) + warp;
   if (tile >= p.ntiles) return;  // the same for the whole warp
   const int ty = tile / p.ntx, tx = tile - ty * p.ntx;
-  backward_warp_pixels<PERSP>(p.sc, p.vdot, p.vattr, tx * PIX_W + (lane & (PIX_W - 1)), ty * PIX_H + lane / PIX_W);
+  backward_warp_pixels<PERSP>(p.sc, p.vdot, p.vattr, tx * PIX_W + (lane & (PIX_W - 1)), ty * PIX_H + lane / PIX_W,
+                              tx + ty);
 }
 
 // Sums of all vertices into the gradient arrays (grad_finish_chunk).
@@ -34,7 +35,7 @@ __global__ void __launch_bounds__(GRAD_CHUNK) k_backward_finish(const __grid_con
 
 using namespace piko;
 
-// acc: V accumulators, zero before and after the call; vdot: n . L per vertex
+// acc: acc_room >= V accumulators, zero before and after the call; vdot: n . L per vertex
 // of the vertex stage launched just before (Lambert), vattr (or NULL): colour
 // and n . L in its place.  set: the gradients are stored (a dlight that is
 // wanted being zero already); needs V > 0, T > 0 and a gradient to write.
@@ -42,11 +43,12 @@ int piko_backward_launch(int W, int H, int mode, int unclamped, int T, int V, co
                          const float* vdot, const float4* vattr, const float* color, const float* normal,
                          const float* light,
                          const float* invw, const float* pos, const float* mvp, const unsigned long long* key,
-                         const float* dl_drgba, float4* acc, float* dcolor, float* dnormal, float* dlight, int set,
-                         int num_sms, cudaStream_t s) {
+                         const float* dl_drgba, float4* acc, long long acc_room, float* dcolor, float* dnormal,
+                         float* dlight, int set, int num_sms, cudaStream_t s) {
   const bool lambert = mode == PIKO_SHADE_LAMBERT;
   GradAcc f;
   f.V = V; f.acc = acc; f.set = set;
+  f.copies = grad_copies((long long)W * H, V, acc_room);
   f.normal = lambert ? normal : nullptr;
   f.light = light;
   f.color = nullptr;
@@ -61,7 +63,7 @@ int piko_backward_launch(int W, int H, int mode, int unclamped, int T, int V, co
   c.tris = tris; c.vtx = vtx; c.color = color; c.normal = normal; c.light = light; c.invw = invw;
   c.pos = reinterpret_cast<const float4*>(pos); c.mvp = mvp;
   c.key = key; c.dl = reinterpret_cast<const float4*>(dl_drgba);
-  c.acc = acc;
+  c.acc = acc; c.copies = f.copies;
   p.vdot = vdot;
   p.vattr = vattr;
   p.ntx = (W + PIX_W - 1) / PIX_W;

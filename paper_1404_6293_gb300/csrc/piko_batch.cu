@@ -42,6 +42,7 @@ struct BatchScene {
   // backward
   const float4* dl;
   float4* acc;  // the gradient sums of the scene's vertices (NULL: no gradients wanted)
+  int copies;   // of acc, V apart
   const float4* attr;  // colour and n . L of the vertices for the backward (Lambert)
 };
 
@@ -555,7 +556,7 @@ __device__ __forceinline__ void fill_bwd_scene(const BatchBwdParams& b, const Ba
   c.invw = b.invw ? b.invw + d.vtx_base : nullptr;
   c.pos = nullptr;  // batches do not clip
   c.mvp = nullptr;
-  c.key = d.key_out; c.dl = d.dl; c.acc = d.acc;
+  c.key = d.key_out; c.dl = d.dl; c.acc = d.acc; c.copies = d.copies;
 }
 
 // Colour and n . L of the vertices of each group of Lambert scenes: the
@@ -604,7 +605,8 @@ __global__ void __launch_bounds__(PIX_THREADS, 4) k_batch_backward_pixel(BatchBw
     const int lt = i - __ldg(b.pblock_prefix + s);
     const int ntx = (c.W + PIX_W - 1) / PIX_W;
     const int ty = lt / ntx, tx = lt - ty * ntx;
-    backward_warp_pixels<PERSP>(c, nullptr, d.attr, tx * PIX_W + (lane & (PIX_W - 1)), ty * PIX_H + lane / PIX_W);
+    backward_warp_pixels<PERSP>(c, nullptr, d.attr, tx * PIX_W + (lane & (PIX_W - 1)), ty * PIX_H + lane / PIX_W,
+                                tx + ty);
   }
 }
 
@@ -638,6 +640,10 @@ int ilog2i(int v) {
 }
 
 }  // namespace
+
+// Gradient accumulators beyond one per vertex (16 MB): copies for scenes of few
+// vertices and many pixels (grad_copies).
+constexpr long long BATCH_GACC_EXTRA = 1 << 20;
 
 // Everything the batch keeps between calls; owned by the handle.
 struct BatchState {
@@ -678,6 +684,7 @@ struct BatchState {
   std::vector<BatchScene> host_desc;  // the uploaded descriptors
   size_t smem = 0;
   int grid = 0;
+  size_t grid_smem = 0;  // the shared memory that grid was sized for
   int num_sms = 0;
   int n = 0;
   int persp = 0;               // the layout's attribute interpolation (perspective-correct or not)
@@ -805,8 +812,8 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   if ((r = grow_dev(&bs->rect, &bs->tcap, tt, false, err)) != PIKO_OK) return r;
   if ((r = grow_dev(&bs->marks, &bs->mcap, (tt + 31) / 32, false, err)) != PIKO_OK) return r;
   // here and not in the backward call, which may be recorded into a graph
-  if (tv > bs->gcap) bs->gacc_dirty = true;
-  if ((r = grow_dev(&bs->gacc, &bs->gcap, tv, false, err)) != PIKO_OK) return r;
+  if (tv + BATCH_GACC_EXTRA > bs->gcap) bs->gacc_dirty = true;
+  if ((r = grow_dev(&bs->gacc, &bs->gcap, tv + BATCH_GACC_EXTRA, false, err)) != PIKO_OK) return r;
   if (tb > bs->bcap) {
     // counts must start at zero; offsets/cursors/chunk states are rewritten
     cudaFree(bs->cnt); cudaFree(bs->bin_off); cudaFree(bs->cursor); cudaFree(bs->chunk_state);
@@ -904,14 +911,19 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
     err = "batch shared memory request refused";
     return PIKO_ERR_CUDA;
   }
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kf, BATCH_THREADS, bs->smem) != cudaSuccess ||
-      per_sm < 1) {
-    cudaGetLastError();
-    err = "batch kernel does not fit on an SM";
-    return PIKO_ERR_CUDA;
+  // (the two kernels share their register cap; the query is repeated only for another layout)
+  if (bs->grid == 0 || bs->grid_smem != bs->smem || bs->persp != (persp ? 1 : 0)) {
+    int per_sm = 0, per_sm_p = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kf, BATCH_THREADS, bs->smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_p, kp, BATCH_THREADS, bs->smem) != cudaSuccess ||
+        per_sm < 1 || per_sm_p < 1) {
+      cudaGetLastError();
+      err = "batch kernel does not fit on an SM";
+      return PIKO_ERR_CUDA;
+    }
+    bs->grid = (per_sm < per_sm_p ? per_sm : per_sm_p) * num_sms;
+    bs->grid_smem = bs->smem;
   }
-  bs->grid = per_sm * num_sms;
   bs->num_sms = num_sms;
   bs->desc_bytes = total;
   bs->group_off = group_off;
@@ -934,7 +946,8 @@ int batch_launch_forward(BatchState* bs, DevStatus* st, bool persistent, cudaStr
   b.capacity = (unsigned long long)bs->ecap;
   b.bin_tris = bs->bin_tris;
   b.epoch = ++bs->epoch;
-  if (cudaMemsetAsync(bs->sync, 0, sizeof(BatchSync), stream) != cudaSuccess) {
+  // (the separate launches use only its queue head, which the scan resets)
+  if (persistent && cudaMemsetAsync(bs->sync, 0, sizeof(BatchSync), stream) != cudaSuccess) {
     err = "batch barrier reset failed";
     return PIKO_ERR_CUDA;
   }
@@ -1001,7 +1014,7 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
   std::vector<BatchScene> d = bs->host_desc;
   std::vector<GradAcc> groups;
   std::vector<int> chunk_prefix(1, 0);
-  long long acc_used = 0;
+  std::vector<long long> group_px;
   for (int i = 0; i < n; ++i) {
     if (scenes[i].num_triangles != d[i].T || scenes[i].num_vertices != d[i].V ||
         reinterpret_cast<unsigned long long*>(fbs[i].key) != d[i].key_out) {
@@ -1028,24 +1041,43 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
     g.dnormal = dn && lambert ? dn[i] : nullptr;
     g.dlight = dlt && lambert ? dlt[i] : nullptr;
     d[i].acc = nullptr;
+    d[i].copies = 0;
     d[i].attr = nullptr;
     if (!d[i].dl || d[i].mode == PIKO_SHADE_GBUFFER || g.V == 0 || (!g.dcolor && !g.dnormal && !g.dlight)) continue;
     if (!groups.empty()) {
       const GradAcc& q = groups.back();
       if (q.V == g.V && q.normal == g.normal && q.light == g.light && q.color == g.color && q.dcolor == g.dcolor &&
           q.dnormal == g.dnormal && q.dlight == g.dlight) {
-        d[i].acc = q.acc;
         d[i].attr = q.attr;
+        d[i].copies = (int)groups.size();  // (the group, until its accumulators are dealt below)
+        group_px.back() += (long long)d[i].g.W * d[i].g.H;
         continue;
       }
     }
-    g.acc = d[i].acc = bs->gacc + acc_used;
     d[i].attr = g.attr;
-    acc_used += g.V;  // at most the batch's vertices
     groups.push_back(g);
+    d[i].copies = (int)groups.size();
+    group_px.push_back((long long)d[i].g.W * d[i].g.H);
     chunk_prefix.push_back(chunk_prefix.back() + (g.V + GRAD_CHUNK - 1) / GRAD_CHUNK);
   }
   if (groups.empty()) return PIKO_OK;  // nothing to add
+  // accumulators: one per vertex of each group (at most the batch's vertices),
+  // and copies from what is left
+  long long used = 0, spare = bs->gcap;
+  for (const GradAcc& g : groups) spare -= g.V;
+  for (size_t k = 0; k < groups.size(); ++k) {
+    GradAcc& g = groups[k];
+    g.copies = grad_copies(group_px[k], g.V, g.V + spare);
+    g.acc = bs->gacc + used;
+    used += (long long)g.copies * g.V;
+    spare -= (long long)(g.copies - 1) * g.V;
+  }
+  for (BatchScene& x : d) {
+    if (x.copies == 0) continue;
+    const GradAcc& g = groups[x.copies - 1];
+    x.acc = g.acc;
+    x.copies = g.copies;
+  }
   if (bs->gacc_dirty) {
     if (cudaMemsetAsync(bs->gacc, 0, (size_t)bs->gcap * sizeof(float4), stream) != cudaSuccess) {
       err = "gradient sums reset failed";

@@ -53,6 +53,7 @@ struct BwdScene {
   const unsigned long long* key;
   const float4* dl;
   float4* acc;  // per vertex: sums of g s b (colour) and of G b (zero between calls)
+  int copies;   // of acc, V apart
 };
 
 // ------------------------------------------------------------ accumulators
@@ -70,6 +71,7 @@ __device__ __forceinline__ void grad_add(float4* acc, float c0, float c1, float 
 // several scenes of a batch that share their attributes and gradient arrays.
 struct GradAcc {
   int V;
+  int copies;  // of the accumulators, V apart (grad_copies)
   float4* acc;
   const float* normal;  // Lambert (NULL for Gouraud: no normal or light gradients)
   const float* light;
@@ -80,6 +82,22 @@ struct GradAcc {
   float* dlight;
   int set;  // 1: dcolor and dnormal are stored, not added to (dlight is zero before the call)
 };
+
+// Copies of a group's accumulators: neighbouring blocks of pixels add to
+// different ones, and the finishing pass adds the copies up.  A vertex of
+// triangles of hundreds of pixels takes hundreds of sums one after the other
+// into one float; with several copies the rounding error falls with their
+// number, as does the queue at one address of the L2.  px: pixels of the
+// group's framebuffers; room: accumulators that may be used.
+constexpr int GRAD_MAX_COPIES = 8;
+// (A soup's vertices belong to one triangle each and take few sums: with copies
+// by the pixels per triangle a batch of 64 uneven scenes took 1684 us, by the
+// pixels per vertex, or without, 1624.)
+inline int grad_copies(long long px, long long V, long long room) {
+  int k = 1;
+  while (k < GRAD_MAX_COPIES && px >= 64 * k * V && 2 * k * V <= room) k *= 2;
+  return k;
+}
 
 constexpr int GRAD_CHUNK = 256;  // vertices per CTA step of the finishing pass, one per thread
 
@@ -95,9 +113,15 @@ struct GradFinishSmem {
 __device__ __forceinline__ void grad_finish_chunk(const GradAcc& f, int chunk, GradFinishSmem& sm) {
   const int tid = threadIdx.x, lane = tid & 31, base = chunk * GRAD_CHUNK, v = base + tid;
   float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (v < f.V) a = __ldcg(f.acc + v);
-  const bool hit = a.x != 0.f || a.y != 0.f || a.z != 0.f || a.w != 0.f;
-  if (hit) f.acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+  bool hit = false;
+  for (int k = 0; k < f.copies && v < f.V; ++k) {
+    float4* at = f.acc + (size_t)k * f.V + v;
+    const float4 c = __ldcg(at);
+    if (c.x == 0.f && c.y == 0.f && c.z == 0.f && c.w == 0.f) continue;
+    hit = true;
+    *at = make_float4(0.f, 0.f, 0.f, 0.f);
+    a.x += c.x; a.y += c.y; a.z += c.z; a.w += c.w;
+  }
   if (!__syncthreads_or(hit) && !f.set) return;  // (the barrier also ends the last chunk's reads of sm)
   sm.a[tid] = a;
   if (f.normal && f.dlight) {
@@ -138,10 +162,12 @@ constexpr int PIX_THREADS = 256;     // CTA size of the backward kernels: 8 warp
 constexpr int PIX_W = 16, PIX_H = 2;  // pixels of a warp
 
 // Pixel (x, y) of each lane (lane mod PIX_W along x).  vattr: colour and n . L
-// per vertex; without it vdot: n . L (Lambert).
+// per vertex; without it vdot: n . L (Lambert).  block: the warp's block of
+// pixels, which picks the copy of the accumulators.
 template <bool PERSP>
 __device__ __forceinline__ void backward_warp_pixels(const BwdScene& sc, const float* __restrict__ vdot,
-                                                     const float4* __restrict__ vattr, int x, int y) {
+                                                     const float4* __restrict__ vattr, int x, int y,
+                                                     int block) {
   const int lane = threadIdx.x & 31;
   // the key and dL/drgba do not come from the vertex stage before this kernel
   const size_t o = (size_t)y * sc.W + x;
@@ -257,9 +283,10 @@ __device__ __forceinline__ void backward_warp_pixels(const BwdScene& sc, const f
     }
   }
   if (hit && ((heads >> lane) & 1u)) {
-    grad_add(sc.acc + ia, v[0], v[3], v[6], v[9]);
-    grad_add(sc.acc + ib, v[1], v[4], v[7], v[10]);
-    grad_add(sc.acc + ic, v[2], v[5], v[8], v[11]);
+    float4* acc = sc.acc + (size_t)(block & (sc.copies - 1)) * sc.V;
+    grad_add(acc + ia, v[0], v[3], v[6], v[9]);
+    grad_add(acc + ib, v[1], v[4], v[7], v[10]);
+    grad_add(acc + ic, v[2], v[5], v[8], v[11]);
   }
 }
 

@@ -68,23 +68,19 @@ class DeviceScene:
         return int(self.tris.shape[0])
 
     def c_struct(self) -> L.PikoScene:
-        for name in ("pos", "tris", "color", "normal", "mvp", "light_dir"):
-            v = getattr(self, name)
-            if v is not None and (not v.is_cuda or not v.is_contiguous()):
+        # one pass over the tensors: a batch call builds a structure per scene
+        ptrs = []
+        for v in (self.pos, self.tris, self.color, self.normal, self.mvp, self.light_dir):
+            if v is None:
+                ptrs.append(None)
+                continue
+            if not (v.is_cuda and v.is_contiguous()):
+                name = ("pos", "tris", "color", "normal", "mvp", "light_dir")[len(ptrs)]
                 raise ValueError(f"{name} must be a contiguous CUDA tensor")
-        if self.pos.dtype != torch.float32 or self.tris.dtype != torch.int32:
+            ptrs.append(v.data_ptr())
+        if self.pos.dtype is not torch.float32 or self.tris.dtype is not torch.int32:
             raise TypeError("pos must be float32 and tris int32")
-        s = L.PikoScene()
-        s.width, s.height = self.width, self.height
-        s.num_vertices, s.num_triangles = self.num_vertices, self.num_triangles
-        s.pos, s.tris = self.pos.data_ptr(), self.tris.data_ptr()
-        s.color = None if self.color is None else self.color.data_ptr()
-        s.normal = None if self.normal is None else self.normal.data_ptr()
-        s.mvp = None if self.mvp is None else self.mvp.data_ptr()
-        s.light_dir = None if self.light_dir is None else self.light_dir.data_ptr()
-        s.shade_mode = self.shade_mode
-        s.reserved = 0
-        return s
+        return L.PikoScene(self.width, self.height, self.pos.shape[0], self.tris.shape[0], *ptrs, self.shade_mode, 0)
 
 
 @dataclass
@@ -153,12 +149,9 @@ class Framebuffer:
         return Framebuffer(key, torch.empty((height, width, 4), dtype=torch.float32, device=device) if rgba else None)
 
     def c_struct(self) -> L.PikoFramebuffer:
-        f = L.PikoFramebuffer()
-        f.key = self.key.data_ptr()
-        f.rgba = None if self.rgba is None else self.rgba.data_ptr()
-        f.gbuf_normal = None if self.gbuf_normal is None else self.gbuf_normal.data_ptr()
-        f.gbuf_albedo = None if self.gbuf_albedo is None else self.gbuf_albedo.data_ptr()
-        return f
+        return L.PikoFramebuffer(self.key.data_ptr(), None if self.rgba is None else self.rgba.data_ptr(),
+                                 None if self.gbuf_normal is None else self.gbuf_normal.data_ptr(),
+                                 None if self.gbuf_albedo is None else self.gbuf_albedo.data_ptr())
 
     def key_numpy(self) -> np.ndarray:
         return self.key.cpu().numpy().view(np.uint64)
