@@ -184,8 +184,9 @@ class Rasterizer:
 
     @staticmethod
     def _stream(stream) -> C.c_void_p:
-        s = torch.cuda.current_stream() if stream is None else stream
-        return C.c_void_p(s.cuda_stream)
+        if stream is None:  # the raw handle: torch.cuda.current_stream() builds an object for 4 us
+            return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+        return C.c_void_p(stream.cuda_stream)
 
     def close(self):
         if getattr(self, "_h", None):
