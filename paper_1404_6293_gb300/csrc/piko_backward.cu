@@ -60,7 +60,7 @@ int piko_backward_launch(int W, int H, int mode, int unclamped, int T, int V, co
   BackwardParams p;
   BwdScene& c = p.sc;
   c.W = W; c.H = H; c.mode = mode; c.unclamped = unclamped; c.T = T; c.V = V;
-  c.tris = tris; c.vtx = vtx; c.color = color; c.normal = normal; c.light = light; c.invw = invw;
+  c.tris = tris; c.vtx = vtx; c.color = color; c.invw = invw;
   c.pos = reinterpret_cast<const float4*>(pos); c.mvp = mvp;
   c.key = key; c.dl = reinterpret_cast<const float4*>(dl_drgba);
   c.acc = acc; c.copies = f.copies;

@@ -542,7 +542,6 @@ struct BatchBwdParams {
   const int* pblock_prefix;  // [n+1] 16 x 2 pixel blocks per scene
   int total_pblocks;
   const int4* vtx;
-  float4* vattr;      // colour and n . L per vertex, rewritten here for the first scene of each group
   const float* invw;  // as in BatchParams
   // accumulators (GradAcc) of the finishing pass and the prefix of their chunks
   int ngroups, total_chunks;
@@ -552,7 +551,7 @@ struct BatchBwdParams {
 
 __device__ __forceinline__ void fill_bwd_scene(const BatchBwdParams& b, const BatchScene& d, BwdScene& c) {
   c.W = d.g.W; c.H = d.g.H; c.mode = d.mode; c.unclamped = d.unclamped; c.T = d.T; c.V = d.V;
-  c.tris = d.tris; c.vtx = b.vtx + d.vtx_base; c.color = d.color; c.normal = d.normal; c.light = d.light;
+  c.tris = d.tris; c.vtx = b.vtx + d.vtx_base; c.color = d.color;
   c.invw = b.invw ? b.invw + d.vtx_base : nullptr;
   c.pos = nullptr;  // batches do not clip
   c.mvp = nullptr;
@@ -1107,7 +1106,6 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
   p.pblock_prefix = bs->params.pblock_prefix;
   p.total_pblocks = bs->params.total_pblocks;
   p.vtx = bs->vtx;
-  p.vattr = bs->vattr;
   p.invw = bs->params.invw;  // the interpolation of the last forward_batch
   p.ngroups = (int)groups.size();
   p.total_chunks = chunk_prefix.back();

@@ -45,8 +45,6 @@ struct BwdScene {
   const int* tris;
   const int4* vtx;
   const float* color;
-  const float* normal;
-  const float* light;
   const float* invw;  // 1 / clip w per vertex: perspective-correct attributes (NULL: screen-space)
   const float4* pos;  // near/far clipping: positions and matrix of clipped winners (NULL: off)
   const float* mvp;

@@ -174,7 +174,7 @@ def _close(a, b):
     assert np.abs(a - b).max() <= 1e-4 * max(np.abs(b).max(), 1e-30)
 
 
-@pytest.mark.parametrize("quads", [(60, 40), (6, 5)])  # pixel form, tile form
+@pytest.mark.parametrize("quads", [(60, 40), (6, 5)])  # tiny and large triangles
 @pytest.mark.parametrize("color", [True, False])
 def test_stored_gradients_equal_added_ones(quads, color):
     torch = _torch()
