@@ -174,7 +174,7 @@ __device__ void phase_vertex(const BatchParams& b) {
     } else {
       b.vtx[i] = snap_vertex(__ldg(d.pos + v), d.mvp, (float)d.g.W, (float)d.g.H);
     }
-    if (d.mode == PIKO_SHADE_LAMBERT) {
+    if (d.mode == PIKO_SHADE_LAMBERT && d.normal) {  // (without triangles there may be no normals)
       const float* n = d.normal + 3 * (size_t)v;
       const float* c = d.color + 3 * (size_t)v;
       float4 a = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -67,6 +67,9 @@ void launch_vertex(int W, int H, int V, const float* pos, const float* mvp, int4
                    unsigned long long* dkeys, DevStatus* clip_st, const float* color, float4* vattr,
                    float* zero3) {
   if (V <= 0) return;
+  // a Lambert scene without triangles may come without normals: it has no light
+  // terms, and nothing reads them
+  if (!normal) vdot = nullptr;
   // one vertex per thread: every load is in flight at once; at least a wave
   // of CTAs when there are keys to clear
   int blocks = (V + 255) / 256;

@@ -1,0 +1,86 @@
+"""Calls at the edges of what the entry points accept: scenes without
+triangles or normals, odd light counts, attribute arrays longer than the
+scene, scratch reserved ahead of a capture, and replayed graphs whose inputs
+change between replays."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_1404_6293_gb300 import scenes as S
+
+pytestmark = pytest.mark.gpu
+
+EMPTY = -1  # the all-ones key, as int64
+
+
+def _torch():
+    import torch
+    return torch
+
+
+def _bare_lambert(W, H, color):
+    """A Lambert scene of 300 vertices, no triangles and no normals."""
+    from paper_1404_6293_gb300.raster import DeviceScene
+    s = S.heightfield(W, H, 24, 11, seed=2, with_color=True)
+    ds = DeviceScene.from_host(s)
+    assert ds.num_vertices == 300 and ds.shade_mode == S.SHADE_LAMBERT
+    ds.tris = ds.tris[:0].contiguous()
+    ds.normal = None
+    if not color:
+        ds.color = None
+    return ds
+
+
+@pytest.mark.parametrize("color", [True, False])
+def test_lambert_scene_without_triangles_needs_no_normals(color):
+    """Every call that takes a scene: an empty frame, and no gradient."""
+    torch = _torch()
+    from paper_1404_6293_gb300 import _lib as L
+    from paper_1404_6293_gb300.raster import DeviceScene, Framebuffer, HostScene, Rasterizer
+    W, H = 64, 48
+    ds = _bare_lambert(W, H, color)
+    r = Rasterizer(W, H)
+
+    def check(fb, what):
+        torch.cuda.synchronize()
+        assert r.status()[0] == 0, what
+        assert bool((fb.key == EMPTY).all()) and not bool(fb.rgba.any()), what
+
+    for check_capacity in (1, 0):
+        r.set_option(L.PIKO_OPT_CHECK_CAPACITY, check_capacity)
+        check(r.forward(ds), "forward")
+    r.set_option(L.PIKO_OPT_CHECK_CAPACITY, 1)
+    full = S.heightfield(W, H, 30, 20, seed=3, with_color=True)
+    dfull = DeviceScene.from_host(full)
+    fbs = r.forward_batch([dfull, ds])
+    check(fbs[1], "batch")
+    assert np.array_equal(fbs[0].key_numpy(), oracle.raster_bbox(full)[0])
+
+    hs = HostScene.from_host(full)
+    hs.tris, hs.normal = hs.tris[:0].contiguous(), None
+    check(r.forward_host(hs), "host")
+
+    fb = Framebuffer.allocate(W, H, ds.shade_mode)
+    status = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    f = L.load().piko_raster_forward_noalloc
+    f.argtypes = [C.POINTER(L.PikoScene), C.POINTER(L.PikoFramebuffer), C.c_int, C.c_int, C.c_int, C.c_void_p,
+                  C.c_void_p]
+    f.restype = C.c_int
+    cs, cf = ds.c_struct(), fb.c_struct()
+    assert f(C.byref(cs), C.byref(cf), 16, 16, 0, C.c_void_p(status.data_ptr()),
+             C.c_void_p(torch.cuda.current_stream().cuda_stream)) == L.PIKO_OK
+    check(fb, "without allocation")
+    assert int(status.item()) == L.PIKO_OK
+
+    g = torch.ones((H, W, 4), device="cuda")
+    dc = torch.full((ds.num_vertices, 3), 2.0, device="cuda")
+    dl = torch.full((3,), 2.0, device="cuda")
+    r.backward(ds, fb, g, dc if color else None, None, dl)
+    gc, gn, gl = r.gradients(ds, fb, g, color=color, normal=False)
+    r.backward_batch([dfull, ds], fbs, [g, g], [None, dc if color else None], None, [None, dl])
+    torch.cuda.synchronize()
+    assert bool((dc == 2.0).all()) and bool((dl == 2.0).all())  # added to: nothing
+    assert gn is None and not bool(gl.any()) and (gc is None or not bool(gc.any()))
+    r.close()
