@@ -99,7 +99,9 @@ __device__ __forceinline__ float light_pairs(const LightPair* lights, int npairs
   return a0 + a1;
 }
 
-// The same sum for any lights, one by one.
+// The same sum for any lights, one by one (and for the last of an odd number:
+// half a pair padded with a light of intensity 0 would add 0 * inf = NaN where a
+// binary16 normal is infinite).
 __device__ __forceinline__ float light_singles(const float4* __restrict__ lights, int n_lights, float4 n, float sx,
                                                float sy, float sz, float inv_r2) {
   float acc = 0.f;
@@ -121,12 +123,11 @@ __global__ void __launch_bounds__(256) k_deferred_light(int W, int H, const unsi
                                                         float4* __restrict__ rgba) {
   extern __shared__ __align__(16) float slights[];
   const float D = (float)max(W, H);
-  const int npairs = (n_lights + 1) / 2;
+  const int npairs = n_lights / 2;
   bool odd_light = false;
   for (int i = threadIdx.x; i < 2 * npairs; i += blockDim.x) {
-    float4 p = lights[min(i, n_lights - 1)];
+    const float4 p = lights[i];
     odd_light |= !ordinary_light(p, D);
-    if (i >= n_lights) p.w = 0.f;  // the last pair's second light
     float* s = slights + 8 * (i >> 1) + (i & 1);
     s[0] = p.x; s[2] = p.y; s[4] = p.z; s[6] = p.w;
   }
@@ -146,8 +147,10 @@ __global__ void __launch_bounds__(256) k_deferred_light(int W, int H, const unsi
   const float4 a = unpack_half4(__ldg(galb + i));
   const float sx = (float)x + 0.5f, sy = (float)y + 0.5f;
   const float sz = (float)(unsigned)(k >> 32) * zscale;
-  const float acc = singles ? light_singles(lights, n_lights, n, sx, sy, sz, inv_r2)
-                            : light_pairs(reinterpret_cast<const LightPair*>(slights), npairs, n, sx, sy, sz, inv_r2);
+  float acc = 0.f;
+  if (!singles) acc = light_pairs(reinterpret_cast<const LightPair*>(slights), npairs, n, sx, sy, sz, inv_r2);
+  const int paired = singles ? 0 : 2 * npairs;
+  if (paired < n_lights) acc += light_singles(lights + paired, n_lights - paired, n, sx, sy, sz, inv_r2);
   rgba[i] = make_float4(a.x * acc, a.y * acc, a.z * acc, 1.0f);
 }
 
@@ -156,7 +159,7 @@ void launch_deferred_light(int W, int H, const unsigned long long* key, const ui
   (void)num_sms;
   const long long npix = (long long)W * H;
   const int blocks = (int)((npix + 255) / 256);
-  k_deferred_light<<<blocks, 256, (size_t)((n_lights + 1) / 2) * sizeof(LightPair), s>>>(W, H, key, gnorm, galb, lights,
+  k_deferred_light<<<blocks, 256, (size_t)(n_lights / 2) * sizeof(LightPair), s>>>(W, H, key, gnorm, galb, lights,
                                                                                          n_lights, rgba);
 }
 

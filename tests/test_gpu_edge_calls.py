@@ -84,3 +84,32 @@ def test_lambert_scene_without_triangles_needs_no_normals(color):
     assert bool((dc == 2.0).all()) and bool((dl == 2.0).all())  # added to: nothing
     assert gn is None and not bool(gl.any()) and (gc is None or not bool(gc.any()))
     r.close()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 64, 65])
+def test_light_pass_with_an_infinite_normal(n):
+    """A binary16 normal that overflowed gives an infinite sum where a light
+    shines on it and nothing where none does, for odd and even counts; never
+    NaN.  Other pixels are the oracle's."""
+    torch = _torch()
+    from paper_1404_6293_gb300.raster import Framebuffer, Rasterizer
+    W, H = 61, 45
+    key, gn, ga = S.gbuffer_inputs(W, H, empty_frac=0.0)
+    lights = S.point_lights(W, H, n)
+    lights[:, 2] = -5.0  # on the viewer's side of every sample
+    facing, away = (7, 11), (30, 20)
+    gn[facing] = (0.0, 0.0, -np.inf, 0.0)
+    gn[away] = (0.0, 0.0, np.inf, 0.0)
+    finite = gn.copy()
+    finite[facing] = finite[away] = 0
+    ref = oracle.light_pass(key, finite.view(np.uint16), ga.view(np.uint16), lights)
+    r = Rasterizer(W, H)
+    fb = Framebuffer(torch.from_numpy(key.view(np.int64)).cuda(), None, torch.from_numpy(gn).cuda(),
+                     torch.from_numpy(ga).cuda())
+    out = r.deferred_light(fb, torch.from_numpy(lights).cuda()).cpu().numpy()
+    assert (ga[facing][:3] > 0).all() and (lights[:, 3] > 0).all()
+    assert np.isposinf(out[facing][:3]).all()
+    assert (out[away][:3] == 0.0).all()
+    out[facing] = ref[facing]
+    assert np.abs(out - ref).max() <= 1e-5
+    r.close()
