@@ -79,7 +79,6 @@ struct piko_raster {
   uint2* heavy = nullptr;
   unsigned heavy_epoch = 0;
   unsigned long long* dkeys = nullptr;  // a key per pixel of directly rasterized triangles (piko_direct.cuh)
-  long long dkcap = 0;
   unsigned* busy = nullptr;             // tiles with bin entries, of a frame with direct keys
   // fragment buffers of the unfused pipeline (PIKO_SCHED_UNFUSED)
   unsigned* frag_pix = nullptr;
@@ -294,6 +293,16 @@ static float4* packed_attributes(piko_raster* h, const piko_scene* s) {
   return s->shade_mode == PIKO_SHADE_LAMBERT && s->color ? h->vattr : nullptr;
 }
 
+// Allocates the keys of direct rasterization, one per pixel, if they are not
+// there yet; false without the memory.
+static bool allocate_direct_keys(piko_raster* h) {
+  if (!h->dkeys && cudaMalloc(&h->dkeys, sizeof(unsigned long long) * (size_t)h->W * h->H) != cudaSuccess) {
+    cudaGetLastError();
+    h->dkeys = nullptr;
+  }
+  return h->dkeys != nullptr;
+}
+
 // The keys of direct rasterization for a frame of T triangles, or NULL when
 // every triangle is binned: a frame of larger triangles, one whose work is
 // counted or binned exactly, or no memory for the keys (nothing is allocated
@@ -302,11 +311,9 @@ static unsigned long long* direct_keys(piko_raster* h, int T, int V, cudaStream_
   if (h->stats || h->exact_bins || h->small_px < 1 || h->schedule > PIKO_SCHED_HARDWARE ||
       !direct_scene(T, V, h->W, h->H))
     return nullptr;
-  const long long need = (long long)h->W * h->H;
-  if (need > h->dkcap) {
+  if (!h->dkeys) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
-        grow(h, &h->dkeys, &h->dkcap, need, "direct keys") != PIKO_OK) {
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone || !allocate_direct_keys(h)) {
       cudaGetLastError();
       return nullptr;
     }
@@ -385,11 +392,9 @@ int piko_raster_reserve(piko_raster* h, int64_t max_vertices, int64_t max_triang
   if ((r = grow_vertices(h, max_vertices)) != PIKO_OK) return r;
   if ((r = grow_triangles(h, max_triangles)) != PIKO_OK) return r;
   if ((r = grow(h, &h->bin_tris, &h->ecap, max_bin_entries, "bin lists")) != PIKO_OK) return r;
-  // keys of direct rasterization, if such scenes can take it (else, or without
-  // the memory, every triangle is binned)
-  if (direct_scene(max_triangles, max_vertices, h->W, h->H) &&
-      grow(h, &h->dkeys, &h->dkcap, (long long)h->W * h->H, "direct keys") != PIKO_OK)
-    cudaGetLastError();
+  // keys of direct rasterization, if any scene within the sizes can take it
+  // (else, or without the memory, every triangle is binned)
+  if (direct_scene_within(max_triangles, max_vertices, h->W, h->H)) allocate_direct_keys(h);
   cudaError_t e = cudaDeviceSynchronize();
   return e == cudaSuccess ? PIKO_OK : cuda_fail(h, e, "reserve");
 }

@@ -44,6 +44,12 @@ inline bool direct_scene(long long T, long long V, int W, int H) {
   return V > 0 && (V < 2 * T ? 16 : 4) * T >= (long long)W * H;
 }
 
+// Whether some scene of at most max_t triangles and max_v vertices is one: a
+// mesh, which takes fewer triangles than a soup, of as many as there may be.
+inline bool direct_scene_within(long long max_t, long long max_v, int W, int H) {
+  return max_v > 0 && max_t > 0 && direct_scene(max_t, 1, W, H);
+}
+
 // A triangle of at most 128 pixels a side (its snapped extents below 2^15, so
 // that areas and edge functions are exact in 32 bits) whose box, clipped to
 // the screen, has at most max_px samples.

@@ -113,3 +113,45 @@ def test_light_pass_with_an_infinite_normal(n):
     out[facing] = ref[facing]
     assert np.abs(out - ref).max() <= 1e-5
     r.close()
+
+
+def test_reserve_covers_the_keys_of_every_mesh_within_the_sizes():
+    """Sizes with two vertices a triangle and more, of which a mesh at 4 to 16
+    pixels a triangle makes up a part: its forward allocates nothing and is
+    captured as it runs uncaptured."""
+    torch = _torch()
+    from paper_1404_6293_gb300 import _lib as L
+    from paper_1404_6293_gb300.raster import DeviceScene, Framebuffer, Rasterizer
+    W, H = 1280, 1024  # 10 MB of keys
+    s = S.heightfield(W, H, 400, 200, seed=12, with_color=True)
+    T = s.num_triangles
+    assert 4 * T < W * H <= 16 * T and s.num_vertices < 2 * T
+    ds = DeviceScene.from_host(s)
+    ref = oracle.raster_bbox(s, threads=8)[0]
+    fb = Framebuffer.allocate(W, H, s.shade_mode)
+    warm = Rasterizer(W, H)  # loads the kernels
+    warm.forward(ds, fb)
+    warm.set_option(L.PIKO_OPT_CHECK_CAPACITY, 0)
+    warm.forward(ds, fb)
+    torch.cuda.synchronize()
+    assert warm.status()[0] == 0
+    r = Rasterizer(W, H)
+    r.reserve(2 * T, T, 4 * T)
+    r.set_option(L.PIKO_OPT_CHECK_CAPACITY, 0)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    fb.key.fill_(0)
+    r.forward(ds, fb)
+    torch.cuda.synchronize()
+    assert r.status()[0] == 0
+    assert np.array_equal(fb.key_numpy(), ref)
+    assert torch.cuda.mem_get_info()[0] == free
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        r.forward(ds, fb)
+    fb.key.fill_(0)
+    g.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(fb.key_numpy(), ref)
+    r.close()
+    warm.close()
