@@ -71,13 +71,11 @@ struct piko_raster {
   unsigned* bin_off = nullptr;    // nbins + 1
   unsigned* cursor = nullptr;
   unsigned long long* chunk_state = nullptr;  // look-back state of the scan
-  unsigned scan_epoch = 0;
   unsigned* bin_tris = nullptr;
   long long ecap = 0;
   // AssignBin's list of heavy triangles (chunks of (triangle, bin) pairs
   // spread over whole CTAs), and the count pass's parity
   uint2* heavy = nullptr;
-  unsigned heavy_epoch = 0;
   unsigned long long* dkeys = nullptr;  // a key per pixel of directly rasterized triangles (piko_direct.cuh)
   unsigned* busy = nullptr;             // tiles with bin entries, of a frame with direct keys
   // fragment buffers of the unfused pipeline (PIKO_SCHED_UNFUSED)
@@ -610,13 +608,12 @@ static int scatter_and_process(piko_raster* h, const piko_scene* s, piko_framebu
   p.st = h->status;
   if (direct.keys) {
     const cudaError_t e = launch_scatter_shade(p, h->rect, h->cursor, h->bin_tris, (unsigned long long)h->ecap,
-                                               h->num_sms, st, clip_cap, h->heavy, heavy_cap(h), h->heavy_epoch,
-                                               direct.marks);
+                                               h->num_sms, st, clip_cap, h->heavy, heavy_cap(h), direct.marks);
     if (e != cudaSuccess) return cuda_fail(h, e, "scatter launch");
   } else {
     launch_scatter(h->g, T, h->rect, h->bin_off, h->cursor, h->bin_tris, (unsigned long long)h->ecap, h->status,
                    h->num_sms, st, clip_tris, clip_cap, h->exact_bins ? s->tris : nullptr, V, h->vtx, h->heavy,
-                   heavy_cap(h), h->heavy_epoch);
+                   heavy_cap(h));
   }
   if (ev) cudaEventRecord(h->stage_ev[4], st);
   int grid = h->nbins;
@@ -682,7 +679,6 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
     // a frame of one scan chunk of bins is scanned by the count pass's last
     // CTA (one launch fewer on the chain); larger frames take the scan kernel
     // (with stage events on, the count and scan launches stay apart)
-    const unsigned heavy_epoch = ++h->heavy_epoch, scan_epoch = ++h->scan_epoch;
     ScanReport report;
     if (check) {
       report.host = h->h_needed;
@@ -690,15 +686,14 @@ int piko_raster_forward(piko_raster* h, const piko_scene* s, piko_framebuffer* f
     }
     const bool fused = !ev && launch_count_and_scan(h->g, T, s->tris, V, h->vtx, h->rect, h->bin_count, h->status,
                                                     h->stats, h->num_sms, st, clip_tris, clip_cap, h->exact_bins,
-                                                    h->heavy, heavy_cap(h), heavy_epoch, h->bin_off, h->cursor,
-                                                    (unsigned long long)h->ecap, h->chunk_state, scan_epoch, direct,
-                                                    report);
+                                                    h->heavy, heavy_cap(h), h->bin_off, h->cursor,
+                                                    (unsigned long long)h->ecap, h->chunk_state, direct, report);
     if (!fused) {
       launch_setup_count(h->g, T, s->tris, V, h->vtx, h->rect, h->bin_count, h->status, h->stats, h->num_sms, st,
-                         clip_tris, clip_cap, h->exact_bins, h->heavy, heavy_cap(h), heavy_epoch, direct);
+                         clip_tris, clip_cap, h->exact_bins, h->heavy, heavy_cap(h), direct);
       if (ev) cudaEventRecord(h->stage_ev[2], st);
       launch_scan(h->nbins, h->bin_count, h->bin_off, h->cursor, (unsigned long long)h->ecap, h->status,
-                  h->chunk_state, scan_epoch, st, h->wait_budget, h->withhold, &report, direct.busy);
+                  h->chunk_state, st, h->wait_budget, h->withhold, &report, direct.busy);
       if (ev) cudaEventRecord(h->stage_ev[3], st);
     }
     if ((r = scatter_and_process(h, s, fb, st, ev, direct, vattr, clip_tris, clip_cap)) != PIKO_OK) return r;

@@ -12,6 +12,7 @@
 //
 // Every wait (grid barrier, scan look-back) is bounded by a clock budget;
 // on expiry PIKO_ERR_TIMEOUT is recorded and every later phase is skipped.
+#include <cstddef>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -50,7 +51,7 @@ struct BatchSync {
   unsigned count;     // CTAs arrived at the current grid barrier
   unsigned gen;       // barrier generation
   unsigned dyn_head;  // dynamic tile queue
-  unsigned pad;
+  unsigned epoch;     // tag of the scan's chunk states; each count phase advances it (never cleared)
 };
 
 struct BatchParams {
@@ -75,7 +76,6 @@ struct BatchParams {
   unsigned* bin_off;
   unsigned* cursor;
   unsigned long long* chunk_state;
-  unsigned epoch;
   unsigned* bin_tris;
   unsigned long long capacity;
   DevStatus* st;
@@ -304,6 +304,12 @@ __device__ void phase_count(const BatchParams& b) {
   if (lane == 0 && sum) atomicAdd(&b.st->direct_entries, sum);
 }
 
+// By one thread, before the launch or barrier that the scan waits for.
+__device__ void prepare_scan(const BatchParams& b) {
+  b.st->scan_ticket = 0u;
+  b.sync->epoch += 1u;
+}
+
 __device__ void phase_scan(const BatchParams& b, ScanSmem& sm) {
   const int chunk_bins = (int)blockDim.x * SCAN_PER;
   const int nchunks = (b.total_bins + chunk_bins - 1) / chunk_bins;
@@ -320,7 +326,7 @@ __device__ void phase_scan(const BatchParams& b, ScanSmem& sm) {
     __syncthreads();
     const int chunk = sm.chunk;
     if (chunk < 0 || chunk >= nchunks) break;
-    scan_chunk(chunk, nchunks, b.total_bins, b.cnt, b.bin_off, b.cursor, b.capacity, b.st, b.chunk_state, b.epoch,
+    scan_chunk(chunk, nchunks, b.total_bins, b.cnt, b.bin_off, b.cursor, b.capacity, b.st, b.chunk_state, &b.sync->epoch,
                sm, &b.sync->dyn_head, b.wait_budget, b.withhold);
     __syncthreads();  // sm.chunk is rewritten for the next ticket
   }
@@ -486,7 +492,7 @@ __global__ void __maxnreg__(PIKO_BATCH_MAXNREG) k_batch_forward(BatchParams b) {
   phase_vertex<PERSP>(b);
   const bool skip = (b.withhold & TEST_WITHHOLD_BARRIER) && blockIdx.x == 0;
   if (!grid_barrier(b.sync, b.st, b.wait_budget, skip)) return;
-  if (blockIdx.x == 0 && threadIdx.x == 0) b.st->scan_ticket = 0u;  // the scan runs after a barrier
+  if (blockIdx.x == 0 && threadIdx.x == 0) prepare_scan(b);  // the scan runs after a barrier
   phase_count(b);
   if (!grid_barrier(b.sync, b.st, b.wait_budget)) return;
   phase_scan(b, scan_sm);
@@ -510,7 +516,7 @@ __global__ void __launch_bounds__(256, 4) k_batch_count(BatchParams b) {
   pdl_wait();
   pdl_launch_dependents();
   if (cta_should_stop(b.st)) return;
-  if (blockIdx.x == 0 && threadIdx.x == 0) b.st->scan_ticket = 0u;  // the scan runs after this kernel
+  if (blockIdx.x == 0 && threadIdx.x == 0) prepare_scan(b);  // the scan runs after this kernel
   phase_count(b);
 }
 __global__ void __launch_bounds__(BATCH_THREADS) k_batch_scan(BatchParams b) {
@@ -672,7 +678,6 @@ struct BatchState {
   long long gcap = 0;
   bool gacc_dirty = false;  // gacc is not zero: new, or a backward launch failed
   BatchSync* sync = nullptr;
-  unsigned epoch = 0;
   // host staging (pinned) and the last layout
   void* staging = nullptr;
   size_t staging_cap = 0;
@@ -944,9 +949,8 @@ int batch_launch_forward(BatchState* bs, DevStatus* st, bool persistent, cudaStr
   b.withhold = withhold;
   b.capacity = (unsigned long long)bs->ecap;
   b.bin_tris = bs->bin_tris;
-  b.epoch = ++bs->epoch;
   // (the separate launches use only its queue head, which the scan resets)
-  if (persistent && cudaMemsetAsync(bs->sync, 0, sizeof(BatchSync), stream) != cudaSuccess) {
+  if (persistent && cudaMemsetAsync(bs->sync, 0, offsetof(BatchSync, epoch), stream) != cudaSuccess) {
     err = "batch barrier reset failed";
     return PIKO_ERR_CUDA;
   }

@@ -308,8 +308,8 @@ constexpr unsigned HEAVY_NONE = 0xFFFFFFFFu;  // a chunk slot of a triangle that
 
 // Read after the grid dependency wait: the count pass that wrote it has
 // completed, so a plain (read-only path) load sees its final value.
-__device__ __forceinline__ unsigned heavy_count(const DevStatus* st, unsigned epoch, unsigned cap) {
-  const unsigned n = __ldg(&st->heavy_n[epoch & 1u]);
+__device__ __forceinline__ unsigned heavy_count(const DevStatus* st, unsigned cap) {
+  const unsigned n = __ldg(&st->heavy_n);
   return n < cap ? n : cap;
 }
 
@@ -351,7 +351,7 @@ constexpr int SCAN_CHUNK = FWD_SCAN_CHUNK;
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan(int nbins, unsigned* __restrict__ cnt,
                                                        unsigned* __restrict__ bin_off, unsigned* __restrict__ cursor,
                                                        unsigned long long capacity, DevStatus* st,
-                                                       unsigned long long* __restrict__ chunk_state, unsigned epoch,
+                                                       unsigned long long* __restrict__ chunk_state,
                                                        long long wait_budget, int withhold, ScanReport report,
                                                        unsigned* __restrict__ busy) {
   __shared__ ScanSmem sm;
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan(int nbins, unsigned* __re
   const int chunk = sm.chunk;
   const int nchunks = (nbins + SCAN_CHUNK - 1) / SCAN_CHUNK;
   if (chunk >= nchunks) return;  // only with a corrupted ticket; the count pass resets it every frame
-  scan_chunk(chunk, nchunks, nbins, cnt, bin_off, cursor, capacity, st, chunk_state, epoch, sm, &st->queue_head,
+  scan_chunk(chunk, nchunks, nbins, cnt, bin_off, cursor, capacity, st, chunk_state, &st->scan_epoch, sm, &st->queue_head,
              wait_budget, withhold, report, busy);
   // one CTA per chunk: every ticket was taken before the last chunk's
   // look-back ended, so the last chunk may reset the ticket
@@ -527,7 +527,6 @@ struct FusedScan {
   unsigned* cursor;
   unsigned long long capacity;
   unsigned long long* chunk_state;
-  unsigned epoch;
   ScanReport report;
 };
 
@@ -539,7 +538,7 @@ __global__ void __launch_bounds__(256, EXACT || DIRECT ? 4 : 8) k_setup_count(Ra
                                                      unsigned* __restrict__ cnt, int nbins, DevStatus* st,
                                                      int stats, const int4* __restrict__ clip_tris,
                                                      unsigned clip_cap, uint2* __restrict__ heavy,
-                                                     unsigned heavy_cap, unsigned heavy_epoch, FusedScan fs,
+                                                     unsigned heavy_cap, FusedScan fs,
                                                      DirectRaster direct) {
   unsigned dentries = 0u;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -548,10 +547,9 @@ __global__ void __launch_bounds__(256, EXACT || DIRECT ? 4 : 8) k_setup_count(Ra
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     st->scan_ticket = 0u;  // the scan runs after this kernel (or in its last CTA)
     st->busy_n = 0u;
-    // the other parity's heavy counter is the next count pass's: nothing reads it until then
-    st->heavy_n[(heavy_epoch + 1u) & 1u] = 0u;
+    st->scan_epoch += 1u;
   }
-  unsigned* heavy_n = &st->heavy_n[heavy_epoch & 1u];
+  unsigned* heavy_n = &st->heavy_n;
   pdl_wait();  // snapped vertices
   pdl_launch_dependents();
   const unsigned lt_mask = (1u << lane) - 1u;
@@ -610,7 +608,7 @@ __global__ void __launch_bounds__(256, EXACT || DIRECT ? 4 : 8) k_setup_count(Ra
     if (s_last) {
       __threadfence();
       if (threadIdx.x == 0) st->count_done = 0u;  // for the next frame
-      scan_chunk(0, 1, nbins, cnt, fs.bin_off, fs.cursor, fs.capacity, st, fs.chunk_state, fs.epoch, scan_sm,
+      scan_chunk(0, 1, nbins, cnt, fs.bin_off, fs.cursor, fs.capacity, st, fs.chunk_state, &st->scan_epoch, scan_sm,
                  &st->queue_head, WAIT_BUDGET_CYCLES, 0, fs.report, direct.busy);
     }
   }
@@ -630,7 +628,7 @@ static int resident_per_sm(K kernel, int threads) {
 void launch_setup_count(const RasterGeom& g, int T, const int* tris, int V, const int4* vtx, BinRect* rect,
                         unsigned* bin_count, DevStatus* st, int stats, int num_sms, cudaStream_t s,
                         const int4* clip_tris, unsigned clip_cap, int exact, uint2* heavy, unsigned heavy_cap,
-                        unsigned heavy_epoch, DirectRaster direct) {
+                        DirectRaster direct) {
   static const int per_sm_of[2] = {resident_per_sm(k_setup_count<false>, 256),
                                    resident_per_sm(k_setup_count<false, false, true>, 256)};
   const int per_sm = per_sm_of[direct.keys != nullptr];
@@ -641,14 +639,14 @@ void launch_setup_count(const RasterGeom& g, int T, const int* tris, int V, cons
   blocks = blocks < num_sms * per_sm ? blocks : num_sms * per_sm;
   if (blocks < 1) blocks = 1;  // with no triangles the kernel still resets the scan ticket
   launch_pdl(kernel, blocks, 256, 0, s, g, T, tris, V, vtx, rect, bin_count, g.nbx * g.nby, st, stats, clip_tris,
-             clip_cap, heavy_cap ? heavy : nullptr, heavy_cap, heavy_epoch, FusedScan{}, direct);
+             clip_cap, heavy_cap ? heavy : nullptr, heavy_cap, FusedScan{}, direct);
 }
 
 bool launch_count_and_scan(const RasterGeom& g, int T, const int* tris, int V, const int4* vtx, BinRect* rect,
                            unsigned* bin_count, DevStatus* st, int stats, int num_sms, cudaStream_t s,
                            const int4* clip_tris, unsigned clip_cap, int exact, uint2* heavy, unsigned heavy_cap,
-                           unsigned heavy_epoch, unsigned* bin_off, unsigned* cursor, unsigned long long capacity,
-                           unsigned long long* chunk_state, unsigned scan_epoch, DirectRaster direct,
+                           unsigned* bin_off, unsigned* cursor, unsigned long long capacity,
+                           unsigned long long* chunk_state, DirectRaster direct,
                            const ScanReport& report) {
   const int nbins = g.nbx * g.nby;
   // one chunk of the count pass's 256 threads x SCAN_PER bins
@@ -668,18 +666,17 @@ bool launch_count_and_scan(const RasterGeom& g, int T, const int* tris, int V, c
   fs.cursor = cursor;
   fs.capacity = capacity;
   fs.chunk_state = chunk_state;
-  fs.epoch = scan_epoch;
   fs.report = report;
   launch_pdl(kernel, blocks, 256, 0, s, g, T, tris, V, vtx, rect, bin_count, nbins, st, stats, clip_tris, clip_cap,
-             heavy_cap ? heavy : nullptr, heavy_cap, heavy_epoch, fs, direct);
+             heavy_cap ? heavy : nullptr, heavy_cap, fs, direct);
   return true;
 }
 
 void launch_scan(int nbins, unsigned* bin_count, unsigned* bin_off, unsigned* cursor, unsigned long long capacity,
-                 DevStatus* st, unsigned long long* chunk_state, unsigned epoch, cudaStream_t s, long long wait_budget,
+                 DevStatus* st, unsigned long long* chunk_state, cudaStream_t s, long long wait_budget,
                  int withhold, const ScanReport* report, unsigned* busy) {
   launch_pdl(k_scan, scan_chunks(nbins), SCAN_THREADS, 0, s, nbins, bin_count, bin_off, cursor, capacity, st,
-             chunk_state, epoch, wait_budget, withhold, report ? *report : ScanReport(), busy);
+             chunk_state, wait_budget, withhold, report ? *report : ScanReport(), busy);
 }
 
 // ======================================================================
@@ -759,12 +756,12 @@ __device__ __forceinline__ void scatter_cta(const RasterGeom& g, int T, const Bi
                                             unsigned* __restrict__ bin_tris, unsigned long long capacity,
                                             const DevStatus* st, const int4* __restrict__ clip_tris, unsigned clip_cap,
                                             const int* __restrict__ tris, int V, const int4* __restrict__ vtx,
-                                            const uint2* __restrict__ heavy, unsigned heavy_cap, unsigned heavy_epoch,
+                                            const uint2* __restrict__ heavy, unsigned heavy_cap,
                                             const unsigned char* __restrict__ marks, int block, int nblocks) {
   const int T_in = T;
   T = frame_triangles(T, clip_tris, clip_cap, st);
   // the heavy list's length is loaded now and used after the per-warp work
-  const unsigned nheavy = heavy ? heavy_count(st, heavy_epoch, heavy_cap) : 0u;
+  const unsigned nheavy = heavy ? heavy_count(st, heavy_cap) : 0u;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int step = nblocks * (blockDim.x >> 5) * 32;
   BinRect none;
@@ -828,13 +825,12 @@ __global__ void __launch_bounds__(256, EXACT ? 4 : 8) k_scatter(RasterGeom g, in
                                                  unsigned long long capacity, const DevStatus* st,
                                                  const int4* __restrict__ clip_tris, unsigned clip_cap,
                                                  const int* __restrict__ tris, int V, const int4* __restrict__ vtx,
-                                                 const uint2* __restrict__ heavy, unsigned heavy_cap,
-                                                 unsigned heavy_epoch) {
+                                                 const uint2* __restrict__ heavy, unsigned heavy_cap) {
   pdl_wait();  // offsets, cursors and the status of the scan
   pdl_launch_dependents();
   if (st->flags & STATUS_SKIP_MASK) return;
   scatter_cta<EXACT, false>(g, T, rect, bin_off, cursor, bin_tris, capacity, st, clip_tris, clip_cap, tris, V, vtx,
-                            heavy, heavy_cap, heavy_epoch, nullptr, blockIdx.x, gridDim.x);
+                            heavy, heavy_cap, nullptr, blockIdx.x, gridDim.x);
 }
 
 // A frame with direct keys: the first scatter_blocks CTAs scatter, the others
@@ -852,7 +848,7 @@ struct ScatterShade {
   const DevStatus* st;
   unsigned clip_cap;
   const uint2* heavy;
-  unsigned heavy_cap, heavy_epoch;
+  unsigned heavy_cap;
   const unsigned char* marks;
   int scatter_blocks;
 };
@@ -865,7 +861,7 @@ __global__ void __launch_bounds__(256, CLIP ? 4 : 5) k_scatter_shade(const __gri
   const RasterGeom& g = sc.g;
   if ((int)blockIdx.x < a.scatter_blocks) {
     scatter_cta<false, true>(g, sc.T, a.rect, a.bin_off, a.cursor, a.bin_tris, a.capacity, a.st, sc.clip_tris,
-                             a.clip_cap, nullptr, 0, nullptr, a.heavy, a.heavy_cap, a.heavy_epoch, a.marks, blockIdx.x,
+                             a.clip_cap, nullptr, 0, nullptr, a.heavy, a.heavy_cap, a.marks, blockIdx.x,
                              a.scatter_blocks);
     return;
   }
@@ -918,7 +914,7 @@ __global__ void __launch_bounds__(256, CLIP ? 4 : 5) k_scatter_shade(const __gri
 void launch_scatter(const RasterGeom& g, int T, const BinRect* rect, const unsigned* bin_off, unsigned* cursor,
                     unsigned* bin_tris, unsigned long long capacity, DevStatus* st, int num_sms, cudaStream_t s,
                     const int4* clip_tris, unsigned clip_cap, const int* tris, int V, const int4* vtx,
-                    const uint2* heavy, unsigned heavy_cap, unsigned heavy_epoch) {
+                    const uint2* heavy, unsigned heavy_cap) {
   const long long TT = (long long)T + (clip_tris ? clip_cap : 0u);
   if (TT <= 0) return;
   static const int per_sm = resident_per_sm(k_scatter<false>, 256);
@@ -926,20 +922,19 @@ void launch_scatter(const RasterGeom& g, int T, const BinRect* rect, const unsig
   int blocks = (warps + 7) / 8;
   blocks = blocks < num_sms * per_sm ? blocks : num_sms * per_sm;
   launch_pdl(tris ? k_scatter<true> : k_scatter<false>, blocks, 256, 0, s, g, T, rect, bin_off, cursor, bin_tris,
-             capacity, st, clip_tris, clip_cap, tris, V, vtx, heavy_cap ? heavy : nullptr, heavy_cap, heavy_epoch);
+             capacity, st, clip_tris, clip_cap, tris, V, vtx, heavy_cap ? heavy : nullptr, heavy_cap);
 }
 
 cudaError_t launch_scatter_shade(const ProcessParams& p, const BinRect* rect, unsigned* cursor, unsigned* bin_tris,
                                  unsigned long long capacity, int num_sms, cudaStream_t s, unsigned clip_cap,
-                                 const uint2* heavy, unsigned heavy_cap, unsigned heavy_epoch,
-                                 const unsigned char* marks) {
+                                 const uint2* heavy, unsigned heavy_cap, const unsigned char* marks) {
   const long long TT = (long long)p.num_triangles + (p.clip_tris ? clip_cap : 0u);
   const long long need = ((TT + 31) / 32 + 7) / 8;
   ScatterShade a;
   a.sc = scene_of(p);
   a.rect = rect; a.bin_off = p.bin_off; a.cursor = cursor; a.bin_tris = bin_tris; a.capacity = capacity; a.st = p.st;
   a.clip_cap = clip_cap;
-  a.heavy = heavy_cap ? heavy : nullptr; a.heavy_cap = heavy_cap; a.heavy_epoch = heavy_epoch;
+  a.heavy = heavy_cap ? heavy : nullptr; a.heavy_cap = heavy_cap;
   a.marks = marks;
   // two CTAs of scattering warps per SM: a warp looks at 32 batches with one load
   a.scatter_blocks = (int)(need < 2LL * num_sms ? need : 2LL * num_sms);

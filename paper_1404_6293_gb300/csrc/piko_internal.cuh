@@ -57,7 +57,8 @@ struct DevStatus {
   unsigned long long frags;     // covered samples
   unsigned long long shaded;    // covered pixels after the depth test
   unsigned long long binned;    // triangles that reached at least one bin
-  unsigned int heavy_n[2];      // chunks in the heavy-triangle list of AssignBin, by count-pass parity
+  unsigned int heavy_n;         // chunks in the heavy-triangle list of AssignBin (0 after the Process stage)
+  unsigned int scan_epoch;      // tag of the last scan's chunk states; each count pass advances it
   unsigned int count_done;      // count-pass CTAs finished (its last CTA scans small frames; then 0 again)
   unsigned int busy_n;          // bins with entries (listed by the scan of a frame with direct keys; 0 before it)
   unsigned long long direct_entries;  // bin entries of the triangles the count pass rasterized itself (0 after the scan)
@@ -394,14 +395,11 @@ constexpr unsigned HEAVY_LIST_CAP = 16384;
 
 // heavy (optional, heavy_cap entries): triangles spanning many bins are
 // listed there in chunks of pairs, whose entries launch_scatter writes
-// spread over whole CTAs; heavy_epoch
-// must change between consecutive count passes of a handle (its parity
-// picks the list's counter; the pass clears the other one).
+// spread over whole CTAs; the Process stage clears the list for the next frame.
 void launch_setup_count(const RasterGeom& g, int T, const int* tris, int V, const int4* vtx,
                         BinRect* rect, unsigned* bin_count, DevStatus* st, int stats, int num_sms, cudaStream_t s,
                         const int4* clip_tris = nullptr, unsigned clip_cap = 0, int exact = 0,
-                        uint2* heavy = nullptr, unsigned heavy_cap = 0, unsigned heavy_epoch = 0,
-                        DirectRaster direct = DirectRaster());
+                        uint2* heavy = nullptr, unsigned heavy_cap = 0, DirectRaster direct = DirectRaster());
 // Count pass and scan in one launch for a frame of at most one scan chunk of
 // bins (scan_chunks(nbins) == 1): the count pass's last CTA scans.  Returns
 // false (nothing launched) for larger frames, which take launch_setup_count
@@ -409,35 +407,33 @@ void launch_setup_count(const RasterGeom& g, int T, const int* tris, int V, cons
 bool launch_count_and_scan(const RasterGeom& g, int T, const int* tris, int V, const int4* vtx, BinRect* rect,
                            unsigned* bin_count, DevStatus* st, int stats, int num_sms, cudaStream_t s,
                            const int4* clip_tris, unsigned clip_cap, int exact, uint2* heavy, unsigned heavy_cap,
-                           unsigned heavy_epoch, unsigned* bin_off, unsigned* cursor, unsigned long long capacity,
-                           unsigned long long* chunk_state, unsigned scan_epoch, DirectRaster direct,
+                           unsigned* bin_off, unsigned* cursor, unsigned long long capacity,
+                           unsigned long long* chunk_state, DirectRaster direct,
                            const ScanReport& report);
 // Near/far clipping of the triangles with a rejected vertex: sub-triangles
 // (3 snapped points each) and their triangle's index appended at
 // st->clip_count (PIKO_ERR_OVERFLOW past cap).
 void launch_clip(int W, int H, int T, const int* tris, int V, const float* pos, const float* mvp, const int4* vtx,
                  int4* clip_tris, unsigned* clip_orig, unsigned cap, DevStatus* st, int num_sms, cudaStream_t s);
-// chunk_state: scan_chunks(nbins) words, zero at allocation; epoch must
-// differ between consecutive scans on the same state array.  wait_budget:
+// chunk_state: scan_chunks(nbins) words, zero at allocation (told apart from
+// the last scan's by st->scan_epoch).  wait_budget:
 // clock cycles a look-back wait may take before PIKO_ERR_TIMEOUT; withhold:
 // test hook bits (piko_scan.cuh).
 void launch_scan(int nbins, unsigned* bin_count, unsigned* bin_off, unsigned* cursor, unsigned long long capacity,
-                 DevStatus* st, unsigned long long* chunk_state, unsigned epoch, cudaStream_t s,
+                 DevStatus* st, unsigned long long* chunk_state, cudaStream_t s,
                  long long wait_budget = 40000000, int withhold = 0, const ScanReport* report = nullptr,
                  unsigned* busy = nullptr);
 int scan_chunks(int nbins);
 void launch_scatter(const RasterGeom& g, int T, const BinRect* rect, const unsigned* bin_off, unsigned* cursor,
                     unsigned* bin_tris, unsigned long long capacity, DevStatus* st, int num_sms, cudaStream_t s,
                     const int4* clip_tris = nullptr, unsigned clip_cap = 0, const int* tris = nullptr, int V = 0,
-                    const int4* vtx = nullptr, const uint2* heavy = nullptr, unsigned heavy_cap = 0,
-                    unsigned heavy_epoch = 0);
+                    const int4* vtx = nullptr, const uint2* heavy = nullptr, unsigned heavy_cap = 0);
 cudaError_t launch_process(const ProcessParams& p, int threads, int grid, cudaStream_t s);
 // launch_scatter of a frame with direct keys (default binning), and the
 // shading of the tiles without bin entries, in one launch.
 cudaError_t launch_scatter_shade(const ProcessParams& p, const BinRect* rect, unsigned* cursor, unsigned* bin_tris,
                                  unsigned long long capacity, int num_sms, cudaStream_t s, unsigned clip_cap,
-                                 const uint2* heavy, unsigned heavy_cap, unsigned heavy_epoch,
-                                 const unsigned char* marks);
+                                 const uint2* heavy, unsigned heavy_cap, const unsigned char* marks);
 cudaError_t process_occupancy(const ProcessParams& p, int threads, int* blocks_per_sm);
 
 // Boxes (pixels of a triangle's bounding box inside a tile) up to this size

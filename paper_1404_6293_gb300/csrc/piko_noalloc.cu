@@ -16,7 +16,6 @@
 // loads this library keeps until the process exits.
 #include <cuda.h>
 
-#include <atomic>
 #include <mutex>
 
 #include "piko_internal.cuh"
@@ -50,7 +49,6 @@ constexpr size_t SCRATCH_BYTES = align256(OFF_ENTRIES + sizeof(unsigned) * (size
 // address comes from cudaGetSymbolAddress below.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[SCRATCH_BYTES];
 
-std::atomic<unsigned> g_scan_epoch{0};
 std::mutex g_setup_lock;
 
 // The array's device address belongs to the module instance of one CUDA
@@ -204,7 +202,7 @@ extern "C" int piko_raster_forward_noalloc(const piko_scene* s, piko_framebuffer
                 lambert ? vdot : nullptr, nullptr, num_sms, st);
   launch_setup_count(g, s->num_triangles, s->tris, s->num_vertices, vtx, rect, bin_count, status, 0, num_sms, st);
   launch_scan(nbins, bin_count, bin_off, cursor, (unsigned long long)PIKO_NOALLOC_MAX_BIN_ENTRIES, status, chunk_state,
-              ++g_scan_epoch, st);
+              st);
   launch_scatter(g, s->num_triangles, rect, bin_off, cursor, bin_tris, (unsigned long long)PIKO_NOALLOC_MAX_BIN_ENTRIES,
                  status, num_sms, st);
 

@@ -71,6 +71,9 @@ __global__ void __maxnreg__(PIKO_PROCESS_MAXNREG) k_process(const __grid_constan
   };
   if (!p.busy) clear_keys();
   pdl_wait();  // bin lists and status of the scatter pass
+  // the heavy list is scattered: empty for the next frame (also after one that
+  // was skipped, and in every replay of a captured one)
+  if (blockIdx.x == 0 && tid == 0) p.st->heavy_n = 0u;
   // with direct keys the tiles without entries are shaded already: a frame of
   // tiny triangles ends here after one look at the list's length
   const int ntiles = p.busy ? (int)min(__ldcg(&p.st->busy_n), (unsigned)p.ntiles) : p.ntiles;

@@ -5,7 +5,10 @@
 // A single-pass decoupled look-back scan: chunks are taken in ticket order,
 // so every predecessor of a chunk has started.  Each chunk publishes its
 // aggregate, then its inclusive prefix, in a 64-bit state word tagged with
-// the frame's epoch (so the words never need clearing):
+// the frame's epoch (so the words never need clearing).  The epoch lives in
+// device memory and a kernel before the scan advances it, so that a captured
+// frame gets a new one at every replay; a tag from the host would be the same
+// each time, and a chunk would take its predecessor's state of the replay before:
 //   bits 63..62 kind (1 aggregate, 2 inclusive prefix), 61..46 epoch, 45..0 value.
 // off[b] = entries of all earlier bins; the scatter cursor of a bin starts
 // after its single-bin part; both count arrays are zeroed for the next frame.
@@ -75,12 +78,11 @@ struct ScanReport {
 __device__ __forceinline__ void scan_chunk(int chunk, int nchunks, int nbins, unsigned* __restrict__ cnt,
                                            unsigned* __restrict__ bin_off, unsigned* __restrict__ cursor,
                                            unsigned long long capacity, DevStatus* st,
-                                           unsigned long long* __restrict__ chunk_state, unsigned epoch, ScanSmem& sm,
+                                           unsigned long long* __restrict__ chunk_state, const unsigned* epoch, ScanSmem& sm,
                                            unsigned* queue_to_reset, long long wait_budget = WAIT_BUDGET_CYCLES,
                                            int withhold = 0, ScanReport report = ScanReport(),
                                            unsigned* __restrict__ busy = nullptr) {
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
-  const unsigned long long tag = (unsigned long long)(epoch & 0xFFFFu) << 46;
   unsigned* __restrict__ multi = cnt + nbins;
   const bool vec = (nbins & 3) == 0;  // second array 16-byte aligned
   const int b0 = chunk * (int)blockDim.x * SCAN_PER + tid * SCAN_PER;
@@ -110,6 +112,7 @@ __device__ __forceinline__ void scan_chunk(int chunk, int nchunks, int nbins, un
   __syncthreads();
   const unsigned long long agg = sm.warp_sums[nw - 1];
   if (tid == 0) {
+    const unsigned long long tag = (unsigned long long)(__ldcg(epoch) & 0xFFFFu) << 46;
     unsigned long long excl = 0;
     if (chunk == 0) {
       if (!(withhold & TEST_WITHHOLD_SCAN)) st_release_u64(chunk_state, SCAN_KIND_PREFIX | tag | (agg & SCAN_VALUE_MASK));

@@ -3,6 +3,7 @@ triangles or normals, odd light counts, attribute arrays longer than the
 scene, scratch reserved ahead of a capture, and replayed graphs whose inputs
 change between replays."""
 import ctypes as C
+import dataclasses
 
 import numpy as np
 import pytest
@@ -155,3 +156,101 @@ def test_reserve_covers_the_keys_of_every_mesh_within_the_sizes():
     assert np.array_equal(fb.key_numpy(), ref)
     r.close()
     warm.close()
+
+
+def _cameras(n):
+    """Zooms and shifts of the identity camera, each unlike the one before it."""
+    out = []
+    for k in range(n):
+        m = np.eye(4, dtype=np.float32)
+        m[0, 0] = m[1, 1] = (1.0, 0.3, 1.6, 0.7, 2.0, 0.5)[k % 6]
+        m[0, 3], m[1, 3] = 0.4 * np.cos(2.0 * k), 0.4 * np.sin(2.0 * k)
+        out.append(m.ravel())
+    return out
+
+
+@pytest.mark.parametrize("schedule", ["static", "dynamic"])
+@pytest.mark.parametrize("kind", ["binned", "direct"])
+def test_replays_of_a_captured_frame_follow_the_camera(kind, schedule):
+    """16,384 bins (eight scan chunks, which look back at each other) and
+    triangles across hundreds of them, captured once and replayed with another
+    camera each time: every replay is the oracle's frame."""
+    torch = _torch()
+    from paper_1404_6293_gb300 import _lib as L
+    from paper_1404_6293_gb300.raster import DeviceScene, Framebuffer, Rasterizer
+    W = H = 1024
+    large = S.random_triangles(W, H, 60, 400.0, seed=31)
+    if kind == "binned":
+        s = S.random_triangles(W, H, 3000, 12.0, seed=32)
+    else:
+        s = S.random_triangles(W, H, 400000, 2.0, seed=33)
+    pos = np.concatenate([s.pos, large.pos])
+    s = S.Scene(W, H, pos, np.arange(len(pos), dtype=np.int32).reshape(-1, 3),
+                color=np.concatenate([s.color, large.color]), mvp=np.eye(4, dtype=np.float32).ravel())
+    ds = DeviceScene.from_host(s)
+    fb = Framebuffer.allocate(W, H, s.shade_mode)
+    r = Rasterizer(W, H, 8, 8, schedule)
+    r.reserve(s.num_vertices, s.num_triangles, 4_000_000)
+    r.set_option(L.PIKO_OPT_CHECK_CAPACITY, 0)
+    r.forward(ds, fb)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        r.forward(ds, fb)
+    for k, m in enumerate(_cameras(7)):
+        ds.mvp.copy_(torch.from_numpy(m))
+        fb.key.fill_(0)
+        for _ in range(1 + k % 2):  # (also twice without a change)
+            g.replay()
+        torch.cuda.synchronize()
+        assert r.status()[0] == 0
+        ref = oracle.raster_bbox(dataclasses.replace(s, mvp=m), threads=8)[0]
+        assert np.array_equal(fb.key_numpy(), ref), f"replay {k}"
+    ref = oracle.raster_bbox(s, threads=8)[0]  # an ordinary call among the replays
+    ds.mvp.copy_(torch.from_numpy(s.mvp))
+    r.forward(ds, fb)
+    torch.cuda.synchronize()
+    assert np.array_equal(fb.key_numpy(), ref)
+    r.close()
+
+
+@pytest.mark.parametrize("launch", [0, 1])
+def test_replays_of_a_captured_batch_follow_the_cameras(launch):
+    """12,288 bins of three scenes: a dozen scan chunks."""
+    torch = _torch()
+    from paper_1404_6293_gb300 import _lib as L
+    from paper_1404_6293_gb300.raster import DeviceScene, Rasterizer
+    W = H = 512
+    host = [S.random_triangles(W, H, 2000, 9.0, seed=41), S.random_triangles(W, H, 100000, 2.0, seed=42),
+            S.random_triangles(W, H, 100, 150.0, seed=43)]
+    host = [dataclasses.replace(s, mvp=np.eye(4, dtype=np.float32).ravel()) for s in host]
+    ds = [DeviceScene.from_host(s) for s in host]
+    r = Rasterizer(W, H, 8, 8)
+    r.set_option(L.PIKO_OPT_BATCH_LAUNCH, launch)
+    cams = _cameras(6)
+    big = torch.from_numpy(cams[4])  # the most bin entries: sizes the lists
+    for d in ds:
+        d.mvp.copy_(big)
+    fbs = r.forward_batch(ds)
+    for m in cams:
+        for d in ds:
+            d.mvp.copy_(torch.from_numpy(m))
+        r.forward_batch(ds, fbs)
+    r.set_option(L.PIKO_OPT_CHECK_CAPACITY, 0)
+    r.forward_batch(ds, fbs)
+    torch.cuda.synchronize()
+    assert r.status()[0] == 0
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        r.forward_batch(ds, fbs)
+    for k in range(7):
+        for i, d in enumerate(ds):
+            d.mvp.copy_(torch.from_numpy(cams[(k + i) % 6]))
+        for _ in range(1 + k % 2):
+            g.replay()
+        torch.cuda.synchronize()
+        assert r.status()[0] == 0
+        for i, s in enumerate(host):
+            ref = oracle.raster_bbox(dataclasses.replace(s, mvp=cams[(k + i) % 6]), threads=8)[0]
+            assert np.array_equal(fbs[i].key_numpy(), ref), f"replay {k}, scene {i}"
+    r.close()
