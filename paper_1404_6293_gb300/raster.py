@@ -336,9 +336,14 @@ class Rasterizer:
                   light=True, stream=None):
         """The gradients of ``backward`` in new tensors (None for those not
         asked for), which the kernels write without a clear before them."""
-        dc = torch.empty_like(scene.color) if color else None
-        dn = torch.empty_like(scene.normal) if normal else None
-        dl = torch.empty_like(scene.light_dir) if light else None
+        def new(t, n):
+            # the kernels write n floats; an array longer than the scene (padded) is zero behind them
+            return torch.empty_like(t) if t.numel() == n else torch.zeros_like(t)
+
+        n = 3 * scene.num_vertices
+        dc = new(scene.color, n) if color else None
+        dn = new(scene.normal, n) if normal else None
+        dl = new(scene.light_dir, 3) if light else None
         cs, cf = scene.c_struct(), fb.c_struct()
         g = dl_drgba.contiguous()
         self._check(self.lib.piko_raster_backward_set(self._h, C.byref(cs), C.byref(cf), _ptr(g), _ptr(dc), _ptr(dn),

@@ -254,3 +254,31 @@ def test_replays_of_a_captured_batch_follow_the_cameras(launch):
             ref = oracle.raster_bbox(dataclasses.replace(s, mvp=cams[(k + i) % 6]), threads=8)[0]
             assert np.array_equal(fbs[i].key_numpy(), ref), f"replay {k}, scene {i}"
     r.close()
+
+
+def test_gradients_of_arrays_longer_than_the_scene():
+    """Attribute arrays padded past the scene's vertices (a buffer reused for
+    several meshes): the padding's gradient is zero through autograd."""
+    torch = _torch()
+    from paper_1404_6293_gb300.autograd import render
+    from paper_1404_6293_gb300.raster import DeviceScene, Rasterizer
+    s = S.heightfield(97, 61, 30, 20, seed=8, with_color=True)
+    ds = DeviceScene.from_host(s)
+    V, r = s.num_vertices, Rasterizer(97, 61)
+
+    def padded(t, rows):
+        return torch.cat([t, torch.ones((rows,) + tuple(t.shape[1:]), device="cuda")]).requires_grad_(True)
+
+    g = torch.randn((61, 97, 4), device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    plain = [t.clone().requires_grad_(True) for t in (ds.color, ds.normal, ds.light_dir)]
+    long = [padded(ds.color, 400), padded(ds.normal, 400), padded(ds.light_dir, 2)]
+    want = torch.autograd.grad(render(r, ds, *plain)[0], plain, g)
+    rgba = render(r, ds, *long)[0]
+    junk = [torch.full_like(t, float("nan")) for t in long]  # freed, so that new tensors hold them
+    del junk
+    got = torch.autograd.grad(rgba, long, g)
+    torch.cuda.synchronize()
+    for a, b, n in zip(got, want, (V, V, 3)):
+        assert not bool(a[n:].any())
+        assert float((a[:n] - b).abs().max()) <= 1e-4 * float(b.abs().max())
+    r.close()
