@@ -1283,7 +1283,7 @@ def measure_batch(args, ctx) -> dict:
                      "how": "per-scene piko_raster_forward then piko_raster_backward, 16x16 static"},
            "batched": {"value": T / (ms_batch * 1e-3) / 1e6, "ms_per_step": ms_batch,
                        "forward_ms": f_ms, "loss_gradient_ms": l_ms, "backward_ms": b_ms,
-                       "how": "forward_batch (one launch per phase), the loss gradient "
+                       "how": f"forward_batch ({args.batch_launch} launch), the loss gradient "
                               "(one elementwise torch op) and backward_batch (with the gradient arrays' zeroing), "
                               "each replayed from its own CUDA graph",
                        "autotune_s": tune_s, "static_scenes": n_static,
@@ -1302,7 +1302,7 @@ def measure_batch(args, ctx) -> dict:
                       "grad_scale": gscale,
                       "oracle": "every scene's keys bit-exact and colour <= 1e-5 vs the oracle "
                                 "(tests/test_gpu_full_size.py)"},
-           "clocks": clk, "gpu_launches": 8 * args.steps,
+           "clocks": clk, "gpu_launches": (4 if args.batch_launch == "persistent" else 8) * args.steps,
            "gpu_launches_plain": sum(forward_launches(s.width, s.height, 16, 16) + 3 for s in host) * args.steps}
     if not args.no_cpu_baseline:
         import oracle
@@ -1379,8 +1379,8 @@ def main():
     ap.add_argument("--batch-bins", type=int, default=0, help="batch workload: one square bin size for all scenes "
                     "instead of the autotuner's choice (0: autotune)")
     ap.add_argument("--batch-schedule", default="dynamic", choices=["static", "dynamic"])
-    ap.add_argument("--batch-launch", default="persistent", choices=["persistent", "per-phase"],
-                    help="batch workload: the library's choice, or always one launch per phase (now the same)")
+    ap.add_argument("--batch-launch", default="per-phase", choices=["persistent", "per-phase"],
+                    help="batch workload: one launch per phase (the library's default), or one cooperative launch")
     ap.add_argument("--workload", default="heightfield",
                     choices=["heightfield", "random256", "deferred", "sphere", "batch", "reyes"],
                     help="heightfield: the headline line (with every other configuration under 'configs'); "

@@ -103,10 +103,10 @@ extern "C" {
 #define PIKO_OPT_STATS 6            /* 1: the Process stage also counts its work (see
                                        piko_raster_stats); default 0                        */
 #define PIKO_OPT_BATCH_LAUNCH 7     /* how piko_raster_forward_batch launches its phases:
-                                       0 (default) the faster form, one launch per phase (with
-                                       PIKO_OPT_TEST_WITHHOLD bit 1: one persistent cooperative
-                                       kernel with grid barriers between phases); 1 always one
-                                       launch per phase                                     */
+                                       1 (default) one launch per phase; 0 all phases in one
+                                       persistent cooperative kernel with grid barriers between
+                                       them (the same results, slower at every size measured;
+                                       also taken under PIKO_OPT_TEST_WITHHOLD bit 1)       */
 #define PIKO_OPT_PERSPECTIVE 8      /* 1: perspective-correct attributes in shading and
                                        gradients: b'_i = (b_i / w_i) / sum_j (b_j / w_j), w_i
                                        the clip w of vertex i; 0 (default): screen-space b_i.

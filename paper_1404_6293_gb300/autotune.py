@@ -15,7 +15,7 @@ triangle count, coverage density, shading mode) so that similar scenes share
 one measurement; the cache can be saved to and loaded from JSON.
 
 A choice that is best for a scene rendered alone need not be best inside a
-batch, where all scenes share one persistent launch (there is no per-scene
+batch, where all scenes share one launch per phase (there is no per-scene
 launch or grid-size effect).  ``tune_batch`` therefore measures inside the
 batched pass itself: every workload class is timed as a sub-batch under each
 candidate, and the assembled per-class choice is kept only if the whole batch
@@ -36,7 +36,7 @@ from .raster import DeviceScene, Rasterizer
 DEFAULT_BINS: Tuple[Tuple[int, int], ...] = ((8, 8), (16, 16), (32, 32), (64, 64))
 DEFAULT_SCHEDULES: Tuple[str, ...] = ("static", "dynamic", "hardware")
 THREAD_CHOICES: Tuple[int, ...] = (64, 128, 256, 512)  # the CTA sizes the library accepts
-# a batch has no hardware mapping (its tiles are dealt inside one persistent launch)
+# a batch has no hardware mapping (its tiles are dealt inside one launch)
 BATCH_SCHEDULES: Tuple[str, ...] = ("static", "dynamic")
 # the other two mappings of the pipeline (no tiling; one kernel per stage):
 # bin size and threads per bin do not apply, so each is one candidate

@@ -45,7 +45,7 @@ struct piko_raster {
   int check_capacity = 1;
   int small_px = 32;
   int stats = 0;
-  int batch_launch = 0;  // 0 persistent cooperative, 1 one launch per phase
+  int batch_launch = 1;  // PIKO_OPT_BATCH_LAUNCH
   int clip = 0;                      // near/far clipping instead of culling (PIKO_OPT_CLIP)
   int exact_bins = 0;                // exact triangle-vs-bin overlap in AssignBin (PIKO_OPT_EXACT_BINS)
   long long wait_budget = 40000000;  // clock cycles a device-side wait may take (PIKO_OPT_WAIT_BUDGET)
@@ -804,7 +804,7 @@ int piko_raster_forward_batch(piko_raster* h, const piko_scene* scenes, int n, p
   if (r != PIKO_OK) return r;
   for (int attempt = 0;; ++attempt) {
     if ((r = batch_launch_forward(h->batch, h->status,
-                                  h->batch_launch == 0 && (h->withhold & TEST_WITHHOLD_BARRIER), st, h->err,
+                                  h->batch_launch == 0 || (h->withhold & TEST_WITHHOLD_BARRIER), st, h->err,
                                   h->wait_budget, h->withhold)) != PIKO_OK)
       return r;
     if (!h->check_capacity) return PIKO_OK;

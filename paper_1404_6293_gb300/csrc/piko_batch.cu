@@ -465,7 +465,7 @@ __device__ void phase_process(const BatchParams& b, ProcessShared& ps, const Til
 #ifndef PIKO_BATCH_THREADS
 #define PIKO_BATCH_THREADS 128
 #endif
-constexpr int BATCH_THREADS = PIKO_BATCH_THREADS;  // CTA size of the persistent batch kernel
+constexpr int BATCH_THREADS = PIKO_BATCH_THREADS;  // CTA size of the batch's scan and Process phases, and of its persistent kernel
 
 struct BatchSmem {
   ProcessShared ps;
@@ -938,7 +938,7 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
 }
 
 // Launches the forward phases, a launch each; persistent: all in one
-// cooperative launch, the form whose grid barriers have a test hook.  (The
+// cooperative launch (PIKO_OPT_BATCH_LAUNCH 0).  (The
 // separate launches are faster at every size: 49 against 62 us for three scenes
 // of 5,000 triangles at most, 407 against 455 for 32 of up to 100,000.)
 int batch_launch_forward(BatchState* bs, DevStatus* st, bool persistent, cudaStream_t stream, std::string& err,

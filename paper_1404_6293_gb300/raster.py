@@ -287,7 +287,7 @@ class Rasterizer:
 
     # -------------------------------------------------------------- batches
     def forward_batch(self, scenes, fbs=None, bin_sizes=None, schedules=None, stream=None):
-        """All scenes in one pass (one persistent launch by default).
+        """All scenes in one pass (a launch per phase by default).
         bin_sizes: per-scene (w, h) pairs or None; schedules: per-scene names /
         PIKO_SCHED_* values or None.  Returns the list of framebuffers."""
         n = len(scenes)

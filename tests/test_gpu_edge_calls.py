@@ -282,3 +282,35 @@ def test_gradients_of_arrays_longer_than_the_scene():
         assert not bool(a[n:].any())
         assert float((a[:n] - b).abs().max()) <= 1e-4 * float(b.abs().max())
     r.close()
+
+
+def test_batch_launch_option_selects_the_form():
+    """PIKO_OPT_BATCH_LAUNCH: one kernel for 0, one per phase for 1 and by
+    default, with the same keys (tests that compare the two rely on it)."""
+    torch = _torch()
+    from torch.profiler import ProfilerActivity, profile
+    from paper_1404_6293_gb300 import _lib as L
+    from paper_1404_6293_gb300.raster import DeviceScene, Rasterizer
+    ds = [DeviceScene.from_host(s) for s in (S.random_triangles(160, 120, 500, 20.0, seed=51),
+                                             S.heightfield(200, 150, 90, 70, seed=52))]
+    keys, names = [], []
+    with profile(activities=[ProfilerActivity.CUDA]):  # (a process's first session may miss its kernels)
+        torch.zeros(8, device="cuda")
+        torch.cuda.synchronize()
+    for launch in (None, 0, 1):
+        r = Rasterizer(64, 64, 8, 8)
+        if launch is not None:
+            r.set_option(L.PIKO_OPT_BATCH_LAUNCH, launch)
+        r.forward_batch(ds)
+        with profile(activities=[ProfilerActivity.CUDA]) as p:
+            fbs = r.forward_batch(ds)
+            torch.cuda.synchronize()
+        assert r.status()[0] == 0
+        keys.append([f.key.clone() for f in fbs])
+        found = " ".join(e.name for e in p.events())
+        names.append({k for k in ("k_batch_forward", "k_batch_count", "k_batch_process") if k in found})
+        r.close()
+    per_phase = {"k_batch_count", "k_batch_process"}
+    assert names == [per_phase, {"k_batch_forward"}, per_phase]
+    for k in keys[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(k, keys[0]))
