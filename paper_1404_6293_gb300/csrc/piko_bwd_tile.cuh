@@ -213,18 +213,18 @@ __device__ __forceinline__ void backward_warp_pixels(const BwdScene& sc, const f
       const int dx1 = p0.x - p2.x, dy1 = p0.y - p2.y, dx2 = p1.x - p0.x, dy2 = p1.y - p0.y;
       const int ux = 256 * x + 128 - p0.x, uy = 256 * y + 128 - p0.y;
       if (A == (long long)(int)A) {  // the covered pixel's edge functions lie in [0, A]: exact in 32 bits
-        const float rA = __frcp_rn((float)(int)A);
+        const float fA = (float)(int)A;
         const int w1 = (int)((unsigned)dx1 * (unsigned)uy - (unsigned)dy1 * (unsigned)ux);
         const int w2 = (int)((unsigned)dx2 * (unsigned)uy - (unsigned)dy2 * (unsigned)ux);
-        b[0] = (float)((int)A - w1 - w2) * rA;
-        b[1] = (float)w1 * rA;
-        b[2] = (float)w2 * rA;
+        b[0] = __fdiv_rn((float)((int)A - w1 - w2), fA);
+        b[1] = __fdiv_rn((float)w1, fA);
+        b[2] = __fdiv_rn((float)w2, fA);
       } else {
-        const float rA = __frcp_rn(f32_from_i64(A));
+        const float fA = f32_from_i64(A);
         const long long w1 = (long long)dx1 * uy - (long long)dy1 * ux, w2 = (long long)dx2 * uy - (long long)dy2 * ux;
-        b[0] = f32_from_i64(A - w1 - w2) * rA;
-        b[1] = f32_from_i64(w1) * rA;
-        b[2] = f32_from_i64(w2) * rA;
+        b[0] = __fdiv_rn(f32_from_i64(A - w1 - w2), fA);
+        b[1] = __fdiv_rn(f32_from_i64(w1), fA);
+        b[2] = __fdiv_rn(f32_from_i64(w2), fA);
       }
       if (PERSP)
         perspective_bary(b[0], b[1], b[2], __ldg(sc.invw + vid[0]), __ldg(sc.invw + vid[1]), __ldg(sc.invw + vid[2]));

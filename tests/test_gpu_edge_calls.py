@@ -314,3 +314,50 @@ def test_batch_launch_option_selects_the_form():
     assert names == [per_phase, {"k_batch_forward"}, per_phase]
     for k in keys[1:]:
         assert all(torch.equal(a, b) for a, b in zip(k, keys[0]))
+
+
+def _pixel_triangles(W, H, corners, order):
+    """A triangle per pixel of a W x H frame (powers of two), its corners at
+    offsets (1/256 pixel) from the pixel's centre, in the vertex array at
+    order[t] + (0, 1, 2)."""
+    y, x = np.divmod(np.arange(W * H), W)
+    c = np.stack([x + 0.5, y + 0.5], 1)[:, None, :] + np.asarray(corners, np.float64) / 256.0
+    pos = np.zeros((int(order[-1]) + 3, 4), np.float32)
+    tris = (order[:, None] + np.arange(3)).astype(np.int32)
+    pos[:, 3] = 1.0
+    pos[tris, 0] = c[..., 0] * (2.0 / W) - 1.0
+    pos[tris, 1] = 1.0 - c[..., 1] * (2.0 / H)
+    return pos, tris
+
+
+def test_gradient_weights_are_correctly_rounded():
+    """dL/dc of a vertex of a one-pixel Gouraud triangle under dL/drgb = 1 is the
+    pixel's weight: the correctly rounded quotient of its edge function and the
+    triangle's area."""
+    torch = _torch()
+    from paper_1404_6293_gb300.raster import DeviceScene, Rasterizer
+    W, H = 64, 32
+    T = W * H
+    rng = np.random.default_rng(6)
+    # around the centre, in three sectors, so that it is inside; all distinct
+    ang = np.array([0.3, 2.4, 4.5]) + rng.uniform(-0.4, 0.4, (T, 3))
+    rad = rng.uniform(40, 120, (T, 3))
+    off = np.rint(np.stack([rad * np.cos(ang), rad * np.sin(ang)], -1)).astype(np.int64)
+    pos, tris = _pixel_triangles(W, H, off, np.arange(0, 3 * T, 3))
+    s = S.Scene(W, H, pos, tris, color=np.ones((3 * T, 3), np.float32))
+    ds, r = DeviceScene.from_host(s), Rasterizer(W, H)
+    fb = r.forward(ds)
+    torch.cuda.synchronize()
+    assert np.array_equal(fb.key_numpy().ravel() & 0xFFFFFFFF, np.arange(T))
+    dc, _, _ = r.gradients(ds, fb, torch.ones((H, W, 4), device="cuda"), normal=False, light=False)
+
+    def cross(a, b):
+        return a[:, 0] * b[:, 1] - a[:, 1] * b[:, 0]
+
+    w = np.stack([cross(off[:, 1], off[:, 2]), cross(off[:, 2], off[:, 0]), cross(off[:, 0], off[:, 1])], 1)
+    A = w.sum(1, keepdims=True)
+    want = (w.astype(np.float64) / A).astype(np.float32)  # (both below 2^17: no double rounding)
+    got = dc.cpu().numpy().reshape(T, 3, 3)
+    for c in range(3):
+        assert np.array_equal(got[:, :, c], want)
+    r.close()
