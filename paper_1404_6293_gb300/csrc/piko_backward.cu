@@ -26,9 +26,12 @@ __global__ void __launch_bounds__(PIX_THREADS, 5) k_backward_pixel(const __grid_
 // Sums of all vertices into the gradient arrays (grad_finish_chunk).
 __global__ void __launch_bounds__(GRAD_CHUNK) k_backward_finish(const __grid_constant__ GradAcc f) {
   __shared__ GradFinishSmem sm;
+  cluster_arrive();
   pdl_wait();  // the accumulators
   const int chunks = (f.V + GRAD_CHUNK - 1) / GRAD_CHUNK;
-  for (int c = blockIdx.x; c < chunks; c += gridDim.x) grad_finish_chunk(f, c, sm);
+  double lacc = 0.0;
+  for (int c = blockIdx.x; c < chunks; c += gridDim.x) grad_finish_chunk(f, c, sm, lacc);
+  grad_add_light_cluster(&f, lacc, true);
 }
 
 }  // namespace piko
@@ -73,7 +76,12 @@ int piko_backward_launch(int W, int H, int mode, int unclamped, int T, int V, co
       launch_pdl(invw ? k_backward_pixel<true> : k_backward_pixel<false>, blocks, PIX_THREADS, 0, s, p);
   if (e != cudaSuccess) return 1;
   const int chunks = (V + GRAD_CHUNK - 1) / GRAD_CHUNK;
-  return launch_pdl(k_backward_finish, chunks < 8 * num_sms ? chunks : 8 * num_sms, GRAD_CHUNK, 0, s, f) == cudaSuccess
+  // all CTAs take as many chunks as the fullest: no fewer steps in a row, and fewer
+  // additions to the light gradient
+  const int steps = (chunks + 8 * num_sms - 1) / (8 * num_sms), ctas = (chunks + steps - 1) / steps;
+  const int cluster = chunks > 1024 ? FINISH_CLUSTER_MAX : FINISH_CLUSTER;
+  return launch_pdl_cluster(cluster, k_backward_finish, (ctas + cluster - 1) / cluster * cluster, GRAD_CHUNK, 0, s,
+                            f) == cudaSuccess
              ? 0
              : 1;
 }

@@ -618,14 +618,25 @@ __global__ void __launch_bounds__(PIX_THREADS, 4) k_batch_backward_pixel(BatchBw
 // Sums of all vertices into the gradient arrays, a chunk of one group per CTA step.
 __global__ void __launch_bounds__(GRAD_CHUNK) k_batch_finish(BatchBwdParams b) {
   __shared__ GradFinishSmem sm;
+  cluster_arrive();
   pdl_wait();  // the accumulators
-  const int per = (b.total_chunks + (int)gridDim.x - 1) / (int)gridDim.x, first = (int)blockIdx.x * per;
-  if (first >= b.total_chunks) return;
-  int g = find_scene(b.chunk_prefix, b.ngroups, first);
-  for (int i = first; i < min(first + per, b.total_chunks); ++i) {
-    while (__ldg(b.chunk_prefix + g + 1) <= i) ++g;
-    grad_finish_chunk(b.groups[g], i - __ldg(b.chunk_prefix + g), sm);
+  const int per = (b.total_chunks + (int)gridDim.x - 1) / (int)gridDim.x;
+  auto end_of = [&](int cta) { return min((cta + 1) * per, b.total_chunks); };  // one past a CTA's last chunk
+  const int first = (int)blockIdx.x * per, end = end_of(blockIdx.x);
+  const bool any = first < end;
+  int g = any ? find_scene(b.chunk_prefix, b.ngroups, first) : 0;
+  double lacc = 0.0;
+  for (int i = first; i < end; ++i) {
+    if (__ldg(b.chunk_prefix + g + 1) <= i) {  // (every group has a chunk)
+      grad_add_light(b.groups[g], lacc);
+      lacc = 0.0;
+      ++g;
+    }
+    grad_finish_chunk(b.groups[g], i - __ldg(b.chunk_prefix + g), sm, lacc);
   }
+  // whether the last group reaches back to the last chunk of the cluster's first CTA
+  const int head_end = end_of((int)blockIdx.x / FINISH_CLUSTER * FINISH_CLUSTER);
+  grad_add_light_cluster(any ? b.groups + g : nullptr, lacc, any && __ldg(b.chunk_prefix + g) < head_end);
 }
 
 }  // namespace piko
@@ -1125,7 +1136,8 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
     k_batch_backward_pixel<false><<<pblocks, PIX_THREADS, 0, stream>>>(p);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)
-    e = launch_pdl(k_batch_finish, chunk_blocks, GRAD_CHUNK, 0, stream, p);
+    e = launch_pdl_cluster(FINISH_CLUSTER, k_batch_finish, (chunk_blocks + FINISH_CLUSTER - 1) / FINISH_CLUSTER * FINISH_CLUSTER,
+                           GRAD_CHUNK, 0, stream, p);
   if (e != cudaSuccess) {
     bs->gacc_dirty = true;
     err = std::string("batch backward launch: ") + cudaGetErrorString(e);
