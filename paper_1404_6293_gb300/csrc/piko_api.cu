@@ -2,8 +2,10 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <string>
 
+#include "piko_bwd_tile.cuh"
 #include "piko_direct.cuh"
 #include "piko_internal.cuh"
 #include "piko_scan.cuh"
@@ -27,13 +29,22 @@ int piko_backward_launch(int W, int H, int mode, int unclamped, int T, int V, co
                          const float* vdot, const float4* vattr, const float* color, const float* normal,
                          const float* light,
                          const float* invw, const float* pos, const float* mvp, const unsigned long long* key,
-                         const float* dl_drgba, float4* acc, long long acc_room, float* dcolor, float* dnormal,
-                         float* dlight, int set, int num_sms, cudaStream_t s);
+                         const float* dl_drgba, float4* acc, long long acc_room, float* dcolor,
+                         float* dnormal, float* dlight, int set, int num_sms, cudaStream_t s);
+
+// Per-vertex arrays of a handle: bytes a vertex without the copies below.
+constexpr long long VERTEX_BYTES = sizeof(int4) + 2 * sizeof(float4) + 2 * sizeof(float);
 
 // Gradient accumulators of a handle beyond one per vertex: copies for scenes of
-// few vertices and many pixels, three at most (1 MB at most).  Not more, as an
-// allocation past a megabyte costs a first frame 75 us more than one below.
-inline long long gacc_extra(long long vertices) { return 3 * vertices < 65536 ? 3 * vertices : 65536; }
+// few vertices and many pixels (grad_copies), which take fewer than two per
+// GRAD_COPY_PX pixels.  Where they alone would take the block past a megabyte,
+// what fits below it or three copies: a first frame's allocation past a megabyte
+// costs it 75 us more than one below.
+inline long long gacc_extra(long long vertices, long long px) {
+  const long long all = std::min((GRAD_MAX_COPIES - 1) * vertices, 2 * px / GRAD_COPY_PX);
+  const long long room = ((1 << 20) - VERTEX_BYTES * vertices) / (long long)sizeof(float4);
+  return room < 0 ? all : std::min(all, std::max(room, 3 * vertices));
+}
 
 struct piko_raster {
   int W, H, bin_w, bin_h, schedule;
@@ -60,7 +71,8 @@ struct piko_raster {
   long long vcap = 0;
   int4* vtx = nullptr;      // snapped position
   float4* vattr = nullptr;  // colour and n . L, for Lambert with colours
-  float4* gacc = nullptr;   // gradient sums, zero between calls; gacc_extra(vcap) more of them for copies
+  float4* gacc = nullptr;   // gradient sums, zero between calls: gacc_room of them, for copies too
+  long long gacc_room = 0;
   float* vdot = nullptr;    // n . L, for Lambert without colours
   float* invw = nullptr;    // 1 / clip w, with perspective-correct attributes
   bool gacc_dirty = false;  // gacc is not zero: new, or a backward launch failed
@@ -156,7 +168,6 @@ int grow_vertices(piko_raster* h, long long need) {
   char* block = static_cast<char*>(h->vertex_block);
   long long cap = 0;
   h->vcap = 0;
-  const long long per_vertex = sizeof(int4) + 2 * sizeof(float4) + 2 * sizeof(float);
   // a quarter more than needed, so that slowly growing scenes do not allocate each time
   cap = (need + need / 4 + 255) / 256 * 256;
   long long bytes = 0;
@@ -167,7 +178,8 @@ int grow_vertices(piko_raster* h, long long need) {
     cudaFree(block);
     block = nullptr;
   }
-  bytes = cap * per_vertex + gacc_extra(cap) * (long long)sizeof(float4);
+  const long long extra = gacc_extra(cap, (long long)h->W * h->H);
+  bytes = cap * VERTEX_BYTES + extra * (long long)sizeof(float4);
   if (cudaMalloc(reinterpret_cast<void**>(&block), (size_t)bytes) != cudaSuccess) {
     cudaGetLastError();
     return fail(h, PIKO_ERR_OOM, "cudaMalloc of vertex buffer failed");
@@ -176,7 +188,8 @@ int grow_vertices(piko_raster* h, long long need) {
   h->vtx = reinterpret_cast<int4*>(block);
   h->vattr = reinterpret_cast<float4*>(h->vtx + cap);
   h->gacc = h->vattr + cap;
-  h->vdot = reinterpret_cast<float*>(h->gacc + cap + gacc_extra(cap));
+  h->gacc_room = cap + extra;
+  h->vdot = reinterpret_cast<float*>(h->gacc + h->gacc_room);
   h->invw = h->vdot + cap;
   h->gacc_dirty = true;
   h->vcap = cap;
@@ -887,7 +900,7 @@ static int backward_pass(piko_raster* h, const piko_scene* s, const piko_framebu
     if (e != cudaSuccess) return cuda_fail(h, e, "gradient clear");
   }
   if (h->gacc_dirty) {
-    const cudaError_t e = cudaMemsetAsync(h->gacc, 0, (size_t)(h->vcap + gacc_extra(h->vcap)) * sizeof(float4), st);
+    const cudaError_t e = cudaMemsetAsync(h->gacc, 0, (size_t)h->gacc_room * sizeof(float4), st);
     if (e != cudaSuccess) return cuda_fail(h, e, "gradient sums");
     // a captured clear has not run
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -902,7 +915,7 @@ static int backward_pass(piko_raster* h, const piko_scene* s, const piko_framebu
   if (piko_backward_launch(h->W, h->H, s->shade_mode, h->unclamped, s->num_triangles, s->num_vertices, s->tris,
                            h->vtx, h->vdot, vattr, s->color, s->normal, s->light_dir, invw, h->clip ? s->pos : nullptr,
                            s->mvp, reinterpret_cast<const unsigned long long*>(fwd->key), dl_drgba, h->gacc,
-                           h->vcap + gacc_extra(h->vcap), dl_dcolor, dl_dnormal, dl_dlight, set ? 1 : 0, h->num_sms, st) != 0) {
+                           h->gacc_room, dl_dcolor, dl_dnormal, dl_dlight, set ? 1 : 0, h->num_sms, st) != 0) {
     h->gacc_dirty = true;
     return cuda_fail(h, cudaGetLastError(), "backward launch");
   }

@@ -23,14 +23,19 @@ __global__ void __launch_bounds__(PIX_THREADS, 5) k_backward_pixel(const __grid_
                               tx + ty);
 }
 
-// Sums of all vertices into the gradient arrays (grad_finish_chunk).
-__global__ void __launch_bounds__(GRAD_CHUNK) k_backward_finish(const __grid_constant__ GradAcc f) {
+// Sums of all vertices into the gradient arrays (grad_finish_chunk).  Copies come
+// with few vertices, where the time is that of a chain of loads: eight at a time
+// there (16 copies of 3,721 vertices: 6.2 us, 10.7 two at a time), and few enough
+// registers for every warp of the SM without copies.
+template <bool COPIES>
+__global__ void __launch_bounds__(GRAD_CHUNK, COPIES ? 4 : 8)
+    k_backward_finish(const __grid_constant__ GradAcc f) {
   __shared__ GradFinishSmem sm;
   cluster_arrive();
   pdl_wait();  // the accumulators
   const int chunks = (f.V + GRAD_CHUNK - 1) / GRAD_CHUNK;
   double lacc = 0.0;
-  for (int c = blockIdx.x; c < chunks; c += gridDim.x) grad_finish_chunk(f, c, sm, lacc);
+  for (int c = blockIdx.x; c < chunks; c += gridDim.x) grad_finish_chunk<COPIES ? 8 : 1>(f, c, sm, lacc);
   grad_add_light_cluster(&f, lacc, true);
 }
 
@@ -51,7 +56,7 @@ int piko_backward_launch(int W, int H, int mode, int unclamped, int T, int V, co
   const bool lambert = mode == PIKO_SHADE_LAMBERT;
   GradAcc f;
   f.V = V; f.acc = acc; f.set = set;
-  f.copies = grad_copies((long long)W * H, V, acc_room);
+  f.copies = grad_copies((long long)W * H, V, acc_room, GRAD_COPY_PX, GRAD_MAX_COPIES);
   f.normal = lambert ? normal : nullptr;
   f.light = light;
   f.color = nullptr;
@@ -80,8 +85,8 @@ int piko_backward_launch(int W, int H, int mode, int unclamped, int T, int V, co
   // additions to the light gradient
   const int steps = (chunks + 8 * num_sms - 1) / (8 * num_sms), ctas = (chunks + steps - 1) / steps;
   const int cluster = chunks > 1024 ? FINISH_CLUSTER_MAX : FINISH_CLUSTER;
-  return launch_pdl_cluster(cluster, k_backward_finish, (ctas + cluster - 1) / cluster * cluster, GRAD_CHUNK, 0, s,
-                            f) == cudaSuccess
+  return launch_pdl_cluster(cluster, f.copies > 1 ? k_backward_finish<true> : k_backward_finish<false>,
+                            (ctas + cluster - 1) / cluster * cluster, GRAD_CHUNK, 0, s, f) == cudaSuccess
              ? 0
              : 1;
 }

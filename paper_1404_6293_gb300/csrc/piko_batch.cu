@@ -12,6 +12,7 @@
 //
 // Every wait (grid barrier, scan look-back) is bounded by a clock budget;
 // on expiry PIKO_ERR_TIMEOUT is recorded and every later phase is skipped.
+#include <algorithm>
 #include <cstddef>
 #include <cstring>
 #include <string>
@@ -616,7 +617,7 @@ __global__ void __launch_bounds__(PIX_THREADS, 4) k_batch_backward_pixel(BatchBw
 }
 
 // Sums of all vertices into the gradient arrays, a chunk of one group per CTA step.
-__global__ void __launch_bounds__(GRAD_CHUNK) k_batch_finish(BatchBwdParams b) {
+__global__ void __launch_bounds__(GRAD_CHUNK, 8) k_batch_finish(BatchBwdParams b) {
   __shared__ GradFinishSmem sm;
   cluster_arrive();
   pdl_wait();  // the accumulators
@@ -632,7 +633,7 @@ __global__ void __launch_bounds__(GRAD_CHUNK) k_batch_finish(BatchBwdParams b) {
       lacc = 0.0;
       ++g;
     }
-    grad_finish_chunk(b.groups[g], i - __ldg(b.chunk_prefix + g), sm, lacc);
+    grad_finish_chunk<4>(b.groups[g], i - __ldg(b.chunk_prefix + g), sm, lacc);
   }
   // whether the last group reaches back to the last chunk of the cluster's first CTA
   const int head_end = end_of((int)blockIdx.x / FINISH_CLUSTER * FINISH_CLUSTER);
@@ -657,8 +658,9 @@ int ilog2i(int v) {
 
 }  // namespace
 
-// Gradient accumulators beyond one per vertex (16 MB): copies for scenes of few
-// vertices and many pixels (grad_copies).
+// Gradient accumulators beyond one per vertex, 16 MB of them at most: copies for
+// scenes of few vertices and many pixels (grad_copies), which take fewer than one
+// per BATCH_COPY_PX pixels.
 constexpr long long BATCH_GACC_EXTRA = 1 << 20;
 
 // Everything the batch keeps between calls; owned by the handle.
@@ -766,7 +768,7 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   if (n < 1 || !scenes || !fbs) { err = "batch needs n >= 1 scenes and framebuffers"; return PIKO_ERR_INVALID_ARG; }
   std::vector<BatchScene> d(n);
   std::vector<int> pv(n + 1), pt(n + 1), pb(n + 1), ps(n + 1), pd(n + 1), pq(n + 1);
-  long long tv = 0, tt = 0, tb = 0, tsd = 0, tdy = 0, tq = 0, tk = 0;
+  long long tv = 0, tt = 0, tb = 0, tsd = 0, tdy = 0, tq = 0, tk = 0, px_total = 0;
   int max_bin_px = 64;
   for (int i = 0; i < n; ++i) {
     const piko_scene& s = scenes[i];
@@ -794,6 +796,7 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
     x.vtx_base = (int)tv; x.tri_base = (int)tt; x.bin_base = (int)tb;
     // key indices are 32-bit; scenes past that, or without the memory below, bin every triangle
     const long long px = (long long)s.width * s.height;
+    px_total += px;
     if (direct_scene(x.T, x.V, s.width, s.height) && tk + px < (1LL << 32)) {
       x.direct = 1;
       x.key_base = (unsigned)tk;
@@ -827,8 +830,9 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
   if ((r = grow_dev(&bs->rect, &bs->tcap, tt, false, err)) != PIKO_OK) return r;
   if ((r = grow_dev(&bs->marks, &bs->mcap, (tt + 31) / 32, false, err)) != PIKO_OK) return r;
   // here and not in the backward call, which may be recorded into a graph
-  if (tv + BATCH_GACC_EXTRA > bs->gcap) bs->gacc_dirty = true;
-  if ((r = grow_dev(&bs->gacc, &bs->gcap, tv + BATCH_GACC_EXTRA, false, err)) != PIKO_OK) return r;
+  const long long copies = std::min(std::min(px_total / BATCH_COPY_PX, (BATCH_MAX_COPIES - 1) * tv), BATCH_GACC_EXTRA);
+  if (tv + copies > bs->gcap) bs->gacc_dirty = true;
+  if ((r = grow_dev(&bs->gacc, &bs->gcap, tv + copies, false, err)) != PIKO_OK) return r;
   if (tb > bs->bcap) {
     // counts must start at zero; offsets/cursors/chunk states are rewritten
     cudaFree(bs->cnt); cudaFree(bs->bin_off); cudaFree(bs->cursor); cudaFree(bs->chunk_state);
@@ -1081,7 +1085,7 @@ int batch_launch_backward(BatchState* bs, const piko_scene* scenes, int n, const
   for (const GradAcc& g : groups) spare -= g.V;
   for (size_t k = 0; k < groups.size(); ++k) {
     GradAcc& g = groups[k];
-    g.copies = grad_copies(group_px[k], g.V, g.V + spare);
+    g.copies = grad_copies(group_px[k], g.V, g.V + spare, BATCH_COPY_PX, BATCH_MAX_COPIES);
     g.acc = bs->gacc + used;
     used += (long long)g.copies * g.V;
     spare -= (long long)(g.copies - 1) * g.V;

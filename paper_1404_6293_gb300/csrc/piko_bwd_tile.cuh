@@ -89,13 +89,21 @@ struct GradAcc {
 // into one float; with several copies the rounding error falls with their
 // number, as does the queue at one address of the L2.  px: pixels of the
 // group's framebuffers; room: accumulators that may be used.
-constexpr int GRAD_MAX_COPIES = 8;
+//
+// A copy per GRAD_COPY_PX pixels a vertex makes a single scene's sums as exact as
+// sums over tiles of 16 x 16 pixels (relative error of dL/dcolour at 46 pixels a
+// vertex: 1.2e-7, with a copy per 64 pixels 1.7e-7, by tiles 1.4e-7; at 1,180
+// pixels a vertex 1.9, 2.7 and 2.4e-7).  Batches are there with a copy per 64
+// (1.9e-7 against 2.0e-7 by tiles on 12 uneven scenes); with one per 16, up to 32,
+// their finishing pass took 163 us instead of 89 (64 scenes).
+constexpr int GRAD_MAX_COPIES = 16, GRAD_COPY_PX = 8;
+constexpr int BATCH_MAX_COPIES = 8, BATCH_COPY_PX = 64;
 // (A soup's vertices belong to one triangle each and take few sums: with copies
 // by the pixels per triangle a batch of 64 uneven scenes took 1684 us, by the
 // pixels per vertex, or without, 1624.)
-inline int grad_copies(long long px, long long V, long long room) {
+inline int grad_copies(long long px, long long V, long long room, int per_px, int most) {
   int k = 1;
-  while (k < GRAD_MAX_COPIES && px >= 64 * k * V && 2 * k * V <= room) k *= 2;
+  while (k < most && px >= per_px * k * V && 2 * k * V <= room) k *= 2;
   return k;
 }
 
@@ -111,17 +119,37 @@ struct GradFinishSmem {
 // gradient arrays (three floats a vertex) are added to in whole sectors.
 // Atomic, as several calls on different streams may share the arrays.
 // lacc: the light gradient's component tid of the CTA's chunks (threads 0 to 2).
+// FLIGHT: copies loaded at a time (1: there is only one).
+template <int FLIGHT>
 __device__ __forceinline__ void grad_finish_chunk(const GradAcc& f, int chunk, GradFinishSmem& sm, double& lacc) {
   const int tid = threadIdx.x, lane = tid & 31, base = chunk * GRAD_CHUNK, v = base + tid;
   float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
   bool hit = false;
-  for (int k = 0; k < f.copies && v < f.V; ++k) {
-    float4* at = f.acc + (size_t)k * f.V + v;
-    const float4 c = __ldcg(at);
-    if (c.x == 0.f && c.y == 0.f && c.z == 0.f && c.w == 0.f) continue;
+  auto take = [&](float4* at, const float4& c) {
+    if (c.x == 0.f && c.y == 0.f && c.z == 0.f && c.w == 0.f) return;
     hit = true;
     *at = make_float4(0.f, 0.f, 0.f, 0.f);
     a.x += c.x; a.y += c.y; a.z += c.z; a.w += c.w;
+  };
+  if (v < f.V) {
+    float4* at = f.acc + v;
+    if (FLIGHT == 1 || f.copies == 1) {
+      take(at, __ldcg(at));
+    } else if (f.copies < FLIGHT) {  // (a power of two)
+      for (int k = 0; k < f.copies; k += 2, at += 2 * (size_t)f.V) {
+        const float4 c0 = __ldcg(at), c1 = __ldcg(at + f.V);
+        take(at, c0);
+        take(at + f.V, c1);
+      }
+    } else {
+      for (int k0 = 0; k0 < f.copies; k0 += FLIGHT, at += FLIGHT * (size_t)f.V) {
+        float4 c[FLIGHT];
+#pragma unroll
+        for (int k = 0; k < FLIGHT; ++k) c[k] = __ldcg(at + (size_t)k * f.V);
+#pragma unroll
+        for (int k = 0; k < FLIGHT; ++k) take(at + (size_t)k * f.V, c[k]);
+      }
+    }
   }
   if (!__syncthreads_or(hit) && !f.set) return;  // (the barrier also ends the last chunk's reads of sm)
   sm.a[tid] = a;

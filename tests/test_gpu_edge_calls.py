@@ -427,3 +427,32 @@ def test_batch_light_gradient_of_groups_that_share_ctas():
             assert np.array_equal(dc[s.tris][:, :, 0], np.tile(np.float32([0.25, 0.25, 0.5]), (T, 1)))
             assert dc.sum(dtype=np.float64) == T
     r.close()
+
+
+def test_colour_sums_of_a_vertex_of_many_pixels():
+    """A vertex that takes the same sum r from each of 8,192 rows (one column of a
+    triangle whose weight is constant along it): 8,192 r to within one rounding
+    (half of 2^-24 on average) for each of 512 additions to one of 16 copies and of
+    the 16 that join them.  2,048 additions to a copy are off by 1.9e-5 to 2.2e-5."""
+    torch = _torch()
+    from paper_1404_6293_gb300.raster import DeviceScene, Rasterizer
+    W, H = 32, 8192
+    px = np.array([(-20000.0, 4096.0), (100.0, -5000.0), (100.0, 13192.0)])
+    pos = np.tile(np.float32([0, 0, 0, 1]), (300, 1))  # (the other vertices are unused)
+    pos[:3, 0], pos[:3, 1] = px[:, 0] * (2.0 / W) - 1.0, 1.0 - px[:, 1] * (2.0 / H)
+    s = S.Scene(W, H, pos, np.array([[0, 1, 2]], np.int32), color=np.ones((300, 3), np.float32))
+    ds, r = DeviceScene.from_host(s), Rasterizer(W, H)
+    fb = r.forward(ds)
+    torch.cuda.synchronize()
+    assert bool((fb.key != EMPTY).all())
+
+    def sum_of(rows, x):
+        g = torch.zeros((H, W, 4), device="cuda")
+        g[:rows, x, 0] = 1.0
+        return float(r.gradients(ds, fb, g, normal=False, light=False)[0][0, 0])
+
+    for x in (3, 9, 15, 21):
+        one = sum_of(1, x)
+        assert abs(one - (99.5 - x) / 20100.0) <= 1e-6
+        assert abs(sum_of(H, x) - H * one) <= 528 * 2.0 ** -25 * H * one
+    r.close()
