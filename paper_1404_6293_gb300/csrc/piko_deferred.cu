@@ -99,9 +99,18 @@ __device__ __forceinline__ float light_pairs(const LightPair* lights, int npairs
   return a0 + a1;
 }
 
-// The same sum for any lights, one by one (and for the last of an odd number:
-// half a pair padded with a light of intensity 0 would add 0 * inf = NaN where a
-// binary16 normal is infinite).
+// The term of one ordinary light, the first of a record: the last of an odd number.
+// (A pair padded with a light of intensity 0 would add 0 * inf = NaN where a
+// binary16 normal is infinite.)
+__device__ __forceinline__ float light_last(const float* s, float4 n, float sx, float sy, float sz, float inv_r2) {
+  const float dx = s[0] - sx, dy = s[2] - sy, dz = s[4] - sz;
+  const float d2 = dx * dx + dy * dy + dz * dz;
+  const float nd = n.x * dx + n.y * dy + n.z * dz;
+  const float t = __fmaf_rn(d2, inv_r2, 1.0f);
+  return s[6] * fmaxf(nd, 0.f) * rsqrt_normal(fmaxf(d2 * t * t, 1.17549435e-38f));
+}
+
+// The same sum for any lights, one by one.
 __device__ __forceinline__ float light_singles(const float4* __restrict__ lights, int n_lights, float4 n, float sx,
                                                float sy, float sz, float inv_r2) {
   float acc = 0.f;
@@ -125,7 +134,7 @@ __global__ void __launch_bounds__(256) k_deferred_light(int W, int H, const unsi
   const float D = (float)max(W, H);
   const int npairs = n_lights / 2;
   bool odd_light = false;
-  for (int i = threadIdx.x; i < 2 * npairs; i += blockDim.x) {
+  for (int i = threadIdx.x; i < n_lights; i += blockDim.x) {
     const float4 p = lights[i];
     odd_light |= !ordinary_light(p, D);
     float* s = slights + 8 * (i >> 1) + (i & 1);
@@ -148,9 +157,12 @@ __global__ void __launch_bounds__(256) k_deferred_light(int W, int H, const unsi
   const float sx = (float)x + 0.5f, sy = (float)y + 0.5f;
   const float sz = (float)(unsigned)(k >> 32) * zscale;
   float acc = 0.f;
-  if (!singles) acc = light_pairs(reinterpret_cast<const LightPair*>(slights), npairs, n, sx, sy, sz, inv_r2);
-  const int paired = singles ? 0 : 2 * npairs;
-  if (paired < n_lights) acc += light_singles(lights + paired, n_lights - paired, n, sx, sy, sz, inv_r2);
+  if (singles) {
+    acc = light_singles(lights, n_lights, n, sx, sy, sz, inv_r2);
+  } else {
+    if (n_lights & 1) acc = light_last(slights + 8 * npairs, n, sx, sy, sz, inv_r2);
+    acc += light_pairs(reinterpret_cast<const LightPair*>(slights), npairs, n, sx, sy, sz, inv_r2);
+  }
   rgba[i] = make_float4(a.x * acc, a.y * acc, a.z * acc, 1.0f);
 }
 
@@ -159,7 +171,7 @@ void launch_deferred_light(int W, int H, const unsigned long long* key, const ui
   (void)num_sms;
   const long long npix = (long long)W * H;
   const int blocks = (int)((npix + 255) / 256);
-  k_deferred_light<<<blocks, 256, (size_t)(n_lights / 2) * sizeof(LightPair), s>>>(W, H, key, gnorm, galb, lights,
+  k_deferred_light<<<blocks, 256, (size_t)((n_lights + 1) / 2) * sizeof(LightPair), s>>>(W, H, key, gnorm, galb, lights,
                                                                                          n_lights, rgba);
 }
 
