@@ -827,35 +827,23 @@ __device__ __forceinline__ void process_tile(const TileScene& p, int tile, unsig
       __syncthreads();
     }
   }
-  // shade, write, and leave the key tile cleared for the next tile; the
-  // indices of a thread's next winner are loaded before it shades one
-  auto take = [&](int i) {
-    unsigned long long k = KEY_EMPTY;
-    if (i < bin_px) {
-      k = skey[i];
-      skey[i] = KEY_EMPTY;
-    }
-    return k;
-  };
-  unsigned long long k = take(tid);
-  int3 id = make_int3(0, 0, 0), idn = id;
-  if (k != KEY_EMPTY) id = tri_indices(p.tris, (unsigned)k);
+  // shade, write, and leave the key tile cleared for the next tile.  (Loading the
+  // indices of a thread's next winner ahead took 1 to 2% longer: 94.7 against 92.6 us
+  // for a 1920x1080 mesh of 115,200 triangles at 16 x 16, 149 against 147 for a
+  // power-law G-buffer of 290,000.)
   for (int i = tid; i < bin_px; i += nt) {
-    const unsigned long long kn = take(i + nt);
-    if (kn != KEY_EMPTY) idn = tri_indices(p.tris, (unsigned)kn);
+    const unsigned long long k = skey[i];
+    skey[i] = KEY_EMPTY;
     const int x = x0 + (i & (bin_w - 1)), y = y0 + (i >> p.g.bshift_x);
-    if (x <= x1 && y <= y1) {
-      const size_t o = (size_t)y * p.g.W + x;
-      p.key_out[o] = k;
-      if (k == KEY_EMPTY) {
-        write_empty(p, o);
-      } else {
-        if (STATS) ++st.shaded;
-        shade_winner<PERSP, CLIP>(p, id, x, y, o);
-      }
+    if (x > x1 || y > y1) continue;
+    const size_t o = (size_t)y * p.g.W + x;
+    p.key_out[o] = k;
+    if (k == KEY_EMPTY) {
+      write_empty(p, o);
+    } else {
+      if (STATS) ++st.shaded;
+      shade_winner<PERSP, CLIP>(p, tri_indices(p.tris, (unsigned)k), x, y, o);
     }
-    k = kn;
-    id = idn;
   }
   __syncthreads();
 }
