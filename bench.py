@@ -499,10 +499,9 @@ def size_and_count(r, ds, fb):
 
 def small_triangle_frame(scene) -> bool:
     """Whether the library rasterizes the scene's small triangles in the count
-    pass and shades tiles without bin entries in the scatter launch
-    (direct_scene in csrc/piko_direct.cuh)."""
-    V, T = scene.num_vertices, scene.num_triangles
-    return V > 0 and (16 if V < 2 * T else 4) * T >= scene.width * scene.height
+    pass and shades tiles without bin entries in the scatter launch."""
+    from paper_1404_6293_gb300 import _lib as L
+    return bool(L.load().piko_raster_direct_scene(scene.width, scene.height, scene.num_triangles, scene.num_vertices))
 
 
 def process_stage_ms(scene, stage_ms) -> float:

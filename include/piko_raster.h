@@ -298,6 +298,12 @@ int piko_raster_backward_batch(piko_raster *h, const piko_scene *scenes, int n, 
 int piko_raster_reserve(piko_raster *h, int64_t max_vertices, int64_t max_triangles,
                         int64_t max_bin_entries);
 
+/* 1 if piko_raster_forward with default options rasterizes the small triangles of
+ * a scene of these counts and this framebuffer size in the count pass and shades
+ * tiles without bin entries in the scatter launch, 0 if it bins every triangle
+ * (for tools that attribute the time of the stages; the output is the same). */
+int piko_raster_direct_scene(int width, int height, int64_t num_triangles, int64_t num_vertices);
+
 /* Sets a PIKO_OPT_* option.  Returns PIKO_ERR_INVALID_ARG for unknown keys
  * or values. */
 int piko_raster_set_option(piko_raster *h, int key, int value);

@@ -82,6 +82,7 @@ def _declare(lib):
     lib.piko_raster_backward_set.argtypes = lib.piko_raster_backward.argtypes
     lib.piko_raster_deferred_light.argtypes = [P, C.POINTER(PikoFramebuffer), P, i32, P, P]
     lib.piko_raster_reserve.argtypes = [P, i64, i64, i64]
+    lib.piko_raster_direct_scene.argtypes = [i32, i32, i64, i64]
     lib.piko_raster_set_option.argtypes = [P, i32, i32]
     lib.piko_raster_status.argtypes = [P, C.POINTER(C.c_int64)]
     lib.piko_raster_last_error.argtypes = [P]
@@ -91,7 +92,7 @@ def _declare(lib):
     lib.piko_raster_stats.argtypes = [P, C.POINTER(C.c_int64)]
     for name in ("piko_raster_forward", "piko_raster_forward_host", "piko_raster_backward",
                  "piko_raster_backward_set", "piko_raster_deferred_light",
-                 "piko_raster_reserve", "piko_raster_set_option", "piko_raster_status",
+                 "piko_raster_reserve", "piko_raster_direct_scene", "piko_raster_set_option", "piko_raster_status",
                  "piko_raster_version", "piko_raster_set_stage_events", "piko_raster_stats"):
         getattr(lib, name).restype = i32
     lib.piko_raster_forward_batch.argtypes = [P, C.POINTER(PikoScene), i32, C.POINTER(PikoFramebuffer), P, P, P]

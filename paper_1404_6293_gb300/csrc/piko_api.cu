@@ -320,7 +320,7 @@ static bool allocate_direct_keys(piko_raster* h) {
 // while the stream is being captured).
 static unsigned long long* direct_keys(piko_raster* h, int T, int V, cudaStream_t st) {
   if (h->stats || h->exact_bins || h->small_px < 1 || h->schedule > PIKO_SCHED_HARDWARE ||
-      !direct_scene(T, V, h->W, h->H))
+      !direct_scene(T, V, (long long)h->W * h->H, false))
     return nullptr;
   if (!h->dkeys) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -405,9 +405,13 @@ int piko_raster_reserve(piko_raster* h, int64_t max_vertices, int64_t max_triang
   if ((r = grow(h, &h->bin_tris, &h->ecap, max_bin_entries, "bin lists")) != PIKO_OK) return r;
   // keys of direct rasterization, if any scene within the sizes can take it
   // (else, or without the memory, every triangle is binned)
-  if (direct_scene_within(max_triangles, max_vertices, h->W, h->H)) allocate_direct_keys(h);
+  if (direct_scene_within(max_triangles, max_vertices, (long long)h->W * h->H)) allocate_direct_keys(h);
   cudaError_t e = cudaDeviceSynchronize();
   return e == cudaSuccess ? PIKO_OK : cuda_fail(h, e, "reserve");
+}
+
+int piko_raster_direct_scene(int width, int height, int64_t num_triangles, int64_t num_vertices) {
+  return direct_scene(num_triangles, num_vertices, (long long)width * height, false) ? 1 : 0;
 }
 
 int piko_raster_status(piko_raster* h, int64_t* needed_bin_entries) {

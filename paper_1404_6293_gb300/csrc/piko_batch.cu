@@ -797,7 +797,7 @@ int batch_prepare(BatchState*& bs, int num_sms, const piko_scene* scenes, int n,
     // key indices are 32-bit; scenes past that, or without the memory below, bin every triangle
     const long long px = (long long)s.width * s.height;
     px_total += px;
-    if (direct_scene(x.T, x.V, s.width, s.height) && tk + px < (1LL << 32)) {
+    if (direct_scene(x.T, x.V, px, true) && tk + px < (1LL << 32)) {
       x.direct = 1;
       x.key_base = (unsigned)tk;
       tk += px;

@@ -33,21 +33,41 @@ __device__ __forceinline__ void clear_keys(unsigned long long* keys, size_t n) {
   if ((n & 1) && first == 0) keys[n - 1] = KEY_EMPTY;
 }
 
-// Scenes worth it: triangles small on average, fewer than 16 pixels of the
-// framebuffer for each in a mesh, whose triangles share vertices and are of
-// similar size, and fewer than 4 in a soup of separate triangles, where large
-// ones among them leave every tile with both kinds to merge and a pixel's
-// vertices are shared with none of its neighbours'.  (Terrain at 7 pixels a
-// triangle: 41 us with the line at 16, 49 at 4; a power-law soup at 4.1 pixels
-// a triangle: 265 and 250 us.)
-inline bool direct_scene(long long T, long long V, int W, int H) {
-  return V > 0 && (V < 2 * T ? 16 : 4) * T >= (long long)W * H;
+// Scenes worth it: triangles small on average, at most this many pixels of the
+// framebuffer for each.  The lines lie where the route stops paying against binning
+// every triangle (us on the direct route / binned, Lambert mesh at 16 x 16 bins):
+//   1920x1080   9 pixels a triangle 57 / 81, 10 67 / 84, 11 84 / 87, 12 98 / 90
+//   1280x720    9 41 / 46, 10 42 / 47, 11 53 / 49
+//   900x600     7 36 / 39, 9 41 / 41, 10 50 / 42
+//   640x400     6 25 / 27, 7 25 / 27, 8 35 / 27
+//   320x240     4 21 / 23, 5 (sphere) 27 / 24, 7 31 / 23
+// as beyond them most tiles hold triangles of both kinds and both routes' launches
+// have work; small frames are bound by these launches.  Soups of separate triangles
+// share no vertices, and their sizes differ more (power law / equal sizes of three
+// times the framebuffer in all, direct / binned):
+//   1920x1080   2.5 290 / 311 and 219 / 231, 3 270 / 270 and 215 / 219, 3.5 252 / 229 and 213 / 198
+//   560x420     2.5 62 / 67 and 53 / 58, 3 63 / 62 and 55 / 55, 3.5 59 / 56 and 55 / 52
+//   320x240     1.5 49 / 50 and 35 / 39, 2 46 / 44 and 39 / 35, 3 47 / 43 and 41 / 35
+// (Soups of one-pixel triangles that cover a quarter of the framebuffer would gain up
+// to 4 pixels a triangle and beyond, 63 / 89 at 3.9, but counts do not tell them.)
+// In a batch the launches are shared and all tiles are one launch's: meshes pay up to
+// 10 pixels a triangle (16 heightfields of 600x600: 9 197 / 221, 11 235 / 234) and soups
+// to 4 in frames of any size (three of 300x300: 3.9 42 / 49 and 62 / 62; 64 uneven
+// scenes 1,663 with the line at 4 and 1,677 at 3).
+inline bool direct_scene(long long T, long long V, long long px, bool batch) {
+  const bool mesh = V < 2 * T;
+  int line;
+  if (batch) line = mesh ? 10 : 4;
+  else if (px < 1 << 17) line = mesh ? 4 : 2;
+  else if (px < 3 << 18) line = mesh ? 7 : 3;
+  else line = mesh ? 10 : 3;
+  return V > 0 && line * T >= px;
 }
 
 // Whether some scene of at most max_t triangles and max_v vertices is one: a
 // mesh, which takes fewer triangles than a soup, of as many as there may be.
-inline bool direct_scene_within(long long max_t, long long max_v, int W, int H) {
-  return max_v > 0 && max_t > 0 && direct_scene(max_t, 1, W, H);
+inline bool direct_scene_within(long long max_t, long long max_v, long long px) {
+  return max_v > 0 && max_t > 0 && direct_scene(max_t, 1, px, false);
 }
 
 // A triangle of at most 128 pixels a side (its snapped extents below 2^15, so

@@ -456,3 +456,30 @@ def test_colour_sums_of_a_vertex_of_many_pixels():
         assert abs(one - (99.5 - x) / 20100.0) <= 1e-6
         assert abs(sum_of(H, x) - H * one) <= 528 * 2.0 ** -25 * H * one
     r.close()
+
+
+@pytest.mark.parametrize("size,bins", [((131, 137), 8), ((150, 70), 64), ((700, 300), 16), ((1200, 700), 32)])
+def test_boxes_at_the_limits_on_the_direct_route(size, bins):
+    """Boxes of 31 to 33 samples and 128 pixels, as many as the direct route asks
+    for in small, medium and large frames."""
+    from test_gpu_direct_raster import _LIMITS, _check, _triangles
+    from paper_1404_6293_gb300 import _lib as L
+    W, H = size
+    copies = -(-W * H // (2 * len(_LIMITS))) + 1
+    s = _triangles(W, H, _LIMITS, 5 * bins + W, copies)
+    assert L.load().piko_raster_direct_scene(W, H, s.num_triangles, s.num_vertices) == 1
+    _check(s, bins, "dynamic").close()
+
+
+def test_meshes_on_both_sides_of_the_direct_lines():
+    """Heightfields one step of tessellation apart around each line."""
+    from test_gpu_direct_raster import _check
+    from paper_1404_6293_gb300 import _lib as L
+    for W, H, line in ((301, 211, 4), (640, 400, 7), (1100, 800, 10)):
+        taken = []
+        for px in (line * 0.9, line * 1.1):
+            q = int((W * H / px / 2) ** 0.5)
+            s = S.heightfield(W, H, q, q, seed=q, with_color=True)
+            taken.append(L.load().piko_raster_direct_scene(W, H, s.num_triangles, s.num_vertices))
+            _check(s, 16, "static").close()
+        assert taken == [1, 0]
