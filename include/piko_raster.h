@@ -60,7 +60,10 @@ extern "C" {
 #define PIKO_SCHED_STATIC 0   /* DirectMap: persistent CTA c takes tiles c, c+G, c+2G, ...   */
 #define PIKO_SCHED_DYNAMIC 1  /* LoadBalance: persistent CTAs pop tiles from an atomic queue */
 #define PIKO_SCHED_HARDWARE 2 /* one CTA per tile, balanced by the hardware block scheduler
-                                 (the schedule elimination of Sec. 5.2.2)                   */
+                                 (the schedule elimination of Sec. 5.2.2).  In frames whose
+                                 small triangles never reach a tile (piko_raster_direct_scene)
+                                 the few tiles that are left are dealt from the queue, as
+                                 with DYNAMIC                                               */
 /* Two other mappings of the same pipeline, for the design-space comparison of
  * Sec. 7.2 (same keys and colours; bin size and threads per tile unused):   */
 #define PIKO_SCHED_FUSED 3    /* full fusion without tiling (the FreePipe-style point of
@@ -197,8 +200,8 @@ void piko_raster_destroy(piko_raster *h);
  * scene->width/height must equal the handle's.  Writes every pixel of
  * fb->key and of fb->rgba (if not NULL; zero where empty) or, in GBUFFER
  * mode, of fb->gbuf_normal and fb->gbuf_albedo.  Asynchronous unless
- * PIKO_OPT_CHECK_CAPACITY is 1 (the default), which adds one host sync
- * after the scan.  Returns PIKO_ERR_INVALID_ARG for bad sizes, NULL
+ * PIKO_OPT_CHECK_CAPACITY is 1 (the default): then the call waits until the
+ * scan has reported, while the later kernels run.  Returns PIKO_ERR_INVALID_ARG for bad sizes, NULL
  * required pointers, misaligned pos/tris, or a shade mode without the
  * attributes it needs.  The stages after the vertex stage are launched with
  * programmatic dependent launch: each may start while the one before it

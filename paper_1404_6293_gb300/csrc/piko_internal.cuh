@@ -196,13 +196,6 @@ __device__ __forceinline__ float f32_from_i64(long long v) {
   return v < 0 ? -f : f;
 }
 
-// Edge function of a pixel centre P for edge (a -> b): (Xb - Xa)(Py - Ya) -
-// (Yb - Ya)(Px - Xa).  The wrapping 32-bit form is exact whenever the true
-// value lies in [-2^31, 2^31), e.g. for a pixel the triangle covers when its
-// doubled area A is below 2^31 (then the value lies in [0, A]).
-__device__ __forceinline__ int edge_fn_wrap32(int Xa, int Ya, int Xb, int Yb, int Px, int Py) {
-  return (int)((unsigned)(Xb - Xa) * (unsigned)(Py - Ya) - (unsigned)(Yb - Ya) * (unsigned)(Px - Xa));
-}
 
 // floor(n / A) for A > 0 and |n / A| < 2^25, exact.  The float estimate
 // (relative error below 2^-21) is within a few units of the quotient; the
